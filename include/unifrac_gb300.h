@@ -83,9 +83,13 @@ typedef enum {
  * point (value * 2^F, F chosen per call from an upper bound of the sums, so
  * that one grid step is about 1e-18 of a tree's root-to-tip distance) and
  * end with one FP64 num / den division.
- * UF_FP64   branch embeddings and per-branch updates in IEEE FP64 on CUDA
- *           cores, partial sums in FP64 before each fixed-point rounding;
- *           every numerator is a sum of nonnegative terms (no cancellation).
+ * UF_FP64   branch embeddings in IEEE FP64.  Weighted and unweighted methods:
+ *           each embedded value rounded once to a 64-bit fixed-point grid
+ *           (about 2^-60 of a root-to-tip distance), every per-branch update
+ *           and sum after that in exact integers.  Generalized and
+ *           variance-adjusted: per-branch updates in FP64 on CUDA cores,
+ *           partial sums in FP64 before each fixed-point rounding, every
+ *           numerator a sum of nonnegative terms (no cancellation).
  *           Distances d within 1e-10 * |d| + 1e-15 of an FP64 per-pair
  *           evaluation: relative 1e-10 down to d = 1e-5, and the grid's
  *           absolute rounding below that (near-identical samples).

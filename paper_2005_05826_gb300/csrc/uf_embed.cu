@@ -6,6 +6,8 @@
 // embedding row of a branch is then f(count[k] / total[k]) for every sample
 // k, written over a padded width so that the stripe kernel can read the
 // partner column k + d without a modulo.
+#include <type_traits>
+
 #include "uf_device.cuh"
 #include "uf_embed.h"
 
@@ -165,7 +167,7 @@ __global__ void k_emb_rows(int64_t b0, const int32_t *__restrict__ nodes,
                            const double *__restrict__ counts, int64_t ld,
                            const double *__restrict__ length, const double *__restrict__ total,
                            const float *__restrict__ inv_total_f, T *__restrict__ X, int64_t pitch,
-                           const TabDesc *__restrict__ tabs, int n_tabs) {
+                           const TabDesc *__restrict__ tabs, int n_tabs, double row_scale) {
   const int64_t v = nodes ? (int64_t)nodes[blockIdx.x] : b0 + blockIdx.x;
   const double *c = counts + (int64_t)slot_of_node[v] * ld;
   const double l = length[v];
@@ -175,7 +177,9 @@ __global__ void k_emb_rows(int64_t b0, const int32_t *__restrict__ nodes,
     int64_t k = j - tb.x_col;
     while (k >= tb.n) k -= tb.n;
     k += tb.off;
-    x[j] = emb_value<T, KIND>(c[k], l, total[k], inv_total_f[k]);
+    if constexpr (std::is_same_v<T, unsigned long long>)
+      x[j] = __double2ull_rn(emb_value<double, KIND>(c[k], l, total[k], 0.f) * row_scale);
+    else x[j] = emb_value<T, KIND>(c[k], l, total[k], inv_total_f[k]);
   }
 }
 
@@ -251,7 +255,7 @@ cudaError_t launch_emb_rows(int kind, bool fp32, int64_t b0, int rows,
                             const int32_t *slot_of_node, const double *counts, int64_t ld,
                             const double *length, const double *total, const float *inv_total_f,
                             void *X, int64_t pitch, const TabDesc *tabs, int n_tabs, cudaStream_t st,
-                            const int32_t *nodes) {
+                            const int32_t *nodes, double row_scale) {
   if (rows <= 0) return cudaSuccess;
   if (kind == EMB_VAW) {
     if (!nodes) return cudaErrorInvalidValue;
@@ -263,14 +267,14 @@ cudaError_t launch_emb_rows(int kind, bool fp32, int64_t b0, int rows,
   }
 #define UF_EMB(T, K)                                                                                 \
   return launch_k(k_emb_rows<T, K>, dim3(rows), dim3(256), 0, st, b0, nodes, slot_of_node, counts, ld, length, \
-                  total, inv_total_f, (T *)X, pitch, tabs, n_tabs)
+                  total, inv_total_f, (T *)X, pitch, tabs, n_tabs, row_scale)
   if (fp32) {
     if (kind == EMB_SCALED) UF_EMB(float, EMB_SCALED);
     if (kind == EMB_PRESENCE) UF_EMB(float, EMB_PRESENCE);
     UF_EMB(float, EMB_PROP);
   }
-  if (kind == EMB_SCALED) UF_EMB(double, EMB_SCALED);
-  if (kind == EMB_PRESENCE) UF_EMB(double, EMB_PRESENCE);
+  if (kind == EMB_SCALED) UF_EMB(unsigned long long, EMB_SCALED);
+  if (kind == EMB_PRESENCE) UF_EMB(unsigned long long, EMB_PRESENCE);
   UF_EMB(double, EMB_PROP);
 #undef UF_EMB
 }

@@ -349,7 +349,7 @@ namespace {
 //   variance-adjusted (den, N): den <= w_max (D_k + D_j), with the weight
 //                             1 / sqrt(m_v (m - m_v)) <= w_max = max(1, 1 / c_min)
 //                             (both factors are sums of counts >= c_min, or 0)
-double accum_bound(uf_tree *tree, uf_table *table, int kind) {
+double accum_bound_of(uf_tree *tree, uf_table *table, int kind) {
   if (kind == EMB_SCALED) return tree->max_tip_dist;
   if (kind == EMB_VAW) return 2.0 * tree->max_tip_dist * std::max(1.0, 1.0 / table->min_count);
   double pres;
@@ -412,12 +412,30 @@ uf_status check_args(const uf_tree *tree, const uf_table *table, uf_method metho
 }  // namespace
 
 namespace ufg {
+double accum_bound(const uf_tree *tree, const uf_table *table, int kind) {
+  return accum_bound_of(const_cast<uf_tree *>(tree), const_cast<uf_table *>(table), kind);
+}
+
 // Fixed-point scale 2^F of the accumulators: 2 * bound * 2^F <= 2^61.
 double accum_scale(const uf_tree *tree, const uf_table *table, int kind) {
-  const double B = accum_bound(const_cast<uf_tree *>(tree), const_cast<uf_table *>(table), kind);
+  const double B = accum_bound(tree, table, kind);
   int F = 100;
   if (B > 0.0 && std::isfinite(B)) F = std::min(100, std::max(0, 60 - (int)std::ceil(std::log2(B))));
   return std::ldexp(1.0, F);
+}
+
+int fixed_row_shift(double scale, double bound, const double *len, int64_t n, int chunk) {
+  double most = 0.0;
+  for (int64_t i = 0; i < n; i += chunk) {
+    double x = 0.0;
+    for (int64_t j = i; j < std::min<int64_t>(n, i + chunk); j++) x += len[j];
+    most = std::max(most, x);
+  }
+  // the margin covers the rounding of each value, of the sums here and of the bound
+  const double room = std::ldexp(1.0, 63) * (1.0 - 1.0 / 1024), use = std::min(bound, most) * scale;
+  int e = 0;
+  while (e < 32 && std::ldexp(use, e + 1) <= room) e++;
+  return e;
 }
 }  // namespace ufg
 

@@ -66,16 +66,17 @@ struct TabDesc {
 // A stripe s whose bit (s mod 8) is set in the call's abs mask holds
 // A = sum |x_k - x_j| (abs form) instead of M = sum min(x_k, x_j) (min form).
 // FP32: stripes 1, 3, 5, 7 of every 8, so that the ALU and FMA pipes share
-// the load (see uf_stripe.cu).  FP64: every stripe, so that no numerator is
-// formed by cancellation (D_k + D_j - 2M) and its error stays relative to
-// the distance itself, however close the two samples are.
+// the load (see uf_stripe.cu).  FP64: every stripe; its rows are 64-bit fixed
+// point and a cell holds 2 R, R = sum max(x_j - x_k, 0), so that
+// A = 2 R + D_k - D_j in exact integers (k_stripe_u64; FinalArgs::relu).
 constexpr unsigned FP32_ABS_ROW_MASK = 0xAAu;
 constexpr unsigned FP64_ABS_ROW_MASK = 0xFFu;
 __host__ __device__ constexpr unsigned abs_row_mask(bool fp32) { return fp32 ? FP32_ABS_ROW_MASK : FP64_ABS_ROW_MASK; }
 __host__ __device__ constexpr bool abs_row(unsigned mask, int64_t s) { return (mask >> (s & 7)) & 1u; }
 
 struct StripeArgs {
-  const void *X;        // [rows][pitch] float or double, one segment per table
+  const void *X;        // [rows][pitch] float, double or (FP64 ACC_MIN) 64-bit fixed point,
+                        // one segment per table
   const double *len;    // per-row branch length (generalized only), [rows]
   int rows;             // branches in this launch
   int64_t pitch;        // elements per row (all segments)
@@ -95,6 +96,9 @@ struct StripeArgs {
   // this many elements after its first word (M and M2 cells; Dg); the FP32
   // kernels keep one word
   int64_t m_lo_off, d_lo_off;
+  // FP64 ACC_MIN: the rows of X are x * 2^(F + x_shift), 0 <= x_shift <= 32,
+  // with every column's sum over a work unit's rows below 2^63
+  int x_shift;
   // FP32 min kernel: 0xFF runs every stripe in the abs form (methods whose
   // numerator must not come from a difference of sums); anything else the
   // default FP32_ABS_ROW_MASK
@@ -109,9 +113,10 @@ int stripe_shapes(int acc, bool fp32, unsigned abs_mask);
 // default rows per work unit
 int stripe_chunk_rows();
 cudaError_t launch_stripe_acc(int acc, bool fp32, const StripeArgs &a, cudaStream_t st);
-// D[k] += sum of the launch's rows at column k (ACC_MIN only), with the
-// stripe kernel's operation order; scratch holds diag_scratch_bytes() (valid
-// for every chunk size the StripeArgs may carry)
+// D[k] += sum of the launch's rows at column k (ACC_MIN only): FP32 with the
+// stripe kernel's operation order, in scratch of diag_scratch_bytes() (valid
+// for every chunk size the StripeArgs may carry); FP64 rows are integers,
+// summed in any order
 size_t diag_scratch_bytes(bool fp32, int rows, int n_cols);
 cudaError_t launch_diag(bool fp32, const StripeArgs &a, void *scratch, cudaStream_t st);
 
@@ -139,8 +144,15 @@ bool table_host_view(const ::uf_table *t, TableView *v);
 }  // namespace ufg
 
 namespace ufg {
-// Fixed-point scale 2^F for the accumulators of an embedding kind (uf_host.cpp).
+// Upper bound of every accumulated value of an embedding kind, and the
+// fixed-point scale 2^F it gives (uf_host.cpp).
+double accum_bound(const ::uf_tree *tree, const ::uf_table *table, int kind);
 double accum_scale(const ::uf_tree *tree, const ::uf_table *table, int kind);
+// Largest StripeArgs::x_shift for FP64 ACC_MIN rows: the sum of any column
+// over the rows of one work unit is at most the accumulator's bound and at
+// most the unit's summed branch lengths (n lengths len[], units of `chunk`
+// rows from len[0] on), and stays below 2^63 on the rows' grid.
+int fixed_row_shift(double scale, double bound, const double *len, int64_t n, int chunk);
 // Set the calling thread's uf_last_error() text and return st (uf_host.cpp).
 uf_status set_last_error(uf_status st, const char *msg);
 // UF_OK when p is device (or managed) memory usable on the current device;

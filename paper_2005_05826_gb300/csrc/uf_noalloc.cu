@@ -31,6 +31,7 @@
 // race on the area; the call waits for its own work before returning, so
 // calls from one thread in sequence are safe.
 #include <algorithm>
+#include <cmath>
 #include <cstdio>
 #include <cstring>
 #include <exception>
@@ -241,6 +242,11 @@ uf_status compute_noalloc(const uf_tree *tree, const uf_table *table, uf_method 
   if (p[14]) UF_TRY(cudaMemsetAsync(p[14], 0, (size_t)S * n * 8 * words, st));
   if (p[15]) UF_TRY(cudaMemsetAsync(p[15], 0, (size_t)n * 8 * words, st));
 
+  // FP64 min kernel: 64-bit fixed-point rows (StripeArgs::x_shift)
+  const bool fixed_rows = !fp32 && acc == ACC_MIN;
+  const int x_shift =
+      fixed_rows ? fixed_row_shift(scale, accum_bound(tree, table, kind), tv.length, nb, stripe_chunk_rows()) : 0;
+
   const int32_t *d_lists = (const int32_t *)p[5], *d_slot = (const int32_t *)p[4];
   double *d_counts = (double *)p[11];
   if (rows > 0) {
@@ -252,7 +258,7 @@ uf_status compute_noalloc(const uf_tree *tree, const uf_table *table, uf_method 
                                 (const int32_t *)p[2], (const int32_t *)p[3], d_slot, d_counts, n, st));
     UF_TRY(launch_emb_rows(kind, fp32, 0, rows, d_slot, d_counts, n, (const double *)p[0],
                            (const double *)p[9], (const float *)p[10], p[12], pitch,
-                           (const TabDesc *)p[18], 1, st));
+                           (const TabDesc *)p[18], 1, st, nullptr, fixed_rows ? std::ldexp(scale, x_shift) : 0.0));
     StripeArgs sa{};
     sa.X = p[12];
     sa.len = (const double *)p[0];
@@ -271,6 +277,7 @@ uf_status compute_noalloc(const uf_tree *tree, const uf_table *table, uf_method 
     sa.counter = (int *)p[17];
     sa.m_lo_off = fp32 ? 0 : (int64_t)S * n;
     sa.d_lo_off = fp32 ? 0 : n;
+    sa.x_shift = x_shift;
     UF_TRY(launch_stripe_acc(acc, fp32, sa, st));
     if (acc == ACC_MIN) UF_TRY(launch_diag(fp32, sa, p[16], st));
   }
@@ -281,6 +288,7 @@ uf_status compute_noalloc(const uf_tree *tree, const uf_table *table, uf_method 
   fa.s1 = S;
   fa.full = 1;
   fa.abs_mask = acc == ACC_MIN ? abs_row_mask(fp32) : 0u;
+  fa.relu = fixed_rows;
   fa.gen_abs = acc == ACC_GEN && !fp32;
   fa.M = (const unsigned long long *)p[13];
   fa.M2 = (const unsigned long long *)p[14];

@@ -1120,7 +1120,9 @@ uf_status run_stripes(uf_tree *tree, const BatchJob &J, int device, uf_method me
   const auto key = tune_key(acc, (fp32 ? (amask == 0xFFu ? 2 : 1) : 0) + 4 * (forced + 1), n_tiles, xrows);
   int chunk = stripe_chunk_rows(), shape = forced > 0 ? forced : 0;
   bool tune = false;
-  if (g_autotune.load() && !split.dense.empty()) {
+  // (the FP64 min kernel's sums are exact for any chunk: not tuned)
+  const bool fixed_rows = !fp32 && acc == ACC_MIN;
+  if (g_autotune.load() && !split.dense.empty() && !fixed_rows) {
     std::lock_guard<std::mutex> g(g_tune_mu);
     auto it = g_tuned_chunk.find(key);
     if (it != g_tuned_chunk.end()) {
@@ -1137,6 +1139,15 @@ uf_status run_stripes(uf_tree *tree, const BatchJob &J, int device, uf_method me
     n_tiles = shape_tiles[sh];
   };
   use_shape(shape);
+  int x_shift = 0;  // grid of the FP64 min kernel's rows (StripeArgs::x_shift)
+  if (fixed_rows) {
+    double bound = 0.0;
+    for (const TableJob &t : J.tabs) bound = std::max(bound, accum_bound(tree, t.table, kind));
+    x_shift = 32;
+    for (size_t b = 0; b + 1 < split.dense_ptr.size(); b++)
+      x_shift = std::min(x_shift, fixed_row_shift(scale, bound, split.dense_len.data() + split.dense_ptr[b],
+                                                  split.dense_ptr[b + 1] - split.dense_ptr[b], chunk));
+  }
   // the launch sequence goes into a CUDA graph unless it is timed per phase
   Capture cap(g_graph.load() != 0 && !timer.on && !tune, st, device);
   const cudaStream_t ls = cap.stream();
@@ -1175,7 +1186,7 @@ uf_status run_stripes(uf_tree *tree, const BatchJob &J, int device, uf_method me
     if (nd > 0) {
       ck(launch_emb_rows(kind, fp32, b0, (int)nd, in.pd->slot_of_node, counts.as<double>(), ld,
                          in.td->length, total.as<double>(), inv_total.as<float>(), X.p, pitch,
-                         d_tabs, (int)nt, ls, d_dense + d0),
+                         d_tabs, (int)nt, ls, d_dense + d0, fixed_rows ? std::ldexp(scale, x_shift) : 0.0),
          "embedding rows");
       kernels++;
     }
@@ -1201,6 +1212,7 @@ uf_status run_stripes(uf_tree *tree, const BatchJob &J, int device, uf_method me
     sa.m_lo_off = fp32 ? 0 : cells;
     sa.d_lo_off = fp32 ? 0 : n_cols;
     sa.abs_mask = amask;
+    sa.x_shift = x_shift;
     if (tune && !tuned) {
       std::vector<const TabDesc *> tp;
       for (size_t o : o_shape_tabs) tp.push_back(meta.at<TabDesc>(o));
@@ -1230,7 +1242,7 @@ uf_status run_stripes(uf_tree *tree, const BatchJob &J, int device, uf_method me
       timer.begin(2);
       ck(launch_diag(fp32, sa, diag_tmp.p, ls), "diagonal accumulate");
       timer.end();
-      kernels += 2;
+      kernels += fp32 ? 2 : 1;
     }
   }
   if (split.n_sparse > 0 && !side.ev_fork) {  // not launched beside a dense block
@@ -1249,6 +1261,7 @@ uf_status run_stripes(uf_tree *tree, const BatchJob &J, int device, uf_method me
     fa.s1 = J.tabs[t].stop;
     fa.full = J.tabs[t].start == 0 && J.tabs[t].stop == tabs[t].n / 2;
     fa.abs_mask = amask;
+    fa.relu = fixed_rows;
     fa.gen_abs = acc == ACC_VAW || (acc == ACC_GEN && !fp32);
     fa.clamps = clamps.as<unsigned long long>();
     fa.M = M.as<unsigned long long>() + tabs[t].m_off;

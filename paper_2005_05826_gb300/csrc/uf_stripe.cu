@@ -14,10 +14,11 @@
 // one abs-form update is half an FSUB2 plus one FADD (FMA pipe).  The FP32
 // kernel gives stripes 1, 3, 5 and 7 of every 8 the abs form so the two pipes
 // share the load (odd micro-tile rows read their partner pairs at even,
-// register-pair aligned offsets).  The FP64 kernel uses the abs form on every
-// stripe: its numerators are then sums of nonnegative terms, never a
-// difference of two nearly equal sums, so their error stays relative to the
-// distance however close two samples are.  Generalized UniFrac keeps two
+// register-pair aligned offsets).  The FP64 path's rows are 64-bit fixed
+// point, and its kernel (k_stripe_u64) adds R = sum max(x_j - x_k, 0) in
+// integers, A = 2 R + D_k - D_j: GB300 has 2 FP64 lanes per clock per SM but
+// 64 integer ones, and integer sums are exact, so the only rounding is that
+// of a row's value to the grid, and no difference of two sums cancels.  Generalized UniFrac keeps two
 // accumulators, den = sum l s^a and, FP32, Q = sum l min(u, v) s^(a-1) with
 // num = den - 2Q or, FP64, N = sum l |u - v| s^(a-1) = num.
 //
@@ -31,7 +32,8 @@
 // updates an RD x RK register micro-tile.  Shared rows are XOR-swizzled in
 // 16-byte units so the per-thread 16-byte reads are free of bank conflicts.
 //
-// Precision.  Register partials over B1 = 64 branches are summed into a
+// Precision (the kernels on FP32 and FP64 rows).  Register partials over
+// B1 = 64 branches are summed into a
 // second level kept in shared memory in the path's own precision (FP32 for
 // the paper's fp32 mode, Sec. 4, FP64 otherwise); at the end of the unit that
 // level is scaled by 2^F and rounded once to an int64 fixed-point value (FP64:
@@ -216,14 +218,14 @@ __device__ __forceinline__ void commit_cells(unsigned long long *M, const Mid *m
   }
 }
 
-// ---- weighted / unweighted ----
+// ---- weighted / unweighted, FP32 ----
 // rows i of the micro-tile with bit i of ABSM clear: M += min(x_k, x_j);
 // with it set: A += |x_k - x_j|
-template <typename T, int RD, int RK, unsigned ABSM, int MINB>
+template <int RD, int RK, unsigned ABSM, int MINB>
 __global__ void __launch_bounds__(NT, MINB) k_stripe_min(const StripeArgs a) {
+  using T = float;
   using G = Geo<T, RD, RK, 1>;
   using Mid = typename G::Mid;
-  constexpr bool F32 = sizeof(T) == 4;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T *stg = reinterpret_cast<T *>(smem_raw);
   Mid *mid = reinterpret_cast<Mid *>(smem_raw + (size_t)G::NSTAGE * G::STAGE * sizeof(T));
@@ -274,34 +276,24 @@ __global__ void __launch_bounds__(NT, MINB) k_stripe_min(const StripeArgs a) {
         for (int q = 0; q < G::NV; q++)
           *reinterpret_cast<uint4 *>(&v[q * G::VEC]) =
               *reinterpret_cast<const uint4 *>(vrow + swz<T>(w0 + q * G::VEC));
-        if constexpr (F32) {
 #pragma unroll
-          for (int i = 0; i < RD; i++)
+        for (int i = 0; i < RD; i++)
 #pragma unroll
-            for (int j = 0; j < RK; j += 2) {
-              if (!((ABSM >> i) & 1u)) {  // two mins, one paired add
-                float2 a2 = make_float2(acc[i][j], acc[i][j + 1]);
-                const float2 m2 = make_float2(fminf(u[j], v[i + j + 1]), fminf(u[j + 1], v[i + j + 2]));
-                a2 = __fadd2_rn(a2, m2);
-                acc[i][j] = a2.x;
-                acc[i][j + 1] = a2.y;
-              } else {  // one paired difference, one paired add of absolute values
-                const float2 d2 = fsub2(make_float2(u[j], u[j + 1]), make_float2(v[i + j + 1], v[i + j + 2]));
-                float2 a2 = make_float2(acc[i][j], acc[i][j + 1]);
-                a2 = __fadd2_rn(a2, make_float2(fabsf(d2.x), fabsf(d2.y)));
-                acc[i][j] = a2.x;
-                acc[i][j + 1] = a2.y;
-              }
+          for (int j = 0; j < RK; j += 2) {
+            if (!((ABSM >> i) & 1u)) {  // two mins, one paired add
+              float2 a2 = make_float2(acc[i][j], acc[i][j + 1]);
+              const float2 m2 = make_float2(fminf(u[j], v[i + j + 1]), fminf(u[j + 1], v[i + j + 2]));
+              a2 = __fadd2_rn(a2, m2);
+              acc[i][j] = a2.x;
+              acc[i][j + 1] = a2.y;
+            } else {  // one paired difference, one paired add of absolute values
+              const float2 d2 = fsub2(make_float2(u[j], u[j + 1]), make_float2(v[i + j + 1], v[i + j + 2]));
+              float2 a2 = make_float2(acc[i][j], acc[i][j + 1]);
+              a2 = __fadd2_rn(a2, make_float2(fabsf(d2.x), fabsf(d2.y)));
+              acc[i][j] = a2.x;
+              acc[i][j + 1] = a2.y;
             }
-        } else {
-#pragma unroll
-          for (int i = 0; i < RD; i++)
-#pragma unroll
-            for (int j = 0; j < RK; j++) {
-              if ((ABSM >> i) & 1u) acc[i][j] += fabs(u[j] - v[i + j + 1]);
-              else acc[i][j] += tmin<T>(u[j], v[i + j + 1]);
-            }
-        }
+          }
       }
       in_sub += G::RB;
       if (in_sub == B1 || it == nst - 1) {
@@ -317,6 +309,95 @@ __global__ void __launch_bounds__(NT, MINB) k_stripe_min(const StripeArgs a) {
     }
     cp_async_wait<0>();
     commit_cells<T, RD, RK>(a.M, mid, a, U, U.s0 + RD * ts, U.k0 + RK * tk);
+  }
+}
+
+// ---- weighted / unweighted, FP64: 64-bit fixed-point rows ----
+// c += max(v - u, 0) for u, v < 2^63: a 64-bit difference, a test of its sign
+// and a predicated 64-bit add, 5 integer instructions.
+__device__ __forceinline__ void add_relu(unsigned long long &c, unsigned long long u, unsigned long long v) {
+  asm("{\n .reg .pred p;\n .reg .u32 u0, u1, v0, v1, c0, c1, d0, d1;\n"
+      " mov.b64 {u0, u1}, %1;\n mov.b64 {v0, v1}, %2;\n mov.b64 {c0, c1}, %0;\n"
+      " sub.cc.u32 d0, v0, u0;\n subc.u32 d1, v1, u1;\n setp.ge.s32 p, d1, 0;\n"
+      " @p add.cc.u32 c0, c0, d0;\n @p addc.u32 c1, c1, d1;\n mov.b64 %0, {c0, c1};\n}\n"
+      : "+l"(c)
+      : "l"(u), "l"(v));
+}
+
+// Integer pipe bound: 5 instructions per update at 64 lanes per clock per SM
+// is 12.8 updates per clock; in a loop over resident rows this form reaches
+// 14.7 (some of the adds issue elsewhere), the 64-bit min 12.6, the FP64 form
+// |u - v| 0.8.  The sums stay in registers for the whole unit (they are exact,
+// so there is no second level) and go to the two-word accumulators at its end.
+template <int RD, int RK, int MINB>
+__global__ void __launch_bounds__(NT, MINB) k_stripe_u64(const StripeArgs a) {
+  using T = unsigned long long;
+  using G = Geo<T, RD, RK, 0>;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  T *stg = reinterpret_cast<T *>(smem_raw);
+  __shared__ int s_unit;
+  const int tk = threadIdx.x & 15, ts = threadIdx.x >> 4;
+  const int w0 = RK * tk + RD * ts;
+  Unit U;
+  while (next_unit(a, G::TS, G::TK, &s_unit, &U)) {
+    const int nst = (U.r1 - U.r0 + G::RB - 1) / G::RB;
+#pragma unroll
+    for (int p = 0; p < G::NSTAGE - 1; p++) {
+      if (p < nst) load_stage<T, RD, RK, 0, false>(stg + p * G::STAGE, a, U.r0 + p * G::RB, U.r1, U.x_col + U.k0,
+                                        U.x_col + U.k0 + U.s0);
+      cp_async_commit();
+    }
+    T acc[RD][RK];
+#pragma unroll
+    for (int i = 0; i < RD; i++)
+#pragma unroll
+      for (int j = 0; j < RK; j++) acc[i][j] = 0;
+    for (int it = 0; it < nst; it++) {
+      cp_async_wait<G::NSTAGE - 2>();
+      __syncthreads();
+      {
+        const int nx = it + G::NSTAGE - 1;
+        if (nx < nst)
+          load_stage<T, RD, RK, 0, false>(stg + (nx % G::NSTAGE) * G::STAGE, a, U.r0 + nx * G::RB, U.r1,
+                                          U.x_col + U.k0, U.x_col + U.k0 + U.s0);
+        cp_async_commit();
+      }
+      const T *stage = stg + (it % G::NSTAGE) * G::STAGE;
+#pragma unroll 2
+      for (int r = 0; r < G::RB; r++) {
+        const T *urow = stage + r * G::ROW;
+        const T *vrow = urow + G::UW;
+        T u[RK], v[G::NV * G::VEC];
+#pragma unroll
+        for (int q = 0; q < RK / G::VEC; q++)
+          *reinterpret_cast<uint4 *>(&u[q * G::VEC]) =
+              *reinterpret_cast<const uint4 *>(urow + swz<T>(RK * tk + q * G::VEC));
+#pragma unroll
+        for (int q = 0; q < G::NV; q++)
+          *reinterpret_cast<uint4 *>(&v[q * G::VEC]) =
+              *reinterpret_cast<const uint4 *>(vrow + swz<T>(w0 + q * G::VEC));
+#pragma unroll
+        for (int i = 0; i < RD; i++)
+#pragma unroll
+          for (int j = 0; j < RK; j++) add_relu(acc[i][j], u[j], v[i + j + 1]);
+      }
+    }
+    cp_async_wait<0>();
+    // 2 R as hi (units of 2^-F) and lo (2^-(F+32)) words
+    const unsigned long long mask = (1ull << a.x_shift) - 1ull;
+#pragma unroll
+    for (int i = 0; i < RD; i++) {
+      const int s = U.s0 + RD * ts + i;
+      if (s < U.s_lo || s > U.s_hi) continue;
+      unsigned long long *row = a.M + U.m_off + (int64_t)(s - U.s_lo) * U.n;
+#pragma unroll
+      for (int j = 0; j < RK; j++) {
+        const int k = U.k0 + RK * tk + j;
+        if (k >= U.n || acc[i][j] == 0) continue;
+        atomicAdd(row + k, (acc[i][j] >> a.x_shift) << 1);
+        atomicAdd(row + k + a.m_lo_off, (acc[i][j] & mask) << (33 - a.x_shift));
+      }
+    }
   }
 }
 
@@ -634,44 +715,62 @@ __device__ __forceinline__ int table_of_col(const TabDesc *tabs, int n_tabs, int
   return lo;
 }
 
-template <typename T>
-__global__ void k_diag_partial(const StripeArgs a, T *__restrict__ part) {
+__global__ void k_diag_partial(const StripeArgs a, float *__restrict__ part) {
   const int kg = blockIdx.x * blockDim.x + threadIdx.x;
   if (kg >= a.n_cols) return;
   const TabDesc &tb = a.tabs[a.n_tabs == 1 ? 0 : table_of_col(a.tabs, a.n_tabs, kg)];
   const int64_t k = tb.x_col + (kg - tb.off);  // the sample's column in its segment
   const int sb = blockIdx.y;
-  const T *X = (const T *)a.X;
+  const float *X = (const float *)a.X;
   const int per_chunk = (a.chunk + B1 - 1) / B1;
   const int c = sb / per_chunk;
   const int e0 = c * a.chunk + (sb - c * per_chunk) * B1;
   const int e1 = min(min(a.rows, (c + 1) * a.chunk), e0 + B1);
-  T acc = T(0);
+  float acc = 0.f;
   for (int e = e0; e < e1; e++) {
-    const T x = X[(int64_t)e * a.pitch + k];
-    acc += tmin<T>(x, x);
+    const float x = X[(int64_t)e * a.pitch + k];
+    acc += fminf(x, x);
   }
   part[(int64_t)sb * a.n_cols + kg] = acc;
 }
 
-// Phase 2: a chunk's sub-block partials summed in order in the path's
-// precision, then rounded to fixed point (the stripe kernels' second level).
-template <typename T>
-__global__ void k_diag_reduce(const StripeArgs a, const T *__restrict__ part, int n_sb) {
+// Phase 2: a chunk's sub-block partials summed in order in FP32, then rounded
+// to fixed point (the stripe kernels' second level).
+__global__ void k_diag_reduce(const StripeArgs a, const float *__restrict__ part, int n_sb) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= a.n_cols) return;
   const int per_chunk = (a.chunk + B1 - 1) / B1;
-  Fx2 d{0, 0};
-  T mid = T(0);
+  long long d = 0;
+  float mid = 0.f;
   for (int sb = 0; sb < n_sb; sb++) {
     mid += part[(int64_t)sb * a.n_cols + k];
     if ((sb + 1) % per_chunk == 0 || sb == n_sb - 1) {
-      d = fx_add(d, to_fixed2(mid, a.scale));
-      mid = T(0);
+      d += to_fixed(mid, a.scale);
+      mid = 0.f;
     }
   }
-  a.Dg[k] += (unsigned long long)d.hi;
-  if constexpr (sizeof(T) == 8) a.Dg[k + a.d_lo_off] += (unsigned long long)d.lo;
+  a.Dg[k] += (unsigned long long)d;
+}
+
+// FP64: the fixed-point rows' sums, each value split into its two words
+// (one thread per column and DIAG_ROWS rows, integers in any order).
+constexpr int DIAG_ROWS = 64;
+__global__ void k_diag_u64(const StripeArgs a) {
+  const int kg = blockIdx.x * blockDim.x + threadIdx.x;
+  if (kg >= a.n_cols) return;
+  const TabDesc &tb = a.tabs[a.n_tabs == 1 ? 0 : table_of_col(a.tabs, a.n_tabs, kg)];
+  const unsigned long long *X = (const unsigned long long *)a.X + tb.x_col + (kg - tb.off);
+  const int e0 = blockIdx.y * DIAG_ROWS, e1 = min(a.rows, e0 + DIAG_ROWS);
+  const unsigned long long mask = (1ull << a.x_shift) - 1ull;
+  unsigned long long hi = 0, lo = 0;  // lo < DIAG_ROWS * 2^32
+#pragma unroll 4
+  for (int e = e0; e < e1; e++) {
+    const unsigned long long x = X[(int64_t)e * a.pitch];
+    hi += x >> a.x_shift;
+    lo += (x & mask) << (32 - a.x_shift);
+  }
+  if (hi) atomicAdd(a.Dg + kg, hi);
+  if (lo) atomicAdd(a.Dg + kg + a.d_lo_off, lo);
 }
 
 template <typename K>
@@ -695,15 +794,26 @@ int units_of(const StripeArgs &a) {
   return n_chunks * a.n_tiles;
 }
 
-template <typename T, int RD, int RK, unsigned ABSM, int MINB>
+template <int RD, int RK, unsigned ABSM, int MINB>
 cudaError_t run_min(const StripeArgs &a, cudaStream_t st) {
-  using G = Geo<T, RD, RK, 1>;
+  using G = Geo<float, RD, RK, 1>;
   int grid = 0;
-  cudaError_t e = prepare(k_stripe_min<T, RD, RK, ABSM, MINB>, G::SMEM, &grid, units_of(a));
+  cudaError_t e = prepare(k_stripe_min<RD, RK, ABSM, MINB>, G::SMEM, &grid, units_of(a));
   if (e != cudaSuccess) return e;
   e = cudaMemsetAsync(a.counter, 0, sizeof(int), st);
   if (e != cudaSuccess) return e;
-  return launch_k(k_stripe_min<T, RD, RK, ABSM, MINB>, dim3(grid), dim3(NT), G::SMEM, st, a);
+  return launch_k(k_stripe_min<RD, RK, ABSM, MINB>, dim3(grid), dim3(NT), G::SMEM, st, a);
+}
+
+template <int RD, int RK, int MINB>
+cudaError_t run_u64(const StripeArgs &a, cudaStream_t st) {
+  using G = Geo<unsigned long long, RD, RK, 0>;
+  int grid = 0;
+  cudaError_t e = prepare(k_stripe_u64<RD, RK, MINB>, G::SMEM, &grid, units_of(a));
+  if (e != cudaSuccess) return e;
+  e = cudaMemsetAsync(a.counter, 0, sizeof(int), st);
+  if (e != cudaSuccess) return e;
+  return launch_k(k_stripe_u64<RD, RK, MINB>, dim3(grid), dim3(NT), G::SMEM, st, a);
 }
 
 template <typename T, int RD, int RK, int MINB>
@@ -730,12 +840,13 @@ cudaError_t run_gen(const StripeArgs &a, cudaStream_t st, int max_per_sm = 0) {
 
 }  // namespace
 
-// micro-tiles: min kernels 8 x 8 (shape 1 of the FP32 min kernel: 4 x 8
+// micro-tiles: FP32 min kernel 8 x 8 (shape 1: 4 x 8
 // at three CTAs per SM, 64-stripe tiles that waste fewer stripes of small
-// tables), generalized 4 x 8 (two accumulators), variance-adjusted 4 x 4
+// tables), FP64 min kernel 4 x 8 (64-bit sums at two CTAs per SM), generalized
+// 4 x 8 (two accumulators), variance-adjusted 4 x 4
 // (two accumulators, three planes)
 void stripe_tile_shape(int acc, bool fp32, int *tile_s, int *tile_k, int shape) {
-  *tile_s = acc == ACC_MIN && !(fp32 && shape == 1) ? 16 * 8 : 16 * 4;
+  *tile_s = acc == ACC_MIN && fp32 && shape == 0 ? 16 * 8 : 16 * 4;
   *tile_k = acc == ACC_VAW ? 16 * 4 : 16 * 8;
 }
 
@@ -748,10 +859,9 @@ int stripe_chunk_rows() { return 2048; }
 cudaError_t launch_stripe_acc(int acc, bool fp32, const StripeArgs &a, cudaStream_t st) {
   if (a.rows <= 0 || a.n_tiles <= 0) return cudaSuccess;
   if (acc == ACC_MIN) {
-    if (!fp32) return run_min<double, 8, 8, FP64_ABS_ROW_MASK, 1>(a, st);
-    if (a.abs_mask == 0xFFu) return run_min<float, 8, 8, 0xFFu, 2>(a, st);
-    return a.shape == 1 ? run_min<float, 4, 8, FP32_ABS_ROW_MASK, 3>(a, st)
-                        : run_min<float, 8, 8, FP32_ABS_ROW_MASK, 2>(a, st);
+    if (!fp32) return run_u64<4, 8, 2>(a, st);
+    if (a.abs_mask == 0xFFu) return run_min<8, 8, 0xFFu, 2>(a, st);
+    return a.shape == 1 ? run_min<4, 8, FP32_ABS_ROW_MASK, 3>(a, st) : run_min<8, 8, FP32_ABS_ROW_MASK, 2>(a, st);
   }
   if (acc == ACC_VAW) return fp32 ? run_vaw<float, 4, 4, 2>(a, st) : run_vaw<double, 4, 4, 1>(a, st);
   const bool half = a.alpha == 0.5;
@@ -760,26 +870,23 @@ cudaError_t launch_stripe_acc(int acc, bool fp32, const StripeArgs &a, cudaStrea
 }
 
 size_t diag_scratch_bytes(bool fp32, int rows, int n_cols) {
+  if (!fp32) return 0;
   // sub-blocks of any chunk size >= 1,024 rows that is a multiple of B1
   const int64_t n_sb = (rows + B1 - 1) / B1 + (rows + 1023) / 1024;
-  return (size_t)std::max<int64_t>(n_sb, 1) * n_cols * (fp32 ? 4 : 8);
+  return (size_t)std::max<int64_t>(n_sb, 1) * n_cols * 4;
 }
 
 cudaError_t launch_diag(bool fp32, const StripeArgs &a, void *scratch, cudaStream_t st) {
   if (a.rows <= 0) return cudaSuccess;
+  const int gx = (a.n_cols + 127) / 128;
+  if (!fp32)
+    return launch_k(k_diag_u64, dim3(gx, (a.rows + DIAG_ROWS - 1) / DIAG_ROWS), dim3(128), 0, st, a);
   const int per_chunk = (a.chunk + B1 - 1) / B1;
   const int n_chunks = (a.rows + a.chunk - 1) / a.chunk;
   const int n_sb = (n_chunks - 1) * per_chunk + ((a.rows - (n_chunks - 1) * a.chunk) + B1 - 1) / B1;
-  dim3 g1((a.n_cols + 127) / 128, n_sb);
-  const int g2 = (a.n_cols + 127) / 128;
-  if (fp32) {
-    const cudaError_t e = launch_k(k_diag_partial<float>, g1, dim3(128), 0, st, a, (float *)scratch);
-    if (e != cudaSuccess) return e;
-    return launch_k(k_diag_reduce<float>, dim3(g2), dim3(128), 0, st, a, (const float *)scratch, n_sb);
-  }
-  const cudaError_t e = launch_k(k_diag_partial<double>, g1, dim3(128), 0, st, a, (double *)scratch);
+  const cudaError_t e = launch_k(k_diag_partial, dim3(gx, n_sb), dim3(128), 0, st, a, (float *)scratch);
   if (e != cudaSuccess) return e;
-  return launch_k(k_diag_reduce<double>, dim3(g2), dim3(128), 0, st, a, (const double *)scratch, n_sb);
+  return launch_k(k_diag_reduce, dim3(gx), dim3(128), 0, st, a, (const float *)scratch, n_sb);
 }
 
 }  // namespace ufg
