@@ -80,7 +80,7 @@ struct StripeArgs {
   const double *len;    // per-row branch length (generalized only), [rows]
   int rows;             // branches in this launch
   int64_t pitch;        // elements per row (all segments)
-  int chunk;            // rows per work unit: a multiple of 64, >= 1,024
+  int chunk;            // rows per work unit: a multiple of 64 (FP32 min) or 16
   const TabDesc *tabs;  // device array of n_tabs tables
   int n_tabs;
   int n_tiles;          // tiles of all tables (per row chunk)
@@ -106,16 +106,30 @@ struct StripeArgs {
   int shape;            // tile shape (stripe_tile_shape); the descriptors must match it
 };
 // stripes and samples per CTA tile of the accumulate kernel; `shape` picks
-// one of stripe_shapes() tile shapes (0: the default)
+// a tile shape (0: the default; 1 and, FP32 min kernel, 2: the small tiles last)
 void stripe_tile_shape(int acc, bool fp32, int *tile_s, int *tile_k, int shape = 0);
-// tile shapes the accumulate kernel of (acc, precision, abs mask) offers
+// tile shapes of (acc, precision, abs mask) for problems that fill the GPU
 int stripe_shapes(int acc, bool fp32, unsigned abs_mask);
+// the shape of small tiles
+int stripe_small_shape(int acc, bool fp32);
+// Tile shape and rows per unit for problems that do not fill it: the small
+// tiles where the shape's own pad their tables' stripes and samples out to
+// more work, and units of fewer than `chunk` rows (split) until there are four
+// waves of them.  Counted over the tables' full stripe ranges (n samples
+// each), so that a stripe range's units have the rows of the full run's and
+// its results the same bits.
+struct SmallPlan {
+  int shape, chunk;
+  bool split;
+};
+SmallPlan stripe_small_plan(int acc, bool fp32, const int *n, size_t n_tabs, int rows, int chunk,
+                            int shape, bool shape_free, int sms);
 // default rows per work unit
 int stripe_chunk_rows();
 cudaError_t launch_stripe_acc(int acc, bool fp32, const StripeArgs &a, cudaStream_t st);
 // D[k] += sum of the launch's rows at column k (ACC_MIN only): FP32 with the
-// stripe kernel's operation order, in scratch of diag_scratch_bytes() (valid
-// for every chunk size the StripeArgs may carry); FP64 rows are integers,
+// stripe kernel's operation order, in scratch of diag_scratch_bytes(); FP64
+// rows are integers,
 // summed in any order
 size_t diag_scratch_bytes(bool fp32, int rows, int n_cols);
 cudaError_t launch_diag(bool fp32, const StripeArgs &a, void *scratch, cudaStream_t st);

@@ -116,8 +116,15 @@ uf_status compute_noalloc(const uf_tree *tree, const uf_table *table, uf_method 
   const bool fp32 = precision == UF_MIXED;
   const size_t es = fp32 ? 4 : 8;
   const size_t words = fp32 ? 1 : 2;
+  int device = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&device);
+  const bool usable = e == cudaSuccess && device >= 0 && device < UF_NOALLOC_MAX_DEVICES &&
+                      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) == cudaSuccess;
+  const unsigned amask = acc == ACC_MIN ? abs_row_mask(fp32) : 0u;
+  const SmallPlan plan = stripe_small_plan(acc, fp32, &n, 1, (int)std::max<int64_t>(tv.n_nodes - 1, 1),
+                                           stripe_chunk_rows(), 0, true, sms);
   int tile_s = 0, tile_k = 0;
-  stripe_tile_shape(acc, fp32, &tile_s, &tile_k);
+  stripe_tile_shape(acc, fp32, &tile_s, &tile_k, plan.shape);
   const int m_hi = (int)((S - 1) / tile_s);
   const int64_t pitch = round_up(round_up(n, tile_k) + (int64_t)(m_hi + 1) * tile_s, 32);
   const int64_t N = tv.n_nodes, nb = N - 1;
@@ -184,9 +191,7 @@ uf_status compute_noalloc(const uf_tree *tree, const uf_table *table, uf_method 
     return noalloc_fail(UF_ENOMEM, msg);
   }
 
-  int device = 0;
-  cudaError_t e = cudaGetDevice(&device);
-  if (e != cudaSuccess || device < 0 || device >= UF_NOALLOC_MAX_DEVICES) {
+  if (!usable) {
     cudaGetLastError();
     return noalloc_fail(UF_ECUDA, "no usable CUDA device");
   }
@@ -245,7 +250,7 @@ uf_status compute_noalloc(const uf_tree *tree, const uf_table *table, uf_method 
   // FP64 min kernel: 64-bit fixed-point rows (StripeArgs::x_shift)
   const bool fixed_rows = !fp32 && acc == ACC_MIN;
   const int x_shift =
-      fixed_rows ? fixed_row_shift(scale, accum_bound(tree, table, kind), tv.length, nb, stripe_chunk_rows()) : 0;
+      fixed_rows ? fixed_row_shift(scale, accum_bound(tree, table, kind), tv.length, nb, plan.chunk) : 0;
 
   const int32_t *d_lists = (const int32_t *)p[5], *d_slot = (const int32_t *)p[4];
   double *d_counts = (double *)p[11];
@@ -264,7 +269,8 @@ uf_status compute_noalloc(const uf_tree *tree, const uf_table *table, uf_method 
     sa.len = (const double *)p[0];
     sa.rows = rows;
     sa.pitch = pitch;
-    sa.chunk = stripe_chunk_rows();
+    sa.chunk = plan.chunk;
+    sa.shape = plan.shape;
     sa.tabs = (const TabDesc *)p[18];
     sa.n_tabs = 1;
     sa.n_tiles = tab.n_ktiles * (m_hi + 1);
@@ -287,7 +293,7 @@ uf_status compute_noalloc(const uf_tree *tree, const uf_table *table, uf_method 
   fa.s0 = 0;
   fa.s1 = S;
   fa.full = 1;
-  fa.abs_mask = acc == ACC_MIN ? abs_row_mask(fp32) : 0u;
+  fa.abs_mask = amask;
   fa.relu = fixed_rows;
   fa.gen_abs = acc == ACC_GEN && !fp32;
   fa.M = (const unsigned long long *)p[13];

@@ -1012,11 +1012,12 @@ uf_status run_stripes(uf_tree *tree, const BatchJob &J, int device, uf_method me
   // the descriptors of every tile shape the kernel offers (shape 0 above; the
   // others have shorter stripe tiles, so the rows' pitch of shape 0 fits them)
   const int n_shapes = stripe_shapes(acc, fp32, amask);
+  const int small_shape = stripe_small_shape(acc, fp32), n_all_shapes = small_shape + 1;
   // option "tile_shape": a forced shape when the kernel has it, else tuned (or 0)
   const int forced = g_tile_shape.load() >= 0 && g_tile_shape.load() < n_shapes ? (int)g_tile_shape.load() : -1;
   std::vector<std::vector<TabDesc>> shape_tabs(1, tabs);
   std::vector<int> shape_tiles(1, n_tiles), shape_ts(1, tile_s), shape_tk(1, tile_k);
-  for (int sh = 1; sh < n_shapes; sh++) {
+  for (int sh = 1; sh < n_all_shapes; sh++) {
     int ts2 = 0, tk2 = 0, nt2 = 0;
     stripe_tile_shape(acc, fp32, &ts2, &tk2, sh);
     std::vector<TabDesc> tb2(tabs);
@@ -1079,7 +1080,7 @@ uf_status run_stripes(uf_tree *tree, const BatchJob &J, int device, uf_method me
   Meta meta;
   const size_t o_tabs = meta.add(tabs);
   std::vector<size_t> o_shape_tabs(1, o_tabs);
-  for (int sh = 1; sh < n_shapes; sh++) o_shape_tabs.push_back(meta.add(shape_tabs[sh]));
+  for (int sh = 1; sh < n_all_shapes; sh++) o_shape_tabs.push_back(meta.add(shape_tabs[sh]));
   const size_t o_cnt = meta.add(split.cnt_lists);
   const size_t o_dense = meta.add(split.dense);
   const size_t o_dlen = meta.add(split.dense_len);
@@ -1122,7 +1123,16 @@ uf_status run_stripes(uf_tree *tree, const BatchJob &J, int device, uf_method me
   bool tune = false;
   // (the FP64 min kernel's sums are exact for any chunk: not tuned)
   const bool fixed_rows = !fp32 && acc == ACC_MIN;
-  if (g_autotune.load() && !split.dense.empty() && !fixed_rows) {
+  // problems too small to fill the GPU: the rule's shape and shorter units, nothing tuned
+  int sms = 0;
+  ck(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device), "cudaDeviceGetAttribute");
+  std::vector<int> ns(nt);
+  for (size_t t = 0; t < nt; t++) ns[t] = tabs[t].n;
+  auto small_plan = [&](bool shape_free) {
+    return stripe_small_plan(acc, fp32, ns.data(), nt, (int)xrows, chunk, shape, shape_free, sms);
+  };
+  const SmallPlan small = small_plan(forced < 0);
+  if (g_autotune.load() && !split.dense.empty() && !fixed_rows && !small.split && small.shape != small_shape) {
     std::lock_guard<std::mutex> g(g_tune_mu);
     auto it = g_tuned_chunk.find(key);
     if (it != g_tuned_chunk.end()) {
@@ -1131,6 +1141,8 @@ uf_status run_stripes(uf_tree *tree, const BatchJob &J, int device, uf_method me
     } else {
       tune = true;
     }
+  } else {
+    shape = small.shape;
   }
   auto use_shape = [&](int sh) {
     shape = sh;
@@ -1139,6 +1151,9 @@ uf_status run_stripes(uf_tree *tree, const BatchJob &J, int device, uf_method me
     n_tiles = shape_tiles[sh];
   };
   use_shape(shape);
+  // a chunk is the rows a unit sums before it rounds; small problems cut it
+  // so that every SM has units (tuned chunks are found with enough of them)
+  int unit_rows = small.split && !tune ? small_plan(false).chunk : chunk;
   int x_shift = 0;  // grid of the FP64 min kernel's rows (StripeArgs::x_shift)
   if (fixed_rows) {
     double bound = 0.0;
@@ -1146,7 +1161,7 @@ uf_status run_stripes(uf_tree *tree, const BatchJob &J, int device, uf_method me
     x_shift = 32;
     for (size_t b = 0; b + 1 < split.dense_ptr.size(); b++)
       x_shift = std::min(x_shift, fixed_row_shift(scale, bound, split.dense_len.data() + split.dense_ptr[b],
-                                                  split.dense_ptr[b + 1] - split.dense_ptr[b], chunk));
+                                                  split.dense_ptr[b + 1] - split.dense_ptr[b], unit_rows));
   }
   // the launch sequence goes into a CUDA graph unless it is timed per phase
   Capture cap(g_graph.load() != 0 && !timer.on && !tune, st, device);
@@ -1197,7 +1212,7 @@ uf_status run_stripes(uf_tree *tree, const BatchJob &J, int device, uf_method me
     sa.len = d_dlen + d0;
     sa.rows = (int)nd;
     sa.pitch = pitch;
-    sa.chunk = chunk;
+    sa.chunk = unit_rows;
     sa.shape = shape;
     sa.tabs = meta.at<TabDesc>(o_shape_tabs[shape]);
     sa.n_tabs = (int)nt;
@@ -1215,8 +1230,8 @@ uf_status run_stripes(uf_tree *tree, const BatchJob &J, int device, uf_method me
     sa.x_shift = x_shift;
     if (tune && !tuned) {
       std::vector<const TabDesc *> tp;
-      for (size_t o : o_shape_tabs) tp.push_back(meta.at<TabDesc>(o));
-      std::vector<int> tiles(shape_tiles);
+      for (int sh = 0; sh < n_shapes; sh++) tp.push_back(meta.at<TabDesc>(o_shape_tabs[sh]));
+      std::vector<int> tiles(shape_tiles.begin(), shape_tiles.begin() + n_shapes);
       if (forced >= 0) {  // only the forced shape is a candidate
         for (size_t sh = 0; sh < tp.size(); sh++)
           if ((int)sh != forced) tiles[sh] = -1;
@@ -1224,6 +1239,7 @@ uf_status run_stripes(uf_tree *tree, const BatchJob &J, int device, uf_method me
       const std::pair<int, int> best = tune_chunk(acc, fp32, sa, tp, tiles, m_bytes, ls);
       use_shape(best.first);
       chunk = best.second;
+      unit_rows = chunk;
       sa.chunk = chunk;
       sa.shape = shape;
       sa.tabs = tp[shape];

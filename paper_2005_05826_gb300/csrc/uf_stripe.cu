@@ -56,7 +56,8 @@ namespace ufg {
 
 namespace {
 
-constexpr int NT = 256;       // threads per CTA: 16 (stripe) x 16 (sample)
+// Threads of a CTA: TX (stripe) x TX (sample), TX = 16 or, for small problems,
+// 8 (tiles of a quarter of the cells: less padding and more units in flight).
 constexpr int B1 = 64;        // inner partial length (branches)
 
 // Shared rows are stored in 16-byte units with unit j placed at
@@ -71,14 +72,15 @@ __host__ __device__ constexpr int swz(int elem) {
   return (j ^ ((j >> 3) & MASK)) * VEC + elem % VEC;
 }
 
-template <typename T, int RD, int RK, int NACC>
+template <typename T, int RD, int RK, int NACC, int TX>
 struct Geo {
+  static constexpr int NT = TX * TX;
   // branch rows per pipeline stage and cp.async stages: FP32 16 rows in two
   // stages (half the block barriers of 8-row stages), FP64 8 rows in three
   static constexpr int RB = sizeof(T) == 4 ? 16 : 8;
   static constexpr int NSTAGE = sizeof(T) == 4 ? 2 : 3;
-  static constexpr int TS = 16 * RD;             // stripes per tile
-  static constexpr int TK = 16 * RK;             // samples per tile
+  static constexpr int TS = TX * RD;             // stripes per tile
+  static constexpr int TK = TX * RK;             // samples per tile
   static constexpr int VEC = 16 / sizeof(T);     // elements per 16-byte copy
   static constexpr int UW = TK;                  // u window
   static constexpr int VW = TK + TS;             // partner window (needs TK + TS - 1, shifted by one)
@@ -162,12 +164,12 @@ __device__ __forceinline__ bool next_unit(const StripeArgs &a, int tile_s, int t
 
 // Stage loader: G::RB branch rows [e0, e0 + G::RB) of the u window (columns from
 // ucol) and the partner window (columns from vcol).
-template <typename T, int RD, int RK, int NACC, bool LEN>
+template <typename T, int RD, int RK, int NACC, int TX, bool LEN>
 __device__ __forceinline__ void load_stage(T *stage, const StripeArgs &a, int e0, int e_end, int64_t ucol,
                                            int64_t vcol) {
-  using G = Geo<T, RD, RK, NACC>;
+  using G = Geo<T, RD, RK, NACC, TX>;
   const T *X = (const T *)a.X;
-  for (int c = threadIdx.x; c < G::RB * G::CH; c += NT) {
+  for (int c = threadIdx.x; c < G::RB * G::CH; c += G::NT) {
     const int r = c / G::CH, q = c - r * G::CH;
     T *row = stage + r * G::ROW;
     const int e = e0 + r;
@@ -198,7 +200,7 @@ __device__ __forceinline__ void load_stage(T *stage, const StripeArgs &a, int e0
 }
 
 // Add one thread's second-level cells (fixed point) into the accumulator.
-template <typename T, int RD, int RK, typename Mid>
+template <typename T, int RD, int RK, int TX, typename Mid>
 __device__ __forceinline__ void commit_cells(unsigned long long *M, const Mid *mid, const StripeArgs &a,
                                              const Unit &U, int s_base, int k_base) {
 #pragma unroll
@@ -210,7 +212,7 @@ __device__ __forceinline__ void commit_cells(unsigned long long *M, const Mid *m
     for (int j = 0; j < RK; j++) {
       const int k = k_base + j;
       if (k < U.n) {
-        const Fx2 q = to_fixed2(mid[(i * RK + j) * NT + threadIdx.x], a.scale);
+        const Fx2 q = to_fixed2(mid[(i * RK + j) * (TX * TX) + threadIdx.x], a.scale);
         atomicAdd(row + k, (unsigned long long)q.hi);
         if constexpr (sizeof(T) == 8) atomicAdd(row + k + a.m_lo_off, (unsigned long long)q.lo);
       }
@@ -221,16 +223,17 @@ __device__ __forceinline__ void commit_cells(unsigned long long *M, const Mid *m
 // ---- weighted / unweighted, FP32 ----
 // rows i of the micro-tile with bit i of ABSM clear: M += min(x_k, x_j);
 // with it set: A += |x_k - x_j|
-template <int RD, int RK, unsigned ABSM, int MINB>
-__global__ void __launch_bounds__(NT, MINB) k_stripe_min(const StripeArgs a) {
+template <int RD, int RK, int TX, unsigned ABSM, int MINB>
+__global__ void __launch_bounds__(TX *TX, MINB) k_stripe_min(const StripeArgs a) {
   using T = float;
-  using G = Geo<T, RD, RK, 1>;
+  using G = Geo<T, RD, RK, 1, TX>;
+  constexpr int NT = G::NT;
   using Mid = typename G::Mid;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T *stg = reinterpret_cast<T *>(smem_raw);
   Mid *mid = reinterpret_cast<Mid *>(smem_raw + (size_t)G::NSTAGE * G::STAGE * sizeof(T));
   __shared__ int s_unit;
-  const int tk = threadIdx.x & 15, ts = threadIdx.x >> 4;
+  const int tk = threadIdx.x % TX, ts = threadIdx.x / TX;
   const int w0 = RK * tk + RD * ts;  // partner window of this thread, used from w0 + 1
   Unit U;
   while (next_unit(a, G::TS, G::TK, &s_unit, &U)) {
@@ -239,7 +242,7 @@ __global__ void __launch_bounds__(NT, MINB) k_stripe_min(const StripeArgs a) {
     const int nst = (U.r1 - U.r0 + G::RB - 1) / G::RB;
 #pragma unroll
     for (int p = 0; p < G::NSTAGE - 1; p++) {
-      if (p < nst) load_stage<T, RD, RK, 1, false>(stg + p * G::STAGE, a, U.r0 + p * G::RB, U.r1, U.x_col + U.k0,
+      if (p < nst) load_stage<T, RD, RK, 1, TX, false>(stg + p * G::STAGE, a, U.r0 + p * G::RB, U.r1, U.x_col + U.k0,
                                         U.x_col + U.k0 + U.s0);
       cp_async_commit();
     }
@@ -255,7 +258,7 @@ __global__ void __launch_bounds__(NT, MINB) k_stripe_min(const StripeArgs a) {
       {
         const int nx = it + G::NSTAGE - 1;
         if (nx < nst)
-          load_stage<T, RD, RK, 1, false>(stg + (nx % G::NSTAGE) * G::STAGE, a, U.r0 + nx * G::RB, U.r1,
+          load_stage<T, RD, RK, 1, TX, false>(stg + (nx % G::NSTAGE) * G::STAGE, a, U.r0 + nx * G::RB, U.r1,
                                           U.x_col + U.k0, U.x_col + U.k0 + U.s0);
         cp_async_commit();
       }
@@ -308,7 +311,7 @@ __global__ void __launch_bounds__(NT, MINB) k_stripe_min(const StripeArgs a) {
       }
     }
     cp_async_wait<0>();
-    commit_cells<T, RD, RK>(a.M, mid, a, U, U.s0 + RD * ts, U.k0 + RK * tk);
+    commit_cells<T, RD, RK, TX>(a.M, mid, a, U, U.s0 + RD * ts, U.k0 + RK * tk);
   }
 }
 
@@ -329,21 +332,21 @@ __device__ __forceinline__ void add_relu(unsigned long long &c, unsigned long lo
 // 14.7 (some of the adds issue elsewhere), the 64-bit min 12.6, the FP64 form
 // |u - v| 0.8.  The sums stay in registers for the whole unit (they are exact,
 // so there is no second level) and go to the two-word accumulators at its end.
-template <int RD, int RK, int MINB>
-__global__ void __launch_bounds__(NT, MINB) k_stripe_u64(const StripeArgs a) {
+template <int RD, int RK, int TX, int MINB>
+__global__ void __launch_bounds__(TX *TX, MINB) k_stripe_u64(const StripeArgs a) {
   using T = unsigned long long;
-  using G = Geo<T, RD, RK, 0>;
+  using G = Geo<T, RD, RK, 0, TX>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T *stg = reinterpret_cast<T *>(smem_raw);
   __shared__ int s_unit;
-  const int tk = threadIdx.x & 15, ts = threadIdx.x >> 4;
+  const int tk = threadIdx.x % TX, ts = threadIdx.x / TX;
   const int w0 = RK * tk + RD * ts;
   Unit U;
   while (next_unit(a, G::TS, G::TK, &s_unit, &U)) {
     const int nst = (U.r1 - U.r0 + G::RB - 1) / G::RB;
 #pragma unroll
     for (int p = 0; p < G::NSTAGE - 1; p++) {
-      if (p < nst) load_stage<T, RD, RK, 0, false>(stg + p * G::STAGE, a, U.r0 + p * G::RB, U.r1, U.x_col + U.k0,
+      if (p < nst) load_stage<T, RD, RK, 0, TX, false>(stg + p * G::STAGE, a, U.r0 + p * G::RB, U.r1, U.x_col + U.k0,
                                         U.x_col + U.k0 + U.s0);
       cp_async_commit();
     }
@@ -358,7 +361,7 @@ __global__ void __launch_bounds__(NT, MINB) k_stripe_u64(const StripeArgs a) {
       {
         const int nx = it + G::NSTAGE - 1;
         if (nx < nst)
-          load_stage<T, RD, RK, 0, false>(stg + (nx % G::NSTAGE) * G::STAGE, a, U.r0 + nx * G::RB, U.r1,
+          load_stage<T, RD, RK, 0, TX, false>(stg + (nx % G::NSTAGE) * G::STAGE, a, U.r0 + nx * G::RB, U.r1,
                                           U.x_col + U.k0, U.x_col + U.k0 + U.s0);
         cp_async_commit();
       }
@@ -403,9 +406,10 @@ __global__ void __launch_bounds__(NT, MINB) k_stripe_u64(const StripeArgs a) {
 
 // ---- generalized: den += l s w and, FP32, Q += l min(u, v) w or, FP64,
 //      N += l |u - v| w, with w = s^(alpha - 1) ----
-template <typename T, int RD, int RK, int MODE, int MINB>
-__global__ void __launch_bounds__(NT, MINB) k_stripe_gen(const StripeArgs a) {
-  using G = Geo<T, RD, RK, 2>;
+template <typename T, int RD, int RK, int TX, int MODE, int MINB>
+__global__ void __launch_bounds__(TX *TX, MINB) k_stripe_gen(const StripeArgs a) {
+  using G = Geo<T, RD, RK, 2, TX>;
+  constexpr int NT = G::NT;
   using Mid = typename G::Mid;
   constexpr bool F32 = sizeof(T) == 4;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -413,7 +417,7 @@ __global__ void __launch_bounds__(NT, MINB) k_stripe_gen(const StripeArgs a) {
   Mid *midd = reinterpret_cast<Mid *>(smem_raw + (size_t)G::NSTAGE * G::STAGE * sizeof(T));
   Mid *midq = midd + RD * RK * NT;
   __shared__ int s_unit;
-  const int tk = threadIdx.x & 15, ts = threadIdx.x >> 4;
+  const int tk = threadIdx.x % TX, ts = threadIdx.x / TX;
   const int w0 = RK * tk + RD * ts;
   const T am1 = (T)(a.alpha - 1.0);
   Unit U;
@@ -423,7 +427,7 @@ __global__ void __launch_bounds__(NT, MINB) k_stripe_gen(const StripeArgs a) {
     const int nst = (U.r1 - U.r0 + G::RB - 1) / G::RB;
 #pragma unroll
     for (int p = 0; p < G::NSTAGE - 1; p++) {
-      if (p < nst) load_stage<T, RD, RK, 2, true>(stg + p * G::STAGE, a, U.r0 + p * G::RB, U.r1, U.x_col + U.k0,
+      if (p < nst) load_stage<T, RD, RK, 2, TX, true>(stg + p * G::STAGE, a, U.r0 + p * G::RB, U.r1, U.x_col + U.k0,
                                        U.x_col + U.k0 + U.s0);
       cp_async_commit();
     }
@@ -439,7 +443,7 @@ __global__ void __launch_bounds__(NT, MINB) k_stripe_gen(const StripeArgs a) {
       {
         const int nx = it + G::NSTAGE - 1;
         if (nx < nst)
-          load_stage<T, RD, RK, 2, true>(stg + (nx % G::NSTAGE) * G::STAGE, a, U.r0 + nx * G::RB, U.r1,
+          load_stage<T, RD, RK, 2, TX, true>(stg + (nx % G::NSTAGE) * G::STAGE, a, U.r0 + nx * G::RB, U.r1,
                                          U.x_col + U.k0, U.x_col + U.k0 + U.s0);
         cp_async_commit();
       }
@@ -517,8 +521,8 @@ __global__ void __launch_bounds__(NT, MINB) k_stripe_gen(const StripeArgs a) {
       }
     }
     cp_async_wait<0>();
-    commit_cells<T, RD, RK>(a.M, midd, a, U, U.s0 + RD * ts, U.k0 + RK * tk);
-    commit_cells<T, RD, RK>(a.M2, midq, a, U, U.s0 + RD * ts, U.k0 + RK * tk);
+    commit_cells<T, RD, RK, TX>(a.M, midd, a, U, U.s0 + RD * ts, U.k0 + RK * tk);
+    commit_cells<T, RD, RK, TX>(a.M2, midq, a, U, U.s0 + RD * ts, U.k0 + RK * tk);
   }
 }
 
@@ -529,12 +533,13 @@ __global__ void __launch_bounds__(NT, MINB) k_stripe_gen(const StripeArgs a) {
 // Rows hold three planes (u, c, r) of `pitch` elements each.  A stage carries
 // RB rows of all three planes; the micro-tile is RD x RK with two
 // accumulators per cell.
-template <typename T, int RD, int RK>
+template <typename T, int RD, int RK, int TX>
 struct GeoV {
+  static constexpr int NT = TX * TX;
   static constexpr int RB = sizeof(T) == 4 ? 8 : 4;  // rows per stage
   static constexpr int NSTAGE = 2;
   static constexpr int NPL = 3;                       // planes: u, c, r
-  static constexpr int TS = 16 * RD, TK = 16 * RK;
+  static constexpr int TS = TX * RD, TK = TX * RK;
   static constexpr int VEC = 16 / sizeof(T);
   static constexpr int UW = TK, VW = TK + TS, ROW = UW + VW;
   static constexpr int STAGE = RB * NPL * ROW;  // rows past the unit are zero (w = 0)
@@ -549,12 +554,12 @@ struct GeoV {
   static __device__ __forceinline__ int at(int elem) { return sizeof(T) == 4 ? elem : swz<T>(elem); }
 };
 
-template <typename T, int RD, int RK>
+template <typename T, int RD, int RK, int TX>
 __device__ __forceinline__ void load_stage_vaw(T *stage, const StripeArgs &a, int e0, int e_end, int64_t ucol,
                                                int64_t vcol) {
-  using G = GeoV<T, RD, RK>;
+  using G = GeoV<T, RD, RK, TX>;
   const T *X = (const T *)a.X;
-  for (int c = threadIdx.x; c < G::RB * G::NPL * G::CH; c += NT) {
+  for (int c = threadIdx.x; c < G::RB * G::NPL * G::CH; c += G::NT) {
     const int rp = c / G::CH, q = c - rp * G::CH;  // rp = row * NPL + plane
     const int r = rp / G::NPL, pl = rp - r * G::NPL;
     T *row = stage + rp * G::ROW;
@@ -591,15 +596,16 @@ __device__ __forceinline__ double vaw_weight<double>(double prod) {
   return prod > 0.0 ? rsqrt(prod) : 0.0;
 }
 
-template <typename T, int RD, int RK, int MINB>
-__global__ void __launch_bounds__(NT, MINB) k_stripe_vaw(const StripeArgs a) {
-  using G = GeoV<T, RD, RK>;
+template <typename T, int RD, int RK, int TX, int MINB>
+__global__ void __launch_bounds__(TX *TX, MINB) k_stripe_vaw(const StripeArgs a) {
+  using G = GeoV<T, RD, RK, TX>;
+  constexpr int NT = G::NT;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T *stg = reinterpret_cast<T *>(smem_raw);
   T *midd = reinterpret_cast<T *>(smem_raw + (size_t)G::NSTAGE * G::STAGE * sizeof(T));
   T *midn = midd + RD * RK * NT;
   __shared__ int s_unit;
-  const int tk = threadIdx.x & 15, ts = threadIdx.x >> 4;
+  const int tk = threadIdx.x % TX, ts = threadIdx.x / TX;
   const int w0 = RK * tk + RD * ts;
   Unit U;
   while (next_unit(a, G::TS, G::TK, &s_unit, &U)) {
@@ -607,7 +613,7 @@ __global__ void __launch_bounds__(NT, MINB) k_stripe_vaw(const StripeArgs a) {
     for (int c = 0; c < RD * RK; c++) midd[c * NT + threadIdx.x] = midn[c * NT + threadIdx.x] = T(0);
     const int nst = (U.r1 - U.r0 + G::RB - 1) / G::RB;
     if (nst > 0)
-      load_stage_vaw<T, RD, RK>(stg, a, U.r0, U.r1, U.x_col + U.k0, U.x_col + U.k0 + U.s0);
+      load_stage_vaw<T, RD, RK, TX>(stg, a, U.r0, U.r1, U.x_col + U.k0, U.x_col + U.k0 + U.s0);
     cp_async_commit();
     T accd[RD][RK], accn[RD][RK];
 #pragma unroll
@@ -619,7 +625,7 @@ __global__ void __launch_bounds__(NT, MINB) k_stripe_vaw(const StripeArgs a) {
       cp_async_wait<0>();
       __syncthreads();
       if (it + 1 < nst)
-        load_stage_vaw<T, RD, RK>(stg + ((it + 1) % G::NSTAGE) * G::STAGE, a, U.r0 + (it + 1) * G::RB, U.r1,
+        load_stage_vaw<T, RD, RK, TX>(stg + ((it + 1) % G::NSTAGE) * G::STAGE, a, U.r0 + (it + 1) * G::RB, U.r1,
                                   U.x_col + U.k0, U.x_col + U.k0 + U.s0);
       cp_async_commit();
       const T *stage = stg + (it % G::NSTAGE) * G::STAGE;
@@ -695,8 +701,8 @@ __global__ void __launch_bounds__(NT, MINB) k_stripe_vaw(const StripeArgs a) {
       }
     }
     cp_async_wait<0>();
-    commit_cells<T, RD, RK>(a.M, midd, a, U, U.s0 + RD * ts, U.k0 + RK * tk);
-    commit_cells<T, RD, RK>(a.M2, midn, a, U, U.s0 + RD * ts, U.k0 + RK * tk);
+    commit_cells<T, RD, RK, TX>(a.M, midd, a, U, U.s0 + RD * ts, U.k0 + RK * tk);
+    commit_cells<T, RD, RK, TX>(a.M2, midn, a, U, U.s0 + RD * ts, U.k0 + RK * tk);
   }
 }
 
@@ -773,81 +779,57 @@ __global__ void k_diag_u64(const StripeArgs a) {
   if (lo) atomicAdd(a.Dg + kg + a.d_lo_off, lo);
 }
 
+// A persistent launch: as many CTAs as fit (or units, if fewer), after the
+// unit counter is reset.
 template <typename K>
-cudaError_t prepare(K kernel, size_t smem, int *grid, int units, int max_per_sm = 0) {
+cudaError_t run_units(K kernel, int threads, size_t smem, const StripeArgs &a, cudaStream_t st) {
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   int per_sm = 0, dev = 0, sms = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, NT, smem);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem);
   if (e != cudaSuccess) return e;
   e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  if (max_per_sm > 0) per_sm = std::min(per_sm, max_per_sm);
-  *grid = std::max(1, std::min(units, std::max(per_sm, 1) * sms));
-  return cudaSuccess;
+  const int n_chunks = (a.rows + a.chunk - 1) / a.chunk, units = n_chunks * a.n_tiles;
+  const int grid = std::max(1, std::min(units, std::max(per_sm, 1) * sms));
+  e = cudaMemsetAsync(a.counter, 0, sizeof(int), st);
+  if (e != cudaSuccess) return e;
+  return launch_k(kernel, dim3(grid), dim3(threads), smem, st, a);
 }
 
-int units_of(const StripeArgs &a) {
-  const int n_chunks = (a.rows + a.chunk - 1) / a.chunk;
-  return n_chunks * a.n_tiles;
-}
-
-template <int RD, int RK, unsigned ABSM, int MINB>
+template <int RD, int RK, int TX, unsigned ABSM, int MINB>
 cudaError_t run_min(const StripeArgs &a, cudaStream_t st) {
-  using G = Geo<float, RD, RK, 1>;
-  int grid = 0;
-  cudaError_t e = prepare(k_stripe_min<RD, RK, ABSM, MINB>, G::SMEM, &grid, units_of(a));
-  if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(a.counter, 0, sizeof(int), st);
-  if (e != cudaSuccess) return e;
-  return launch_k(k_stripe_min<RD, RK, ABSM, MINB>, dim3(grid), dim3(NT), G::SMEM, st, a);
+  return run_units(k_stripe_min<RD, RK, TX, ABSM, MINB>, TX * TX, Geo<float, RD, RK, 1, TX>::SMEM, a, st);
 }
-
-template <int RD, int RK, int MINB>
+template <int RD, int RK, int TX, int MINB>
 cudaError_t run_u64(const StripeArgs &a, cudaStream_t st) {
-  using G = Geo<unsigned long long, RD, RK, 0>;
-  int grid = 0;
-  cudaError_t e = prepare(k_stripe_u64<RD, RK, MINB>, G::SMEM, &grid, units_of(a));
-  if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(a.counter, 0, sizeof(int), st);
-  if (e != cudaSuccess) return e;
-  return launch_k(k_stripe_u64<RD, RK, MINB>, dim3(grid), dim3(NT), G::SMEM, st, a);
+  return run_units(k_stripe_u64<RD, RK, TX, MINB>, TX * TX, Geo<unsigned long long, RD, RK, 0, TX>::SMEM, a, st);
 }
-
-template <typename T, int RD, int RK, int MINB>
+template <typename T, int RD, int RK, int TX, int MINB>
 cudaError_t run_vaw(const StripeArgs &a, cudaStream_t st) {
-  using G = GeoV<T, RD, RK>;
-  int grid = 0;
-  cudaError_t e = prepare(k_stripe_vaw<T, RD, RK, MINB>, G::SMEM, &grid, units_of(a));
-  if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(a.counter, 0, sizeof(int), st);
-  if (e != cudaSuccess) return e;
-  return launch_k(k_stripe_vaw<T, RD, RK, MINB>, dim3(grid), dim3(NT), G::SMEM, st, a);
+  return run_units(k_stripe_vaw<T, RD, RK, TX, MINB>, TX * TX, GeoV<T, RD, RK, TX>::SMEM, a, st);
 }
-
-template <typename T, int RD, int RK, int MODE, int MINB>
-cudaError_t run_gen(const StripeArgs &a, cudaStream_t st, int max_per_sm = 0) {
-  using G = Geo<T, RD, RK, 2>;
-  int grid = 0;
-  cudaError_t e = prepare(k_stripe_gen<T, RD, RK, MODE, MINB>, G::SMEM, &grid, units_of(a), max_per_sm);
-  if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(a.counter, 0, sizeof(int), st);
-  if (e != cudaSuccess) return e;
-  return launch_k(k_stripe_gen<T, RD, RK, MODE, MINB>, dim3(grid), dim3(NT), G::SMEM, st, a);
+template <typename T, int RD, int RK, int TX, int MODE, int MINB>
+cudaError_t run_gen(const StripeArgs &a, cudaStream_t st) {
+  return run_units(k_stripe_gen<T, RD, RK, TX, MODE, MINB>, TX * TX, Geo<T, RD, RK, 2, TX>::SMEM, a, st);
 }
 
 }  // namespace
 
-// micro-tiles: FP32 min kernel 8 x 8 (shape 1: 4 x 8
-// at three CTAs per SM, 64-stripe tiles that waste fewer stripes of small
-// tables), FP64 min kernel 4 x 8 (64-bit sums at two CTAs per SM), generalized
-// 4 x 8 (two accumulators), variance-adjusted 4 x 4
-// (two accumulators, three planes)
+// Shapes of (accumulator, precision): micro-tiles of the FP32 min kernel 8 x 8
+// (shape 1: 4 x 8 at three CTAs per SM, 64-stripe tiles that waste fewer
+// stripes of small tables), FP64 min kernel 4 x 8 (64-bit sums at two CTAs per
+// SM), generalized 4 x 8 (two accumulators), variance-adjusted 4 x 4 (two
+// accumulators, three planes), all on 16 x 16 threads; the last shape of each
+// is the small one, 8 x 8 threads of a 4 x 8 (4 x 4) micro-tile.
+int stripe_small_shape(int acc, bool fp32) { return acc == ACC_MIN && fp32 ? 2 : 1; }
+
 void stripe_tile_shape(int acc, bool fp32, int *tile_s, int *tile_k, int shape) {
-  *tile_s = acc == ACC_MIN && fp32 && shape == 0 ? 16 * 8 : 16 * 4;
-  *tile_k = acc == ACC_VAW ? 16 * 4 : 16 * 8;
+  const bool min8 = acc == ACC_MIN && fp32, small = shape == stripe_small_shape(acc, fp32);
+  *tile_s = small ? 32 : (min8 && shape == 0 ? 128 : 64);
+  *tile_k = acc == ACC_VAW ? (small ? 32 : 64) : (small ? 64 : 128);
 }
 
 int stripe_shapes(int acc, bool fp32, unsigned abs_mask) {
@@ -856,23 +838,76 @@ int stripe_shapes(int acc, bool fp32, unsigned abs_mask) {
 
 int stripe_chunk_rows() { return 2048; }
 
+SmallPlan stripe_small_plan(int acc, bool fp32, const int *n, size_t n_tabs, int rows, int chunk,
+                            int shape, bool shape_free, int sms) {
+  auto tiles_of = [&](int sh, int64_t *cells) {
+    int ts = 0, tk = 0;
+    stripe_tile_shape(acc, fp32, &ts, &tk, sh);
+    int64_t t = 0;
+    for (size_t i = 0; i < n_tabs; i++) t += (int64_t)((n[i] / 2 + ts - 1) / ts) * ((n[i] + tk - 1) / tk);
+    *cells = t * ts * tk;
+    return t;
+  };
+  SmallPlan p{shape, chunk, false};
+  int64_t cells = 0;
+  int64_t tiles = tiles_of(shape, &cells);
+  const int small = stripe_small_shape(acc, fp32);
+  if (shape_free && shape != small) {
+    // the small tiles stage twice the bytes per update; FP64 generalized and
+    // variance-adjusted updates are bound by the FP64 pipe either way
+    const double rate = !fp32 && acc != ACC_MIN ? 1.0 : 0.85;
+    int64_t cells_s = 0;
+    const int64_t tiles_s = tiles_of(small, &cells_s);
+    if ((double)cells_s < rate * (double)cells) {
+      p.shape = small;
+      tiles = tiles_s;
+    }
+  }
+  // units in flight: CTAs of 256 threads run two per SM (FP64 generalized and
+  // variance-adjusted: one), the small ones eight
+  const int64_t slots = (int64_t)sms * (p.shape == small ? 8 : (!fp32 && acc != ACC_MIN ? 1 : 2)), want = 4 * slots;
+  // kernels whose chunk is tuned are cut only where the smallest candidate
+  // leaves under two waves (1,003 samples generalized, three waves of tuned
+  // units: cut to four they took 2 % longer)
+  const bool tuned = fp32 || acc != ACC_MIN;
+  const int64_t least = tuned ? std::min(chunk, 1024) : chunk;
+  if (tiles > 0 && tiles * ((rows + least - 1) / least) < (tuned ? 2 * slots : want)) {
+    const int step = acc == ACC_MIN && fp32 ? B1 : 16;
+    const int64_t c = ((int64_t)rows * tiles / want + step) / step * step;
+    p.chunk = (int)std::min<int64_t>(chunk, std::max<int64_t>(c, step));
+    p.split = true;
+  }
+  return p;
+}
+
 cudaError_t launch_stripe_acc(int acc, bool fp32, const StripeArgs &a, cudaStream_t st) {
   if (a.rows <= 0 || a.n_tiles <= 0) return cudaSuccess;
   if (acc == ACC_MIN) {
-    if (!fp32) return run_u64<4, 8, 2>(a, st);
-    if (a.abs_mask == 0xFFu) return run_min<8, 8, 0xFFu, 2>(a, st);
-    return a.shape == 1 ? run_min<4, 8, FP32_ABS_ROW_MASK, 3>(a, st) : run_min<8, 8, FP32_ABS_ROW_MASK, 2>(a, st);
+    if (!fp32) return a.shape == 1 ? run_u64<4, 8, 8, 8>(a, st) : run_u64<4, 8, 16, 2>(a, st);
+    if (a.abs_mask == 0xFFu)
+      return a.shape == 2 ? run_min<4, 8, 8, 0xFFu, 8>(a, st) : run_min<8, 8, 16, 0xFFu, 2>(a, st);
+    if (a.shape == 2) return run_min<4, 8, 8, FP32_ABS_ROW_MASK, 8>(a, st);
+    return a.shape == 1 ? run_min<4, 8, 16, FP32_ABS_ROW_MASK, 3>(a, st)
+                        : run_min<8, 8, 16, FP32_ABS_ROW_MASK, 2>(a, st);
   }
-  if (acc == ACC_VAW) return fp32 ? run_vaw<float, 4, 4, 2>(a, st) : run_vaw<double, 4, 4, 1>(a, st);
+  const bool small = a.shape == 1;
+  if (acc == ACC_VAW) {
+    if (fp32) return small ? run_vaw<float, 4, 4, 8, 8>(a, st) : run_vaw<float, 4, 4, 16, 2>(a, st);
+    return small ? run_vaw<double, 4, 4, 8, 4>(a, st) : run_vaw<double, 4, 4, 16, 1>(a, st);
+  }
   const bool half = a.alpha == 0.5;
-  if (fp32) return half ? run_gen<float, 4, 8, 0, 2>(a, st) : run_gen<float, 4, 8, 1, 2>(a, st);
-  return half ? run_gen<double, 4, 8, 0, 1>(a, st) : run_gen<double, 4, 8, 1, 1>(a, st);
+  if (fp32) {
+    if (small) return half ? run_gen<float, 4, 8, 8, 0, 8>(a, st) : run_gen<float, 4, 8, 8, 1, 8>(a, st);
+    return half ? run_gen<float, 4, 8, 16, 0, 2>(a, st) : run_gen<float, 4, 8, 16, 1, 2>(a, st);
+  }
+  if (small) return half ? run_gen<double, 4, 8, 8, 0, 4>(a, st) : run_gen<double, 4, 8, 8, 1, 4>(a, st);
+  return half ? run_gen<double, 4, 8, 16, 0, 1>(a, st) : run_gen<double, 4, 8, 16, 1, 1>(a, st);
 }
 
 size_t diag_scratch_bytes(bool fp32, int rows, int n_cols) {
   if (!fp32) return 0;
-  // sub-blocks of any chunk size >= 1,024 rows that is a multiple of B1
-  const int64_t n_sb = (rows + B1 - 1) / B1 + (rows + 1023) / 1024;
+  // one sub-block of B1 rows after another (chunks are multiples of B1)
+  const int64_t n_sb = (rows + B1 - 1) / B1;
   return (size_t)std::max<int64_t>(n_sb, 1) * n_cols * 4;
 }
 

@@ -55,7 +55,7 @@ def test_tile_edges(n):
 @pytest.mark.parametrize("tips", [2, 4, 5, 8, 9, 13, 33, 1024, 1025, 1030, 2100])
 def test_row_edges(tips):
     tree_s = yule_tree(tips, seed=720 + tips)
-    check(tree_s, table_iid(21, tips, max(0.05, 3.0 / tips), seed=721 + tips), f"tips={tips}")
+    check(tree_s, table_iid(21, tips, min(1.0, max(0.05, 3.0 / tips)), seed=721 + tips), f"tips={tips}")
 
 
 def test_lengths_of_every_size():
