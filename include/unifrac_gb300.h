@@ -85,8 +85,9 @@ typedef enum {
  * end with one FP64 num / den division.
  * UF_FP64   branch embeddings in IEEE FP64.  Weighted and unweighted methods:
  *           each embedded value rounded once to a 64-bit fixed-point grid
- *           (about 2^-60 of a root-to-tip distance), every per-branch update
- *           and sum after that in exact integers.  Generalized and
+ *           (about 2^-60 of a root-to-tip distance; UF_UNWEIGHTED, on the
+ *           tensor cores, lengths to 2^-63 of the longest), every per-branch
+ *           update and sum after that in exact integers.  Generalized and
  *           variance-adjusted: per-branch updates in FP64 on CUDA cores,
  *           partial sums in FP64 before each fixed-point rounding, every
  *           numerator a sum of nonnegative terms (no cancellation).
@@ -153,9 +154,10 @@ typedef struct {
  *                    branches per embedding block (>= 1), e.g. to bound memory
  *   "kernel_timing"  0 (default) or 1: time each phase with CUDA events and
  *                    fill the t_*_ms fields of uf_report (adds a stream sync)
- *   "tensor_path"    1 (default): UF_UNWEIGHTED with UF_MIXED runs on the
+ *   "tensor_path"    1 (default): UF_UNWEIGHTED runs on the
  *                    tcgen05 tensor cores when the gram tiles its stripes need
- *                    (128 x 256 int64 cells each, the diagonal tiles included)
+ *                    (128 x 256 int64 cells each, two words with UF_FP64, the
+ *                    diagonal tiles included)
  *                    and the sparse rows' stripe cells fit in half the device
  *                    memory that is free or held unused by the stream-ordered
  *                    pool, else on the CUDA-core stripe kernels
@@ -284,7 +286,7 @@ int64_t uf_table_samples(const uf_table *table);
  * device and is returned before the work completes on the stream.
  * Errors: UF_EINVAL, UF_ERANGE, UF_ETABLE (table of another tree),
  *   UF_ENOMEM, UF_ECUDA; UF_ETIMEOUT when a bounded wait of the tensor-core
- *   kernel (unweighted, mixed) ran out.  An asynchronous call does not wait
+ *   kernel (unweighted) ran out.  An asynchronous call does not wait
  *   to learn that: every value it writes is then NaN instead.
  */
 uf_status uf_compute(const uf_tree *tree, const uf_table *table, uf_method method, double alpha,

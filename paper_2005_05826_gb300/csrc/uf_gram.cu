@@ -9,8 +9,19 @@
 // l = l_hi + l_mid + l_lo (each product is exact; the sum of the three terms
 // carries l to about 24 bits), accumulated in FP32 in tensor memory.
 //
-// Layout: Pl[4][npad_tot][K_pad] BF16, plane 0 = P, planes 1-3 = A_hi, A_mid,
-// A_lo, branches contiguous (K-major for both MMA operands); the tables of a
+// FP64 calls take the same contraction exactly: each length is a 63-bit fixed
+// point integer in seven signed digits of 9 bits (-256 .. 255, exact in BF16),
+// A_t = P diag(digit t), and a digit's sum over a unit is an integer below
+// 2^23, so FP32 accumulation holds it exactly (the error-free splitting of
+// Ozaki et al., Numer. Algorithms 59, 2012, on integer digits).  A unit sums
+// two digits in two accumulators and adds them, shifted to their places, to
+// two-word fixed point: num and den are then exact up to the rounding of a
+// length to 2^-63 of the longest one.  It replaces 64-bit integer sums on the
+// CUDA cores (3.6e12 updates/s): seven digits at the tensor cores' BF16 rate
+// are 7/3 of the mixed call's time.
+//
+// Layout: Pl[4][npad_tot][K_pad] BF16 (FP64: [8]), plane 0 = P, planes 1-3 = A_hi, A_mid,
+// A_lo (1-7: the digits), branches contiguous (K-major for both MMA operands); the tables of a
 // batch occupy consecutive row ranges of every plane.  A work unit is
 // (K chunk of `kc` branches, tile of GM = 128 samples i x GN = 256 samples j of
 // one table).  Only the tiles a call needs are scheduled and stored: those
@@ -26,8 +37,9 @@
 // order-free, so the result does not depend on the order chunks land in.
 //
 // Roles (192 threads): warp 0 issues TMA loads (128-byte swizzled boxes into a
-// two-stage ring), warp 1 allocates tensor memory and issues the MMAs, warps
-// 2-5 drain the accumulators.  Every wait on an mbarrier gives up after two
+// two-stage ring; FP64: three stages of two digit boxes), warp 1 allocates tensor
+// memory and issues the MMAs, warps
+// 2-5 drain the accumulators (FP64: one pair, drained before the next unit).  Every wait on an mbarrier gives up after two
 // seconds, raises an abort flag seen by all roles and reports through
 // `err`; the kernel then waits (again bounded) for its own outstanding copies
 // and MMAs, frees its tensor memory and returns.
@@ -47,11 +59,16 @@ namespace {
 constexpr int GM = GRAM_TM;                          // samples i per tile (TMEM lanes)
 constexpr int GN = GRAM_TN;                          // samples j per tile (TMEM columns)
 constexpr int GK = 64;                               // branches per stage: 128 bytes of BF16
-constexpr int NSPLIT = 3;
-constexpr int GSTAGES = 2;
 constexpr int A_BYTES = GM * GK * 2;                 // 16 KB
 constexpr int B_BYTES = GN * GK * 2;                 // 32 KB
-constexpr int STAGE_BYTES = NSPLIT * A_BYTES + B_BYTES;  // 80 KB
+// A boxes per stage and stages: 2 x 80 KB, or 3 x 64 KB with digits
+template <bool DIGITS>
+struct GramGeo {
+  static constexpr int NA = DIGITS ? 2 : GRAM_SPLITS;
+  static constexpr int STAGES = DIGITS ? 3 : 2;
+  static constexpr int STAGE_BYTES = NA * A_BYTES + B_BYTES;
+  static constexpr size_t SMEM = (size_t)STAGES * STAGE_BYTES + 1024;
+};
 constexpr int G_THREADS = 192;
 constexpr uint32_t TMEM_COLS = 512;                  // two accumulator buffers of GN columns
 constexpr unsigned long long WAIT_NS = 2000000000ull;  // bounded waits: 2 s
@@ -142,14 +159,33 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
+        "=r"(r[15])
+      : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+
 struct GUnit {
   int t;               // stored tile
   int bi, bj, k0, nk;  // its block coordinates, first branch and number of GK steps
   int n, row_base;
+  int a0, na;          // first A plane and number of A planes
 };
 
+// Unit u: chunk-major, with digits then pair of digits, then tile.
+template <bool DIGITS>
 __device__ __forceinline__ GUnit gram_unit(const GramArgs &a, int u) {
-  const int c = u / a.n_tiles, t = u - c * a.n_tiles;
+  int c = u / a.n_tiles;
+  const int t = u - c * a.n_tiles;
+  int pair = 0;
+  if constexpr (DIGITS) {
+    pair = c % GRAM_PAIRS;
+    c /= GRAM_PAIRS;
+  }
   const GramTab &tb = a.tabs[a.tile_tab[t]];
   GUnit g;
   g.t = t;
@@ -159,11 +195,16 @@ __device__ __forceinline__ GUnit gram_unit(const GramArgs &a, int u) {
   g.nk = (min(a.kc, a.k_len - g.k0) + GK - 1) / GK;
   g.n = tb.n;
   g.row_base = tb.row_base;
+  g.a0 = DIGITS ? 1 + 2 * pair : 1;
+  g.na = DIGITS ? min(2, GRAM_DIGITS - 2 * pair) : GRAM_SPLITS;
   return g;
 }
 
+template <bool DIGITS>
 __global__ void __launch_bounds__(G_THREADS, 1)
     k_gram(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, const GramArgs a) {
+  using GG = GramGeo<DIGITS>;
+  constexpr int GSTAGES = GG::STAGES, STAGE_BYTES = GG::STAGE_BYTES, NA = GG::NA;
   extern __shared__ unsigned char smem_dyn[];
   unsigned char *smem = (unsigned char *)(((uintptr_t)smem_dyn + 1023) & ~(uintptr_t)1023);
   __shared__ __align__(8) uint64_t full[GSTAGES], empty[GSTAGES], acc_full[2], acc_empty[2], mma_done, never;
@@ -200,18 +241,18 @@ __global__ void __launch_bounds__(G_THREADS, 1)
     // ---- producer: TMA loads into the stage ring ----
     int stage = 0;
     uint32_t phase = 0;
-    uint32_t armed[GSTAGES] = {0, 0};  // times each stage was armed
+    uint32_t armed[GSTAGES] = {};  // times each stage was armed
     for (int u = blockIdx.x; u < a.n_units && !s_abort; u += gridDim.x) {
-      const GUnit g = gram_unit(a, u);
+      const GUnit g = gram_unit<DIGITS>(a, u);
       for (int ks = 0; ks < g.nk; ks++) {
         if (!mbar_wait(&empty[stage], phase ^ 1, &s_abort)) break;
-        mbar_expect_tx(&full[stage], STAGE_BYTES);
+        mbar_expect_tx(&full[stage], g.na * A_BYTES + B_BYTES);
         armed[stage]++;
         unsigned char *base = smem + stage * STAGE_BYTES;
         const int kx = g.k0 + ks * GK;
-        for (int t = 0; t < NSPLIT; t++)
-          tma_load_2d(base + t * A_BYTES, &mapA, &full[stage], kx, (1 + t) * a.npad_tot + g.row_base + g.bi * GM);
-        tma_load_2d(base + NSPLIT * A_BYTES, &mapB, &full[stage], kx, g.row_base + g.bj * GN);
+        for (int t = 0; t < g.na; t++)
+          tma_load_2d(base + t * A_BYTES, &mapA, &full[stage], kx, (g.a0 + t) * a.npad_tot + g.row_base + g.bi * GM);
+        tma_load_2d(base + NA * A_BYTES, &mapB, &full[stage], kx, g.row_base + g.bj * GN);
         if (++stage == GSTAGES) {
           stage = 0;
           phase ^= 1;
@@ -232,9 +273,10 @@ __global__ void __launch_bounds__(G_THREADS, 1)
     int ul = 0;
     if (a.wait_test) mbar_wait(&never, 0, &s_abort);  // runs out after WAIT_NS and raises the abort
     for (int u = blockIdx.x; u < a.n_units && !s_abort; u += gridDim.x, ul++) {
-      const GUnit g = gram_unit(a, u);
-      const int b = ul & 1;
-      if (!mbar_wait(&acc_empty[b], ((ul >> 1) & 1) ^ 1, &s_abort)) break;
+      const GUnit g = gram_unit<DIGITS>(a, u);
+      // mixed: two accumulators in turn; digits: both at once, one for each
+      const int b = DIGITS ? 0 : ul & 1, use = DIGITS ? ul : ul >> 1;
+      if (!mbar_wait(&acc_empty[b], (use & 1) ^ 1, &s_abort)) break;
       tc_fence_after();
       const uint32_t d = tmem + (uint32_t)(b * GN);
       bool ok = true;
@@ -245,11 +287,11 @@ __global__ void __launch_bounds__(G_THREADS, 1)
         }
         tc_fence_after();
         const uint32_t base = smem_u32(smem + stage * STAGE_BYTES);
-        for (int t = 0; t < NSPLIT; t++)
+        for (int t = 0; t < g.na; t++)
 #pragma unroll
           for (int k = 0; k < GK / 16; k++)
-            mma_bf16(d, desc_sw128(base + t * A_BYTES + k * 32), desc_sw128(base + NSPLIT * A_BYTES + k * 32),
-                     (ks | t | k) != 0);
+            mma_bf16(DIGITS ? d + (uint32_t)(t * GN) : d, desc_sw128(base + t * A_BYTES + k * 32),
+                     desc_sw128(base + NA * A_BYTES + k * 32), DIGITS ? (ks | k) != 0 : (ks | t | k) != 0);
         mma_commit(&empty[stage]);
         if (++stage == GSTAGES) {
           stage = 0;
@@ -268,24 +310,51 @@ __global__ void __launch_bounds__(G_THREADS, 1)
     // ---- epilogue: TMEM -> fixed point -> atomics into Gt ----
     const int quarter = warp & 3;  // the TMEM lane quarter this warp may access
     const int row = quarter * 32 + lane;
-    const float scale = (float)a.scale;
+    [[maybe_unused]] const float scale = (float)a.scale;
     int ul = 0;
     for (int u = blockIdx.x; u < a.n_units && !s_abort; u += gridDim.x, ul++) {
-      const GUnit g = gram_unit(a, u);
-      const int b = ul & 1;
-      if (!mbar_wait(&acc_full[b], (ul >> 1) & 1, &s_abort)) break;
+      const GUnit g = gram_unit<DIGITS>(a, u);
+      const int b = DIGITS ? 0 : ul & 1, use = DIGITS ? ul : ul >> 1;
+      if (!mbar_wait(&acc_full[b], use & 1, &s_abort)) break;
       tc_fence_after();
       const int i = g.bi * GM + row;
       unsigned long long *tile = a.Gt + (int64_t)g.t * GRAM_TILE_CELLS + row;
-      for (int c = 0; c < GN / 32; c++) {
-        uint32_t r[32];
-        tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * GN + c * 32), r);
+      const uint32_t lanes = tmem + ((uint32_t)(quarter * 32) << 16);
+      if constexpr (DIGITS) {
+        // (S0 + 512 S1) 2^(18 pair + digit_shift) in units of 2^-(F+32)
+        const int sh = GRAM_DIGIT_BITS * (g.a0 - 1) + a.digit_shift;
+        for (int c = 0; c < GN / 16; c++) {
+          uint32_t r0[16], r1[16];
+          tmem_ld16(lanes + (uint32_t)(c * 16), r0);
+          if (g.na == 2) tmem_ld16(lanes + (uint32_t)(GN + c * 16), r1);
 #pragma unroll
-        for (int q = 0; q < 32; q++) {
-          const int j = g.bj * GN + c * 32 + q;
-          if (i <= j && j < g.n) {
-            const long long v = __float2ll_rn(__uint_as_float(r[q]) * scale);
-            atomicAdd(tile + (c * 32 + q) * GM, (unsigned long long)v);
+          for (int q = 0; q < 16; q++) {
+            const int j = g.bj * GN + c * 16 + q;
+            if (i <= j && j < g.n) {
+              long long v = (long long)__float2int_rn(__uint_as_float(r0[q]));
+              if (g.na == 2) v += (long long)__float2int_rn(__uint_as_float(r1[q])) << GRAM_DIGIT_BITS;
+              if (v == 0) continue;
+              unsigned long long *cell = tile + (c * 16 + q) * GM;
+              if (sh >= 32) {
+                atomicAdd(cell, (unsigned long long)v << (sh - 32));
+              } else {
+                atomicAdd(cell, (unsigned long long)(v >> (32 - sh)));
+                atomicAdd(cell + a.gt_lo, ((unsigned long long)v << sh) & 0xffffffffull);
+              }
+            }
+          }
+        }
+      } else {
+        for (int c = 0; c < GN / 32; c++) {
+          uint32_t r[32];
+          tmem_ld32(lanes + (uint32_t)(b * GN + c * 32), r);
+#pragma unroll
+          for (int q = 0; q < 32; q++) {
+            const int j = g.bj * GN + c * 32 + q;
+            if (i <= j && j < g.n) {
+              const long long v = __float2ll_rn(__uint_as_float(r[q]) * scale);
+              atomicAdd(tile + (c * 32 + q) * GM, (unsigned long long)v);
+            }
           }
         }
       }
@@ -315,14 +384,16 @@ __device__ __forceinline__ int gram_table_of_row(const GramTab *tabs, int n_tabs
 }
 
 // Presence and split-length planes of a branch block, transposed to
-// sample-major: Pl[0][k][e] = presence flag, Pl[1 + t][k][e] = presence * l_t,
+// sample-major: Pl[0][k][e] = presence flag, Pl[1 + t][k][e] = presence * l_t
+// (term or digit t of the length),
 // for every plane row k (padding rows of a table are 0).  Branch e of the
 // block is node nodes[e] (b0 + e without a list).
+template <bool DIGITS>
 __global__ void k_gram_prep(int64_t b0, const int32_t *__restrict__ nodes, int rows, int k_len,
                             const int32_t *__restrict__ slot_of_node,
                             const uint8_t *__restrict__ flags, int64_t ld, const double *__restrict__ length,
                             const GramTab *__restrict__ tabs, int n_tabs, int npad_tot, int64_t K_pad,
-                            __nv_bfloat16 *__restrict__ Pl) {
+                            __nv_bfloat16 *__restrict__ Pl, double digit_scale) {
   __shared__ float tile[32][33];
   const int e_base = blockIdx.x * 32, k_base = blockIdx.y * 32;
   {
@@ -346,10 +417,25 @@ __global__ void k_gram_prep(int64_t b0, const int32_t *__restrict__ nodes, int r
   __syncthreads();
   const int e = e_base + threadIdx.x;
   double l = e < rows ? length[nodes ? (int64_t)nodes[e] : b0 + e] : 0.0;
-  const __nv_bfloat16 hi = __double2bfloat16(l);
-  const double r1 = l - (double)__bfloat162float(hi);
-  const __nv_bfloat16 mid = __double2bfloat16(r1);
-  const __nv_bfloat16 lo = __double2bfloat16(r1 - (double)__bfloat162float(mid));
+  constexpr int NT = DIGITS ? GRAM_DIGITS : GRAM_SPLITS;
+  __nv_bfloat16 term[NT];
+  if constexpr (DIGITS) {
+    long long x = __double2ll_rn(l * digit_scale);
+#pragma unroll
+    for (int t = 0; t < NT; t++) {
+      constexpr long long HALF = 1ll << (GRAM_DIGIT_BITS - 1);
+      const long long d = ((x + HALF) & (2 * HALF - 1)) - HALF;
+      term[t] = __float2bfloat16((float)d);
+      x = (x - d) >> GRAM_DIGIT_BITS;
+    }
+  } else {
+    double r = l;
+#pragma unroll
+    for (int t = 0; t < NT; t++) {
+      term[t] = __double2bfloat16(r);
+      r -= (double)__bfloat162float(term[t]);
+    }
+  }
   const __nv_bfloat16 zero = __float2bfloat16(0.f), one = __float2bfloat16(1.f);
   if (e >= k_len) return;
   const int64_t plane = (int64_t)npad_tot * K_pad;
@@ -359,25 +445,34 @@ __global__ void k_gram_prep(int64_t b0, const int32_t *__restrict__ nodes, int r
     const bool on = tile[threadIdx.x][kl] != 0.f;
     const int64_t at = (int64_t)k * K_pad + e;
     Pl[at] = on ? one : zero;
-    Pl[plane + at] = on ? hi : zero;
-    Pl[2 * plane + at] = on ? mid : zero;
-    Pl[3 * plane + at] = on ? lo : zero;
+#pragma unroll
+    for (int t = 0; t < NT; t++) Pl[(1 + t) * plane + at] = on ? term[t] : zero;
   }
+}
+
+// One accumulator as an integer in units of 2^-F (one word) or 2^-(F+32) (two).
+template <typename I>
+__device__ __forceinline__ I word_at(const unsigned long long *p, int64_t i, int64_t lo_off) {
+  if constexpr (sizeof(I) == 8) return (I)(long long)p[i];
+  else return ((I)(long long)p[i] << 32) + (I)(long long)p[i + lo_off];
 }
 
 // Cell (i, j), i <= j, of a table's gram matrix from the compact tiles, or -1
 // (never for a cell of the call's stripes or the diagonal).
-__device__ __forceinline__ long long gram_cell(const GramFinalArgs &a, int64_t i, int64_t j) {
+template <typename I>
+__device__ __forceinline__ I gram_cell(const GramFinalArgs &a, int64_t i, int64_t j) {
   const int64_t bi = i / GM, bj = j / GN;
   const int t = a.tile_map[bi * (a.n_pad / GN) + bj];
   if (t < 0) return -1;
-  return (long long)a.Gt[(int64_t)t * GRAM_TILE_CELLS + (j - bj * GN) * GM + (i - bi * GM)];
+  return word_at<I>(a.Gt, (int64_t)t * GRAM_TILE_CELLS + (j - bj * GN) * GM + (i - bi * GM), a.gt_lo);
 }
 
 // Gram accumulators (plus the sparse rows' terms) -> distances for stripes [s0, s1).
+template <typename I>
 __global__ void k_finalize_gram(const GramFinalArgs a) {
   const int64_t rows = a.s1 - a.s0;
   const int64_t total = rows * a.n;
+  const double inv_scale = sizeof(I) == 8 ? a.inv_scale : a.inv_scale / 4294967296.0;
   const bool aborted = a.err && *a.err != 0;  // a bounded wait gave up: no distance is valid
   unsigned long long clamped = 0;
   for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < total;
@@ -389,23 +484,23 @@ __global__ void k_finalize_gram(const GramFinalArgs a) {
     if (j >= a.n) j -= a.n;
     if (a.full && 2 * (s + 1) == a.n && k >= a.n / 2) continue;
     const int64_t lo = k < j ? k : j, hi = k < j ? j : k;
-    long long g = gram_cell(a, lo, hi);
-    long long wl = gram_cell(a, lo, lo), wh = gram_cell(a, hi, hi);
+    I g = gram_cell<I>(a, lo, hi);
+    I wl = gram_cell<I>(a, lo, lo), wh = gram_cell<I>(a, hi, hi);
     const bool missing = g < 0 || wl < 0 || wh < 0;
-    if (a.Msp) g += (long long)a.Msp[c];
+    if (a.Msp) g += word_at<I>(a.Msp, c, a.m_lo_off);
     if (a.Dsp) {
-      wl += (long long)a.Dsp[lo];
-      wh += (long long)a.Dsp[hi];
+      wl += word_at<I>(a.Dsp, lo, a.d_lo_off);
+      wh += word_at<I>(a.Dsp, hi, a.d_lo_off);
     }
-    const long long w = wl + wh;
-    long long num = w - 2 * g;
-    const long long den = w - g;
+    const I w = wl + wh;
+    I num = w - 2 * g;
+    const I den = w - g;
     if (num < 0) {
       clamped++;
       num = 0;
     }
     const double val = (aborted || missing) ? __longlong_as_double(0x7ff8000000000000ll)
-                       : a.unnormalized    ? (double)num * a.inv_scale
+                       : a.unnormalized    ? (double)num * inv_scale
                        : den > 0           ? (double)num / (double)den
                                            : 0.0;
     const int64_t idx = a.full ? (int64_t)a.n * lo - lo * (lo + 1) / 2 + (hi - lo - 1) : c;
@@ -459,22 +554,23 @@ void gram_tiles(int n, int64_t s0, int64_t s1, std::vector<int32_t> *bi, std::ve
     }
 }
 
-size_t gram_smem_bytes() { return (size_t)GSTAGES * STAGE_BYTES + 1024; }
-
 cudaError_t launch_gram_prep(int64_t b0, int rows, const int32_t *slot_of_node, const uint8_t *flags,
                              int64_t ld, const double *length, const GramTab *tabs, int n_tabs,
-                             int npad_tot, int64_t K_pad, void *Pl, cudaStream_t st, const int32_t *nodes) {
+                             int npad_tot, int64_t K_pad, void *Pl, cudaStream_t st, const int32_t *nodes,
+                             double digit_scale) {
   const int k_len = (int)((rows + GK - 1) / GK * GK);
   dim3 grid((k_len + 31) / 32, (npad_tot + 31) / 32), block(32, 8);
-  return launch_k(k_gram_prep, grid, block, 0, st, b0, nodes, rows, k_len, slot_of_node, flags, ld, length, tabs,
-                  n_tabs, npad_tot, K_pad, (__nv_bfloat16 *)Pl);
+  return launch_k(digit_scale != 0.0 ? k_gram_prep<true> : k_gram_prep<false>, grid, block, 0, st, b0, nodes, rows,
+                  k_len, slot_of_node, flags, ld, length, tabs, n_tabs, npad_tot, K_pad, (__nv_bfloat16 *)Pl,
+                  digit_scale);
 }
 
 cudaError_t launch_gram(const GramArgs &a0, void *Pl, int64_t K_pad, cudaStream_t st) {
   EncodeTiledFn enc = encode_fn();
   if (!enc) return cudaErrorNotSupported;
   CUtensorMap mapA, mapB;
-  const cuuint64_t dims[2] = {(cuuint64_t)K_pad, (cuuint64_t)4 * a0.npad_tot};
+  const cuuint64_t dims[2] = {(cuuint64_t)K_pad,
+                              (cuuint64_t)(1 + (a0.digits ? GRAM_DIGITS : GRAM_SPLITS)) * a0.npad_tot};
   const cuuint64_t strides[1] = {(cuuint64_t)K_pad * 2};
   const cuuint32_t boxA[2] = {GK, GM}, boxB[2] = {GK, GN}, es[2] = {1, 1};
   if (enc(&mapA, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Pl, dims, strides, boxA, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -486,16 +582,17 @@ cudaError_t launch_gram(const GramArgs &a0, void *Pl, int64_t K_pad, cudaStream_
           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return cudaErrorInvalidValue;
   GramArgs a = a0;
-  a.n_units = ((a.k_len + a.kc - 1) / a.kc) * a.n_tiles;
+  a.n_units = ((a.k_len + a.kc - 1) / a.kc) * a.n_tiles * (a.digits ? GRAM_PAIRS : 1);
   if (a.n_units <= 0) return cudaSuccess;
-  const size_t smem = gram_smem_bytes();
-  cudaError_t e = cudaFuncSetAttribute(k_gram, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const size_t smem = a.digits ? GramGeo<true>::SMEM : GramGeo<false>::SMEM;
+  auto kernel = a.digits ? k_gram<true> : k_gram<false>;
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
   const int grid = std::max(1, std::min(a.n_units, sms));
-  return launch_k(k_gram, dim3(grid), dim3(G_THREADS), smem, st, mapA, mapB, a);
+  return launch_k(kernel, dim3(grid), dim3(G_THREADS), smem, st, mapA, mapB, a);
 }
 
 cudaError_t launch_finalize_gram(const GramFinalArgs &a, cudaStream_t st) {
@@ -507,7 +604,8 @@ cudaError_t launch_finalize_gram(const GramFinalArgs &a, cudaStream_t st) {
   if (e != cudaSuccess) return e;
   int64_t blocks = (total + 255) / 256;
   blocks = std::min<int64_t>(blocks, (int64_t)std::max(sms, 1) * 64);  // a grid-stride loop beyond that
-  k_finalize_gram<<<(int)blocks, 256, 0, st>>>(a);
+  if (a.gt_lo != 0) k_finalize_gram<__int128><<<(int)blocks, 256, 0, st>>>(a);
+  else k_finalize_gram<long long><<<(int)blocks, 256, 0, st>>>(a);
   return cudaGetLastError();
 }
 

@@ -19,9 +19,20 @@ struct GramTab {
   int off;              // first column on the combined sample axis
   int64_t map_off;      // first entry of its tile map
 };
+// Terms of a branch length in the A planes: mixed, three BF16 terms of its
+// value; FP64, seven signed digits of GRAM_DIGIT_BITS bits of its 63-bit fixed
+// point (integers -256 .. 255, exact in BF16), summed two at a time.
+constexpr int GRAM_SPLITS = 3;
+constexpr int GRAM_DIGITS = 7;
+constexpr int GRAM_DIGIT_BITS = 9;
+constexpr int GRAM_PAIRS = (GRAM_DIGITS + 1) / 2;
+// A digit's sum over a unit is an integer of at most 256 x GRAM_DIGIT_KC:
+// below 2^23, so that FP32 accumulation is exact.
+constexpr int GRAM_DIGIT_KC = 16384;
 struct GramArgs {
+  int digits;           // 1: FP64 (digit planes, exact sums), 0: mixed
   int k_len;            // branches of this block, rounded up to 64
-  int kc;               // branches per work unit (multiple of 64)
+  int kc;               // branches per work unit (multiple of 64; FP64: at most GRAM_DIGIT_KC)
   int n_tiles;          // tiles of all tables
   int n_units;          // set by launch_gram
   int npad_tot;         // plane rows (sum of n_pad)
@@ -30,6 +41,10 @@ struct GramArgs {
   // fixed point, compact tiles: cell (i, j), i <= j, of stored tile t with
   // block coordinates (bi, bj) at t * GRAM_TILE_CELLS + (j - bj GRAM_TN) GRAM_TM + (i - bi GRAM_TM)
   unsigned long long *Gt;
+  // FP64: second words (units of 2^-(F+32)) this many elements on, and the
+  // digits' unit 2^(digit_shift - F - 32), 0 <= digit_shift
+  int64_t gt_lo;
+  int digit_shift;
   double scale;         // 2^F
   int *err;             // set to 1 when a bounded wait gave up
   int wait_test;        // 1: the MMA issuer first waits on a barrier nothing signals, so its
@@ -44,6 +59,8 @@ struct GramFinalArgs {
   // sparse rows (uf_sparse.cu, min form on presence rows), or null: pair terms
   // in the stripe layout [(s1 - s0)][n] and per-sample terms [n]
   const unsigned long long *Msp, *Dsp;
+  // FP64 calls: second words of Gt, Msp and Dsp this many elements on; 0: one word
+  int64_t gt_lo, m_lo_off, d_lo_off;
   void *out;
   int out_fp32;
   const int *err;                // the gram kernel's abort flag: when set, every output is NaN
@@ -58,11 +75,12 @@ int64_t gram_kpad(int rows);              // branches rounded up to the stage
 // Stripe s holds the pairs at distance d = j - i of s + 1 and n - s - 1.
 void gram_tiles(int n, int64_t s0, int64_t s1, std::vector<int32_t> *bi, std::vector<int32_t> *bj);
 // planes of branches nodes[0 .. rows) (b0 .. b0 + rows - 1 when nodes is null)
-// from their presence flags
+// from their presence flags: 1 + GRAM_SPLITS planes, or with digit_scale != 0
+// (2^g, every length x 2^g below 2^62) 1 + GRAM_DIGITS
 cudaError_t launch_gram_prep(int64_t b0, int rows, const int32_t *slot_of_node, const uint8_t *flags,
                              int64_t ld, const double *length, const GramTab *tabs, int n_tabs,
                              int npad_tot, int64_t K_pad, void *Pl, cudaStream_t st,
-                             const int32_t *nodes = nullptr);
+                             const int32_t *nodes = nullptr, double digit_scale = 0.0);
 cudaError_t launch_gram(const GramArgs &a, void *Pl, int64_t K_pad, cudaStream_t st);
 cudaError_t launch_finalize_gram(const GramFinalArgs &a, cudaStream_t st);
 

@@ -778,7 +778,8 @@ int64_t stripe_cells(const BatchJob &J) {
   return c;
 }
 
-// Unweighted, mixed precision, on the tensor cores: per branch block, counts
+// Unweighted on the tensor cores (mixed: three BF16 terms per length; FP64:
+// seven exact digits and two-word sums): per branch block, counts
 // -> presence / split-length planes of every table -> tcgen05 gram into the
 // stored tiles; the sparse rows scatter into stripe-layout cells; then the
 // gram finalize of every table.  Throws CudaFail on CUDA errors.
@@ -797,19 +798,24 @@ uf_status run_gram(uf_tree *tree, const BatchJob &J, int device, double scale) {
   const int n_cols = G.n_cols, npad_tot = G.npad_tot;
   const int n_tiles = (int)G.n_tiles;
   const int64_t nb = tree->n_nodes - 1;
-  const double tile_bytes = (double)G.n_tiles * GRAM_TILE_CELLS * 8.0;
-  const int64_t rows = block_rows(nb, (double)n_cols + 4.0 * npad_tot * 2.0 + 8.0, tile_bytes + cells * 8.0);
+  const bool digits = !J.fp32;
+  const int words = digits ? 2 : 1, planes = 1 + (digits ? GRAM_DIGITS : GRAM_SPLITS);
+  const int64_t gt_cells = std::max<int64_t>(G.n_tiles, 1) * GRAM_TILE_CELLS;
+  const int64_t rows = block_rows(nb, (double)n_cols + 2.0 * planes * npad_tot + 8.0,
+                                  ((double)gt_cells + (double)cells) * 8.0 * words);
   Inputs in = [&] {
     NvtxRange r("uf: bind inputs");
     return bind_inputs(tree, J, device, rows);
   }();
   const std::shared_ptr<const RowSplit> split_p = [&] {
     NvtxRange r("uf: branch split");
-    return get_split(tree, J, in.P, SPLIT_GRAM, true);
+    return get_split(tree, J, in.P, SPLIT_GRAM, J.fp32);
   }();
   const RowSplit &split = *split_p;
   const int64_t K_pad = gram_kpad((int)std::max<int64_t>(split.max_dense, 1));
   cudaStream_t st = J.st;
+  int sms = 0;
+  ck(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device), "cudaDeviceGetAttribute");
   int64_t kernels = 0, acc_launches = 0;
   PhaseTimer timer(g_kernel_timing.load() != 0, st);
   std::vector<int32_t> tl(G.tile_tab);
@@ -818,27 +824,42 @@ uf_status run_gram(uf_tree *tree, const BatchJob &J, int device, double scale) {
   // presence rows: stride rounded up to 16 bytes for the 16-byte level kernel
   const int64_t ld = round_up(n_cols, 16);
   DevBuf flags((size_t)in.P->n_slots * ld, st, "alloc presence rows");
-  DevBuf Pl((size_t)4 * npad_tot * K_pad * 2, st, "alloc presence planes");
-  DevBuf Gt((size_t)std::max<int64_t>(G.n_tiles, 1) * GRAM_TILE_CELLS * 8, st, "alloc gram tiles");
+  DevBuf Pl((size_t)planes * npad_tot * K_pad * 2, st, "alloc presence planes");
+  DevBuf Gt((size_t)gt_cells * 8 * words, st, "alloc gram tiles");
   DevBuf err(sizeof(int), st, "alloc error flag");
   DevBuf clamps(sizeof(unsigned long long), st, "alloc clamp counter");
   DevBuf Msp;
   Meta meta;  // tile list, table descriptors, tile maps and row lists: one staged upload
   const size_t o_tiles = meta.add(tl), o_tabs = meta.add(G.gt), o_maps = meta.add(G.maps);
   const size_t o_cnt = meta.add(split.cnt_lists), o_dense = meta.add(split.dense);
-  // sparse rows: presence terms (x = l) in FP64, one word, min form, into
-  // stripe-layout cells Msp and the per-sample R
+  // sparse rows: presence terms (x = l) in FP64, one word (FP64 calls: two),
+  // min form, into stripe-layout cells Msp and the per-sample R
   SparseScatter sc;
-  sc.prepare(tree, J, in, split, lay, ACC_MIN, true, false, cells, n_cols, meta, st);
+  sc.prepare(tree, J, in, split, lay, ACC_MIN, true, digits, cells, n_cols, meta, st);
   if (split.n_sparse > 0) {
-    Msp = DevBuf((size_t)cells * 8, st, "alloc sparse stripes");
-    ck(cudaMemsetAsync(Msp.p, 0, (size_t)cells * 8, st), "memset");
+    Msp = DevBuf((size_t)cells * 8 * words, st, "alloc sparse stripes");
+    ck(cudaMemsetAsync(Msp.p, 0, (size_t)cells * 8 * words, st), "memset");
+  }
+  // digits: the lengths' grid 2^-g, the longest dense one below 2^62 on it,
+  // no finer than the second words' 2^-(F+32)
+  int digit_shift = 0;
+  double digit_scale = 0.0;
+  if (digits) {
+    double most = 0.0, bound = 0.0;
+    for (double l : split.dense_len) most = std::max(most, l);
+    // (a branch longer than the accumulators' bound is in no sample)
+    for (const TableJob &t : J.tabs) bound = std::max(bound, accum_bound(tree, t.table, EMB_PRESENCE));
+    most = std::min(most, bound);
+    const int f = std::ilogb(scale) + 32;
+    const int g = most > 0.0 ? std::min(f, 61 - std::ilogb(most)) : f;  // most < 2^(ilogb + 1)
+    digit_shift = f - g;
+    digit_scale = std::ldexp(1.0, g);
   }
   meta.upload(st);
   const int32_t *d_tiles = meta.at<int32_t>(o_tiles);
   const GramTab *d_tabs = meta.at<GramTab>(o_tabs);
   const int32_t *d_cnt = meta.at<int32_t>(o_cnt), *d_dense = meta.at<int32_t>(o_dense);
-  ck(cudaMemsetAsync(Gt.p, 0, (size_t)std::max<int64_t>(G.n_tiles, 1) * GRAM_TILE_CELLS * 8, st), "memset");
+  ck(cudaMemsetAsync(Gt.p, 0, (size_t)gt_cells * 8 * words, st), "memset");
   ck(cudaMemsetAsync(err.p, 0, sizeof(int), st), "memset");
   ck(cudaMemsetAsync(clamps.p, 0, sizeof(unsigned long long), st), "memset");
   // the region scatter's pair updates, counted when the call is timed per phase
@@ -873,15 +894,24 @@ uf_status run_gram(uf_tree *tree, const BatchJob &J, int device, double scale) {
     enqueue_split_presence(in, J, off, split, b, d_cnt, flags.as<uint8_t>(), ld, n_cols, ls, &kernels);
     if (nd > 0) {
       ck(launch_gram_prep(b0, (int)nd, in.pd->slot_of_node, flags.as<uint8_t>(), ld, in.td->length, d_tabs,
-                          (int)nt, npad_tot, K_pad, Pl.p, ls, d_dense + d0),
+                          (int)nt, npad_tot, K_pad, Pl.p, ls, d_dense + d0, digit_scale),
          "presence planes");
       kernels++;
     }
     timer.end();
     if (nd == 0 || n_tiles == 0) continue;
     GramArgs ga{};
+    ga.digits = digits;
     ga.k_len = (int)round_up(nd, 64);
     ga.kc = 4096;
+    if (digits) {
+      // the longest units (a drain per unit is not hidden) that still give
+      // four waves of them
+      const int64_t units = (int64_t)n_tiles * GRAM_PAIRS, want = 4 * (int64_t)sms;
+      ga.kc = (int)std::min<int64_t>(GRAM_DIGIT_KC, std::max<int64_t>(512, round_up(ga.k_len * units / want, 64)));
+    }
+    ga.gt_lo = digits ? gt_cells : 0;
+    ga.digit_shift = digit_shift;
     ga.n_tiles = n_tiles;
     ga.npad_tot = npad_tot;
     ga.tile_tab = d_tiles;
@@ -897,7 +927,7 @@ uf_status run_gram(uf_tree *tree, const BatchJob &J, int device, double scale) {
     timer.end();
     kernels++;
     acc_launches++;
-    exec_flops += 2.0 * 3 * (double)GRAM_TILE_CELLS * ga.k_len * n_tiles;
+    exec_flops += 2.0 * (planes - 1) * (double)GRAM_TILE_CELLS * ga.k_len * n_tiles;
   }
   side.join();
   timer.begin(3);
@@ -912,6 +942,9 @@ uf_status run_gram(uf_tree *tree, const BatchJob &J, int device, double scale) {
     fa.tile_map = meta.at<int32_t>(o_maps) + G.gt[t].map_off;
     fa.Msp = Msp.p ? Msp.as<unsigned long long>() + lay[t].m_off : nullptr;
     fa.Dsp = sc.Dsp.p ? sc.Dsp.as<unsigned long long>() + off[t] : nullptr;
+    fa.gt_lo = digits ? gt_cells : 0;
+    fa.m_lo_off = digits ? cells : 0;
+    fa.d_lo_off = digits ? n_cols : 0;
     fa.out = o.dev[t];
     fa.out_fp32 = J.out_fp32;
     fa.err = err.as<int>();
@@ -1366,12 +1399,13 @@ uf_status run_batch(uf_tree *tree, const BatchJob &J) {
   }
   // (the unweighted numerator alone stays on the CUDA-core kernels: the gram
   // gives it as W_i + W_j - 2G, rounded relative to W rather than to itself)
-  if (method == UF_UNWEIGHTED && J.fp32 && g_tensor_path.load()) {
+  if (method == UF_UNWEIGHTED && g_tensor_path.load()) {
     // the tensor path stores the gram tiles the stripes need (and the
     // diagonal) plus the sparse rows' stripe cells; when those do not fit in
     // half the free memory the CUDA-core stripe kernels take the call
     const GramPlan G = gram_plan(J);
-    const double need = (double)G.n_tiles * GRAM_TILE_CELLS * 8.0 + (double)stripe_cells(J) * 8.0;
+    const double need =
+        ((double)G.n_tiles * GRAM_TILE_CELLS + (double)stripe_cells(J)) * 8.0 * (J.fp32 ? 1 : 2);
     if (need <= 0.5 * available_bytes()) return run_gram(tree, J, device, scale);
   }
   return run_stripes(tree, J, device, method, scale);

@@ -36,8 +36,8 @@ RowSplit split_rows(const uf_tree *tree, const BatchJob &J, const Plan *P, int a
   std::vector<char> is_sparse(std::max<int64_t>(nb, 1), 0);
   if (mode != 0) {
     // accumulator words per cell: FP64 terms are two-word fixed point
-    // (uf_device.cuh) except on the tensor path, whose sparse rows keep one
-    const int n_acc = (acc == ACC_GEN ? 2 : 1) * (fp32 || acc == SPLIT_GRAM ? 1 : 2);
+    // (uf_device.cuh)
+    const int n_acc = (acc == ACC_GEN ? 2 : 1) * (fp32 ? 1 : 2);
     double cells = 0.0, cols = 0.0;  // stripe cells of a full run of every table; samples
     for (size_t t = 0; t < nt; t++) {
       const double n = (double)J.tabs[t].table->n;
@@ -55,7 +55,7 @@ RowSplit split_rows(const uf_tree *tree, const BatchJob &J, const Plan *P, int a
     std::vector<double> pair_cost(nt), entry_cost(nt);
     const double n_regions = regions ? sparse_regions(nt, acc, cells * 8.0 * n_acc) : 1.0;
     double dense_rate;  // cell updates per second of the dense kernel
-    if (acc == SPLIT_GRAM) dense_rate = 2.5e14;
+    if (acc == SPLIT_GRAM) dense_rate = fp32 ? 2.5e14 : 2.5e14 * GRAM_SPLITS / GRAM_DIGITS;
     else dense_rate = fp32 ? (acc == ACC_GEN ? 4e12 : 1.3e13) : (acc == ACC_GEN ? 5e10 : 3.5e12);
     const double visit_rate = fp32 ? 2e12 : (acc == ACC_GEN ? 3e10 : 1e12);
     const double job_cost = 5e-10;
