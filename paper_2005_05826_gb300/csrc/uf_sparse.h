@@ -26,7 +26,8 @@ struct SpTab {
 struct SparseArgs {
   const int32_t *nodes;     // sparse branch nodes of this launch
   int n_nodes;
-  int cap;                  // shared-memory capacity in entries (power of two, >= 128)
+  int cap;                  // most entries of a (row, table) run: a power of two, at least
+                            // SPARSE_SMALL_ENTRIES (the shared-memory capacity above that)
   const int32_t *tip_lo, *tip_hi;  // tips of node v: tip numbers [tip_lo[v], tip_hi[v])
   const double *length;     // branch length of every node
   const SpTab *tabs;
@@ -66,6 +67,7 @@ struct SparseArgs {
 };
 // largest subtree entry count a sparse row may have: scattered directly from
 // shared memory, or written as a list (one table, keys alone in shared memory)
+constexpr int SPARSE_SMALL_ENTRIES = 32;  // scattered by a warp
 constexpr int SPARSE_MAX_ENTRIES = 4096;
 constexpr int SPARSE_LIST_MAX_ENTRIES = 16384;
 static_assert(SPARSE_LIST_MAX_ENTRIES <= 65535, "list cursors are 16-bit");

@@ -30,9 +30,10 @@ RowSplit split_rows(const uf_tree *tree, const BatchJob &J, const Plan *P, int a
   const int mode = acc == ACC_VAW ? 0 : (int)g_sparse.load();
   const int64_t nb = tree->n_nodes - 1;
   const size_t nt = J.tabs.size();
-  const int classes[5] = {128, 512, 2048, SPARSE_MAX_ENTRIES, SPARSE_LIST_MAX_ENTRIES};
-  R.cap.assign(classes, classes + 5);
-  R.sparse.resize(5);
+  constexpr int NC = 6;
+  const int classes[NC] = {SPARSE_SMALL_ENTRIES, 128, 512, 2048, SPARSE_MAX_ENTRIES, SPARSE_LIST_MAX_ENTRIES};
+  R.cap.assign(classes, classes + NC);
+  R.sparse.resize(NC);
   std::vector<char> is_sparse(std::max<int64_t>(nb, 1), 0);
   if (mode != 0) {
     // accumulator words per cell: FP64 terms are two-word fixed point
@@ -80,7 +81,7 @@ RowSplit split_rows(const uf_tree *tree, const BatchJob &J, const Plan *P, int a
     // so the result equals a sequential pass (pair counts are integers < 2^53:
     // their double sums are exact in any order)
     struct Part {
-      std::vector<int32_t> cls[5];
+      std::vector<int32_t> cls[NC];
       int64_t n_sparse = 0;
       double pairs = 0.0;
     };
@@ -125,7 +126,7 @@ RowSplit split_rows(const uf_tree *tree, const BatchJob &J, const Plan *P, int a
         }
       }
     });
-    for (int k = 0; k < 5; k++)
+    for (int k = 0; k < NC; k++)
       for (const Part &pt : part) R.sparse[k].insert(R.sparse[k].end(), pt.cls[k].begin(), pt.cls[k].end());
     for (const Part &pt : part) {
       R.n_sparse += pt.n_sparse;
