@@ -6,6 +6,7 @@
 // embedding row of a branch is then f(count[k] / total[k]) for every sample
 // k, written over a padded width so that the stripe kernel can read the
 // partner column k + d without a modulo.
+#include <algorithm>
 #include <type_traits>
 
 #include "uf_device.cuh"
@@ -13,17 +14,17 @@
 
 namespace ufg {
 
-// One CTA per tip: zero the table's part of the tip's count slot, then
-// scatter its CSC column (counts points at the table's first column).
+// One CTA per tip: zero the table's part of the tip's count row, then
+// scatter its CSC column (counts points at the table's first column; the row
+// of node v is slot v).
 __global__ void k_tip_counts(const int32_t *__restrict__ tip_nodes,
-                             const int32_t *__restrict__ slot_of_node,
                              const int32_t *__restrict__ tip_of_node,
                              const int64_t *__restrict__ col_ptr,
                              const int32_t *__restrict__ col_row,
                              const double *__restrict__ col_val, double *__restrict__ counts,
                              int64_t ld, int n) {
   const int v = tip_nodes[blockIdx.x];
-  double *row = counts + (int64_t)slot_of_node[v] * ld;
+  double *row = counts + (int64_t)v * ld;
   for (int k = threadIdx.x; k < n; k += blockDim.x) row[k] = 0.0;
   __syncthreads();
   const int f = tip_of_node[v];
@@ -31,24 +32,20 @@ __global__ void k_tip_counts(const int32_t *__restrict__ tip_nodes,
   for (int64_t q = col_ptr[f] + threadIdx.x; q < q1; q += blockDim.x) row[col_row[q]] = col_val[q];
 }
 
-// One CTA per node of a list: zero the table's part of the node's count
-// slot, then add the CSC columns of its tips [tip_lo, tip_hi) one after the
-// other (within one tip's column the samples are distinct, so its entries
-// scatter without conflicts).  Serves tips and the nodes whose own subtree
-// is not walked level by level (a branch scattered by the sparse-row path
-// whose parent runs through the dense kernels).  With C = uint8_t the slot
+// One CTA per node of a list (and table, blockIdx.y): zero the table's part of
+// the node's count slot, then add the CSC columns of its tips [tip_lo, tip_hi)
+// one after the other (within one tip's column the samples are distinct, so its
+// entries scatter without conflicts).  Serves tips and the nodes whose own
+// subtree is not walked level by level (a branch scattered by the sparse-row
+// path whose parent runs through the dense kernels).  With C = uint8_t the slot
 // holds presence flags instead (1 where the count is nonzero).
 template <typename C>
-__global__ void k_slice_counts(const int32_t *__restrict__ nodes, const int32_t *__restrict__ tip_lo,
-                               const int32_t *__restrict__ tip_hi, const int32_t *__restrict__ slot_of_node,
-                               const int64_t *__restrict__ col_ptr, const int32_t *__restrict__ col_row,
-                               const double *__restrict__ col_val, C *__restrict__ counts, int64_t ld, int n) {
-  const int v = nodes[blockIdx.x];
-  C *row = counts + (int64_t)slot_of_node[v] * ld;
+__device__ __forceinline__ void slice_row(C *row, int f0, int f1, const int64_t *__restrict__ col_ptr,
+                                          const int32_t *__restrict__ col_row, const double *__restrict__ col_val,
+                                          int n) {
   for (int k = threadIdx.x; k < n; k += blockDim.x) row[k] = C(0);
   __syncthreads();
-  const int f1 = tip_hi[v];
-  for (int f = tip_lo[v]; f < f1; f++) {
+  for (int f = f0; f < f1; f++) {
     const int64_t q1 = col_ptr[f + 1];
     for (int64_t q = col_ptr[f] + threadIdx.x; q < q1; q += blockDim.x) {
       if constexpr (sizeof(C) == 1) row[col_row[q]] = C(1);
@@ -56,6 +53,21 @@ __global__ void k_slice_counts(const int32_t *__restrict__ nodes, const int32_t 
     }
     __syncthreads();
   }
+}
+__global__ void k_slice_counts(const int32_t *__restrict__ nodes, const int32_t *__restrict__ tip_lo,
+                               const int32_t *__restrict__ tip_hi, const int32_t *__restrict__ slot_of_node,
+                               const SliceTab *__restrict__ tabs, double *__restrict__ counts, int64_t ld) {
+  const int v = nodes[blockIdx.x];
+  const SliceTab tb = tabs[blockIdx.y];
+  slice_row<double>(counts + (int64_t)slot_of_node[v] * ld + tb.off, tip_lo[v], tip_hi[v], tb.col_ptr, tb.col_row,
+                    tb.col_val, tb.n);
+}
+__global__ void k_slice_presence(const int32_t *__restrict__ nodes, const int32_t *__restrict__ tip_lo,
+                                 const int32_t *__restrict__ tip_hi, const int32_t *__restrict__ slot_of_node,
+                                 const int64_t *__restrict__ col_ptr, const int32_t *__restrict__ col_row,
+                                 uint8_t *__restrict__ flags, int64_t ld, int n) {
+  const int v = nodes[blockIdx.x];
+  slice_row<uint8_t>(flags + (int64_t)slot_of_node[v] * ld, tip_lo[v], tip_hi[v], col_ptr, col_row, nullptr, n);
 }
 
 // count[v][k] = sum of the children's count[c][k], children in index order
@@ -169,7 +181,7 @@ __global__ void k_emb_rows(int64_t b0, const int32_t *__restrict__ nodes,
                            const float *__restrict__ inv_total_f, T *__restrict__ X, int64_t pitch,
                            const TabDesc *__restrict__ tabs, int n_tabs, double row_scale) {
   const int64_t v = nodes ? (int64_t)nodes[blockIdx.x] : b0 + blockIdx.x;
-  const double *c = counts + (int64_t)slot_of_node[v] * ld;
+  const double *c = counts + (slot_of_node ? (int64_t)slot_of_node[v] : v) * ld;
   const double l = length[v];
   T *x = X + (int64_t)blockIdx.x * pitch;
   for (int64_t j = threadIdx.x; j < pitch; j += blockDim.x) {
@@ -211,37 +223,277 @@ __global__ void k_emb_rows_vaw(const int32_t *__restrict__ nodes, const int32_t 
   }
 }
 
-cudaError_t launch_tip_counts(const int32_t *tip_nodes, int n_list, const int32_t *slot_of_node,
-                              const int32_t *tip_of_node, const int64_t *col_ptr,
+// ---- count rows level by level, with the embedding rows ----
+// A thread keeps one column: its total, its reciprocal and where its value goes
+// in a row (a row repeats its own head, so a value has several places) are
+// read once for all the nodes it visits, and a node's value is written when its
+// count is summed (a second pass over the counts before).  Levels of many
+// elements are a launch each over whole rows: bound by the counts' traffic.
+// The narrow levels, most of them and bound by launching, share one launch: a
+// sample's counts depend on no other sample's, so a CTA owns a slab of `w`
+// columns and walks the levels with a block barrier between them.  2,048
+// samples, 19,331 dense branches, 36 levels: 0.48 ms (0.57 with a launch per
+// level and the rows apart; 0.62 with every level in slabs, whose 32-byte pieces
+// of rows leave L2 apart); FP64 rows of 1,531 samples 0.57 ms (1.70); 64
+// samples, one launch instead of 22.
+template <typename T, int KIND>
+struct RowValue;  // one column's value of an embedding row from its count c and the branch length l
+template <int KIND>
+struct RowValue<float, KIND> {
+  double t;
+  float it;
+  __device__ RowValue(double total, float inv, double) : t(total), it(inv) {}
+  __device__ float operator()(double c, double l) const { return emb_value<float, KIND>(c, l, t, it); }
+};
+// c / t by the reciprocal and one correction of the remainder (Markstein):
+// 3 FP64 instructions per value instead of a division's dozen, on a GPU with
+// 2 FP64 lanes per clock per SM
+struct Quotient {
+  double t, rt;
+  __device__ Quotient(double total) : t(total), rt(1.0 / total) {}
+  __device__ double operator()(double c) const {
+    const double q = c * rt;
+    return fma(fma(-q, t, c), rt, q);
+  }
+};
+template <int KIND>
+struct RowValue<double, KIND> {
+  Quotient q;
+  __device__ RowValue(double total, float, double) : q(total) {}
+  __device__ double operator()(double c, double) const { return q(c); }  // EMB_PROP
+};
+template <int KIND>
+struct RowValue<unsigned long long, KIND> {
+  Quotient q;
+  double scale;
+  __device__ RowValue(double total, float, double row_scale) : q(total), scale(row_scale) {}
+  __device__ unsigned long long operator()(double c, double l) const {
+    const double ls = l * scale;  // exact: scale is a power of two
+    if (KIND == EMB_PRESENCE) return c > 0.0 ? __double2ull_rn(ls) : 0ull;
+    return __double2ull_rn(ls * q(c));
+  }
+};
+
+// Table holding combined sample column k (tables in order of off).
+__device__ __forceinline__ int embed_table_of(const TabDesc *tabs, int n_tabs, int k) {
+  int lo = 0, hi = n_tabs - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (tabs[mid].off <= k) lo = mid;
+    else hi = mid - 1;
+  }
+  return lo;
+}
+
+// What the slab kernel needs of list position p in one 16-byte load: the
+// node's slot, its first and second child's (-1: none; two or more levels of
+// indirection per node otherwise, each a trip to L2), its row of X; more than
+// two children: -2 - node in .z.
+__global__ void k_embed_steps(const EmbedArgs a, int4 *__restrict__ steps, double *__restrict__ len) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= a.n_nodes) return;
+  const int p = a.levels[0] + i, v = a.list[p];
+  const bool built = a.n_levels < 2 || p < a.levels[a.level_step];
+  const int c0 = a.child_ptr[v], nc = built ? 0 : a.child_ptr[v + 1] - c0;
+  int4 q;
+  q.x = a.slot_of_node[v];
+  q.y = nc > 0 ? a.slot_of_node[a.child_idx[c0]] : -1;
+  q.z = nc == 2 ? a.slot_of_node[a.child_idx[c0 + 1]] : nc > 2 ? -2 - v : -1;
+  q.w = a.xrow[p];
+  steps[i] = q;
+  len[i] = a.length[v];
+}
+
+// STEPS: from k_embed_steps' records; else from the tree's arrays (the
+// allocation-free call, which has no room for records)
+template <typename T, int KIND, bool STEPS>
+__global__ void __launch_bounds__(512) k_embed_slab(const EmbedArgs a) {
+  constexpr int U = 4;  // nodes per thread in flight
+  const int per = blockDim.x / a.w, g = threadIdx.x / a.w;  // nodes at a time, this thread's
+  const int k = blockIdx.x * a.w + (threadIdx.x - g * a.w);
+  const bool on = k < a.n_cols;
+  const int kc = on ? k : 0;
+  const int ti = a.n_tabs == 1 ? 0 : embed_table_of(a.tabs, a.n_tabs, kc);
+  const int n = a.tabs[ti].n;
+  const int64_t j0 = a.tabs[ti].x_col + (kc - a.tabs[ti].off);
+  const int64_t j1 = ti + 1 < a.n_tabs ? a.tabs[ti + 1].x_col : a.pitch;
+  const double total = a.total[kc];
+  const float inv = a.inv_total_f[kc];
+  const RowValue<T, KIND == EMB_VAW ? EMB_PROP : KIND> value(total, inv, a.row_scale);
+  T *X = (T *)a.X;
+  double *counts = a.counts + kc;
+  auto put = [&](int row, double l, double c) {
+    if constexpr (KIND == EMB_VAW) {
+      // three planes: l p, the count below and the rest of the total (FP32
+      // rows use the FP32 reciprocal of the total)
+      T *x = X + (int64_t)row * 3 * a.pitch;
+      T y;
+      if constexpr (sizeof(T) == 4) y = (float)l * ((float)c * inv);
+      else y = l * value(c, l);
+      for (int64_t j = j0; j < j1; j += n) {
+        x[j] = y;
+        x[a.pitch + j] = (T)c;
+        x[2 * a.pitch + j] = (T)(total - c);
+      }
+    } else {
+      T *x = X + (int64_t)row * a.pitch;
+      const T y = value(c, l);
+      for (int64_t j = j0; j < j1; j += n) x[j] = y;
+    }
+  };
+  auto more = [&](int v, int c0) {  // the sum over a node's children from c0 on, in index order
+    double s = 0.0;
+    for (int c = c0; c < a.child_ptr[v + 1]; c++) {
+      const int ch = a.child_idx[c];
+      s += counts[(int64_t)(a.slot_of_node ? a.slot_of_node[ch] : ch) * a.ld];
+    }
+    return s;
+  };
+  const int p_first = a.levels[0];
+  for (int lv = a.first ? 0 : a.lv0; lv < a.lv1; lv = max(lv + 1, a.lv0)) {
+    const int pb = a.levels[a.level_step * lv], p1 = a.levels[a.level_step * lv + 1];
+    if (on && (lv > 0 || X)) {
+      if constexpr (STEPS) {
+        for (int p = pb + blockIdx.y * (U * per) + g; p < p1; p += gridDim.y * (U * per)) {
+          int4 q[U];
+          double l[U], s[U];
+#pragma unroll
+          for (int u = 0; u < U; u++) {
+            const int pu = p + u * per;
+            q[u] = pu < p1 ? a.steps[pu - p_first] : make_int4(-1, -1, -1, -1);
+            l[u] = pu < p1 ? a.steps_len[pu - p_first] : 0.0;
+          }
+#pragma unroll
+          for (int u = 0; u < U; u++) {
+            // a built row is read (if it has an embedding row), others summed
+            const int c0 = lv == 0 ? (q[u].w >= 0 ? q[u].x : -1) : q[u].y;
+            s[u] = c0 >= 0 ? counts[(int64_t)c0 * a.ld] : 0.0;
+            if (q[u].z >= 0) s[u] += counts[(int64_t)q[u].z * a.ld];
+          }
+#pragma unroll
+          for (int u = 0; u < U; u++) {
+            if (q[u].z < -1) {
+              const int v = -2 - q[u].z;
+              s[u] = more(v, a.child_ptr[v]);
+            }
+            if (lv > 0 && q[u].x >= 0) counts[(int64_t)q[u].x * a.ld] = s[u];
+            if (X && q[u].w >= 0) put(q[u].w, l[u], s[u]);
+          }
+        }
+      } else {
+        for (int p = pb + g; p < p1; p += per) {
+          const int v = a.list[p];
+          double *at = counts + (int64_t)v * a.ld;
+          const double s = lv == 0 ? *at : more(v, a.child_ptr[v]);
+          if (lv > 0) *at = s;
+          if (X) put(v, a.length[v], s);
+        }
+      }
+    }
+    __syncthreads();  // the level's counts, before its parents read them
+  }
+}
+
+namespace {
+// elements of a level from which it gets a launch of its own
+constexpr int64_t EMBED_WIDE = 1 << 18;
+
+cudaError_t embed_launch(int kind, bool fp32, const EmbedArgs &a, dim3 grid, int nt, cudaStream_t st) {
+  const bool steps = a.steps != nullptr;
+#define UF_SLAB(T, K)                                                                    \
+  return launch_k(steps ? k_embed_slab<T, K, true> : k_embed_slab<T, K, false>, grid, dim3(nt), 0, st, a)
+  if (kind == EMB_VAW) {
+    if (fp32) UF_SLAB(float, EMB_VAW);
+    UF_SLAB(double, EMB_VAW);
+  }
+  if (fp32) {
+    if (kind == EMB_SCALED) UF_SLAB(float, EMB_SCALED);
+    if (kind == EMB_PRESENCE) UF_SLAB(float, EMB_PRESENCE);
+    UF_SLAB(float, EMB_PROP);
+  }
+  if (kind == EMB_SCALED) UF_SLAB(unsigned long long, EMB_SCALED);
+  if (kind == EMB_PRESENCE) UF_SLAB(unsigned long long, EMB_PRESENCE);
+  UF_SLAB(double, EMB_PROP);
+#undef UF_SLAB
+}
+
+}  // namespace
+
+cudaError_t launch_embed(int kind, bool fp32, const EmbedArgs &a0, const int *level_nodes, cudaStream_t st,
+                         int64_t *launches) {
+  if (a0.n_nodes <= 0 || a0.n_cols <= 0) return cudaSuccess;
+  EmbedArgs a = a0;
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  const bool steps = a.steps != nullptr;
+  if (steps) {
+    e = launch_k(k_embed_steps, dim3((unsigned)((a.n_nodes + 255) / 256)), dim3(256), 0, st, a, a.steps, a.steps_len);
+    if (e != cudaSuccess) return e;
+    (*launches)++;
+  }
+  // levels of at least EMBED_WIDE elements: CTAs of 256 columns, enough of
+  // them for eight per SM, each with its share of the level's nodes
+  auto wide = [&](int lv) -> cudaError_t {
+    EmbedArgs w = a;
+    w.lv0 = lv;
+    w.lv1 = lv + 1;
+    w.first = 0;
+    w.w = 256;
+    const int64_t gx = (a.n_cols + 255) / 256;
+    const int64_t gy = std::max<int64_t>(1, std::min<int64_t>((level_nodes[lv] + 3) / 4, 8 * (int64_t)sms / gx + 1));
+    (*launches)++;
+    return embed_launch(kind, fp32, w, dim3((unsigned)gx, (unsigned)gy), 256, st);
+  };
+  auto is_wide = [&](int lv) { return steps && (int64_t)level_nodes[lv] * a.n_cols >= EMBED_WIDE; };
+  a.first = a.X != nullptr && level_nodes[0] > 0;
+  if (a.first && is_wide(0)) {
+    a.first = 0;
+    if ((e = wide(0)) != cudaSuccess) return e;
+  }
+  for (a.lv0 = 1; a.lv0 < a.n_levels && is_wide(a.lv0); a.lv0++)
+    if ((e = wide(a.lv0)) != cudaSuccess) return e;
+  if (a.lv0 >= a.n_levels && !a.first) return cudaSuccess;
+  // the rest in slabs: the widest (whole 128-byte lines at 16) that still give
+  // every SM one
+  a.lv1 = a.n_levels;
+  a.w = 16;
+  while (a.w > 2 && (a.n_cols + a.w - 1) / a.w < sms) a.w /= 2;
+  int most = 1;
+  if (a.first) most = level_nodes[0];
+  for (int l = a.lv0; l < a.n_levels; l++) most = std::max(most, level_nodes[l]);
+  const int nt = (int64_t)most * a.w >= 2048 ? 512 : 128;
+  (*launches)++;
+  return embed_launch(kind, fp32, a, dim3((unsigned)((a.n_cols + a.w - 1) / a.w)), nt, st);
+}
+
+cudaError_t launch_tip_counts(const int32_t *tip_nodes, int n_list, const int32_t *tip_of_node, const int64_t *col_ptr,
                               const int32_t *col_row, const double *col_val, double *counts,
                               int64_t ld, int n, cudaStream_t st) {
   if (n_list <= 0) return cudaSuccess;
-  k_tip_counts<<<n_list, 256, 0, st>>>(tip_nodes, slot_of_node, tip_of_node, col_ptr, col_row,
-                                       col_val, counts, ld, n);
+  k_tip_counts<<<n_list, 256, 0, st>>>(tip_nodes, tip_of_node, col_ptr, col_row, col_val, counts, ld, n);
   return cudaGetLastError();
 }
 
 cudaError_t launch_slice_counts(const int32_t *nodes, int n_list, const int32_t *tip_lo, const int32_t *tip_hi,
-                                const int32_t *slot_of_node, const int64_t *col_ptr, const int32_t *col_row,
-                                const double *col_val, double *counts, int64_t ld, int n, cudaStream_t st) {
-  if (n_list <= 0) return cudaSuccess;
-  return launch_k(k_slice_counts<double>, dim3(n_list), dim3(256), 0, st, nodes, tip_lo, tip_hi, slot_of_node, col_ptr,
-                  col_row, col_val, counts, ld, n);
+                                const int32_t *slot_of_node, const SliceTab *tabs, int n_tabs, double *counts,
+                                int64_t ld, cudaStream_t st) {
+  // tables along grid.y, at most 65,535 of them at a time
+  for (int t = 0; n_list > 0 && t < n_tabs; t += 65535) {
+    const cudaError_t e = launch_k(k_slice_counts, dim3(n_list, std::min(n_tabs - t, 65535)), dim3(256), 0, st, nodes,
+                                   tip_lo, tip_hi, slot_of_node, tabs + t, counts, ld);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 cudaError_t launch_slice_presence(const int32_t *nodes, int n_list, const int32_t *tip_lo, const int32_t *tip_hi,
                                   const int32_t *slot_of_node, const int64_t *col_ptr, const int32_t *col_row,
                                   uint8_t *flags, int64_t ld, int n, cudaStream_t st) {
   if (n_list <= 0) return cudaSuccess;
-  return launch_k(k_slice_counts<uint8_t>, dim3(n_list), dim3(256), 0, st, nodes, tip_lo, tip_hi, slot_of_node,
-                  col_ptr, col_row, (const double *)nullptr, flags, ld, n);
-}
-
-cudaError_t launch_node_counts(const int32_t *nodes, int n_list, const int32_t *child_ptr,
-                               const int32_t *child_idx, const int32_t *slot_of_node,
-                               double *counts, int64_t ld, cudaStream_t st, int64_t n_used) {
-  return launch_node_rows<double>(nodes, n_list, child_ptr, child_idx, slot_of_node, counts, ld,
-                                  n_used < 0 ? ld : n_used, st);
+  return launch_k(k_slice_presence, dim3(n_list), dim3(256), 0, st, nodes, tip_lo, tip_hi, slot_of_node, col_ptr,
+                  col_row, flags, ld, n);
 }
 
 cudaError_t launch_node_presence(const int32_t *nodes, int n_list, const int32_t *child_ptr,

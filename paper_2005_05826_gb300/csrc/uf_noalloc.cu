@@ -130,9 +130,8 @@ uf_status compute_noalloc(const uf_tree *tree, const uf_table *table, uf_method 
   const int64_t N = tv.n_nodes, nb = N - 1;
   const double scale = accum_scale(tree, table, kind);
 
-  // one branch block holding every branch; slot of node v = v
-  std::vector<int32_t> level(N, 0), lists, slot(N);
-  std::vector<std::pair<int64_t, int>> launches;
+  // one branch block holding every branch; slot and row of node v = v
+  std::vector<int32_t> level(N, 0), lists, level_at;
   {
     std::vector<std::vector<int32_t>> lv(1);
     for (int64_t v = 0; v < nb; v++) {
@@ -150,10 +149,10 @@ uf_status compute_noalloc(const uf_tree *tree, const uf_table *table, uf_method 
       lv[L + 1].push_back((int32_t)v);
     }
     for (auto &l : lv) {
-      launches.emplace_back((int64_t)lists.size(), (int)l.size());
+      level_at.push_back((int32_t)lists.size());
       lists.insert(lists.end(), l.begin(), l.end());
     }
-    for (int64_t v = 0; v < N; v++) slot[v] = (int32_t)v;
+    level_at.push_back((int32_t)lists.size());  // at most N entries: the tips and up to N - 2 levels
   }
   const int rows = (int)std::max<int64_t>(nb, 0);
 
@@ -163,7 +162,7 @@ uf_status compute_noalloc(const uf_tree *tree, const uf_table *table, uf_method 
     p[1] = c.take<int32_t>(N);                      // tip_of_node
     p[2] = c.take<int32_t>(N + 1);                  // child_ptr
     p[3] = c.take<int32_t>(std::max<int64_t>(nb, 1));  // child_idx
-    p[4] = c.take<int32_t>(N);                      // slot_of_node
+    p[4] = c.take<int32_t>(level_at.size());        // starts of the levels in the lists, and their end
     p[5] = c.take<int32_t>(std::max<size_t>(lists.size(), 1));  // level lists
     p[6] = c.take<int64_t>(xv.n_features + 1);      // col_ptr
     p[7] = c.take<int32_t>(std::max<int64_t>(xv.nnz, 1));  // col_row
@@ -222,7 +221,7 @@ uf_status compute_noalloc(const uf_tree *tree, const uf_table *table, uf_method 
   UF_TRY(h2d(p[1], tv.tip_of_node, N * 4));
   UF_TRY(h2d(p[2], tv.child_ptr, (N + 1) * 4));
   UF_TRY(h2d(p[3], tv.child_idx, nb * 4));
-  UF_TRY(h2d(p[4], slot.data(), N * 4));
+  UF_TRY(h2d(p[4], level_at.data(), level_at.size() * 4));
   UF_TRY(h2d(p[5], lists.data(), lists.size() * 4));
   UF_TRY(h2d(p[6], xv.col_ptr, (xv.n_features + 1) * 8));
   UF_TRY(h2d(p[7], xv.col_row, xv.nnz * 4));
@@ -252,18 +251,36 @@ uf_status compute_noalloc(const uf_tree *tree, const uf_table *table, uf_method 
   const int x_shift =
       fixed_rows ? fixed_row_shift(scale, accum_bound(tree, table, kind), tv.length, nb, plan.chunk) : 0;
 
-  const int32_t *d_lists = (const int32_t *)p[5], *d_slot = (const int32_t *)p[4];
-  double *d_counts = (double *)p[11];
+  const int32_t *d_lists = (const int32_t *)p[5];
   if (rows > 0) {
-    UF_TRY(launch_tip_counts(d_lists + launches[0].first, launches[0].second, d_slot,
-                             (const int32_t *)p[1], (const int64_t *)p[6], (const int32_t *)p[7],
-                             (const double *)p[8], d_counts, n, n, st));
-    for (size_t l = 1; l < launches.size(); l++)
-      UF_TRY(launch_node_counts(d_lists + launches[l].first, launches[l].second,
-                                (const int32_t *)p[2], (const int32_t *)p[3], d_slot, d_counts, n, st));
-    UF_TRY(launch_emb_rows(kind, fp32, 0, rows, d_slot, d_counts, n, (const double *)p[0],
-                           (const double *)p[9], (const float *)p[10], p[12], pitch,
-                           (const TabDesc *)p[18], 1, st, nullptr, fixed_rows ? std::ldexp(scale, x_shift) : 0.0));
+    UF_TRY(launch_tip_counts(d_lists, level_at[1], (const int32_t *)p[1], (const int64_t *)p[6],
+                             (const int32_t *)p[7], (const double *)p[8], (double *)p[11], n, n, st));
+    EmbedArgs ea{};
+    ea.list = d_lists;
+    ea.levels = (const int32_t *)p[4];
+    ea.level_step = 1;
+    ea.n_levels = (int)level_at.size() - 1;
+    ea.n_nodes = rows;
+    ea.child_ptr = (const int32_t *)p[2];
+    ea.child_idx = (const int32_t *)p[3];
+    ea.counts = (double *)p[11];
+    ea.ld = n;
+    ea.n_cols = n;
+    ea.length = (const double *)p[0];
+    ea.total = (const double *)p[9];
+    ea.inv_total_f = (const float *)p[10];
+    ea.X = n >= EMBED_MIN_SAMPLES ? p[12] : nullptr;
+    ea.pitch = pitch;
+    ea.tabs = (const TabDesc *)p[18];
+    ea.n_tabs = 1;
+    ea.row_scale = fixed_rows ? std::ldexp(scale, x_shift) : 0.0;
+    std::vector<int> level_nodes;
+    for (size_t l = 0; l + 1 < level_at.size(); l++) level_nodes.push_back(level_at[l + 1] - level_at[l]);
+    int64_t launches = 0;
+    UF_TRY(launch_embed(kind, fp32, ea, level_nodes.data(), st, &launches));
+    if (!ea.X)
+      UF_TRY(launch_emb_rows(kind, fp32, 0, rows, nullptr, ea.counts, n, ea.length, ea.total, ea.inv_total_f, p[12],
+                             pitch, ea.tabs, 1, st, nullptr, ea.row_scale));
     StripeArgs sa{};
     sa.X = p[12];
     sa.len = (const double *)p[0];

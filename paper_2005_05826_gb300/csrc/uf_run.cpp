@@ -519,29 +519,9 @@ void fill_reports(uf_tree *tree, const BatchJob &J, const Outputs &o, double ms[
   }
 }
 
-// Count rows of block b that the split needs: CSC-built nodes of every
-// table, then the dense internal levels over the combined axis.
-void enqueue_split_counts(const Inputs &in, const BatchJob &J, const std::vector<int> &off, const RowSplit &split,
-                          size_t b, const int32_t *d_cnt, double *counts, int64_t ld, int64_t n_cols,
-                          cudaStream_t st, int64_t *kernels) {
-  const auto &lb = split.cnt_launch[b];
-  for (size_t t = 0; t < J.tabs.size(); t++) {
-    ck(launch_slice_counts(d_cnt + lb[0].first, lb[0].second, in.td->tip_lo, in.td->tip_hi, in.pd->slot_of_node,
-                           in.xd[t]->col_ptr, in.xd[t]->col_row, in.xd[t]->col_val, counts + off[t], ld,
-                           (int)J.tabs[t].table->n, st),
-       "count rows");
-    *kernels += lb[0].second > 0;
-  }
-  for (size_t l = 1; l < lb.size(); l++) {
-    ck(launch_node_counts(d_cnt + lb[l].first, lb[l].second, in.td->child_ptr, in.td->child_idx,
-                          in.pd->slot_of_node, counts, ld, st, n_cols),
-       "node counts");
-    (*kernels)++;
-  }
-}
-
-// The same rows as presence flags (the tensor-core unweighted path needs
-// nothing else): one byte per sample instead of an FP64 count.
+// Rows of block b that the split needs as presence flags (the tensor-core
+// unweighted path needs nothing else), one byte per sample: CSC-built nodes of
+// every table, then the dense internal levels over the combined axis.
 void enqueue_split_presence(const Inputs &in, const BatchJob &J, const std::vector<int> &off,
                             const RowSplit &split, size_t b, const int32_t *d_cnt, uint8_t *flags, int64_t ld,
                             int64_t n_cols, cudaStream_t st, int64_t *kernels) {
@@ -1090,6 +1070,10 @@ uf_status run_stripes(uf_tree *tree, const BatchJob &J, int device, uf_method me
   const int64_t ld = round_up(n_cols, 16);
   const size_t m_bytes = (size_t)cells * 8 * words, d_bytes = (size_t)n_cols * 8 * words;
   DevBuf counts((size_t)in.P->n_slots * ld * 8, st, "alloc counts");
+  int64_t most_nodes = 1;  // count rows of one block
+  for (const auto &lb : split.cnt_launch)
+    most_nodes = std::max(most_nodes, lb.back().first + lb.back().second - lb[0].first);
+  DevBuf steps((size_t)most_nodes * (sizeof(int4) + sizeof(double)), st, "alloc embedding steps");
   DevBuf X((size_t)xrows * pitch * es * planes, st, "alloc embeddings");
   DevBuf M(m_bytes, st, "alloc stripes");
   DevBuf M2, Dg, diag_tmp, counter(sizeof(int), st, "alloc counter");
@@ -1115,6 +1099,11 @@ uf_status run_stripes(uf_tree *tree, const BatchJob &J, int device, uf_method me
   std::vector<size_t> o_shape_tabs(1, o_tabs);
   for (int sh = 1; sh < n_all_shapes; sh++) o_shape_tabs.push_back(meta.add(shape_tabs[sh]));
   const size_t o_cnt = meta.add(split.cnt_lists);
+  std::vector<SliceTab> slice(nt);
+  for (size_t t = 0; t < nt; t++)
+    slice[t] = SliceTab{in.xd[t]->col_ptr, in.xd[t]->col_row, in.xd[t]->col_val, tabs[t].n, tabs[t].off};
+  const size_t o_slice = meta.add(slice);
+  const size_t o_xrow = meta.add(split.cnt_xrow), o_levels = meta.add(split.cnt_levels);
   const size_t o_dense = meta.add(split.dense);
   const size_t o_dlen = meta.add(split.dense_len);
   std::vector<SpLayout> lay(nt);
@@ -1225,13 +1214,46 @@ uf_status run_stripes(uf_tree *tree, const BatchJob &J, int device, uf_method me
     launch_sparse(ss);
     timer.end();
   }
+  const bool rows_in_slab = *std::min_element(ns.begin(), ns.end()) >= EMBED_MIN_SAMPLES;
   bool tuned = false;
   for (size_t b = 0; b < in.P->b0.size(); b++) {
     const int64_t b0 = in.P->b0[b];
     const int64_t d0 = split.dense_ptr[b], nd = split.dense_ptr[b + 1] - d0;
     timer.begin(0);
-    enqueue_split_counts(in, J, off, split, b, d_cnt, counts.as<double>(), ld, n_cols, ls, &kernels);
-    if (nd > 0) {
+    const auto &built = split.cnt_launch[b][0];
+    ck(launch_slice_counts(d_cnt + built.first, built.second, in.td->tip_lo, in.td->tip_hi, in.pd->slot_of_node,
+                           meta.at<SliceTab>(o_slice), (int)nt, counts.as<double>(), ld, ls),
+       "count rows");
+    kernels += built.second > 0;
+    EmbedArgs ea{};
+    ea.list = d_cnt;
+    ea.levels = meta.at<int32_t>(o_levels) + split.cnt_lev_ptr[b];
+    ea.level_step = 2;
+    ea.n_levels = (int)split.cnt_launch[b].size();
+    ea.n_nodes = (int)(split.cnt_launch[b].back().first + split.cnt_launch[b].back().second -
+                       split.cnt_launch[b][0].first);
+    ea.xrow = meta.at<int32_t>(o_xrow);
+    ea.child_ptr = in.td->child_ptr;
+    ea.child_idx = in.td->child_idx;
+    ea.slot_of_node = in.pd->slot_of_node;
+    ea.counts = counts.as<double>();
+    ea.ld = ld;
+    ea.n_cols = n_cols;
+    ea.length = in.td->length;
+    ea.total = total.as<double>();
+    ea.inv_total_f = inv_total.as<float>();
+    ea.X = rows_in_slab ? X.p : nullptr;
+    ea.pitch = pitch;
+    ea.tabs = d_tabs;
+    ea.n_tabs = (int)nt;
+    ea.row_scale = fixed_rows ? std::ldexp(scale, x_shift) : 0.0;
+    ea.steps = steps.as<int4>();
+    ea.steps_len = (double *)(steps.as<int4>() + most_nodes);
+    std::vector<int> level_nodes;
+    for (const auto &l : split.cnt_launch[b]) level_nodes.push_back(l.second);
+    level_nodes[0] = split.cnt_built_dense[b];
+    ck(launch_embed(kind, fp32, ea, level_nodes.data(), ls, &kernels), "count and embedding rows");
+    if (nd > 0 && !rows_in_slab) {
       ck(launch_emb_rows(kind, fp32, b0, (int)nd, in.pd->slot_of_node, counts.as<double>(), ld,
                          in.td->length, total.as<double>(), inv_total.as<float>(), X.p, pitch,
                          d_tabs, (int)nt, ls, d_dense + d0, fixed_rows ? std::ldexp(scale, x_shift) : 0.0),
@@ -1346,6 +1368,7 @@ uf_status run_stripes(uf_tree *tree, const BatchJob &J, int device, uf_method me
   Dg = DevBuf();
   sc = SparseScatter();
   diag_tmp = DevBuf();
+  steps = DevBuf();
   counter = DevBuf();
   clamps = DevBuf();
   pair_ctr = DevBuf();

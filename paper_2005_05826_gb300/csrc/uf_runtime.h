@@ -298,6 +298,11 @@ struct RowSplit {
   // the dense internal nodes level by level; offsets into cnt_lists
   std::vector<int32_t> cnt_lists;
   std::vector<std::vector<std::pair<int64_t, int>>> cnt_launch;
+  // per list position the branch's dense row in its block, or -1; per block and
+  // level its first and one past its last position (level 0: the dense
+  // branches among the built rows, which come first), from cnt_lev_ptr on
+  std::vector<int32_t> cnt_xrow, cnt_levels, cnt_built_dense;
+  std::vector<int64_t> cnt_lev_ptr;
 };
 
 // Stripe regions of a call's sparse scatter: one table whose accumulators

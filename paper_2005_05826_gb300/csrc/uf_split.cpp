@@ -139,8 +139,8 @@ RowSplit split_rows(const uf_tree *tree, const BatchJob &J, const Plan *P, int a
     return p != root && !is_sparse[p];
   };
   // per list position: bit 0 = built from CSC columns (tips, and sparse
-  // branches under a dense parent), bit 1 = a dense internal node; flagged in
-  // parallel, then gathered in list order
+  // branches under a dense parent), bit 1 = a dense internal node, bit 2 = a
+  // dense branch; flagged in parallel, then gathered in list order
   std::vector<uint8_t> flag(P->lists.size(), 0);
   {
     const int64_t np = (int64_t)P->lists.size();
@@ -154,7 +154,8 @@ RowSplit split_rows(const uf_tree *tree, const BatchJob &J, const Plan *P, int a
         const auto &l0 = P->launches[b][0];
         const int32_t v = P->lists[q];
         const bool tip = q < l0.first + l0.second;
-        flag[q] = (uint8_t)((is_sparse[v] ? parent_dense(v) : tip) | ((!tip && !is_sparse[v]) << 1));
+        flag[q] = (uint8_t)((is_sparse[v] ? parent_dense(v) : tip) | ((!tip && !is_sparse[v]) << 1) |
+                            (!is_sparse[v] << 2));
       }
     });
   }
@@ -163,8 +164,15 @@ RowSplit split_rows(const uf_tree *tree, const BatchJob &J, const Plan *P, int a
     std::vector<std::pair<int64_t, int>> lb;
     const int64_t q0 = ls[0].first, q1 = ls.back().first + ls.back().second;
     const int64_t at0 = (int64_t)R.cnt_lists.size();
-    for (int64_t q = q0; q < q1; q++)
-      if (flag[q] & 1) R.cnt_lists.push_back(P->lists[q]);
+    // (the dense branches among them first: only they get embedding rows)
+    int built_dense = 0;
+    for (int want = 1; want >= 0; want--)
+      for (int64_t q = q0; q < q1; q++)
+        if ((flag[q] & 5) == (want ? 5 : 1)) {
+          R.cnt_lists.push_back(P->lists[q]);
+          built_dense += want;
+        }
+    R.cnt_built_dense.push_back(built_dense);
     lb.emplace_back(at0, (int)((int64_t)R.cnt_lists.size() - at0));
     for (size_t l = 1; l < ls.size(); l++) {
       const int64_t at = (int64_t)R.cnt_lists.size();
@@ -174,15 +182,26 @@ RowSplit split_rows(const uf_tree *tree, const BatchJob &J, const Plan *P, int a
     }
     R.cnt_launch.push_back(std::move(lb));
   }
+  std::vector<int32_t> row_of(std::max<int64_t>(nb, 1), -1);
   R.dense_ptr.push_back(0);
   for (size_t b = 0; b < P->b0.size(); b++) {
     for (int64_t v = P->b0[b]; v < P->b1[b]; v++)
       if (!is_sparse[v]) {
+        row_of[v] = (int32_t)((int64_t)R.dense.size() - R.dense_ptr[b]);
         R.dense.push_back((int32_t)v);
         R.dense_len.push_back(tree->length[v]);
       }
     R.dense_ptr.push_back((int64_t)R.dense.size());
     R.max_dense = std::max(R.max_dense, R.dense_ptr[b + 1] - R.dense_ptr[b]);
+  }
+  R.cnt_xrow.resize(R.cnt_lists.size());
+  for (size_t q = 0; q < R.cnt_lists.size(); q++) R.cnt_xrow[q] = row_of[R.cnt_lists[q]];
+  for (size_t b = 0; b < R.cnt_launch.size(); b++) {
+    R.cnt_lev_ptr.push_back((int64_t)R.cnt_levels.size());
+    for (const auto &l : R.cnt_launch[b]) {
+      R.cnt_levels.push_back((int32_t)l.first);
+      R.cnt_levels.push_back((int32_t)(l.first + (&l == &R.cnt_launch[b][0] ? R.cnt_built_dense[b] : l.second)));
+    }
   }
   return R;
 }

@@ -741,21 +741,17 @@ __global__ void k_diag_partial(const StripeArgs a, float *__restrict__ part) {
 }
 
 // Phase 2: a chunk's sub-block partials summed in order in FP32, then rounded
-// to fixed point (the stripe kernels' second level).
+// to fixed point (the stripe kernels' second level); blockIdx.y is the chunk,
+// whose integers add in any order.
 __global__ void k_diag_reduce(const StripeArgs a, const float *__restrict__ part, int n_sb) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= a.n_cols) return;
   const int per_chunk = (a.chunk + B1 - 1) / B1;
-  long long d = 0;
+  const int sb0 = blockIdx.y * per_chunk, sb1 = min(n_sb, sb0 + per_chunk);
   float mid = 0.f;
-  for (int sb = 0; sb < n_sb; sb++) {
-    mid += part[(int64_t)sb * a.n_cols + k];
-    if ((sb + 1) % per_chunk == 0 || sb == n_sb - 1) {
-      d += to_fixed(mid, a.scale);
-      mid = 0.f;
-    }
-  }
-  a.Dg[k] += (unsigned long long)d;
+#pragma unroll 8
+  for (int sb = sb0; sb < sb1; sb++) mid += part[(int64_t)sb * a.n_cols + k];
+  atomicAdd(a.Dg + k, (unsigned long long)to_fixed(mid, a.scale));
 }
 
 // FP64: the fixed-point rows' sums, each value split into its two words
@@ -921,7 +917,7 @@ cudaError_t launch_diag(bool fp32, const StripeArgs &a, void *scratch, cudaStrea
   const int n_sb = (n_chunks - 1) * per_chunk + ((a.rows - (n_chunks - 1) * a.chunk) + B1 - 1) / B1;
   const cudaError_t e = launch_k(k_diag_partial, dim3(gx, n_sb), dim3(128), 0, st, a, (float *)scratch);
   if (e != cudaSuccess) return e;
-  return launch_k(k_diag_reduce, dim3(gx), dim3(128), 0, st, a, (const float *)scratch, n_sb);
+  return launch_k(k_diag_reduce, dim3(gx, n_chunks), dim3(128), 0, st, a, (const float *)scratch, n_sb);
 }
 
 }  // namespace ufg
