@@ -37,126 +37,43 @@ __global__ void k_tip_counts(const int32_t *__restrict__ tip_nodes,
 // one after the other (within one tip's column the samples are distinct, so its
 // entries scatter without conflicts).  Serves tips and the nodes whose own
 // subtree is not walked level by level (a branch scattered by the sparse-row
-// path whose parent runs through the dense kernels).  With C = uint8_t the slot
-// holds presence flags instead (1 where the count is nonzero).
-template <typename C>
-__device__ __forceinline__ void slice_row(C *row, int f0, int f1, const int64_t *__restrict__ col_ptr,
-                                          const int32_t *__restrict__ col_row, const double *__restrict__ col_val,
-                                          int n) {
-  for (int k = threadIdx.x; k < n; k += blockDim.x) row[k] = C(0);
-  __syncthreads();
-  for (int f = f0; f < f1; f++) {
-    const int64_t q1 = col_ptr[f + 1];
-    for (int64_t q = col_ptr[f] + threadIdx.x; q < q1; q += blockDim.x) {
-      if constexpr (sizeof(C) == 1) row[col_row[q]] = C(1);
-      else row[col_row[q]] += col_val[q];
-    }
-    __syncthreads();
-  }
-}
+// path whose parent runs through the dense kernels).
 __global__ void k_slice_counts(const int32_t *__restrict__ nodes, const int32_t *__restrict__ tip_lo,
                                const int32_t *__restrict__ tip_hi, const int32_t *__restrict__ slot_of_node,
                                const SliceTab *__restrict__ tabs, double *__restrict__ counts, int64_t ld) {
   const int v = nodes[blockIdx.x];
   const SliceTab tb = tabs[blockIdx.y];
-  slice_row<double>(counts + (int64_t)slot_of_node[v] * ld + tb.off, tip_lo[v], tip_hi[v], tb.col_ptr, tb.col_row,
-                    tb.col_val, tb.n);
-}
-__global__ void k_slice_presence(const int32_t *__restrict__ nodes, const int32_t *__restrict__ tip_lo,
-                                 const int32_t *__restrict__ tip_hi, const int32_t *__restrict__ slot_of_node,
-                                 const int64_t *__restrict__ col_ptr, const int32_t *__restrict__ col_row,
-                                 uint8_t *__restrict__ flags, int64_t ld, int n) {
-  const int v = nodes[blockIdx.x];
-  slice_row<uint8_t>(flags + (int64_t)slot_of_node[v] * ld, tip_lo[v], tip_hi[v], col_ptr, col_row, nullptr, n);
-}
-
-// count[v][k] = sum of the children's count[c][k], children in index order
-// (the order the postorder walk adds them in), over all ld columns; for
-// presence flags (C = uint8_t) the OR of the children's flags.
-// grid.x = nodes, grid.y = sample chunks.
-template <typename C>
-__global__ void k_node_counts(const int32_t *__restrict__ nodes,
-                              const int32_t *__restrict__ child_ptr,
-                              const int32_t *__restrict__ child_idx,
-                              const int32_t *__restrict__ slot_of_node,
-                              C *__restrict__ counts, int64_t ld) {
-  const int v = nodes[blockIdx.x];
-  const int64_t k = (int64_t)blockIdx.y * blockDim.x + threadIdx.x;
-  if (k >= ld) return;
-  C s = C(0);
-  for (int c = child_ptr[v]; c < child_ptr[v + 1]; c++) {
-    if constexpr (sizeof(C) == 1) s |= counts[(int64_t)slot_of_node[child_idx[c]] * ld + k];
-    else s += counts[(int64_t)slot_of_node[child_idx[c]] * ld + k];
+  double *row = counts + (int64_t)slot_of_node[v] * ld + tb.off;
+  for (int k = threadIdx.x; k < tb.n; k += blockDim.x) row[k] = 0.0;
+  __syncthreads();
+  const int f1 = tip_hi[v];
+  for (int f = tip_lo[v]; f < f1; f++) {
+    const int64_t q1 = tb.col_ptr[f + 1];
+    for (int64_t q = tb.col_ptr[f] + threadIdx.x; q < q1; q += blockDim.x) row[tb.col_row[q]] += tb.col_val[q];
+    __syncthreads();
   }
-  counts[(int64_t)slot_of_node[v] * ld + k] = s;
 }
 
-// The same with 16 bytes per thread (2 counts or 16 flags) for rows whose
-// stride is a multiple of 16 bytes: each element is still the sum (OR) of
-// the children's elements in index order, so the rows are bitwise those of
-// k_node_counts.  Columns [0, n_used) are written; the ragged end of a row
-// goes element by element.  grid.x = nodes, grid.y = column chunks.
-template <typename C>
-__global__ void k_node_counts_v16(const int32_t *__restrict__ nodes,
-                                  const int32_t *__restrict__ child_ptr,
-                                  const int32_t *__restrict__ child_idx,
-                                  const int32_t *__restrict__ slot_of_node,
-                                  C *__restrict__ counts, int64_t ld, int64_t n_used) {
-  constexpr int V = 16 / (int)sizeof(C);
-  const int v = nodes[blockIdx.x];
-  const int64_t e0 = ((int64_t)blockIdx.y * blockDim.x + threadIdx.x) * V;
-  if (e0 >= n_used) return;
-  const int c0 = child_ptr[v], c1 = child_ptr[v + 1];
-  C *dst = counts + (int64_t)slot_of_node[v] * ld + e0;
-  if (e0 + V <= n_used) {
-    if constexpr (sizeof(C) == 1) {
-      uint4 s = make_uint4(0u, 0u, 0u, 0u);
-      for (int c = c0; c < c1; c++) {
-        const uint4 x = *reinterpret_cast<const uint4 *>(counts + (int64_t)slot_of_node[child_idx[c]] * ld + e0);
-        s.x |= x.x;
-        s.y |= x.y;
-        s.z |= x.z;
-        s.w |= x.w;
-      }
-      *reinterpret_cast<uint4 *>(dst) = s;
-    } else {
-      double2 s = make_double2(0.0, 0.0);
-      for (int c = c0; c < c1; c++) {
-        const double2 x =
-            *reinterpret_cast<const double2 *>(counts + (int64_t)slot_of_node[child_idx[c]] * ld + e0);
-        s.x += x.x;
-        s.y += x.y;
-      }
-      *reinterpret_cast<double2 *>(dst) = s;
+// Presence bits of the same nodes, one warp per node: bit k of its row (word
+// k / 32) is 1 where combined sample k has a count below the node.  The rows of
+// all tables are one: `words` words of 32 samples.
+__global__ void k_slice_bits(const int32_t *__restrict__ nodes, int n_list, const int32_t *__restrict__ tip_lo,
+                             const int32_t *__restrict__ tip_hi, const int32_t *__restrict__ slot_of_node,
+                             const SliceTab *__restrict__ tabs, int n_tabs, uint32_t *__restrict__ bits, int64_t words) {
+  const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (i >= n_list) return;
+  const int v = nodes[i];
+  uint32_t *row = bits + (int64_t)slot_of_node[v] * words;
+  for (int64_t w = lane; w < words; w += 32) row[w] = 0u;
+  __syncwarp();
+  for (int t = 0; t < n_tabs; t++) {
+    const SliceTab &tb = tabs[t];
+    const int64_t q1 = tb.col_ptr[tip_hi[v]];
+    for (int64_t q = tb.col_ptr[tip_lo[v]] + lane; q < q1; q += 32) {
+      const int k = tb.off + tb.col_row[q];
+      atomicOr(row + (k >> 5), 1u << (k & 31));
     }
-    return;
   }
-  for (int64_t e = e0; e < n_used; e++) {
-    C s = C(0);
-    for (int c = c0; c < c1; c++) {
-      if constexpr (sizeof(C) == 1) s |= counts[(int64_t)slot_of_node[child_idx[c]] * ld + e];
-      else s += counts[(int64_t)slot_of_node[child_idx[c]] * ld + e];
-    }
-    counts[(int64_t)slot_of_node[v] * ld + e] = s;
-  }
-}
-
-// Node rows of one level: the 16-byte kernel when the stride and base allow
-// it, else one element per thread.
-template <typename C>
-cudaError_t launch_node_rows(const int32_t *nodes, int n_list, const int32_t *child_ptr, const int32_t *child_idx,
-                             const int32_t *slot_of_node, C *counts, int64_t ld, int64_t n_used,
-                             cudaStream_t st) {
-  if (n_list <= 0 || n_used <= 0) return cudaSuccess;
-  if ((ld * (int64_t)sizeof(C)) % 16 == 0 && reinterpret_cast<uintptr_t>(counts) % 16 == 0) {
-    constexpr int V = 16 / (int)sizeof(C);
-    const int64_t chunks = (n_used + V - 1) / V;
-    const int bt = chunks >= 256 ? 256 : 128;
-    return launch_k(k_node_counts_v16<C>, dim3(n_list, (unsigned)((chunks + bt - 1) / bt)), dim3(bt), 0, st,
-                    nodes, child_ptr, child_idx, slot_of_node, counts, ld, n_used);
-  }
-  return launch_k(k_node_counts<C>, dim3(n_list, (unsigned)((ld + 255) / 256)), dim3(256), 0, st, nodes,
-                  child_ptr, child_idx, slot_of_node, counts, ld);
 }
 
 // Table whose row segment holds column j (segments are contiguous, in order).
@@ -299,9 +216,9 @@ __global__ void k_embed_steps(const EmbedArgs a, int4 *__restrict__ steps, doubl
   q.x = a.slot_of_node[v];
   q.y = nc > 0 ? a.slot_of_node[a.child_idx[c0]] : -1;
   q.z = nc == 2 ? a.slot_of_node[a.child_idx[c0 + 1]] : nc > 2 ? -2 - v : -1;
-  q.w = a.xrow[p];
+  q.w = a.xrow ? a.xrow[p] : -1;
   steps[i] = q;
-  len[i] = a.length[v];
+  if (len) len[i] = a.length[v];
 }
 
 // STEPS: from k_embed_steps' records; else from the tree's arrays (the
@@ -394,12 +311,46 @@ __global__ void __launch_bounds__(512) k_embed_slab(const EmbedArgs a) {
   }
 }
 
+// The same walk for presence bits: a node's words are the OR of its children's.
+__global__ void __launch_bounds__(512) k_bits_slab(const EmbedArgs a) {
+  constexpr int U = 4;
+  const int per = blockDim.x / a.w, g = threadIdx.x / a.w;
+  const int k = blockIdx.x * a.w + (threadIdx.x - g * a.w);
+  uint32_t *bits = a.bits + k;
+  const int p_first = a.levels[0];
+  for (int lv = a.lv0; lv < a.lv1; lv++) {
+    const int p1 = a.levels[a.level_step * lv + 1];
+    if (k < a.n_cols)
+      for (int p = a.levels[a.level_step * lv] + blockIdx.y * (U * per) + g; p < p1; p += gridDim.y * (U * per)) {
+        int4 q[U];
+        uint32_t s[U];
+#pragma unroll
+        for (int u = 0; u < U; u++)
+          q[u] = p + u * per < p1 ? a.steps[p + u * per - p_first] : make_int4(-1, -1, -1, -1);
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+          s[u] = q[u].y >= 0 ? bits[(int64_t)q[u].y * a.ld] : 0u;
+          if (q[u].z >= 0) s[u] |= bits[(int64_t)q[u].z * a.ld];
+        }
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+          if (q[u].z < -1)
+            for (int v = -2 - q[u].z, c = a.child_ptr[v]; c < a.child_ptr[v + 1]; c++)
+              s[u] |= bits[(int64_t)a.slot_of_node[a.child_idx[c]] * a.ld];
+          if (q[u].x >= 0) bits[(int64_t)q[u].x * a.ld] = s[u];
+        }
+      }
+    __syncthreads();
+  }
+}
+
 namespace {
 // elements of a level from which it gets a launch of its own
 constexpr int64_t EMBED_WIDE = 1 << 18;
 
 cudaError_t embed_launch(int kind, bool fp32, const EmbedArgs &a, dim3 grid, int nt, cudaStream_t st) {
   const bool steps = a.steps != nullptr;
+  if (a.bits) return launch_k(k_bits_slab, grid, dim3(nt), 0, st, a);
 #define UF_SLAB(T, K)                                                                    \
   return launch_k(steps ? k_embed_slab<T, K, true> : k_embed_slab<T, K, false>, grid, dim3(nt), 0, st, a)
   if (kind == EMB_VAW) {
@@ -459,7 +410,7 @@ cudaError_t launch_embed(int kind, bool fp32, const EmbedArgs &a0, const int *le
   // every SM one
   a.lv1 = a.n_levels;
   a.w = 16;
-  while (a.w > 2 && (a.n_cols + a.w - 1) / a.w < sms) a.w /= 2;
+  while (a.w > (a.bits ? 1 : 2) && (a.n_cols + a.w - 1) / a.w < sms) a.w /= 2;
   int most = 1;
   if (a.first) most = level_nodes[0];
   for (int l = a.lv0; l < a.n_levels; l++) most = std::max(most, level_nodes[l]);
@@ -488,19 +439,12 @@ cudaError_t launch_slice_counts(const int32_t *nodes, int n_list, const int32_t 
   return cudaSuccess;
 }
 
-cudaError_t launch_slice_presence(const int32_t *nodes, int n_list, const int32_t *tip_lo, const int32_t *tip_hi,
-                                  const int32_t *slot_of_node, const int64_t *col_ptr, const int32_t *col_row,
-                                  uint8_t *flags, int64_t ld, int n, cudaStream_t st) {
+cudaError_t launch_slice_bits(const int32_t *nodes, int n_list, const int32_t *tip_lo, const int32_t *tip_hi,
+                              const int32_t *slot_of_node, const SliceTab *tabs, int n_tabs, uint32_t *bits,
+                              int64_t words, cudaStream_t st) {
   if (n_list <= 0) return cudaSuccess;
-  return launch_k(k_slice_presence, dim3(n_list), dim3(256), 0, st, nodes, tip_lo, tip_hi, slot_of_node, col_ptr,
-                  col_row, flags, ld, n);
-}
-
-cudaError_t launch_node_presence(const int32_t *nodes, int n_list, const int32_t *child_ptr,
-                                 const int32_t *child_idx, const int32_t *slot_of_node,
-                                 uint8_t *flags, int64_t ld, cudaStream_t st, int64_t n_used) {
-  return launch_node_rows<uint8_t>(nodes, n_list, child_ptr, child_idx, slot_of_node, flags, ld,
-                                   n_used < 0 ? ld : n_used, st);
+  return launch_k(k_slice_bits, dim3((n_list + 7) / 8), dim3(256), 0, st, nodes, n_list, tip_lo, tip_hi, slot_of_node,
+                  tabs, n_tabs, bits, words);
 }
 
 cudaError_t launch_emb_rows(int kind, bool fp32, int64_t b0, int rows,

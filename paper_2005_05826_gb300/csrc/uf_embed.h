@@ -22,15 +22,10 @@ struct SliceTab {
 cudaError_t launch_slice_counts(const int32_t *nodes, int n_list, const int32_t *tip_lo, const int32_t *tip_hi,
                                 const int32_t *slot_of_node, const SliceTab *tabs, int n_tabs, double *counts,
                                 int64_t ld, cudaStream_t st);
-// Presence flags (uint8_t, 1 where the count is nonzero) instead of counts.
-cudaError_t launch_slice_presence(const int32_t *nodes, int n_list, const int32_t *tip_lo, const int32_t *tip_hi,
-                                  const int32_t *slot_of_node, const int64_t *col_ptr, const int32_t *col_row,
-                                  uint8_t *flags, int64_t ld, int n, cudaStream_t st);
-// Rows of one level's nodes from their children's rows, columns [0, n_used)
-// of rows with stride ld (n_used < 0: all ld columns).
-cudaError_t launch_node_presence(const int32_t *nodes, int n_list, const int32_t *child_ptr,
-                                 const int32_t *child_idx, const int32_t *slot_of_node,
-                                 uint8_t *flags, int64_t ld, cudaStream_t st, int64_t n_used = -1);
+// Presence bits (`words` words of 32 combined samples a row) instead of counts.
+cudaError_t launch_slice_bits(const int32_t *nodes, int n_list, const int32_t *tip_lo, const int32_t *tip_hi,
+                              const int32_t *slot_of_node, const SliceTab *tabs, int n_tabs, uint32_t *bits,
+                              int64_t words, cudaStream_t st);
 // Count rows of a block's internal nodes, level by level, and the embedding
 // rows of its dense branches.
 struct EmbedArgs {
@@ -44,7 +39,8 @@ struct EmbedArgs {
   const int32_t *xrow;          // per list position its row of X, or -1
   const int32_t *child_ptr, *child_idx;
   const int32_t *slot_of_node;
-  double *counts;               // rows of ld values, one column per combined sample
+  double *counts;               // rows of ld values, one column per combined sample, or:
+  uint32_t *bits;               // rows of ld presence words, n_cols of them used (no X then)
   int64_t ld;
   int n_cols;
   const double *length;         // by node

@@ -74,13 +74,12 @@ int64_t gram_kpad(int rows);              // branches rounded up to the stage
 // diagonal cell, in row-major block order: (bi, bj) appended to bi / bj.
 // Stripe s holds the pairs at distance d = j - i of s + 1 and n - s - 1.
 void gram_tiles(int n, int64_t s0, int64_t s1, std::vector<int32_t> *bi, std::vector<int32_t> *bj);
-// planes of branches nodes[0 .. rows) (b0 .. b0 + rows - 1 when nodes is null)
-// from their presence flags: 1 + GRAM_SPLITS planes, or with digit_scale != 0
+// planes of branches nodes[0 .. rows) from their presence bits (rows of `words`
+// words, uf_embed.h): 1 + GRAM_SPLITS planes, or with digit_scale != 0
 // (2^g, every length x 2^g below 2^62) 1 + GRAM_DIGITS
-cudaError_t launch_gram_prep(int64_t b0, int rows, const int32_t *slot_of_node, const uint8_t *flags,
-                             int64_t ld, const double *length, const GramTab *tabs, int n_tabs,
-                             int npad_tot, int64_t K_pad, void *Pl, cudaStream_t st,
-                             const int32_t *nodes = nullptr, double digit_scale = 0.0);
+cudaError_t launch_gram_prep(const int32_t *nodes, int rows, const int32_t *slot_of_node, const uint32_t *bits,
+                             int64_t words, const double *length, const GramTab *tabs, int n_tabs, int npad_tot,
+                             int64_t K_pad, void *Pl, double digit_scale, cudaStream_t st);
 cudaError_t launch_gram(const GramArgs &a, void *Pl, int64_t K_pad, cudaStream_t st);
 cudaError_t launch_finalize_gram(const GramFinalArgs &a, cudaStream_t st);
 

@@ -519,28 +519,6 @@ void fill_reports(uf_tree *tree, const BatchJob &J, const Outputs &o, double ms[
   }
 }
 
-// Rows of block b that the split needs as presence flags (the tensor-core
-// unweighted path needs nothing else), one byte per sample: CSC-built nodes of
-// every table, then the dense internal levels over the combined axis.
-void enqueue_split_presence(const Inputs &in, const BatchJob &J, const std::vector<int> &off,
-                            const RowSplit &split, size_t b, const int32_t *d_cnt, uint8_t *flags, int64_t ld,
-                            int64_t n_cols, cudaStream_t st, int64_t *kernels) {
-  const auto &lb = split.cnt_launch[b];
-  for (size_t t = 0; t < J.tabs.size(); t++) {
-    ck(launch_slice_presence(d_cnt + lb[0].first, lb[0].second, in.td->tip_lo, in.td->tip_hi, in.pd->slot_of_node,
-                             in.xd[t]->col_ptr, in.xd[t]->col_row, flags + off[t], ld, (int)J.tabs[t].table->n,
-                             st),
-       "presence rows");
-    *kernels += lb[0].second > 0;
-  }
-  for (size_t l = 1; l < lb.size(); l++) {
-    ck(launch_node_presence(d_cnt + lb[l].first, lb[l].second, in.td->child_ptr, in.td->child_idx,
-                            in.pd->slot_of_node, flags, ld, st, n_cols),
-       "node presence");
-    (*kernels)++;
-  }
-}
-
 // Stripe-layout description of the tables of a call for the sparse-row
 // scatter: samples, combined column, stored stripes and first cell of each.
 struct SpLayout {
@@ -779,10 +757,10 @@ uf_status run_gram(uf_tree *tree, const BatchJob &J, int device, double scale) {
   const int n_tiles = (int)G.n_tiles;
   const int64_t nb = tree->n_nodes - 1;
   const bool digits = !J.fp32;
-  const int words = digits ? 2 : 1, planes = 1 + (digits ? GRAM_DIGITS : GRAM_SPLITS);
+  const int acc_words = digits ? 2 : 1, planes = 1 + (digits ? GRAM_DIGITS : GRAM_SPLITS);
   const int64_t gt_cells = std::max<int64_t>(G.n_tiles, 1) * GRAM_TILE_CELLS;
-  const int64_t rows = block_rows(nb, (double)n_cols + 2.0 * planes * npad_tot + 8.0,
-                                  ((double)gt_cells + (double)cells) * 8.0 * words);
+  const int64_t rows = block_rows(nb, (double)n_cols / 8.0 + 2.0 * planes * npad_tot + 8.0,
+                                  ((double)gt_cells + (double)cells) * 8.0 * acc_words);
   Inputs in = [&] {
     NvtxRange r("uf: bind inputs");
     return bind_inputs(tree, J, device, rows);
@@ -801,24 +779,33 @@ uf_status run_gram(uf_tree *tree, const BatchJob &J, int device, double scale) {
   std::vector<int32_t> tl(G.tile_tab);
   tl.insert(tl.end(), G.tile_bi.begin(), G.tile_bi.end());
   tl.insert(tl.end(), G.tile_bj.begin(), G.tile_bj.end());
-  // presence rows: stride rounded up to 16 bytes for the 16-byte level kernel
-  const int64_t ld = round_up(n_cols, 16);
-  DevBuf flags((size_t)in.P->n_slots * ld, st, "alloc presence rows");
+  // presence rows: a bit per combined sample
+  const int64_t words = (n_cols + 31) / 32;
+  DevBuf bits((size_t)in.P->n_slots * words * 4, st, "alloc presence rows");
+  int64_t most_nodes = 1;  // presence rows of one block
+  for (const auto &lb : split.cnt_launch)
+    most_nodes = std::max(most_nodes, lb.back().first + lb.back().second - lb[0].first);
+  DevBuf steps((size_t)most_nodes * sizeof(int4), st, "alloc presence steps");
   DevBuf Pl((size_t)planes * npad_tot * K_pad * 2, st, "alloc presence planes");
-  DevBuf Gt((size_t)gt_cells * 8 * words, st, "alloc gram tiles");
+  DevBuf Gt((size_t)gt_cells * 8 * acc_words, st, "alloc gram tiles");
   DevBuf err(sizeof(int), st, "alloc error flag");
   DevBuf clamps(sizeof(unsigned long long), st, "alloc clamp counter");
   DevBuf Msp;
   Meta meta;  // tile list, table descriptors, tile maps and row lists: one staged upload
   const size_t o_tiles = meta.add(tl), o_tabs = meta.add(G.gt), o_maps = meta.add(G.maps);
   const size_t o_cnt = meta.add(split.cnt_lists), o_dense = meta.add(split.dense);
+  const size_t o_levels = meta.add(split.cnt_levels);
+  std::vector<SliceTab> slice(nt);
+  for (size_t t = 0; t < nt; t++)
+    slice[t] = SliceTab{in.xd[t]->col_ptr, in.xd[t]->col_row, in.xd[t]->col_val, G.gt[t].n, G.gt[t].off};
+  const size_t o_slice = meta.add(slice);
   // sparse rows: presence terms (x = l) in FP64, one word (FP64 calls: two),
   // min form, into stripe-layout cells Msp and the per-sample R
   SparseScatter sc;
   sc.prepare(tree, J, in, split, lay, ACC_MIN, true, digits, cells, n_cols, meta, st);
   if (split.n_sparse > 0) {
-    Msp = DevBuf((size_t)cells * 8 * words, st, "alloc sparse stripes");
-    ck(cudaMemsetAsync(Msp.p, 0, (size_t)cells * 8 * words, st), "memset");
+    Msp = DevBuf((size_t)cells * 8 * acc_words, st, "alloc sparse stripes");
+    ck(cudaMemsetAsync(Msp.p, 0, (size_t)cells * 8 * acc_words, st), "memset");
   }
   // digits: the lengths' grid 2^-g, the longest dense one below 2^62 on it,
   // no finer than the second words' 2^-(F+32)
@@ -839,7 +826,7 @@ uf_status run_gram(uf_tree *tree, const BatchJob &J, int device, double scale) {
   const int32_t *d_tiles = meta.at<int32_t>(o_tiles);
   const GramTab *d_tabs = meta.at<GramTab>(o_tabs);
   const int32_t *d_cnt = meta.at<int32_t>(o_cnt), *d_dense = meta.at<int32_t>(o_dense);
-  ck(cudaMemsetAsync(Gt.p, 0, (size_t)gt_cells * 8 * words, st), "memset");
+  ck(cudaMemsetAsync(Gt.p, 0, (size_t)gt_cells * 8 * acc_words, st), "memset");
   ck(cudaMemsetAsync(err.p, 0, sizeof(int), st), "memset");
   ck(cudaMemsetAsync(clamps.p, 0, sizeof(unsigned long long), st), "memset");
   // the region scatter's pair updates, counted when the call is timed per phase
@@ -868,13 +855,33 @@ uf_status run_gram(uf_tree *tree, const BatchJob &J, int device, double scale) {
     timer.end();
   }
   for (size_t b = 0; b < in.P->b0.size(); b++) {
-    const int64_t b0 = in.P->b0[b];
     const int64_t d0 = split.dense_ptr[b], nd = split.dense_ptr[b + 1] - d0;
     timer.begin(0);
-    enqueue_split_presence(in, J, off, split, b, d_cnt, flags.as<uint8_t>(), ld, n_cols, ls, &kernels);
+    const auto &built = split.cnt_launch[b][0];
+    ck(launch_slice_bits(d_cnt + built.first, built.second, in.td->tip_lo, in.td->tip_hi, in.pd->slot_of_node,
+                         meta.at<SliceTab>(o_slice), (int)nt, bits.as<uint32_t>(), words, ls),
+       "presence rows");
+    kernels += built.second > 0;
+    EmbedArgs ea{};
+    ea.list = d_cnt;
+    ea.levels = meta.at<int32_t>(o_levels) + split.cnt_lev_ptr[b];
+    ea.level_step = 2;
+    ea.n_levels = (int)split.cnt_launch[b].size();
+    ea.n_nodes = (int)(split.cnt_launch[b].back().first + split.cnt_launch[b].back().second - built.first);
+    ea.child_ptr = in.td->child_ptr;
+    ea.child_idx = in.td->child_idx;
+    ea.slot_of_node = in.pd->slot_of_node;
+    ea.bits = bits.as<uint32_t>();
+    ea.ld = words;
+    ea.n_cols = (int)words;
+    ea.length = in.td->length;
+    ea.steps = steps.as<int4>();
+    std::vector<int> level_nodes;
+    for (const auto &l : split.cnt_launch[b]) level_nodes.push_back(l.second);
+    ck(launch_embed(EMB_PRESENCE, true, ea, level_nodes.data(), ls, &kernels), "presence levels");
     if (nd > 0) {
-      ck(launch_gram_prep(b0, (int)nd, in.pd->slot_of_node, flags.as<uint8_t>(), ld, in.td->length, d_tabs,
-                          (int)nt, npad_tot, K_pad, Pl.p, ls, d_dense + d0, digit_scale),
+      ck(launch_gram_prep(d_dense + d0, (int)nd, in.pd->slot_of_node, bits.as<uint32_t>(), words, in.td->length,
+                          d_tabs, (int)nt, npad_tot, K_pad, Pl.p, digit_scale, ls),
          "presence planes");
       kernels++;
     }
@@ -951,7 +958,8 @@ uf_status run_gram(uf_tree *tree, const BatchJob &J, int device, double scale) {
   if (!J.out_is_device)
     for (size_t t = 0; t < nt; t++)
       ck(cudaMemcpyAsync(J.tabs[t].out, o.dev[t], o.bytes[t], cudaMemcpyDeviceToHost, st), "copy out");
-  flags = DevBuf();
+  bits = DevBuf();
+  steps = DevBuf();
   Pl = DevBuf();
   Gt = DevBuf();
   Msp = DevBuf();
