@@ -180,24 +180,37 @@ std::mutex g_ring_mu;
 std::map<int, UploadRing> g_rings;
 }  // namespace
 
-void pinned_upload(void *dst, const void *src, size_t bytes) {
-  if (bytes == 0) return;
+namespace {
+// The current device's ring (set up on first use), or null without pinned
+// memory; the caller holds g_ring_mu.
+UploadRing *upload_ring() {
   int dev = 0;
   ck(cudaGetDevice(&dev), "upload");
-  std::lock_guard<std::mutex> g(g_ring_mu);
   UploadRing &R = g_rings[dev];
   if (!R.ok) {
     bool good = cudaStreamCreateWithFlags(&R.st, cudaStreamNonBlocking) == cudaSuccess;
     for (int i = 0; good && i < UploadRing::NBUF; i++)
       good = cudaHostAlloc((void **)&R.buf[i], UploadRing::CHUNK, cudaHostAllocPortable) == cudaSuccess &&
              cudaEventCreateWithFlags(&R.ev[i], cudaEventDisableTiming) == cudaSuccess;
-    if (!good) {  // no pinned memory: the driver's own staged copy
+    if (!good) {
       cudaGetLastError();
-      ck(cudaMemcpy(dst, src, bytes, cudaMemcpyHostToDevice), "upload");
-      return;
+      return nullptr;
     }
     R.ok = true;
   }
+  return &R;
+}
+}  // namespace
+
+void pinned_upload(void *dst, const void *src, size_t bytes) {
+  if (bytes == 0) return;
+  std::lock_guard<std::mutex> g(g_ring_mu);
+  UploadRing *ring = upload_ring();
+  if (!ring) {  // no pinned memory: the driver's own staged copy
+    ck(cudaMemcpy(dst, src, bytes, cudaMemcpyHostToDevice), "upload");
+    return;
+  }
+  UploadRing &R = *ring;
   const char *s = static_cast<const char *>(src);
   char *d = static_cast<char *>(dst);
   const int nt = std::max(1, std::min(host_threads(), 8));
@@ -216,6 +229,22 @@ void pinned_upload(void *dst, const void *src, size_t bytes) {
   }
   ck(cudaStreamSynchronize(R.st), "upload");
   for (bool &x : R.busy) x = false;
+}
+
+void pinned_upload_parts(char *dst, const std::vector<std::pair<const void *, size_t>> &parts,
+                         const std::vector<size_t> &offs, size_t total) {
+  // (the pool's threads cost more than they copy below a few megabytes)
+  if (total <= (size_t)4 << 20) {
+    std::lock_guard<std::mutex> g(g_ring_mu);
+    if (UploadRing *R = upload_ring()) {
+      for (size_t i = 0; i < parts.size(); i++)
+        if (parts[i].second) memcpy(R->buf[0] + offs[i], parts[i].first, parts[i].second);
+      ck(cudaMemcpyAsync(dst, R->buf[0], total, cudaMemcpyHostToDevice, R->st), "upload");
+      ck(cudaStreamSynchronize(R->st), "upload");
+      return;
+    }
+  }
+  for (size_t i = 0; i < parts.size(); i++) pinned_upload(dst + offs[i], parts[i].first, parts[i].second);
 }
 
 uf_tree::Dev &tree_dev(uf_tree *t, int device) {
@@ -658,7 +687,7 @@ uf_status uf_table_create(int64_t n_samples, int64_t n_features, const int64_t *
   if (nnz > 0 && (!indices || !data)) return fail(UF_EINVAL, "null indices or data");
   try {
     // sample ranges of about equal nonzeros, one per host thread
-    const int T = (int)std::max<int64_t>(1, std::min<int64_t>(host_threads(), nnz / 100000));
+    const int T = (int)std::max<int64_t>(1, std::min<int64_t>(host_threads(), nnz / 20000));
     std::vector<int64_t> k_lo(T + 1, n_samples);
     k_lo[0] = 0;
     for (int c = 1, k = 0; c < T; c++) {

@@ -14,23 +14,72 @@ namespace rt {
 
 namespace {
 
+// A call's small buffers come from slabs of one pool allocation each: calls
+// that take turns on several streams make the pool look for a block among those
+// other streams freed, for every buffer (the host time of a 146-sample call
+// grew from 0.18 to 0.8 ms).  The slabs go back to the pool, in stream order,
+// when the call's arena is destroyed, after all its launches are queued.
+struct Arena {
+  static constexpr size_t SLAB = (size_t)8 << 20, MOST = (size_t)2 << 20;  // slab, largest buffer taken from one
+  cudaStream_t st;
+  std::vector<void *> slabs;
+  char *at = nullptr;
+  size_t left = 0;
+  Arena *outer;
+  explicit Arena(cudaStream_t s);
+  ~Arena();
+  // null when no slab can be had (the buffer then asks the pool itself)
+  void *take(size_t bytes) {
+    bytes = (bytes + 255) & ~(size_t)255;
+    if (bytes > left) {
+      void *p = nullptr;
+      if (cudaMallocAsync(&p, SLAB, st) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+      }
+      slabs.push_back(p);
+      at = (char *)p;
+      left = SLAB;
+    }
+    void *p = at;
+    at += bytes;
+    left -= bytes;
+    return p;
+  }
+};
+thread_local Arena *t_arena = nullptr;  // of the call the thread is in
+Arena::Arena(cudaStream_t s) : st(s), outer(t_arena) {
+  slabs.reserve(16);
+  t_arena = this;
+}
+Arena::~Arena() {
+  t_arena = outer;
+  for (void *p : slabs) cudaFreeAsync(p, st);
+}
+
 struct DevBuf {
   void *p = nullptr;
   cudaStream_t st = nullptr;
+  bool own = false;
   DevBuf() = default;
   DevBuf(size_t bytes, cudaStream_t s, const char *what) : st(s) {
-    ck(cudaMallocAsync(&p, std::max<size_t>(bytes, 256), s), what);
+    bytes = std::max<size_t>(bytes, 256);
+    if (t_arena && t_arena->st == s && bytes <= Arena::MOST) p = t_arena->take(bytes);
+    if (p) return;
+    ck(cudaMallocAsync(&p, bytes, s), what);
+    own = true;
   }
   DevBuf(const DevBuf &) = delete;
   DevBuf &operator=(const DevBuf &) = delete;
-  DevBuf(DevBuf &&o) noexcept : p(o.p), st(o.st) { o.p = nullptr; }
+  DevBuf(DevBuf &&o) noexcept : p(o.p), st(o.st), own(o.own) { o.p = nullptr; }
   DevBuf &operator=(DevBuf &&o) noexcept {
     std::swap(p, o.p);
     std::swap(st, o.st);
+    std::swap(own, o.own);
     return *this;
   }
   ~DevBuf() {
-    if (p) cudaFreeAsync(p, st);
+    if (p && own) cudaFreeAsync(p, st);
   }
   template <typename T>
   T *as() const { return (T *)p; }
@@ -788,8 +837,10 @@ uf_status run_gram(uf_tree *tree, const BatchJob &J, int device, double scale) {
   DevBuf steps((size_t)most_nodes * sizeof(int4), st, "alloc presence steps");
   DevBuf Pl((size_t)planes * npad_tot * K_pad * 2, st, "alloc presence planes");
   DevBuf Gt((size_t)gt_cells * 8 * acc_words, st, "alloc gram tiles");
-  DevBuf err(sizeof(int), st, "alloc error flag");
-  DevBuf clamps(sizeof(unsigned long long), st, "alloc clamp counter");
+  // the clamp counter, then the kernel's abort flag
+  DevBuf flags(2 * sizeof(unsigned long long), st, "alloc flags");
+  unsigned long long *const clamps = flags.as<unsigned long long>();
+  int *const err = (int *)(clamps + 1);
   DevBuf Msp;
   Meta meta;  // tile list, table descriptors, tile maps and row lists: one staged upload
   const size_t o_tiles = meta.add(tl), o_tabs = meta.add(G.gt), o_maps = meta.add(G.maps);
@@ -827,11 +878,13 @@ uf_status run_gram(uf_tree *tree, const BatchJob &J, int device, double scale) {
   const GramTab *d_tabs = meta.at<GramTab>(o_tabs);
   const int32_t *d_cnt = meta.at<int32_t>(o_cnt), *d_dense = meta.at<int32_t>(o_dense);
   ck(cudaMemsetAsync(Gt.p, 0, (size_t)gt_cells * 8 * acc_words, st), "memset");
-  ck(cudaMemsetAsync(err.p, 0, sizeof(int), st), "memset");
-  ck(cudaMemsetAsync(clamps.p, 0, sizeof(unsigned long long), st), "memset");
+  ck(cudaMemsetAsync(flags.p, 0, 2 * sizeof(unsigned long long), st), "memset");
   // the region scatter's pair updates, counted when the call is timed per phase
-  DevBuf pair_ctr(SPARSE_PAIR_SLOTS * sizeof(unsigned long long), st, "alloc pair counter");
-  ck(cudaMemsetAsync(pair_ctr.p, 0, SPARSE_PAIR_SLOTS * sizeof(unsigned long long), st), "memset");
+  DevBuf pair_ctr;
+  if (timer.on) {
+    pair_ctr = DevBuf(SPARSE_PAIR_SLOTS * sizeof(unsigned long long), st, "alloc pair counter");
+    ck(cudaMemsetAsync(pair_ctr.p, 0, SPARSE_PAIR_SLOTS * sizeof(unsigned long long), st), "memset");
+  }
   Outputs o = bind_outputs(J, st);
   double exec_flops = 0.0;
   Capture cap(g_graph.load() != 0 && !timer.on, st, device);
@@ -907,7 +960,7 @@ uf_status run_gram(uf_tree *tree, const BatchJob &J, int device, double scale) {
     ga.tabs = d_tabs;
     ga.Gt = Gt.as<unsigned long long>();
     ga.scale = scale;
-    ga.err = err.as<int>();
+    ga.err = err;
     ga.wait_test = (int)g_tensor_wait_test.load();
     timer.begin(1);
     ck(launch_gram(ga, Pl.p, K_pad, ls), "tensor-core gram");
@@ -934,8 +987,8 @@ uf_status run_gram(uf_tree *tree, const BatchJob &J, int device, double scale) {
     fa.d_lo_off = digits ? n_cols : 0;
     fa.out = o.dev[t];
     fa.out_fp32 = J.out_fp32;
-    fa.err = err.as<int>();
-    fa.clamps = clamps.as<unsigned long long>();
+    fa.err = err;
+    fa.clamps = clamps;
     fa.unnormalized = unnormalized(J.method);
     fa.inv_scale = 1.0 / scale;
     ck(launch_finalize_gram(fa, ls), "finalize");
@@ -948,12 +1001,11 @@ uf_status run_gram(uf_tree *tree, const BatchJob &J, int device, double scale) {
   // the finalize has already written NaN to every output when it is set
   const bool sync = !J.out_is_device || st == nullptr || timer.on;
   const bool pairs_counted = timer.on && sc.region_mode;
-  int h_err = 0;
-  unsigned long long h_clamps = 0, h_pairs[SPARSE_PAIR_SLOTS] = {};
+  unsigned long long h_flags[2] = {}, h_pairs[SPARSE_PAIR_SLOTS] = {};
   if (sync) {
-    ck(cudaMemcpyAsync(&h_err, err.p, sizeof(int), cudaMemcpyDeviceToHost, st), "copy flag");
-    ck(cudaMemcpyAsync(&h_clamps, clamps.p, sizeof h_clamps, cudaMemcpyDeviceToHost, st), "copy count");
-    ck(cudaMemcpyAsync(h_pairs, pair_ctr.p, sizeof h_pairs, cudaMemcpyDeviceToHost, st), "copy count");
+    ck(cudaMemcpyAsync(h_flags, flags.p, sizeof h_flags, cudaMemcpyDeviceToHost, st), "copy flags");
+    if (pairs_counted)
+      ck(cudaMemcpyAsync(h_pairs, pair_ctr.p, sizeof h_pairs, cudaMemcpyDeviceToHost, st), "copy count");
   }
   if (!J.out_is_device)
     for (size_t t = 0; t < nt; t++)
@@ -966,12 +1018,11 @@ uf_status run_gram(uf_tree *tree, const BatchJob &J, int device, double scale) {
   sc = SparseScatter();
   meta.dev = DevBuf();
   o.tmp.clear();
-  err = DevBuf();
-  clamps = DevBuf();
   pair_ctr = DevBuf();
   if (sync) ck(cudaStreamSynchronize(st), "synchronize");
   else ck(cudaGetLastError(), "enqueue");
-  if (h_err) return fail(UF_ETIMEOUT, "tensor-core kernel: a bounded wait gave up");
+  const unsigned long long h_clamps = h_flags[0];
+  if (h_flags[1]) return fail(UF_ETIMEOUT, "tensor-core kernel: a bounded wait gave up");
   double ms[5] = {0, 0, 0, 0, 0};
   timer.collect(ms);
   fill_reports(tree, J, o, ms, kernels, acc_launches, 1, rows, (int64_t)in.P->b0.size(), exec_flops, GRAM_TN,
@@ -1142,8 +1193,11 @@ uf_status run_stripes(uf_tree *tree, const BatchJob &J, int device, uf_method me
   ck(cudaMemsetAsync(M.p, 0, m_bytes, st), "memset");
   ck(cudaMemsetAsync(clamps.p, 0, sizeof(unsigned long long), st), "memset");
   // the region scatter's pair updates, counted when the call is timed per phase
-  DevBuf pair_ctr(SPARSE_PAIR_SLOTS * sizeof(unsigned long long), st, "alloc pair counter");
-  ck(cudaMemsetAsync(pair_ctr.p, 0, SPARSE_PAIR_SLOTS * sizeof(unsigned long long), st), "memset");
+  DevBuf pair_ctr;
+  if (timer.on) {
+    pair_ctr = DevBuf(SPARSE_PAIR_SLOTS * sizeof(unsigned long long), st, "alloc pair counter");
+    ck(cudaMemsetAsync(pair_ctr.p, 0, SPARSE_PAIR_SLOTS * sizeof(unsigned long long), st), "memset");
+  }
   Outputs o = bind_outputs(J, st);
   double exec_flops = 0.0;
   // tile shape and chunk size: tuned once per (accumulator, precision, size
@@ -1363,7 +1417,8 @@ uf_status run_stripes(uf_tree *tree, const BatchJob &J, int device, uf_method me
   unsigned long long h_clamps = 0, h_pairs[SPARSE_PAIR_SLOTS] = {};
   if (sync) {
     ck(cudaMemcpyAsync(&h_clamps, clamps.p, sizeof h_clamps, cudaMemcpyDeviceToHost, st), "copy count");
-    ck(cudaMemcpyAsync(h_pairs, pair_ctr.p, sizeof h_pairs, cudaMemcpyDeviceToHost, st), "copy count");
+    if (pairs_counted)
+      ck(cudaMemcpyAsync(h_pairs, pair_ctr.p, sizeof h_pairs, cudaMemcpyDeviceToHost, st), "copy count");
   }
   if (!J.out_is_device)
     for (size_t t = 0; t < nt; t++)
@@ -1420,6 +1475,7 @@ uf_status run_batch(uf_tree *tree, const BatchJob &J) {
   int device = 0;
   ck(cudaGetDevice(&device), "cudaGetDevice");
   keep_pool_memory(device);
+  const Arena arena(J.st);
   uf_method method = J.method;
   if (method == UF_GENERALIZED && J.alpha == 1.0) method = UF_WEIGHTED_NORMALIZED;  // s^0 == 1
   const int kind = kind_of(method);

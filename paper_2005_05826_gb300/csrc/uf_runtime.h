@@ -97,6 +97,10 @@ struct NoInit : std::allocator<T> {
 // (a plain cudaMemcpy from pageable memory is staged by the driver at a
 // fraction of the link's rate).  Synchronous: returns when dst holds the data.
 void pinned_upload(void *dst, const void *src, size_t bytes);
+// The same for several arrays at their offsets in one device block of `total`
+// bytes: one copy and one wait where they fit one chunk together.
+void pinned_upload_parts(char *dst, const std::vector<std::pair<const void *, size_t>> &parts,
+                         const std::vector<size_t> &offs, size_t total);
 
 // Several host arrays copied into one device allocation at 256-byte aligned
 // offsets: one cudaMalloc per handle instead of one per array.
@@ -116,16 +120,13 @@ struct DevPack {
   char *upload(const char *what) {
     char *d = nullptr;
     ck(cudaMalloc(&d, std::max<size_t>(total, 16)), what);
-    for (size_t i = 0; i < parts.size(); i++) {
-      if (!parts[i].second) continue;
-      try {
-        pinned_upload(d + offs[i], parts[i].first, parts[i].second);
-      } catch (...) {
-        cudaFree(d);
-        throw;
-      }
-      g_h2d += (double)parts[i].second;
+    try {
+      pinned_upload_parts(d, parts, offs, total);
+    } catch (...) {
+      cudaFree(d);
+      throw;
     }
+    for (const auto &p : parts) g_h2d += (double)p.second;
     return d;
   }
   template <typename T>
