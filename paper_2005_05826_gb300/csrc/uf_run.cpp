@@ -593,11 +593,74 @@ struct SparseScatter {
   DevBuf le, lk, lz, Dsp, cur;
   int64_t list_entries = 0;
   std::vector<SpLayout> lay;
+  // tile scatter: rows of the classes from here on, the windows, the offsets
+  bool tiles = false;
+  std::vector<int64_t> tile_off, tile_n;
+  int64_t n_tile_rows = 0, n_tiles = 0;
+  int n_win = 0;
+  size_t o_win = 0;
+  DevBuf toff;
 
-  // acc: ACC_MIN / ACC_GEN; fp64_entries: terms computed in FP64
+  // Places the rows of at least `least` entries in the tile scatter's lists
+  // (after the others, class by class) and allocates its buffers; false when
+  // they do not fit the memory at hand.
+  bool prepare_tiles(uf_tree *tree, const BatchJob &J, const RowSplit &sp, std::vector<int32_t> *all, Meta &meta,
+                     cudaStream_t st) {
+    std::vector<TileWin> win;
+    n_tiles = tile_windows(lay[0].n, lay[0].s_lo, lay[0].s_hi, &win);
+    if (n_tiles > INT32_MAX / 2) return false;
+    // a listed row costs a look at its offsets per tile, a direct one an atomic
+    // per pair: both over the full stripe range, so that a range call splits
+    // the rows as the full run does (FP64 lists have a grid of their own)
+    const double n = lay[0].n, full = 0.5 * n * n;
+    const double rate = full * 16.0 <= 64e6 ? 1.15e11 : 1.25e10;
+    const double row_cost = full / (TILE_I * TILE_J) * 4e-13;
+    const int64_t least = std::max<int64_t>(SPARSE_SMALL_ENTRIES + 1,
+                                            std::min<int64_t>(1024, (int64_t)std::sqrt(2.0 * rate * row_cost)));
+    const auto &cp = J.tabs[0].table->col_ptr;
+    std::vector<int32_t> listed;
+    int64_t entries = 0;
+    for (const auto &c : sp.sparse) {
+      sp_off.push_back((int64_t)all->size());
+      tile_off.push_back((int64_t)listed.size());
+      for (int32_t v : c) {
+        const int64_t ub = cp[tree->tip_hi[v]] - cp[tree->tip_lo[v]];
+        if (ub >= least) {
+          listed.push_back(v);
+          entries += ub;
+        } else {
+          all->push_back(v);
+        }
+      }
+      cls_n.push_back((int64_t)all->size() - sp_off.back());
+      tile_n.push_back((int64_t)listed.size() - tile_off.back());
+    }
+    n_tile_rows = (int64_t)listed.size();
+    const int64_t stride = round_up(std::max<int64_t>(n_tile_rows, 1), 32), blocks = (lay[0].n + TILE_I - 1) / TILE_I + 1;
+    const double need = (double)entries * sizeof(TileEnt) + (double)stride * blocks * 2.0;
+    if (entries >= (int64_t)UINT32_MAX || (need > 64e6 && need > 0.25 * available_bytes())) {
+      sp_off.clear();
+      cls_n.clear();
+      all->clear();
+      return false;
+    }
+    for (int64_t &o : tile_off) o += (int64_t)all->size();
+    all->insert(all->end(), listed.begin(), listed.end());
+    le = DevBuf((size_t)std::max<int64_t>(entries, 1) * sizeof(TileEnt), st, "alloc sparse lists");
+    toff = DevBuf((size_t)(stride * blocks) * 2, st, "alloc list offsets");
+    // per row its place and length, then the running total of entries
+    lz = DevBuf((size_t)(2 * stride + 1) * 4, st, "alloc sparse lists");
+    ck(cudaMemsetAsync(lz.p, 0, (size_t)(2 * stride + 1) * 4, st), "memset");
+    n_win = (int)win.size();
+    o_win = meta.add(win);
+    return true;
+  }
+
+  // acc: ACC_MIN / ACC_GEN; fp64_entries: terms computed in FP64; want_tiles:
+  // the tile scatter where it fits
   void prepare(uf_tree *tree, const BatchJob &J, const Inputs &in, const RowSplit &sp,
                const std::vector<SpLayout> &layout, int acc, bool fp64_entries, bool two_words,
-               int64_t call_cells, int64_t call_cols, Meta &meta, cudaStream_t st) {
+               int64_t call_cells, int64_t call_cols, bool want_tiles, Meta &meta, cudaStream_t st) {
     split = &sp;
     lay = layout;
     two_word = two_words;
@@ -607,12 +670,14 @@ struct SparseScatter {
     const size_t nt = J.tabs.size();
     if (sp.n_sparse == 0) return;
     const int64_t n_regions = (int64_t)sparse_regions(nt, acc, (double)cells * 8.0 * n_acc * (two_word ? 2 : 1));
-    region_mode = n_regions > 1 || sp.lists;
+    std::vector<int32_t> all, members;
+    tiles = want_tiles && prepare_tiles(tree, J, sp, &all, meta, st);
+    region_mode = !tiles && (n_regions > 1 || sp.lists);
     // the generalized method's entries carry each row's proportion as well:
     // two members at most
     fuse_m = !region_mode ? 0 : acc == ACC_MIN ? (int)g_sparse_fuse.load() : (int)std::min<int64_t>(g_sparse_fuse.load(), 2);
-    std::vector<int32_t> all, members;
-    if (fuse_m > 0) {
+    if (tiles) {
+    } else if (fuse_m > 0) {
       // A sparse branch whose parent is a listed head rides in the parent's
       // list (its samples are among the parent's and its pairs among the
       // parent's pairs); with six members per head, so does a sparse child of
@@ -690,7 +755,7 @@ struct SparseScatter {
 
   // base: kind, masks, M / M2, alpha and scale filled by the caller
   void launch(const Meta &meta, const Inputs &in, SparseArgs base, int acc, bool fp64_entries, int64_t region_bytes,
-              cudaStream_t on, int64_t *kernels) const {
+              int sms, cudaStream_t on, int64_t *kernels) const {
     if (!split || split->n_sparse == 0) return;
     const bool f32 = !fp64_entries;
     base.tip_lo = in.td->tip_lo;
@@ -720,6 +785,46 @@ struct SparseScatter {
       sp.cap = split->cap[c];
       if (region_mode) ck(launch_sparse_lists(acc, f32, sp, on), "sparse lists");
       else ck(launch_sparse_rows(acc, f32, sp, on), "sparse rows");
+      (*kernels)++;
+    }
+    if (tiles && n_tile_rows > 0) {
+      const int64_t stride = round_up(n_tile_rows, 32);
+      SparseArgs sp = base;
+      sp.le = le.p;
+      sp.pos = lz.as<uint32_t>();
+      sp.lz = (int *)(sp.pos + stride);
+      sp.total = sp.pos + 2 * stride;
+      sp.off = toff.as<uint16_t>();
+      sp.off_stride = stride;
+      sp.n_blocks = (lay[0].n + TILE_I - 1) / TILE_I;
+      for (size_t c = 0; c < split->sparse.size(); c++) {
+        if (tile_n[c] == 0) continue;
+        sp.row_base = (int)(tile_off[c] - (n_sparse_rows - n_tile_rows));
+        sp.nodes = meta.at<int32_t>(o_sparse) + tile_off[c];
+        sp.n_nodes = (int)tile_n[c];
+        sp.cap = split->cap[c];
+        ck(launch_tile_lists(sp, on), "sparse lists");
+        (*kernels)++;
+      }
+      TileArgs ta{};
+      ta.ent = le.as<TileEnt>();
+      ta.pos = sp.pos;
+      ta.z = sp.lz;
+      ta.off = toff.as<uint16_t>();
+      ta.n_rows = (int)n_tile_rows;
+      ta.stride = stride;
+      ta.n = lay[0].n;
+      ta.s_lo = lay[0].s_lo;
+      ta.s_hi = lay[0].s_hi;
+      ta.M = base.M;
+      ta.win = meta.at<TileWin>(o_win);
+      ta.n_win = n_win;
+      ta.n_tiles = (int)n_tiles;
+      // three waves of two CTAs per SM
+      ta.parts = (int)std::max<int64_t>(1, std::min<int64_t>(stride / 32, (6 * sms + n_tiles - 1) / n_tiles));
+      ta.x_shift = base.x_shift;
+      ta.m_lo_off = base.m_lo_off;
+      ck(launch_tile_scatter(ta, on), "tile scatter");
       (*kernels)++;
     }
     if (!region_mode) return;
@@ -853,7 +958,7 @@ uf_status run_gram(uf_tree *tree, const BatchJob &J, int device, double scale) {
   // sparse rows: presence terms (x = l) in FP64, one word (FP64 calls: two),
   // min form, into stripe-layout cells Msp and the per-sample R
   SparseScatter sc;
-  sc.prepare(tree, J, in, split, lay, ACC_MIN, true, digits, cells, n_cols, meta, st);
+  sc.prepare(tree, J, in, split, lay, ACC_MIN, true, digits, cells, n_cols, false, meta, st);
   if (split.n_sparse > 0) {
     Msp = DevBuf((size_t)cells * 8 * acc_words, st, "alloc sparse stripes");
     ck(cudaMemsetAsync(Msp.p, 0, (size_t)cells * 8 * acc_words, st), "memset");
@@ -904,7 +1009,7 @@ uf_status run_gram(uf_tree *tree, const BatchJob &J, int device, double scale) {
     sp.M = Msp.as<unsigned long long>();
     sp.alpha = 1.0;
     sp.scale = scale;
-    sc.launch(meta, in, sp, ACC_MIN, true, g_region_bytes.load(), ss, &kernels);
+    sc.launch(meta, in, sp, ACC_MIN, true, g_region_bytes.load(), sms, ss, &kernels);
     timer.end();
   }
   for (size_t b = 0; b < in.P->b0.size(); b++) {
@@ -1168,7 +1273,7 @@ uf_status run_stripes(uf_tree *tree, const BatchJob &J, int device, uf_method me
   std::vector<SpLayout> lay(nt);
   for (size_t t = 0; t < nt; t++) lay[t] = SpLayout{tabs[t].n, tabs[t].off, tabs[t].s_lo, tabs[t].s_hi, tabs[t].m_off};
   SparseScatter sc;
-  sc.prepare(tree, J, in, split, lay, acc, !fp32, !fp32, cells, n_cols, meta, st);
+  sc.prepare(tree, J, in, split, lay, acc, !fp32, !fp32, cells, n_cols, tile_scatter(J, acc, fp32), meta, st);
   meta.upload(st);
   const TabDesc *d_tabs = meta.at<TabDesc>(o_tabs);
   const int32_t *d_cnt = meta.at<int32_t>(o_cnt);
@@ -1238,13 +1343,13 @@ uf_status run_stripes(uf_tree *tree, const BatchJob &J, int device, uf_method me
   // a chunk is the rows a unit sums before it rounds; small problems cut it
   // so that every SM has units (tuned chunks are found with enough of them)
   int unit_rows = small.split && !tune ? small_plan(false).chunk : chunk;
+  double acc_most = 0.0;  // bound of the accumulators
   int x_shift = 0;  // grid of the FP64 min kernel's rows (StripeArgs::x_shift)
   if (fixed_rows) {
-    double bound = 0.0;
-    for (const TableJob &t : J.tabs) bound = std::max(bound, accum_bound(tree, t.table, kind));
+    for (const TableJob &t : J.tabs) acc_most = std::max(acc_most, accum_bound(tree, t.table, kind));
     x_shift = 32;
     for (size_t b = 0; b + 1 < split.dense_ptr.size(); b++)
-      x_shift = std::min(x_shift, fixed_row_shift(scale, bound, split.dense_len.data() + split.dense_ptr[b],
+      x_shift = std::min(x_shift, fixed_row_shift(scale, acc_most, split.dense_len.data() + split.dense_ptr[b],
                                                   split.dense_ptr[b + 1] - split.dense_ptr[b], unit_rows));
   }
   // the launch sequence goes into a CUDA graph unless it is timed per phase
@@ -1261,7 +1366,11 @@ uf_status run_stripes(uf_tree *tree, const BatchJob &J, int device, uf_method me
     sp.M2 = M2.as<unsigned long long>();
     sp.alpha = J.alpha;
     sp.scale = scale;
-    sc.launch(meta, in, sp, acc, !fp32, g_region_bytes.load(), on, &kernels);
+    if (fixed_rows) {  // listed rows on a 64-bit grid like the dense rows'
+      sp.x_shift = fixed_row_shift(scale, acc_most, &acc_most, 1, 1);
+      sp.row_scale = std::ldexp(scale, sp.x_shift);
+    }
+    sc.launch(meta, in, sp, acc, !fp32, g_region_bytes.load(), sms, on, &kernels);
   };
   // with option "sparse_overlap" (default) the sparse-row scatter runs on a
   // side branch beside the count pass, the embeddings and the dense stripe

@@ -314,6 +314,12 @@ extern std::atomic<int64_t> g_region_bytes;
 // split and region path: ACC_MIN or ACC_GEN (CUDA-core stripe kernels) or SPLIT_GRAM (tensor cores)
 constexpr int SPLIT_GRAM = 2;
 double sparse_regions(size_t n_tables, int acc, double acc_bytes);
+// Whether a call's scatter runs in shared-memory tiles (uf_sparse.cu): FP64
+// weighted methods (rows on the dense kernel's 64-bit grid) on one table of
+// TILE_MIN_SAMPLES (fewer make too few tiles) to TILE_MAX_SAMPLES (more leave
+// few of a row's samples in a tile) samples
+constexpr int64_t TILE_MIN_SAMPLES = 512, TILE_MAX_SAMPLES = 4096;
+bool tile_scatter(const BatchJob &J, int acc, bool fp32);
 
 
 // The split of a call, cached on the tree (uf_split.cpp).

@@ -36,8 +36,10 @@
 // z (z - 1) / 2 pairs; each thread takes a contiguous range of the pair
 // numbering and adds each pair to its stripe cell with one atomic per
 // accumulator (two when the pair is the duplicated half stripe of an even n).
+#include <algorithm>
 #include <cmath>
 #include <type_traits>
+#include <vector>
 
 #include "uf_device.cuh"
 #include "uf_sparse.h"
@@ -619,6 +621,245 @@ __global__ void __launch_bounds__(256) k_sparse_lists(const SparseArgs a) {
   if (tid == 0) a.lz[row] = z;
 }
 
+// ---- tile scatter (FP64 weighted) ----
+// A row's list for the tile scatter: as k_sparse_lists, but each entry is the
+// sample and its value on a 64-bit grid (as the dense kernel's rows), the row
+// takes its place in the entry array from a running total (its length is known
+// only here), and it writes where each block of samples starts in it.
+__global__ void __launch_bounds__(256) k_tile_lists(const SparseArgs a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int sh[33];
+  __shared__ uint32_t s_pos;
+  unsigned long long *key = reinterpret_cast<unsigned long long *>(smem_raw);  // (sample << 32) | entry
+  const int v = a.nodes[blockIdx.x], row = a.row_base + blockIdx.x;
+  const SpTab tb = a.tabs[0];
+  const int64_t q0 = tb.col_ptr[a.tip_lo[v]];
+  const int L = (int)(tb.col_ptr[a.tip_hi[v]] - q0);
+  if (L <= 0 || L > a.cap) return;  // the host sizes cap to every run and z starts at 0
+  const int tid = threadIdx.x, NT = blockDim.x;
+  int P2 = 1;
+  while (P2 < L) P2 <<= 1;
+  for (int i = tid; i < P2; i += NT)
+    key[i] = i < L ? ((unsigned long long)(unsigned)tb.col_row[q0 + i] << 32) | (unsigned)i : ~0ull;
+  __syncthreads();
+  int unsorted = 0;
+  for (int i = tid + 1; i < L; i += NT) unsorted |= (key[i] >> 32) <= (key[i - 1] >> 32);
+  if (__syncthreads_or(unsorted)) {
+    for (int k = 2; k <= P2; k <<= 1)
+      for (int j = k >> 1; j > 0; j >>= 1) {
+        for (int i = tid; i < P2; i += NT) {
+          const int ixj = i ^ j;
+          if (ixj > i) {
+            const unsigned long long x = key[i], y = key[ixj];
+            if ((x > y) == ((i & k) == 0)) {
+              key[i] = y;
+              key[ixj] = x;
+            }
+          }
+        }
+        __syncthreads();
+      }
+  }
+  const int EPT = (L + NT - 1) / NT, i0 = tid * EPT, i1 = min(L, i0 + EPT);
+  int heads = 0;
+  for (int i = i0; i < i1; i++) heads += (i == 0 || (key[i] >> 32) != (key[i - 1] >> 32));
+  int z = 0;
+  int u = block_exclusive_scan(heads, sh, &z);
+  if (tid == 0) {
+    s_pos = atomicAdd(a.total, (uint32_t)z);
+    a.pos[row] = s_pos;
+    a.lz[row] = z;
+  }
+  __syncthreads();
+  TileEnt *le = reinterpret_cast<TileEnt *>(a.le) + s_pos;
+  const double l = a.length[v];
+  for (int i = i0; i < i1; i++) {
+    const unsigned smp = (unsigned)(key[i] >> 32);
+    const int prev = i > 0 ? (int)(key[i - 1] >> 32) : -1;
+    // offsets of the blocks that start after the last key
+    if (i == L - 1)
+      for (int b = (int)smp / TILE_I + 1; b <= a.n_blocks; b++) a.off[b * a.off_stride + row] = (uint16_t)z;
+    if (prev == (int)smp) continue;
+    // and of those that start after the sample before and up to this one
+    for (int b = prev < 0 ? 0 : prev / TILE_I + 1; b <= (int)smp / TILE_I; b++) a.off[b * a.off_stride + row] = (uint16_t)u;
+    double c = 0.0;  // in entry order
+    for (int m = i; m < L && (unsigned)(key[m] >> 32) == smp; m++) c += tb.col_val[q0 + (key[m] & 0xffffffffu)];
+    const double x = emb_value<double, EMB_SCALED>(c, l, tb.total[smp], 0.f);
+    TileEnt en;
+    en.k = (int)smp;
+    en.pad = 0;
+    en.x = __double2ull_rn(x * a.row_scale);
+    const unsigned long long mask = (1ull << a.x_shift) - 1ull;
+    atomicAdd(a.Dsp + tb.off + smp, en.x >> a.x_shift);
+    atomicAdd(a.Dsp + tb.off + smp + a.d_lo_off, (en.x & mask) << (32 - a.x_shift));
+    le[u] = en;
+    u++;
+  }
+}
+
+// One CTA per tile (and part of the rows).  A thread reads a row's four offsets
+// (coalesced; many rows have no pair in a tile) and the warp queues the rows
+// that do; it then takes them one by one and adds the smaller value of each pair
+// of a row's samples to the tile's cell: a 64-bit sum in two 32-bit words, the
+// carry from the first word's old value (two native 32-bit atomics, 1.6e12 adds
+// per second on random cells; a 64-bit one in shared memory is a
+// compare-and-swap loop, 2.6 times slower).  The cells go to the two-word
+// accumulators once per tile.  Without tiles every pair was two 64-bit atomics
+// into L2, 1.5e11 pairs/s on 1,531 samples; here 4.2e11.  One-word FP32 terms are
+// one L2 atomic a pair, 2.3e11/s, and no faster in tiles (3.2e11/s less the
+// lists), and with 25,000 samples (8 pairs per row and tile) tiles are slower
+// than regions: tile_scatter() says which calls come here.
+constexpr int TS_THREADS = 512, TS_WARPS = TS_THREADS / 32, TS_QUEUE = 64;
+constexpr size_t TS_SMEM = (size_t)TILE_I * TILE_J * 8 + (size_t)TS_WARPS * TS_QUEUE * sizeof(uint4);
+
+__global__ void __launch_bounds__(TS_THREADS, 2) k_tile_scatter(const TileArgs a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int s_next;
+  uint32_t *lo = reinterpret_cast<uint32_t *>(smem_raw), *hi = lo + TILE_I * TILE_J;
+  uint4 *queue = reinterpret_cast<uint4 *>(hi + TILE_I * TILE_J) + (threadIdx.x >> 5) * TS_QUEUE;
+  const int lane = threadIdx.x & 31;
+  for (int i = threadIdx.x; i < 2 * TILE_I * TILE_J; i += TS_THREADS) lo[i] = 0u;
+  if (threadIdx.x == 0) s_next = 0;
+  // the tile's window and block of samples i
+  int w = 0;
+  {
+    int top = a.n_win - 1;
+    while (w < top) {
+      const int mid = (w + top + 1) >> 1;
+      if (a.win[mid].tile0 <= (int)blockIdx.x) w = mid;
+      else top = mid - 1;
+    }
+  }
+  const TileWin win = a.win[w];
+  const int q = blockIdx.x - win.tile0;
+  const int ib = q < win.a_n ? win.a_lo + q : win.b_lo + (q - win.a_n);
+  const int i0 = ib * TILE_I, j0 = w * TILE_J, j1 = min(a.n, j0 + TILE_J);
+  // the part of the window that pairs of the stripes reach, when only one of
+  // the two distance ranges [s_lo + 1, s_hi + 1], [n - s_hi - 1, n - s_lo - 1] does
+  int ja = j0, jb = j1 - 1;
+  {
+    const int a0 = i0 + a.s_lo + 1, a1 = i0 + TILE_I - 1 + a.s_hi + 1;
+    const int b0 = i0 + a.n - a.s_hi - 1, b1 = i0 + TILE_I - 1 + a.n - a.s_lo - 1;
+    const bool in_a = a0 <= jb && a1 >= ja, in_b = b0 <= jb && b1 >= ja;
+    if (in_a != in_b) {
+      ja = max(ja, in_a ? a0 : b0);
+      jb = min(jb, in_a ? a1 : b1);
+    }
+  }
+  const uint16_t *oi = a.off + (int64_t)ib * a.stride;
+  const uint16_t *oj0 = a.off + (int64_t)(ja / TILE_I) * a.stride, *oj1 = a.off + (int64_t)(jb / TILE_I + 1) * a.stride;
+  __syncthreads();
+
+  // The first m queued rows, one after the other: a lane holds one of the row's
+  // samples i and two of its samples j (64 at a time), and the warp passes the
+  // samples i around; the next row's entries are on their way meanwhile.
+  struct Visit {
+    const TileEnt *j;
+    int ni, nj;
+    TileEnt own, e0, e1;
+  };
+  const int off_c = -i0 * TILE_J - j0;
+  const TileEnt none{0, -1, 0};
+  auto fetch = [&](int v, int m) {
+    Visit x;
+    const uint4 e = v < m ? queue[v] : make_uint4(0, 0, 0, 0);  // first entry i, entries i, first entry j, entries j
+    x.j = a.ent + e.z;
+    x.ni = (int)e.y;
+    x.nj = (int)e.w;
+    x.own = lane < x.ni ? a.ent[e.x + lane] : none;
+    x.e0 = lane < x.nj ? x.j[lane] : none;
+    x.e1 = lane + 32 < x.nj ? x.j[lane + 32] : none;
+    return x;
+  };
+  auto add = [&](unsigned long long xi, int ki, int ci, const TileEnt &ej) {
+    if (ki >= ej.k) return;  // (no entry: k = -1)
+    const unsigned long long x = xi < ej.x ? xi : ej.x;
+    const uint32_t x0 = (uint32_t)x, old = atomicAdd(lo + ci + ej.k, x0);
+    const uint32_t x1 = (uint32_t)(x >> 32) + (old + x0 < x0 ? 1u : 0u);
+    if (x1) atomicAdd(hi + ci + ej.k, x1);
+  };
+  auto process = [&](int m) {
+    Visit cur = fetch(0, m);
+    for (int v = 0; v < m; v++) {
+      const Visit next = fetch(v + 1, m);
+      for (int jc = lane;;) {
+        for (int ia = 0; ia < cur.ni; ia++) {
+          const unsigned long long xi = __shfl_sync(0xffffffffu, cur.own.x, ia);
+          const int ki = __shfl_sync(0xffffffffu, cur.own.k, ia), ci = ki * TILE_J + off_c;
+          add(xi, ki, ci, cur.e0);
+          add(xi, ki, ci, cur.e1);
+        }
+        jc += 64;
+        if (jc - lane >= cur.nj) break;
+        cur.e0 = jc < cur.nj ? cur.j[jc] : none;
+        cur.e1 = jc + 32 < cur.nj ? cur.j[jc + 32] : none;
+      }
+      cur = next;
+    }
+  };
+  int queued = 0;
+  const int groups = (int)(a.stride / 32);
+  for (;;) {
+    int g = 0;
+    if (lane == 0) g = atomicAdd(&s_next, 1);
+    g = __shfl_sync(0xffffffffu, g, 0) * a.parts + (int)blockIdx.y;
+    if (g >= groups) break;
+    const int r = g * 32 + lane;
+    uint32_t fi = 0, ni = 0, fj = 0, nj = 0;
+    if (r < a.n_rows) {
+      fi = oi[r];
+      ni = oi[r + a.stride] - fi;
+      fj = oj0[r];
+      nj = oj1[r] - fj;
+    }
+    const bool has = ni != 0 && nj != 0;
+    const unsigned who = __ballot_sync(0xffffffffu, has);
+    if (has) {
+      const uint32_t p = a.pos[r];
+      queue[queued + __popc(who & ((1u << lane) - 1u))] = make_uint4(p + fi, ni, p + fj, nj);
+    }
+    queued += __popc(who);
+    __syncwarp();
+    if (queued >= 32) {
+      process(32);
+      __syncwarp();
+      // the rest (fewer than 32) moves to the front
+      const uint4 e = lane < queued - 32 ? queue[32 + lane] : make_uint4(0, 0, 0, 0);
+      __syncwarp();
+      if (lane < queued - 32) queue[lane] = e;
+      queued -= 32;
+      __syncwarp();
+    }
+  }
+  process(queued);
+  __syncthreads();
+
+  // cells to stripes: a warp takes a diagonal, whose 32 cells are neighbours of
+  // one stripe
+  const unsigned long long mask = (1ull << a.x_shift) - 1ull;
+  for (int t = threadIdx.x >> 5; t < TILE_I + TILE_J - 1; t += TS_WARPS) {
+    const int d = j0 - i0 + t - (TILE_I - 1);  // k_j - k_i of the diagonal
+    if (d <= 0) continue;
+    const bool near = 2 * (int64_t)d <= a.n;
+    const int s = near ? d - 1 : a.n - d - 1;
+    if (s < a.s_lo || s > a.s_hi) continue;
+    const int jr = t - (TILE_I - 1) + lane;
+    if (jr < 0 || jr >= TILE_J || j0 + jr >= a.n) continue;
+    const int c = lane * TILE_J + jr;
+    const unsigned long long x = ((unsigned long long)hi[c] << 32) | lo[c];
+    if (x == 0) continue;
+    unsigned long long *cell = a.M + (int64_t)(s - a.s_lo) * a.n + (near ? i0 + lane : j0 + jr);
+    // -2 min, as every abs-form cell
+    const unsigned long long v = 0ull - ((x >> a.x_shift) << 1), u = 0ull - ((x & mask) << (33 - a.x_shift));
+    atomicAdd(cell, v);
+    atomicAdd(cell + a.m_lo_off, u);
+    if (2 * (int64_t)d == a.n) {
+      atomicAdd(cell + d, v);
+      atomicAdd(cell + d + a.m_lo_off, u);
+    }
+  }
+}
+
 // first index in [lo, hi) of the ascending samples K with K[i] >= key
 __device__ __forceinline__ int lower_index(const int *K, int lo, int hi, int key) {
   while (lo < hi) {
@@ -839,6 +1080,55 @@ cudaError_t launch_sparse_lists(int acc, bool fp32, const SparseArgs &a, cudaStr
   if (acc == ACC_MIN) return fp32 ? go(k_sparse_lists<float, ACC_MIN, 0>) : go(k_sparse_lists<double, ACC_MIN, 0>);
   if (fp32) return mode == 0 ? go(k_sparse_lists<float, ACC_GEN, 0>) : go(k_sparse_lists<float, ACC_GEN, 1>);
   return mode == 0 ? go(k_sparse_lists<double, ACC_GEN, 0>) : go(k_sparse_lists<double, ACC_GEN, 1>);
+}
+
+int64_t tile_windows(int n, int s_lo, int s_hi, std::vector<TileWin> *win) {
+  auto fdiv = [](int64_t a, int64_t b) { return a >= 0 ? a / b : -((-a + b - 1) / b); };
+  const int64_t s0 = s_lo, s1 = (int64_t)s_hi + 1;  // distances [s0 + 1, s1] and [n - s1, n - s0 - 1]
+  int64_t tiles = 0;
+  for (int64_t j0 = 0; j0 < n; j0 += TILE_J) {
+    const int64_t j1 = std::min<int64_t>(n, j0 + TILE_J);
+    // blocks b with i0 = b TILE_I whose distances j - i, [max(1, j0 - i0 - 31), j1 - 1 - i0], meet [lo, hi]
+    auto range = [&](int64_t lo, int64_t hi, int *first, int *count) {
+      const int64_t b0 = std::max<int64_t>(0, fdiv(j0 - (TILE_I - 1) - hi + TILE_I - 1, TILE_I));
+      const int64_t b1 = fdiv(j1 - 1 - lo, TILE_I);
+      *first = (int)b0;
+      *count = (int)std::max<int64_t>(0, b1 - b0 + 1);
+    };
+    TileWin w{};
+    w.tile0 = (int)tiles;
+    range(s0 + 1, s1, &w.a_lo, &w.a_n);
+    range(n - s1, n - s0 - 1, &w.b_lo, &w.b_n);
+    // the second range's blocks come before the first's; both where they meet
+    if (w.a_n > 0 && w.b_n > 0 && w.b_lo + w.b_n > w.a_lo) {
+      const int end = std::max(w.a_lo + w.a_n, w.b_lo + w.b_n);
+      w.a_lo = std::min(w.a_lo, w.b_lo);
+      w.a_n = end - w.a_lo;
+      w.b_n = 0;
+    }
+    tiles += w.a_n + w.b_n;
+    win->push_back(w);
+  }
+  return tiles;
+}
+
+cudaError_t launch_tile_scatter(const TileArgs &a, cudaStream_t st) {
+  if (a.n_rows <= 0 || a.n_tiles <= 0) return cudaSuccess;
+  const cudaError_t e = cudaFuncSetAttribute(k_tile_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TS_SMEM);
+  if (e != cudaSuccess) return e;
+  k_tile_scatter<<<dim3((unsigned)a.n_tiles, (unsigned)a.parts), TS_THREADS, TS_SMEM, st>>>(a);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_tile_lists(const SparseArgs &a, cudaStream_t st) {
+  if (a.n_nodes <= 0) return cudaSuccess;
+  if (a.cap < SPARSE_SMALL_ENTRIES || (a.cap & (a.cap - 1)) || a.cap > SPARSE_LIST_MAX_ENTRIES || a.n_tabs != 1)
+    return cudaErrorInvalidValue;
+  const size_t smem = sparse_list_smem_bytes(a.cap);
+  const cudaError_t e = cudaFuncSetAttribute(k_tile_lists, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  k_tile_lists<<<(unsigned)a.n_nodes, a.cap <= 512 ? 128 : 256, smem, st>>>(a);
+  return cudaGetLastError();
 }
 
 }  // namespace ufg

@@ -61,10 +61,55 @@ struct SparseArgs {
   unsigned long long *pair_count;  // non-null: the pair updates made are added to these
                                    // SPARSE_PAIR_SLOTS counters (summed by the host)
   int first_region;         // 1: the call's first region (cursors are searched, not read)
+  // tile lists (launch_tile_lists): le holds TileEnt; row r's entries with a
+  // sample below b TILE_I at off[b * off_stride + r], b <= n_blocks
+  uint32_t *pos, *total;
+  uint16_t *off;
+  int64_t off_stride;
+  int n_blocks;
+  double row_scale;         // the values are x * row_scale, 2^x_shift finer than scale
+  int x_shift;
   uint16_t *cur;            // two cursors per list entry (indices into its row's list, which
                             // holds at most SPARSE_LIST_MAX_ENTRIES): window 1 at cur[e],
   int64_t cur_stride;       // window 2 at cur[cur_stride + e] (regions in increasing order)
 };
+// ---- tile scatter (FP64 weighted, one table) ----
+// The pairs of the listed rows are added in shared memory, tile by tile of
+// TILE_I x TILE_J samples, and each tile's cells go to the accumulators once.
+constexpr int TILE_I = 32;   // samples i of a tile, and the grid of the rows' offsets
+constexpr int TILE_J = 384;  // samples j
+// one distinct sample of a row and its value on the 64-bit grid
+struct alignas(16) TileEnt {
+  unsigned long long x;
+  int k, pad;
+};
+// tiles of the window of samples j in [j0, j0 + TILE_J): those of the blocks of
+// TILE_I samples i that hold a pair of the call's stripes, a_n from block a_lo
+// on and b_n from b_lo on, numbered from tile0
+struct TileWin {
+  int tile0, a_lo, a_n, b_lo, b_n, pad;
+};
+struct TileArgs {
+  const TileEnt *ent;       // the rows' entries in ascending sample, row r's from pos[r] on, z[r] of them
+  const uint32_t *pos;
+  const int *z;
+  const uint16_t *off;      // off[b * stride + r]: entries of row r with a sample below b TILE_I
+  int n_rows;
+  int64_t stride;           // n_rows rounded up to 32
+  int n, s_lo, s_hi;        // samples, stored stripes
+  unsigned long long *M;
+  const TileWin *win;
+  int n_win, n_tiles, parts;  // windows, their tiles, CTAs per tile (each takes every parts-th group of rows)
+  // values in units of 2^-(F + x_shift); the cells' second words m_lo_off on
+  int x_shift;
+  int64_t m_lo_off;
+};
+// windows of an n-sample table's stripes [s_lo, s_hi]; returns the tiles
+int64_t tile_windows(int n, int s_lo, int s_hi, std::vector<TileWin> *win);
+cudaError_t launch_tile_scatter(const TileArgs &a, cudaStream_t st);
+// List mode of the tile scatter: rows nodes[0 .. n_nodes) write their entries
+// where *total places them (pos and z at row_base + row), and their terms to Dsp
+cudaError_t launch_tile_lists(const SparseArgs &a, cudaStream_t st);
 // largest subtree entry count a sparse row may have: scattered directly from
 // shared memory, or written as a list (one table, keys alone in shared memory)
 constexpr int SPARSE_SMALL_ENTRIES = 32;  // scattered by a warp

@@ -13,6 +13,12 @@ double sparse_regions(size_t n_tables, int acc, double acc_bytes) {
   return std::ceil(acc_bytes / budget);
 }
 
+bool tile_scatter(const BatchJob &J, int acc, bool fp32) {
+  if (J.tabs.size() != 1 || fp32 || acc != ACC_MIN || kind_of(J.method) != EMB_SCALED) return false;
+  const int64_t n = J.tabs[0].table->n;
+  return n >= TILE_MIN_SAMPLES && n <= TILE_MAX_SAMPLES;
+}
+
 namespace {
 
 // Per branch v the count entries of table t under v are the CSC run of v's
@@ -47,10 +53,11 @@ RowSplit split_rows(const uf_tree *tree, const BatchJob &J, const Plan *P, int a
     }
     // accumulators beyond L2: one table scatters region by region in L2
     // (sparse_regions), several tables scatter straight into HBM-resident cells
-    const bool regions = sparse_regions(nt, acc, cells * 8.0 * n_acc) > 1;
-    R.lists = regions;
+    const bool tiles = tile_scatter(J, acc, fp32);
+    const bool regions = !tiles && sparse_regions(nt, acc, cells * 8.0 * n_acc) > 1;
+    R.lists = regions || tiles;
     // list mode keeps only sort keys in shared memory: longer runs fit
-    const int64_t max_entries = regions ? SPARSE_LIST_MAX_ENTRIES : SPARSE_MAX_ENTRIES;
+    const int64_t max_entries = R.lists ? SPARSE_LIST_MAX_ENTRIES : SPARSE_MAX_ENTRIES;
     // the scatter runs table by table (its grid's y is the table), so each
     // table's atomics hit L2 when that table's accumulators fit there
     std::vector<double> pair_cost(nt), entry_cost(nt);
@@ -74,7 +81,13 @@ RowSplit split_rows(const uf_tree *tree, const BatchJob &J, const Plan *P, int a
       const double atom_rate = std::floor(n / 2.0) * n * 8.0 * n_acc <= 64e6 || regions ? 2.3e11 : 2.5e10;
       pair_cost[t] = (1.0 / visit_rate + n_acc / atom_rate) * fuse;
       entry_cost[t] = 4.0 / atom_rate;
+      if (tiles) {
+        pair_cost[t] = 2.4e-12;
+        entry_cost[t] = 3e-11;
+      }
     }
+    // a row's offsets read by every tile
+    const double tile_cost = tiles ? cells / (TILE_I * TILE_J) * 4e-13 : 0.0;
     // a dense row also costs its count row and embedding (or planes) in HBM
     const double dense_t = cells / dense_rate + cols * 36.0 / 6e12;
     // node ranges in parallel; each class list is the ranges' lists in order,
@@ -109,7 +122,7 @@ RowSplit split_rows(const uf_tree *tree, const BatchJob &J, const Plan *P, int a
           if (ub == 0) continue;
           const double pr = (double)ub * (double)(ub - 1) / 2.0;
           pairs += pr;
-          cost += job_cost + pr * pair_cost[t] + (double)ub * entry_cost[t];
+          cost += job_cost + pr * pair_cost[t] + (double)ub * entry_cost[t] + tile_cost;
           // one visit per region: a CTA, and each entry's cursors walked to the
           // region (about 7e-12 s per entry and region measured on GB300 with a
           // 113,000-sample table; pairs at 4.3e-12 s)
@@ -213,7 +226,7 @@ RowSplit split_rows(const uf_tree *tree, const BatchJob &J, const Plan *P, int a
 std::shared_ptr<const RowSplit> get_split(uf_tree *tree, const BatchJob &J, const Plan *P, int acc, bool fp32) {
   SplitKey key;
   for (const TableJob &t : J.tabs) std::get<0>(key).push_back(t.table->id);
-  std::get<1>(key) = acc;
+  std::get<1>(key) = acc + (tile_scatter(J, acc, fp32) ? 16 : 0);
   std::get<2>(key) = fp32 ? 1 : 0;
   std::get<3>(key) = (int)(g_sparse.load() * 16 + g_sparse_fuse.load());
   std::get<4>(key) = P->block_rows;
