@@ -726,7 +726,9 @@ struct SparseScatter {
       list_entries = (int64_t)total_e;
       le = DevBuf(total_e * sparse_entry_bytes(!fp64_entries, fuse_m, acc), st, "alloc sparse lists");
       lk = DevBuf(total_e * 4, st, "alloc sparse lists");
-      cur = DevBuf(total_e * 2 * sizeof(uint16_t), st, "alloc sparse list cursors");
+      // (cursors from one region to the next)
+      if (region_stripes(g_region_bytes.load()) <= (int64_t)lay[0].s_hi - lay[0].s_lo)
+        cur = DevBuf(total_e * 2 * sizeof(uint16_t), st, "alloc sparse list cursors");
       lz = DevBuf(std::max<size_t>(all.size(), 1) * 4, st, "alloc sparse lists");
       // rows without entries in the table return before writing their count
       ck(cudaMemsetAsync(lz.p, 0, std::max<size_t>(all.size(), 1) * 4, st), "memset");
@@ -751,6 +753,11 @@ struct SparseScatter {
     const size_t dsp_words = (size_t)n_cols * (two_word ? 2 : 1);
     Dsp = DevBuf(dsp_words * 8, st, "alloc diagonal");
     ck(cudaMemsetAsync(Dsp.p, 0, dsp_words * 8, st), "memset");
+  }
+
+  // stripes whose accumulators fit one region
+  int64_t region_stripes(int64_t region_bytes) const {
+    return std::max<int64_t>(1, (int64_t)((double)region_bytes / (8.0 * n_acc * (two_word ? 2 : 1) * lay[0].n)));
   }
 
   // base: kind, masks, M / M2, alpha and scale filled by the caller
@@ -828,8 +835,7 @@ struct SparseScatter {
       (*kernels)++;
     }
     if (!region_mode) return;
-    const int64_t per =
-        std::max<int64_t>(1, (int64_t)((double)region_bytes / (8.0 * n_acc * (two_word ? 2 : 1) * lay[0].n)));
+    const int64_t per = region_stripes(region_bytes);
     for (int64_t r0 = lay[0].s_lo; r0 <= lay[0].s_hi; r0 += per) {
       SparseArgs sp = base;
       sp.nodes = meta.at<int32_t>(o_sparse);

@@ -913,7 +913,8 @@ __global__ void __launch_bounds__(128) k_sparse_region(const SparseArgs a) {
   // call searches for it.
   // 16-bit cursors: the region kernels stream every entry's state once per
   // region, so its bytes count (a list holds at most SPARSE_LIST_MAX_ENTRIES)
-  uint16_t *cur1 = a.cur + off, *cur2 = a.cur + a.cur_stride + off;
+  // (null: the call has one region)
+  uint16_t *cur1 = a.cur ? a.cur + off : nullptr, *cur2 = a.cur ? a.cur + a.cur_stride + off : nullptr;
   [[maybe_unused]] unsigned n_upd = 0;  // pair updates made by this thread: the cursors' moves
   auto add = [&](const Ent &ea, int ka, int b, int kb) {
     if constexpr (FUSED && ACC == ACC_MIN) add_pair_fused<T, F>(ka, kb, ea, E[b], c);
@@ -932,7 +933,7 @@ __global__ void __launch_bounds__(128) k_sparse_region(const SparseArgs a) {
       [[maybe_unused]] const int b0 = b;
       if (dlo <= dhi)
         for (int kb; b < z && (kb = K[b]) <= ka + dhi; b++) add(ea, ka, b, kb);
-      cur1[ia] = (uint16_t)b;
+      if (cur1) cur1[ia] = (uint16_t)b;
       if constexpr (COUNT) n_upd += (unsigned)(b - b0);
     }
     // window 2: d in [max(n - r1, n/2 + 1), n - r0 - 1], stripe n - d - 1, column k_b;
@@ -943,7 +944,7 @@ __global__ void __launch_bounds__(128) k_sparse_region(const SparseArgs a) {
       [[maybe_unused]] const int e0 = e;
       if (dlo <= dhi)
         for (int kb; e > ia + 1 && (kb = K[e - 1]) >= ka + dlo; e--) add(ea, ka, e - 1, kb);
-      cur2[ia] = (uint16_t)e;
+      if (cur2) cur2[ia] = (uint16_t)e;
       if constexpr (COUNT) n_upd += (unsigned)(e0 - e);
     }
   }

@@ -71,7 +71,7 @@ struct SparseArgs {
   int x_shift;
   uint16_t *cur;            // two cursors per list entry (indices into its row's list, which
                             // holds at most SPARSE_LIST_MAX_ENTRIES): window 1 at cur[e],
-  int64_t cur_stride;       // window 2 at cur[cur_stride + e] (regions in increasing order)
+  int64_t cur_stride;       // (null when the call has one region) window 2 at cur[cur_stride + e] (regions in increasing order)
 };
 // ---- tile scatter (FP64 weighted, one table) ----
 // The pairs of the listed rows are added in shared memory, tile by tile of

@@ -55,7 +55,12 @@ RowSplit split_rows(const uf_tree *tree, const BatchJob &J, const Plan *P, int a
     // (sparse_regions), several tables scatter straight into HBM-resident cells
     const bool tiles = tile_scatter(J, acc, fp32);
     const bool regions = !tiles && sparse_regions(nt, acc, cells * 8.0 * n_acc) > 1;
-    R.lists = regions || tiles;
+    // FP32 min-form terms of one table go through lists even when its
+    // accumulators fit in L2: a fused list's pair is one atomic for three
+    // branches, and the atomics bound the scatter (2,048 samples: 4.77 ms a call
+    // scattered directly, 4.50 through lists in two regions)
+    const bool listed = nt == 1 && acc == ACC_MIN && fp32 && J.tabs[0].table->n >= LIST_MIN_SAMPLES;
+    R.lists = regions || tiles || listed;
     // list mode keeps only sort keys in shared memory: longer runs fit
     const int64_t max_entries = R.lists ? SPARSE_LIST_MAX_ENTRIES : SPARSE_MAX_ENTRIES;
     // the scatter runs table by table (its grid's y is the table), so each
@@ -75,7 +80,7 @@ RowSplit split_rows(const uf_tree *tree, const BatchJob &J, const Plan *P, int a
     // scatter runs beside its gram and ends after it already: its split keeps
     // the unfused costs.
     const int64_t fm = acc == ACC_GEN ? std::min<int64_t>(g_sparse_fuse.load(), 2) : g_sparse_fuse.load();
-    const double fuse = regions && acc != SPLIT_GRAM && fm > 0 ? (fm == 6 ? 0.45 : 0.6) : 1.0;
+    const double fuse = (regions || listed) && acc != SPLIT_GRAM && fm > 0 ? (fm == 6 ? 0.45 : 0.6) : 1.0;
     for (size_t t = 0; t < nt; t++) {
       const double n = (double)J.tabs[t].table->n;
       const double atom_rate = std::floor(n / 2.0) * n * 8.0 * n_acc <= 64e6 || regions ? 2.3e11 : 2.5e10;
