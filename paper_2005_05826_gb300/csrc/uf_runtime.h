@@ -290,7 +290,7 @@ struct RowSplit {
   std::vector<double> dense_len;    // their branch lengths
   std::vector<std::vector<int32_t>> sparse;  // sparse branch nodes by capacity class
   std::vector<int> cap;             // shared-memory entries of each class
-  bool lists = false;               // sample lists: stripe regions, tiles, or FP32 min-form rows of one table
+  bool lists = false;               // sample lists: stripe regions, tiles, or FP32 rows of one table
   int64_t n_sparse = 0;
   double pairs = 0.0;               // both-nonzero pairs scattered, at most (sum over tables)
   int64_t max_dense = 0;            // most dense rows in one block
@@ -311,8 +311,7 @@ struct RowSplit {
 // that every region's cells stay in L2; otherwise one region.
 constexpr double SPARSE_REGION_BYTES_DEFAULT = 48e6;
 extern std::atomic<int64_t> g_region_bytes;
-// Fewest samples of a table whose FP32 min-form scatter goes through (fused)
-// lists when its accumulators fit in L2.
+// Fewest samples of a table whose FP32 scatter goes through (fused) lists when its accumulators fit in L2.
 constexpr int64_t LIST_MIN_SAMPLES = 512;
 // split and region path: ACC_MIN or ACC_GEN (CUDA-core stripe kernels) or SPLIT_GRAM (tensor cores)
 constexpr int SPLIT_GRAM = 2;

@@ -55,11 +55,12 @@ RowSplit split_rows(const uf_tree *tree, const BatchJob &J, const Plan *P, int a
     // (sparse_regions), several tables scatter straight into HBM-resident cells
     const bool tiles = tile_scatter(J, acc, fp32);
     const bool regions = !tiles && sparse_regions(nt, acc, cells * 8.0 * n_acc) > 1;
-    // FP32 min-form terms of one table go through lists even when its
-    // accumulators fit in L2: a fused list's pair is one atomic for three
-    // branches, and the atomics bound the scatter (2,048 samples: 4.77 ms a call
-    // scattered directly, 4.50 through lists in two regions)
-    const bool listed = nt == 1 && acc == ACC_MIN && fp32 && J.tabs[0].table->n >= LIST_MIN_SAMPLES;
+    // FP32 terms of one table go through lists even when its accumulators fit
+    // in L2: a fused list's pair is one atomic (generalized: two) for three
+    // branches, and the atomics bound the scatter (2,048 samples weighted 4.73 ->
+    // 4.35 ms a call, 1,003 generalized 3.13 -> 3.01)
+    const bool listed =
+        nt == 1 && (acc == ACC_MIN || acc == ACC_GEN) && fp32 && J.tabs[0].table->n >= LIST_MIN_SAMPLES;
     R.lists = regions || tiles || listed;
     // list mode keeps only sort keys in shared memory: longer runs fit
     const int64_t max_entries = R.lists ? SPARSE_LIST_MAX_ENTRIES : SPARSE_MAX_ENTRIES;
