@@ -584,6 +584,7 @@ struct SparseScatter {
   const RowSplit *split = nullptr;
   bool region_mode = false;
   int fuse_m = 0;         // members per min-form list row (launch_sparse_region); 0: unfused
+  bool pres = false;      // presence terms (one-byte entries in fused lists)
   bool two_word = false;  // FP64 terms in two words (second words after the first)
   int n_acc = 1;
   int64_t n_sparse_rows = 0, cells = 0, n_cols = 0;
@@ -657,10 +658,10 @@ struct SparseScatter {
   }
 
   // acc: ACC_MIN / ACC_GEN; fp64_entries: terms computed in FP64; want_tiles:
-  // the tile scatter where it fits
+  // the tile scatter where it fits; presence: the rows hold presence terms
   void prepare(uf_tree *tree, const BatchJob &J, const Inputs &in, const RowSplit &sp,
                const std::vector<SpLayout> &layout, int acc, bool fp64_entries, bool two_words,
-               int64_t call_cells, int64_t call_cols, bool want_tiles, Meta &meta, cudaStream_t st) {
+               int64_t call_cells, int64_t call_cols, bool want_tiles, bool presence, Meta &meta, cudaStream_t st) {
     split = &sp;
     lay = layout;
     two_word = two_words;
@@ -673,6 +674,7 @@ struct SparseScatter {
     std::vector<int32_t> all, members;
     tiles = want_tiles && prepare_tiles(tree, J, sp, &all, meta, st);
     region_mode = !tiles && (n_regions > 1 || sp.lists);
+    pres = presence;
     // the generalized method's entries carry each row's proportion as well:
     // two members at most
     fuse_m = !region_mode ? 0 : acc == ACC_MIN ? (int)g_sparse_fuse.load() : (int)std::min<int64_t>(g_sparse_fuse.load(), 2);
@@ -724,7 +726,7 @@ struct SparseScatter {
         lofs[r + 1] = lofs[r] + (cp[tree->tip_hi[all[r]]] - cp[tree->tip_lo[all[r]]]);
       const size_t total_e = (size_t)std::max<int64_t>(lofs.back(), 1);
       list_entries = (int64_t)total_e;
-      le = DevBuf(total_e * sparse_entry_bytes(!fp64_entries, fuse_m, acc), st, "alloc sparse lists");
+      le = DevBuf(total_e * sparse_entry_bytes(!fp64_entries, fuse_m, acc, pres), st, "alloc sparse lists");
       lk = DevBuf(total_e * 4, st, "alloc sparse lists");
       // (cursors from one region to the next)
       if (region_stripes(g_region_bytes.load()) <= (int64_t)lay[0].s_hi - lay[0].s_lo)
@@ -781,6 +783,7 @@ struct SparseScatter {
       base.cur = cur.as<uint16_t>();
       base.cur_stride = list_entries;
       base.fused = fuse_m;
+      base.pres = pres && fuse_m > 0 && acc == ACC_MIN;
       base.members = fuse_m > 0 ? meta.at<int32_t>(o_members) : nullptr;
     }
     for (size_t c = 0; c < split->sparse.size(); c++) {
@@ -964,7 +967,7 @@ uf_status run_gram(uf_tree *tree, const BatchJob &J, int device, double scale) {
   // sparse rows: presence terms (x = l) in FP64, one word (FP64 calls: two),
   // min form, into stripe-layout cells Msp and the per-sample R
   SparseScatter sc;
-  sc.prepare(tree, J, in, split, lay, ACC_MIN, true, digits, cells, n_cols, false, meta, st);
+  sc.prepare(tree, J, in, split, lay, ACC_MIN, true, digits, cells, n_cols, false, true, meta, st);
   if (split.n_sparse > 0) {
     Msp = DevBuf((size_t)cells * 8 * acc_words, st, "alloc sparse stripes");
     ck(cudaMemsetAsync(Msp.p, 0, (size_t)cells * 8 * acc_words, st), "memset");
@@ -1279,7 +1282,8 @@ uf_status run_stripes(uf_tree *tree, const BatchJob &J, int device, uf_method me
   std::vector<SpLayout> lay(nt);
   for (size_t t = 0; t < nt; t++) lay[t] = SpLayout{tabs[t].n, tabs[t].off, tabs[t].s_lo, tabs[t].s_hi, tabs[t].m_off};
   SparseScatter sc;
-  sc.prepare(tree, J, in, split, lay, acc, !fp32, !fp32, cells, n_cols, tile_scatter(J, acc, fp32), meta, st);
+  sc.prepare(tree, J, in, split, lay, acc, !fp32, !fp32, cells, n_cols, tile_scatter(J, acc, fp32), kind == EMB_PRESENCE,
+             meta, st);
   meta.upload(st);
   const TabDesc *d_tabs = meta.at<TabDesc>(o_tabs);
   const int32_t *d_cnt = meta.at<int32_t>(o_cnt);

@@ -263,6 +263,32 @@ __device__ __forceinline__ void add_pair_fused(int ka, int kb, const FuEnt<T, F>
   if (2 * d == c.n) red_add2<T>(c.M + cell + d, c.m_lo_off, t);
 }
 
+// The same for presence rows: the lengths (len[r], fixed point) of the rows in
+// which both samples are present.
+template <typename T, int F>
+__device__ __forceinline__ void add_pair_pres(int ka, int kb, uint8_t ea, uint8_t eb, const PairCtx<T> &c,
+                                              const Fx2 *len) {
+  const int d = kb - ka;
+  int s, kc;
+  if (2 * d <= c.n) {
+    s = d - 1;
+    kc = ka;
+  } else {
+    s = c.n - d - 1;
+    kc = kb;
+  }
+  if (s < c.s_lo || s > c.s_hi) return;
+  const int64_t cell = (int64_t)(s - c.s_lo) * c.n + kc;
+  const unsigned both = ea & eb;
+  Fx2 t = len[0];  // the listed row holds every sample of its list
+#pragma unroll
+  for (int r = 1; r <= F; r++)
+    if ((both >> r) & 1u) t = fx_add(t, len[r]);
+  if (abs_row(c.abs_mask, s)) t = fx_mul(t, -2);
+  red_add2<T>(c.M + cell, c.m_lo_off, t);
+  if (2 * d == c.n) red_add2<T>(c.M + cell + d, c.m_lo_off, t);
+}
+
 // The pair (a, b), k_a < k_b, of a fused generalized list: each row in which
 // both samples are present (u > 0) gives the den and Q (or N) terms of its
 // own update with its own length len[r]; their sums go with one atomic per
@@ -589,7 +615,14 @@ __global__ void __launch_bounds__(256) k_sparse_lists(const SparseArgs a) {
         fu_set(fe, 1 + j, fm);
         dsum = fx_add(dsum, fm);
       }
-      lf[off + u] = fe;
+      if (ACC == ACC_MIN && a.pres) {
+        unsigned m = 1u;
+#pragma unroll
+        for (int j = 0; j < F; j++) m |= cm[j] > 0.0 ? 2u << j : 0u;
+        reinterpret_cast<uint8_t *>(a.le)[off + u] = (uint8_t)m;
+      } else {
+        lf[off + u] = fe;
+      }
       a.lk[off + u] = (int)smp;
       red_add2<T>(a.Dsp + tb.off + smp, a.d_lo_off, dsum);
       u++;
@@ -872,10 +905,12 @@ __device__ __forceinline__ int lower_index(const int *K, int lo, int hi, int key
 
 // COUNT: the instantiation for timed calls, which also counts the pair updates
 // (kept apart: the count costs the counting-free kernel's 32 registers)
-template <typename T, int ACC, int MODE, int F = 0, bool COUNT = false>
+// PRES: fused presence rows, a byte per entry (25,000 samples unweighted: 62 ms
+// with the rows' 48-byte terms per entry, which every region and pair read)
+template <typename T, int ACC, int MODE, int F = 0, bool COUNT = false, bool PRES = false>
 __global__ void __launch_bounds__(128) k_sparse_region(const SparseArgs a) {
   constexpr bool FUSED = F > 0;
-  using Ent = ListEnt<T, ACC, F>;
+  using Ent = std::conditional_t<PRES, uint8_t, ListEnt<T, ACC, F>>;
   const int row = blockIdx.x;
   const SpTab tb = a.tabs[0];
   const int64_t off = a.lofs[row];
@@ -906,6 +941,16 @@ __global__ void __launch_bounds__(128) k_sparse_region(const SparseArgs a) {
   }
   c.am1 = (T)(a.alpha - 1.0);
   c.scale = a.scale;
+  // presence: the fixed-point lengths of the row and its members
+  Fx2 plen[1 + (F > 0 ? F : 1)];
+  if constexpr (PRES) {
+    plen[0] = to_fixed2((T)a.length[a.nodes[row]], a.scale);
+#pragma unroll
+    for (int j = 0; j < F; j++) {
+      const int mv = a.members[(int64_t)F * row + j];
+      plen[1 + j] = mv >= 0 ? to_fixed2((T)a.length[mv], a.scale) : Fx2{0, 0};
+    }
+  }
   // Regions come in increasing stripe order (r0 of one is r1 of the one
   // before), so for a sample a the partners of window 1 move up and those of
   // window 2 move down from region to region: each entry keeps a cursor per
@@ -917,7 +962,8 @@ __global__ void __launch_bounds__(128) k_sparse_region(const SparseArgs a) {
   uint16_t *cur1 = a.cur ? a.cur + off : nullptr, *cur2 = a.cur ? a.cur + a.cur_stride + off : nullptr;
   [[maybe_unused]] unsigned n_upd = 0;  // pair updates made by this thread: the cursors' moves
   auto add = [&](const Ent &ea, int ka, int b, int kb) {
-    if constexpr (FUSED && ACC == ACC_MIN) add_pair_fused<T, F>(ka, kb, ea, E[b], c);
+    if constexpr (PRES) add_pair_pres<T, F>(ka, kb, ea, E[b], c, plen);
+    else if constexpr (FUSED && ACC == ACC_MIN) add_pair_fused<T, F>(ka, kb, ea, E[b], c);
     else if constexpr (FUSED) add_pair_fused_gen<T, MODE, F>(ka, kb, ea, E[b], c, len);
     else add_pair<T, ACC, MODE>(ea, E[b], c);
   };
@@ -987,7 +1033,8 @@ size_t sparse_smem_bytes(bool fp32, int cap) {
   return (size_t)cap * (8 + 8 + (fp32 ? sizeof(SpEnt<float>) : sizeof(SpEnt<double>)));
 }
 
-size_t sparse_entry_bytes(bool fp32, int fused, int acc) {
+size_t sparse_entry_bytes(bool fp32, int fused, int acc, bool pres) {
+  if (pres && fused != 0 && acc == ACC_MIN) return 1;
   if (fused == 2 && acc == ACC_GEN) return fp32 ? sizeof(FuGEnt<float, 2>) : sizeof(FuGEnt<double, 2>);
   if (fused != 0 && acc == ACC_GEN) return 0;
   if (fused == 2) return fp32 ? sizeof(FuEnt<float, 2>) : sizeof(FuEnt<double, 2>);
@@ -1014,7 +1061,17 @@ cudaError_t launch_sparse_rows(int acc, bool fp32, const SparseArgs &a, cudaStre
 template <bool C>
 cudaError_t launch_region(int acc, bool fp32, const SparseArgs &a, dim3 grid, cudaStream_t st) {
   const int mode = a.alpha == 0.5 ? 0 : 1;
-  if (acc == ACC_MIN && a.fused != 0) {
+  if (acc == ACC_MIN && a.fused != 0 && a.pres) {
+    if (a.fused == 2) {
+      if (fp32) k_sparse_region<float, ACC_MIN, 0, 2, C, true><<<grid, 128, 0, st>>>(a);
+      else k_sparse_region<double, ACC_MIN, 0, 2, C, true><<<grid, 128, 0, st>>>(a);
+    } else if (a.fused == 6) {
+      if (fp32) k_sparse_region<float, ACC_MIN, 0, 6, C, true><<<grid, 128, 0, st>>>(a);
+      else k_sparse_region<double, ACC_MIN, 0, 6, C, true><<<grid, 128, 0, st>>>(a);
+    } else {
+      return cudaErrorInvalidValue;
+    }
+  } else if (acc == ACC_MIN && a.fused != 0) {
     if (a.fused == 2) {
       if (fp32) k_sparse_region<float, ACC_MIN, 0, 2, C><<<grid, 128, 0, st>>>(a);
       else k_sparse_region<double, ACC_MIN, 0, 2, C><<<grid, 128, 0, st>>>(a);

@@ -55,6 +55,9 @@ struct SparseArgs {
   // atomic per accumulator; members[fused * (row_base + blockIdx.x) + i] is a
   // node or -1
   int fused;
+  int pres;                 // fused presence rows: an entry is one byte, bit r set where the sample
+                            // is below the row (r = 0) or its r-th member; every such term is the
+                            // row's length
   const int32_t *members;
   // region mode: only pairs whose stripe lies in [r0, r1) (launch_sparse_region)
   int r0, r1;
@@ -118,7 +121,7 @@ constexpr int SPARSE_LIST_MAX_ENTRIES = 16384;
 static_assert(SPARSE_LIST_MAX_ENTRIES <= 65535, "list cursors are 16-bit");
 constexpr int SPARSE_PAIR_SLOTS = 256;
 size_t sparse_smem_bytes(bool fp32, int cap);
-size_t sparse_entry_bytes(bool fp32, int fused = 0, int acc = ACC_MIN);
+size_t sparse_entry_bytes(bool fp32, int fused = 0, int acc = ACC_MIN, bool pres = false);
 cudaError_t launch_sparse_rows(int acc, bool fp32, const SparseArgs &a, cudaStream_t st);
 cudaError_t launch_sparse_lists(int acc, bool fp32, const SparseArgs &a, cudaStream_t st);
 // Pairs of the listed rows (nodes[0 .. n_nodes), lists from a list-mode
