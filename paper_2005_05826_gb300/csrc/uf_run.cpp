@@ -671,71 +671,37 @@ struct SparseScatter {
     const size_t nt = J.tabs.size();
     if (sp.n_sparse == 0) return;
     const int64_t n_regions = (int64_t)sparse_regions(nt, acc, (double)cells * 8.0 * n_acc * (two_word ? 2 : 1));
-    std::vector<int32_t> all, members;
+    std::vector<int32_t> all;
     tiles = want_tiles && prepare_tiles(tree, J, sp, &all, meta, st);
     region_mode = !tiles && (n_regions > 1 || sp.lists);
     pres = presence;
-    // the generalized method's entries carry each row's proportion as well:
-    // two members at most
-    fuse_m = !region_mode ? 0 : acc == ACC_MIN ? (int)g_sparse_fuse.load() : (int)std::min<int64_t>(g_sparse_fuse.load(), 2);
-    if (tiles) {
-    } else if (fuse_m > 0) {
-      // A sparse branch whose parent is a listed head rides in the parent's
-      // list (its samples are among the parent's and its pairs among the
-      // parent's pairs); with six members per head, so does a sparse child of
-      // such a member (two levels below the head).  Parents come before
-      // children in decreasing node order (parent[v] > v), so every head and
-      // member is final when its children are visited.
-      const int F = fuse_m, depth = F == 6 ? 2 : 1;
-      const int64_t nn = tree->n_nodes;
-      std::vector<int8_t> level(nn, -1), used(nn, 0);  // -1: not listed, 0: head, >0: member depth
-      std::vector<int32_t> head_of(nn, -1), mem_of((size_t)nn * F, -1);
-      for (const auto &c : sp.sparse)
-        for (int32_t v : c) level[v] = 0;
-      for (int64_t v = nn - 2; v >= 0; v--) {
-        if (level[v] != 0) continue;
-        const int64_t p = tree->parent[v];
-        if (p < 0 || level[p] < 0 || level[p] >= depth) continue;
-        const int32_t h = level[p] == 0 ? (int32_t)p : head_of[p];
-        if (used[h] >= F) continue;
-        mem_of[(size_t)h * F + used[h]++] = (int32_t)v;
-        level[v] = (int8_t)(level[p] + 1);
-        head_of[v] = h;
-      }
-      for (const auto &c : sp.sparse) {
-        sp_off.push_back((int64_t)all.size());
-        for (int32_t v : c)
-          if (level[v] == 0) {
-            all.push_back(v);
-            members.insert(members.end(), mem_of.begin() + (size_t)v * F, mem_of.begin() + (size_t)v * F + F);
-          }
-        cls_n.push_back((int64_t)all.size() - sp_off.back());
-      }
-    } else {
+    fuse_m = region_mode ? sp.fuse : 0;
+    const RegionLists *rl = region_mode ? &region_lists(tree, J.tabs[0].table, sp) : nullptr;
+    if (rl) {
+      sp_off = rl->cls_off;
+      cls_n = rl->cls_n;
+    } else if (!tiles) {
       for (const auto &c : sp.sparse) {
         sp_off.push_back((int64_t)all.size());
         all.insert(all.end(), c.begin(), c.end());
         cls_n.push_back((int64_t)c.size());
       }
     }
-    n_sparse_rows = (int64_t)all.size();
+    const std::vector<int32_t> &rows = rl ? rl->heads : all;
+    n_sparse_rows = (int64_t)rows.size();
     if (region_mode) {
-      const auto &cp = J.tabs[0].table->col_ptr;
-      std::vector<int64_t> lofs(all.size() + 1, 0);
-      for (size_t r = 0; r < all.size(); r++)
-        lofs[r + 1] = lofs[r] + (cp[tree->tip_hi[all[r]]] - cp[tree->tip_lo[all[r]]]);
-      const size_t total_e = (size_t)std::max<int64_t>(lofs.back(), 1);
+      const size_t total_e = (size_t)std::max<int64_t>(rl->entry_off.back(), 1);
       list_entries = (int64_t)total_e;
       le = DevBuf(total_e * sparse_entry_bytes(!fp64_entries, fuse_m, acc, pres), st, "alloc sparse lists");
       lk = DevBuf(total_e * 4, st, "alloc sparse lists");
       // (cursors from one region to the next)
       if (region_stripes(g_region_bytes.load()) <= (int64_t)lay[0].s_hi - lay[0].s_lo)
         cur = DevBuf(total_e * 2 * sizeof(uint16_t), st, "alloc sparse list cursors");
-      lz = DevBuf(std::max<size_t>(all.size(), 1) * 4, st, "alloc sparse lists");
+      lz = DevBuf(std::max<size_t>(rows.size(), 1) * 4, st, "alloc sparse lists");
       // rows without entries in the table return before writing their count
-      ck(cudaMemsetAsync(lz.p, 0, std::max<size_t>(all.size(), 1) * 4, st), "memset");
-      o_lofs = meta.add(lofs);
-      if (fuse_m > 0) o_members = meta.add(members);
+      ck(cudaMemsetAsync(lz.p, 0, std::max<size_t>(rows.size(), 1) * 4, st), "memset");
+      o_lofs = meta.add(rl->entry_off);
+      if (fuse_m > 0) o_members = meta.add(rl->members);
     }
     std::vector<SpTab> tabs(nt);
     for (size_t t = 0; t < nt; t++) {
@@ -750,7 +716,7 @@ struct SparseScatter {
       tabs[t].s_hi = lay[t].s_hi;
       tabs[t].m_off = lay[t].m_off;
     }
-    o_sparse = meta.add(all);
+    o_sparse = meta.add(rows);
     o_sptabs = meta.add(tabs);
     const size_t dsp_words = (size_t)n_cols * (two_word ? 2 : 1);
     Dsp = DevBuf(dsp_words * 8, st, "alloc diagonal");

@@ -62,6 +62,7 @@ RowSplit split_rows(const uf_tree *tree, const BatchJob &J, const Plan *P, int a
     const bool listed =
         nt == 1 && (acc == ACC_MIN || acc == ACC_GEN) && fp32 && J.tabs[0].table->n >= LIST_MIN_SAMPLES;
     R.lists = regions || tiles || listed;
+    R.fuse = (int)(acc == ACC_GEN ? std::min<int64_t>(g_sparse_fuse.load(), 2) : g_sparse_fuse.load());
     // list mode keeps only sort keys in shared memory: longer runs fit
     const int64_t max_entries = R.lists ? SPARSE_LIST_MAX_ENTRIES : SPARSE_MAX_ENTRIES;
     // the scatter runs table by table (its grid's y is the table), so each
@@ -80,8 +81,7 @@ RowSplit split_rows(const uf_tree *tree, const BatchJob &J, const Plan *P, int a
     // about that share of its own pairs and visits.  The tensor path's
     // scatter runs beside its gram and ends after it already: its split keeps
     // the unfused costs.
-    const int64_t fm = acc == ACC_GEN ? std::min<int64_t>(g_sparse_fuse.load(), 2) : g_sparse_fuse.load();
-    const double fuse = (regions || listed) && acc != SPLIT_GRAM && fm > 0 ? (fm == 6 ? 0.45 : 0.6) : 1.0;
+    const double fuse = (regions || listed) && acc != SPLIT_GRAM && R.fuse > 0 ? (R.fuse == 6 ? 0.45 : 0.6) : 1.0;
     for (size_t t = 0; t < nt; t++) {
       const double n = (double)J.tabs[t].table->n;
       const double atom_rate = std::floor(n / 2.0) * n * 8.0 * n_acc <= 64e6 || regions ? 2.3e11 : 2.5e10;
@@ -152,69 +152,84 @@ RowSplit split_rows(const uf_tree *tree, const BatchJob &J, const Plan *P, int a
       R.pairs += pt.pairs;
     }
   }
-  const int64_t root = tree->n_nodes - 1;
-  auto parent_dense = [&](int64_t v) {
-    const int64_t p = tree->parent[v];
-    return p != root && !is_sparse[p];
-  };
-  // per list position: bit 0 = built from CSC columns (tips, and sparse
-  // branches under a dense parent), bit 1 = a dense internal node, bit 2 = a
-  // dense branch; flagged in parallel, then gathered in list order
-  std::vector<uint8_t> flag(P->lists.size(), 0);
-  {
-    const int64_t np = (int64_t)P->lists.size();
-    const int T = (int)std::max<int64_t>(1, std::min<int64_t>(host_threads(), np / 16384));
-    parallel_for(T, [&](int c) {
-      const int64_t p0 = np * c / T, p1 = np * (c + 1) / T;
-      size_t b = 0;
-      for (int64_t q = p0; q < p1; q++) {
-        // block of position q: blocks cover consecutive ranges of the lists
-        while (b + 1 < P->launches.size() && q >= P->launches[b + 1][0].first) b++;
-        const auto &l0 = P->launches[b][0];
-        const int32_t v = P->lists[q];
-        const bool tip = q < l0.first + l0.second;
-        flag[q] = (uint8_t)((is_sparse[v] ? parent_dense(v) : tip) | ((!tip && !is_sparse[v]) << 1) |
-                            (!is_sparse[v] << 2));
-      }
-    });
-  }
-  for (size_t b = 0; b < P->b0.size(); b++) {
-    const auto &ls = P->launches[b];
-    std::vector<std::pair<int64_t, int>> lb;
-    const int64_t q0 = ls[0].first, q1 = ls.back().first + ls.back().second;
-    const int64_t at0 = (int64_t)R.cnt_lists.size();
-    // (the dense branches among them first: only they get embedding rows)
-    int built_dense = 0;
-    for (int want = 1; want >= 0; want--)
-      for (int64_t q = q0; q < q1; q++)
-        if ((flag[q] & 5) == (want ? 5 : 1)) {
-          R.cnt_lists.push_back(P->lists[q]);
-          built_dense += want;
+  auto count_rows = [&] {
+    const int64_t root = tree->n_nodes - 1;
+    auto parent_dense = [&](int64_t v) {
+      const int64_t p = tree->parent[v];
+      return p != root && !is_sparse[p];
+    };
+    // per list position: bit 0 = built from CSC columns (tips, and sparse
+    // branches under a dense parent), bit 1 = a dense internal node, bit 2 = a
+    // dense branch; flagged in parallel, then gathered in list order
+    std::vector<uint8_t> flag(P->lists.size(), 0);
+    {
+      const int64_t np = (int64_t)P->lists.size();
+      const int T = (int)std::max<int64_t>(1, std::min<int64_t>(host_threads(), np / 16384));
+      parallel_for(T, [&](int c) {
+        const int64_t p0 = np * c / T, p1 = np * (c + 1) / T;
+        size_t b = 0;
+        for (int64_t q = p0; q < p1; q++) {
+          // block of position q: blocks cover consecutive ranges of the lists
+          while (b + 1 < P->launches.size() && q >= P->launches[b + 1][0].first) b++;
+          const auto &l0 = P->launches[b][0];
+          const int32_t v = P->lists[q];
+          const bool tip = q < l0.first + l0.second;
+          flag[q] = (uint8_t)((is_sparse[v] ? parent_dense(v) : tip) | ((!tip && !is_sparse[v]) << 1) |
+                              (!is_sparse[v] << 2));
         }
-    R.cnt_built_dense.push_back(built_dense);
-    lb.emplace_back(at0, (int)((int64_t)R.cnt_lists.size() - at0));
-    for (size_t l = 1; l < ls.size(); l++) {
-      const int64_t at = (int64_t)R.cnt_lists.size();
-      for (int64_t q = ls[l].first; q < ls[l].first + ls[l].second; q++)
-        if (flag[q] & 2) R.cnt_lists.push_back(P->lists[q]);
-      if ((int64_t)R.cnt_lists.size() > at) lb.emplace_back(at, (int)((int64_t)R.cnt_lists.size() - at));
+      });
     }
-    R.cnt_launch.push_back(std::move(lb));
-  }
-  std::vector<int32_t> row_of(std::max<int64_t>(nb, 1), -1);
-  R.dense_ptr.push_back(0);
-  for (size_t b = 0; b < P->b0.size(); b++) {
-    for (int64_t v = P->b0[b]; v < P->b1[b]; v++)
-      if (!is_sparse[v]) {
-        row_of[v] = (int32_t)((int64_t)R.dense.size() - R.dense_ptr[b]);
-        R.dense.push_back((int32_t)v);
-        R.dense_len.push_back(tree->length[v]);
+    for (size_t b = 0; b < P->b0.size(); b++) {
+      const auto &ls = P->launches[b];
+      std::vector<std::pair<int64_t, int>> lb;
+      const int64_t q0 = ls[0].first, q1 = ls.back().first + ls.back().second;
+      const int64_t at0 = (int64_t)R.cnt_lists.size();
+      // (the dense branches among them first: only they get embedding rows)
+      std::vector<int32_t> sparse_built;
+      for (int64_t q = q0; q < q1; q++)
+        if (flag[q] & 1) (flag[q] & 4 ? R.cnt_lists : sparse_built).push_back(P->lists[q]);
+      R.cnt_built_dense.push_back((int)((int64_t)R.cnt_lists.size() - at0));
+      R.cnt_lists.insert(R.cnt_lists.end(), sparse_built.begin(), sparse_built.end());
+      lb.emplace_back(at0, (int)((int64_t)R.cnt_lists.size() - at0));
+      for (size_t l = 1; l < ls.size(); l++) {
+        const int64_t at = (int64_t)R.cnt_lists.size();
+        for (int64_t q = ls[l].first; q < ls[l].first + ls[l].second; q++)
+          if (flag[q] & 2) R.cnt_lists.push_back(P->lists[q]);
+        if ((int64_t)R.cnt_lists.size() > at) lb.emplace_back(at, (int)((int64_t)R.cnt_lists.size() - at));
       }
-    R.dense_ptr.push_back((int64_t)R.dense.size());
-    R.max_dense = std::max(R.max_dense, R.dense_ptr[b + 1] - R.dense_ptr[b]);
-  }
+      R.cnt_launch.push_back(std::move(lb));
+    }
+  };
+  std::vector<int32_t> row_of(std::max<int64_t>(nb, 1));  // of a dense branch
+  auto dense_rows = [&] {
+    R.dense_ptr.push_back(0);
+    for (size_t b = 0; b < P->b0.size(); b++) {
+      for (int64_t v = P->b0[b]; v < P->b1[b]; v++)
+        if (!is_sparse[v]) {
+          row_of[v] = (int32_t)((int64_t)R.dense.size() - R.dense_ptr[b]);
+          R.dense.push_back((int32_t)v);
+          R.dense_len.push_back(tree->length[v]);
+        }
+      R.dense_ptr.push_back((int64_t)R.dense.size());
+      R.max_dense = std::max(R.max_dense, R.dense_ptr[b + 1] - R.dense_ptr[b]);
+    }
+  };
+  // the lists of the scattered branches (a table's tiles make their own), of
+  // the count rows and of the dense rows side by side: none needs another
+  const bool lists = R.lists && R.n_sparse > 0 && !tile_scatter(J, acc, fp32);
+  auto part = [&](int c) {
+    if (c == 0 && lists) region_lists(tree, J.tabs[0].table, R);
+    if (c == 1) count_rows();
+    if (c == 2) dense_rows();
+  };
+  if (nb >= 16384) parallel_for(3, part);
+  else
+    for (int c = 0; c < 3; c++) part(c);
   R.cnt_xrow.resize(R.cnt_lists.size());
-  for (size_t q = 0; q < R.cnt_lists.size(); q++) R.cnt_xrow[q] = row_of[R.cnt_lists[q]];
+  for (size_t q = 0; q < R.cnt_lists.size(); q++) {
+    const int32_t v = R.cnt_lists[q];
+    R.cnt_xrow[q] = is_sparse[v] ? -1 : row_of[v];
+  }
   for (size_t b = 0; b < R.cnt_launch.size(); b++) {
     R.cnt_lev_ptr.push_back((int64_t)R.cnt_levels.size());
     for (const auto &l : R.cnt_launch[b]) {
@@ -226,6 +241,103 @@ RowSplit split_rows(const uf_tree *tree, const BatchJob &J, const Plan *P, int a
 }
 
 }  // namespace
+
+const RegionLists &region_lists(const uf_tree *tree, const uf_table *table, const RowSplit &sp) {
+  RegionLists &L = *sp.region;
+  std::call_once(L.once, [&] {
+    const int F = sp.fuse, depth = F == 0 ? 0 : F == 6 ? 2 : 1;
+    const int64_t nn = tree->n_nodes;
+    // A sparse branch whose parent is a listed head rides in the parent's
+    // list (its samples are among the parent's and its pairs among the
+    // parent's pairs); with six members per head, so does a sparse child of
+    // such a member (two levels below the head).  Parents come before
+    // children in decreasing node order (parent[v] > v), so every head and
+    // member is final when its children are visited.  The pass is sequential
+    // and its choices are near coin flips: written without branches.
+    std::vector<int8_t> level(nn, -1), used(nn, 0);  // -1: not listed, 0: head, >0: member depth
+    std::vector<int32_t> head(nn);                   // a member's head, else the node
+    std::vector<int8_t> slot(nn);
+    for (const auto &c : sp.sparse)
+      for (int32_t v : c) level[v] = 0;
+    head[nn - 1] = (int32_t)(nn - 1);
+    const int64_t *parent = tree->parent.data();
+    for (int64_t v = nn - 2; v >= 0; v--) {
+      const int64_t p = parent[v];
+      const int32_t h = head[p];
+      const int lp = level[p], uh = used[h];
+      const int join = (level[v] == 0) & (lp >= 0) & (lp < depth) & (uh < F);
+      used[h] = (int8_t)(uh + join);
+      slot[v] = (int8_t)uh;
+      level[v] = (int8_t)(level[v] + join * (lp + 1));
+      head[v] = join ? h : (int32_t)v;
+    }
+    // the rest in parallel, in pieces of a class that keep its order
+    struct Piece {
+      size_t k, b, e;
+      int64_t heads = 0, entries = 0;
+    };
+    std::vector<Piece> pc;
+    constexpr size_t PIECE = 8192;
+    for (size_t k = 0; k < sp.sparse.size(); k++)
+      for (size_t b = 0; b < sp.sparse[k].size(); b += PIECE)
+        pc.push_back(Piece{k, b, std::min(b + PIECE, sp.sparse[k].size())});
+    const auto &cp = table->col_ptr;
+    const int T = (int)std::max<int64_t>(1, std::min<int64_t>(host_threads(), (int64_t)pc.size()));
+    auto pieces = [&](const std::function<void(Piece &)> &body) {
+      parallel_for(T, [&](int c) {
+        for (size_t i = pc.size() * c / T; i < pc.size() * (c + 1) / T; i++) body(pc[i]);
+      });
+    };
+    pieces([&](Piece &x) {
+      const std::vector<int32_t> &rows = sp.sparse[x.k];
+      int64_t heads = 0, entries = 0;
+      for (size_t i = x.b; i < x.e; i++) {
+        const int32_t v = rows[i];
+        const int64_t is = level[v] == 0;
+        heads += is;
+        entries += is * (cp[tree->tip_hi[v]] - cp[tree->tip_lo[v]]);
+      }
+      x.heads = heads;
+      x.entries = entries;
+    });
+    L.cls_off.assign(sp.sparse.size(), 0);
+    L.cls_n.assign(sp.sparse.size(), 0);
+    int64_t n_heads = 0, n_entries = 0;
+    for (Piece &x : pc) {  // counts -> first positions
+      L.cls_n[x.k] += x.heads;
+      std::swap(n_heads, x.heads);
+      std::swap(n_entries, x.entries);
+      n_heads += x.heads;
+      n_entries += x.entries;
+    }
+    for (size_t k = 1; k < L.cls_n.size(); k++) L.cls_off[k] = L.cls_off[k - 1] + L.cls_n[k - 1];
+    L.heads.resize(n_heads);
+    L.members.resize((size_t)n_heads * F);
+    L.entry_off.resize(n_heads + 1);
+    L.entry_off[n_heads] = n_entries;
+    pieces([&](Piece &x) {
+      const std::vector<int32_t> &rows = sp.sparse[x.k];
+      int64_t q = x.heads, e = x.entries;
+      for (size_t i = x.b; i < x.e; i++) {
+        const int32_t v = rows[i];
+        if (level[v] != 0) continue;
+        L.heads[q] = v;
+        L.entry_off[q] = e;
+        e += cp[tree->tip_hi[v]] - cp[tree->tip_lo[v]];
+        for (int m = used[v]; m < F; m++) L.members[(size_t)q * F + m] = -1;
+        head[v] = (int32_t)q++;  // (from here a head's position)
+      }
+    });
+    pieces([&](Piece &x) {
+      const std::vector<int32_t> &rows = sp.sparse[x.k];
+      for (size_t i = x.b; i < x.e; i++) {
+        const int32_t v = rows[i];
+        if (level[v] > 0) L.members[(size_t)head[head[v]] * F + slot[v]] = v;
+      }
+    });
+  });
+  return L;
+}
 
 // The split of a call, cached on the tree by its tables and kind (tables are
 // immutable and their ids are never reused).
