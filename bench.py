@@ -313,33 +313,38 @@ def downstream_agreement(mixed_outs, fp64_outs, sub=512, perms=999):
     return res
 
 
-# FP64 instructions per update of the FP64 accumulate kernels: the min / abs
-# kernel one DADD for u - v and one DADD of |u - v| into the accumulator
-# (ncu: 2.02); the generalized kernel (alpha = 1/2) 11.07, as ncu counts them
-# (smsp__inst_executed_pipe_fp64 per update; profiles/fp64_kernels_yule50k_n2048.md).
-FP64_OPS_PER_UPDATE = {"min": 2.0, "gen": 11.07}
-# GB300 FP64 lanes per SM and clock: nominal 1.25 TFLOP/s counting an FMA as two
-FP64_LANES_PER_SM = 2.0
+# FP64 calls: the generalized kernel (alpha = 1/2) is bound by the FP64 pipe, 11.07
+# instructions per update as ncu counts them (profiles/fp64_kernels_yule50k_n2048.md)
+# on 2 lanes per SM and clock (nominal 1.25 TFLOP/s counting an FMA as two); the
+# weighted kernel sums 64-bit integers, 5 instructions per update on 64 lanes; the
+# unweighted gram runs on the tensor cores (seven digit products per term).
+FP64_GEN_OPS_PER_UPDATE, FP64_LANES_PER_SM = 11.07, 2.0
+U64_OPS_PER_UPDATE, INT_LANES_PER_SM = 5.0, 64.0
 
 
-def fp64_rooflines(f_reps, pairs, sm_max):
-    """Roofline objects of the FP64 accumulate kernels from the per-phase
-    device times of the FP64 calls: updates of the dense branches over the
-    FP64 pipe's instruction rate divided by the instructions per update."""
+def fp64_rooflines(f_reps, pairs, sm_max, peaks, peak_src):
+    """Roofline objects of the FP64 calls' accumulate kernels from their
+    per-phase device times: updates of the dense branches over the bounding
+    pipe's instruction rate divided by the instructions per update, or executed
+    tensor flops over the measured BF16 peak."""
     out = {}
     for m, r in f_reps:
         if r.acc_launches == 0 or r.t_accumulate_ms <= 0:
             continue
-        kind = "gen" if m == "generalized" else "min"
-        ach = pairs * r.dense_rows / (r.t_accumulate_ms / 1e3) / 1e12
-        obj = {"kernel": "k_stripe_gen<double,4,8>" if kind == "gen" else "k_stripe_min<double,8,8,abs>",
-               "bound": "alu", "achieved": ach, "unit": "Tupdates/s"}
-        ops = FP64_OPS_PER_UPDATE[kind]
-        if ops:
-            peak = FP64_LANES_PER_SM * SMS * sm_max * 1e6 / ops / 1e12
-            obj.update({"peak": peak, "frac": ach / peak,
-                        "peak_basis": f"FP64 pipe {FP64_LANES_PER_SM:g} lanes/clk/SM x {SMS} SMs x "
-                                      f"{sm_max:.0f} MHz / {ops:g} FP64 instructions per update"})
+        if r.path == 1:
+            ach, peak = r.exec_flops / (r.t_accumulate_ms / 1e3) / 1e12, float(peaks.get("bf16_tflops", 1900.0))
+            obj = {"kernel": "k_gram<digits>", "bound": "tensor", "achieved": ach, "unit": "TFLOP/s", "peak": peak,
+                   "frac": ach / peak, "peak_basis": f"measured bf16 dense ({peak_src})"}
+        else:
+            gen = m == "generalized"
+            ops, lanes = ((FP64_GEN_OPS_PER_UPDATE, FP64_LANES_PER_SM) if gen
+                          else (U64_OPS_PER_UPDATE, INT_LANES_PER_SM))
+            ach = pairs * r.dense_rows / (r.t_accumulate_ms / 1e3) / 1e12
+            peak = lanes * SMS * sm_max * 1e6 / ops / 1e12
+            obj = {"kernel": "k_stripe_gen<double,4,8>" if gen else "k_stripe_u64<4,8>", "bound": "alu",
+                   "achieved": ach, "unit": "Tupdates/s", "peak": peak, "frac": ach / peak,
+                   "peak_basis": f"{'FP64' if gen else 'integer'} pipe {lanes:g} lanes/clk/SM x {SMS} SMs x "
+                                 f"{sm_max:.0f} MHz / {ops:g} instructions per update"}
         out[f"roofline_{m}"] = obj
     return out
 
@@ -815,7 +820,7 @@ def run_ours(args, rank, world, local_rank):
                 "slice": f"stripes [0, {k}) of {S}, all methods of the step (from a slice)",
                 "ms_per_method": {m: r.t_accumulate_ms + r.t_diag_ms + r.t_embed_ms + r.t_finalize_ms
                                   for m, r in f_reps}}
-        fp64.update(fp64_rooflines(f_reps, k * n, sm_max))
+        fp64.update(fp64_rooflines(f_reps, k * n, sm_max, peaks, peak_src))
         if full and not args.no_downstream:
             # the paper's FP32-vs-FP64 check (Sec. 4) on a sample subset: the
             # mixed full matrix's entries of the first `sub` samples against
@@ -849,7 +854,7 @@ def run_ours(args, rank, world, local_rank):
                       for m, r in f_reps}
         fp64 = {"value": updates_step / t64, "unit": "updates/s", "ms_per_step": t64 * 1e3,
                 "ms_per_method": per_method}
-        fp64.update(fp64_rooflines(f_reps, npairs, sm_max))
+        fp64.update(fp64_rooflines(f_reps, npairs, sm_max, peaks, peak_src))
         if keep_host and not args.no_err:
             mixed_err = max_err_vs_fp64(mixed_outs, fp64_outs)
         if keep_host and not args.no_downstream:

@@ -182,8 +182,9 @@ typedef struct {
  *                    faster; 0: every branch through the dense kernels;
  *                    2: every branch that can be scattered is (subtree with
  *                    at most 4,096 entries per table, 16,384 when one table's
- *                    accumulators are scattered region by region, and
- *                    contiguous tip numbers).  Applies to the CUDA-core stripe kernels and
+ *                    branches go through lists (its accumulators scattered
+ *                    region by region, or 512 samples or more with UF_MIXED or,
+ *                    weighted, UF_FP64), and contiguous tip numbers).  Applies to the CUDA-core stripe kernels and
  *                    to the tensor-core unweighted path; the results agree
  *                    within the precision's tolerance.
  *   "sparse_overlap" 1 (default): the sparse-row scatter runs on a second
@@ -196,7 +197,7 @@ typedef struct {
  *                    wait runs out after 2 s: a synchronous call returns
  *                    UF_ETIMEOUT and an asynchronous one writes NaN (for
  *                    testing the abort path; no fault, the context stays usable)
- *   "sparse_fuse"    2 (default), 6 or 0: in the region scatter of a min-form
+ *   "sparse_fuse"    2 (default), 6 or 0: in the list scatter of a min-form
  *                    method (the weighted methods and the tensor path's
  *                    unweighted) a listed branch also carries the terms of its
  *                    scattered children (2), or of its children and their

@@ -58,7 +58,7 @@ RowSplit split_rows(const uf_tree *tree, const BatchJob &J, const Plan *P, int a
     // FP32 terms of one table go through lists even when its accumulators fit
     // in L2: a fused list's pair is one atomic (generalized: two) for three
     // branches, and the atomics bound the scatter (2,048 samples weighted 4.73 ->
-    // 4.35 ms a call, 1,003 generalized 3.13 -> 3.01)
+    // 4.29 ms a call, 1,003 generalized 3.13 -> 2.94)
     const bool listed =
         nt == 1 && (acc == ACC_MIN || acc == ACC_GEN) && fp32 && J.tabs[0].table->n >= LIST_MIN_SAMPLES;
     R.lists = regions || tiles || listed;
@@ -76,7 +76,7 @@ RowSplit split_rows(const uf_tree *tree, const BatchJob &J, const Plan *P, int a
     const double job_cost = 5e-10;
     // region lists are fused (a listed branch carries its sparse children,
     // and for the min form with option sparse_fuse 6 its grandchildren,
-    // uf_run.cpp): on the 113k-sample table about 0.57 (0.43) of the pairs
+    // region_lists): on the 113k-sample table about 0.57 (0.43) of the pairs
     // and 0.54 (0.39) of the list entries remain, so a scattered branch costs
     // about that share of its own pairs and visits.  The tensor path's
     // scatter runs beside its gram and ends after it already: its split keeps
