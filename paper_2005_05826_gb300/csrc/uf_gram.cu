@@ -9,8 +9,9 @@
 // l = l_hi + l_mid + l_lo (each product is exact; the sum of the three terms
 // carries l to about 24 bits), accumulated in FP32 in tensor memory.
 //
-// FP64 calls take the same contraction exactly: each length is a 63-bit fixed
-// point integer in seven signed digits of 9 bits (-256 .. 255, exact in BF16),
+// FP64 calls take the same contraction exactly: each length is a fixed-point
+// integer of at most 2^62 in seven signed digits of 9 bits (-256 .. 255, the top
+// one up to 256; all exact in BF16),
 // A_t = P diag(digit t), and a digit's sum over a unit is an integer below
 // 2^23, so FP32 accumulation holds it exactly (the error-free splitting of
 // Ozaki et al., Numer. Algorithms 59, 2012, on integer digits).  A unit sums
@@ -427,7 +428,9 @@ __global__ void __launch_bounds__(256) k_gram_prep(const int32_t *__restrict__ n
 #pragma unroll
       for (int t = 0; t < NT; t++) {
         constexpr long long HALF = 1ll << (GRAM_DIGIT_BITS - 1);
-        const long long d = ((x + HALF) & (2 * HALF - 1)) - HALF;
+        // the top digit is what is left, up to +256: seven digits of at most 255
+        // end at 0.998 x 2^62
+        const long long d = t == NT - 1 ? x : ((x + HALF) & (2 * HALF - 1)) - HALF;
         term[1 + t][threadIdx.x] = __float2bfloat16((float)d);
         x = (x - d) >> GRAM_DIGIT_BITS;
       }

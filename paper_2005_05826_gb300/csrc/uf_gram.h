@@ -20,8 +20,9 @@ struct GramTab {
   int64_t map_off;      // first entry of its tile map
 };
 // Terms of a branch length in the A planes: mixed, three BF16 terms of its
-// value; FP64, seven signed digits of GRAM_DIGIT_BITS bits of its 63-bit fixed
-// point (integers -256 .. 255, exact in BF16), summed two at a time.
+// value; FP64, seven signed digits of GRAM_DIGIT_BITS bits of its fixed point, an
+// integer of at most 2^62 (digits -256 .. 255, the top one 0 .. 256: all exact in
+// BF16), summed two at a time.
 constexpr int GRAM_SPLITS = 3;
 constexpr int GRAM_DIGITS = 7;
 constexpr int GRAM_DIGIT_BITS = 9;
@@ -76,7 +77,7 @@ int64_t gram_kpad(int rows);              // branches rounded up to the stage
 void gram_tiles(int n, int64_t s0, int64_t s1, std::vector<int32_t> *bi, std::vector<int32_t> *bj);
 // planes of branches nodes[0 .. rows) from their presence bits (rows of `words`
 // words, uf_embed.h): 1 + GRAM_SPLITS planes, or with digit_scale != 0
-// (2^g, every length x 2^g below 2^62) 1 + GRAM_DIGITS
+// (2^g, every length a sample has x 2^g below 2^62) 1 + GRAM_DIGITS
 cudaError_t launch_gram_prep(const int32_t *nodes, int rows, const int32_t *slot_of_node, const uint32_t *bits,
                              int64_t words, const double *length, const GramTab *tabs, int n_tabs, int npad_tot,
                              int64_t K_pad, void *Pl, double digit_scale, cudaStream_t st);

@@ -19,6 +19,16 @@ def olib():
     return oracle.load()
 
 
+@pytest.fixture(scope="session")
+def gpu_library():
+    """The library, built, on a box with a CUDA device."""
+    import torch
+    from paper_2005_05826_gb300 import build
+    build.build()
+    if not torch.cuda.is_available():
+        pytest.fail("GPU tests need a CUDA device")
+
+
 def pytest_terminal_summary(terminalreporter):
     # the precision report of the GPU parity tests: every comparison with the
     # FP64 oracle, largest errors per method and precision
