@@ -85,12 +85,15 @@ typedef enum {
  * end with one FP64 num / den division.
  * UF_FP64   branch embeddings in IEEE FP64.  Weighted and unweighted methods:
  *           each embedded value rounded once to a 64-bit fixed-point grid
- *           (about 2^-60 of a root-to-tip distance; UF_UNWEIGHTED, on the
- *           tensor cores, lengths to 2^-63 of the longest), every per-branch
- *           update and sum after that in exact integers.  Generalized and
- *           variance-adjusted: per-branch updates in FP64 on CUDA cores,
- *           partial sums in FP64 before each fixed-point rounding, every
- *           numerator a sum of nonnegative terms (no cancellation).
+ *           (about 2^-62 of a sample's mean root-to-tip distance, the largest
+ *           of them; UF_UNWEIGHTED, on the tensor cores, lengths to 2^-62 of
+ *           the longest), every per-branch update and sum after that in exact
+ *           integers.  Where a sample's own branches are so much shorter that
+ *           this grid could move its distances by more than 4e-16 of their
+ *           denominator, and for the generalized and variance-adjusted
+ *           methods: per-branch updates in FP64 on CUDA cores, partial sums in
+ *           FP64 before each fixed-point rounding (slower).  Every numerator is
+ *           a sum of nonnegative terms (no cancellation).
  *           Distances d within 1e-10 * |d| + 1e-15 of an FP64 per-pair
  *           evaluation: relative 1e-10 down to d = 1e-5, and the grid's
  *           absolute rounding below that (near-identical samples).

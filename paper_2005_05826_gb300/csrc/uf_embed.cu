@@ -192,7 +192,10 @@ template <int KIND>
 struct RowValue<double, KIND> {
   Quotient q;
   __device__ RowValue(double total, float, double) : q(total) {}
-  __device__ double operator()(double c, double) const { return q(c); }  // EMB_PROP
+  __device__ double operator()(double c, double l) const {
+    if (KIND == EMB_PRESENCE) return c > 0.0 ? l : 0.0;
+    return KIND == EMB_SCALED ? l * q(c) : q(c);
+  }
 };
 template <int KIND>
 struct RowValue<unsigned long long, KIND> {
@@ -200,7 +203,7 @@ struct RowValue<unsigned long long, KIND> {
   double scale;
   __device__ RowValue(double total, float, double row_scale) : q(total), scale(row_scale) {}
   __device__ unsigned long long operator()(double c, double l) const {
-    const double ls = l * scale;  // exact: scale is a power of two
+    const double ls = l * scale;  // exact, and finite for every branch (grid_fits)
     if (KIND == EMB_PRESENCE) return c > 0.0 ? __double2ull_rn(ls) : 0ull;
     return __double2ull_rn(ls * q(c));
   }
@@ -377,8 +380,12 @@ cudaError_t embed_launch(int kind, bool fp32, const EmbedArgs &a, dim3 grid, int
     if (kind == EMB_PRESENCE) UF_SLAB(float, EMB_PRESENCE);
     UF_SLAB(float, EMB_PROP);
   }
-  if (kind == EMB_SCALED) UF_SLAB(unsigned long long, EMB_SCALED);
-  if (kind == EMB_PRESENCE) UF_SLAB(unsigned long long, EMB_PRESENCE);
+  if (a.row_scale != 0.0) {
+    if (kind == EMB_SCALED) UF_SLAB(unsigned long long, EMB_SCALED);
+    if (kind == EMB_PRESENCE) UF_SLAB(unsigned long long, EMB_PRESENCE);
+  }
+  if (kind == EMB_SCALED) UF_SLAB(double, EMB_SCALED);
+  if (kind == EMB_PRESENCE) UF_SLAB(double, EMB_PRESENCE);
   UF_SLAB(double, EMB_PROP);
 #undef UF_SLAB
 }
@@ -501,8 +508,12 @@ cudaError_t launch_emb_rows(int kind, bool fp32, int64_t b0, int rows,
     if (kind == EMB_PRESENCE) UF_EMB(float, EMB_PRESENCE);
     UF_EMB(float, EMB_PROP);
   }
-  if (kind == EMB_SCALED) UF_EMB(unsigned long long, EMB_SCALED);
-  if (kind == EMB_PRESENCE) UF_EMB(unsigned long long, EMB_PRESENCE);
+  if (row_scale != 0.0) {
+    if (kind == EMB_SCALED) UF_EMB(unsigned long long, EMB_SCALED);
+    if (kind == EMB_PRESENCE) UF_EMB(unsigned long long, EMB_PRESENCE);
+  }
+  if (kind == EMB_SCALED) UF_EMB(double, EMB_SCALED);
+  if (kind == EMB_PRESENCE) UF_EMB(double, EMB_PRESENCE);
   UF_EMB(double, EMB_PROP);
 #undef UF_EMB
 }

@@ -50,7 +50,7 @@ struct EmbedArgs {
   int64_t pitch;
   const TabDesc *tabs;
   int n_tabs;
-  double row_scale;             // 64-bit fixed-point rows (FP64, EMB_SCALED and EMB_PRESENCE)
+  double row_scale;             // != 0: 64-bit fixed-point rows (FP64, EMB_SCALED and EMB_PRESENCE)
   int4 *steps;                  // scratch of n_nodes records each, or both null (with xrow and
   double *steps_len;            // slot_of_node null: row and slot v for node v)
   int w, lv0, lv1, first;       // set by launch_embed: columns per CTA, levels of the launch, 1: level 0 too

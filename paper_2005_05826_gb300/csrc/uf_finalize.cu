@@ -6,7 +6,7 @@
 // sample k, partner j = (k + s + 1) mod n), with D the diagonal sums and the
 // cell holding M = sum min(x_k, x_j) (min form) or A = sum |x_k - x_j|
 // (abs form):
-// (FP64: its dense part as 2 R, R = sum max(x_j - x_k, 0), A = 2 R + D_k - D_j):
+// (FP64, fixed rows: its dense part as 2 R, R = sum max(x_j - x_k, 0), A = 2 R + D_k - D_j):
 //   weighted:    num = A  or  D_k + D_j - 2M,      den = D_k + D_j
 //   unweighted:  num = A  or  W_k + W_j - 2G,      den = (W_k + W_j + A) / 2  or  W_k + W_j - G
 //                (W = D, G = M on presence embeddings)

@@ -12,7 +12,7 @@ struct FinalArgs {
   int64_t s0, s1;       // stripes [s0, s1)
   int full;             // 1: condensed output, 0: stripe-major
   unsigned abs_mask;    // ACC_MIN: stripes s with abs_row(abs_mask, s) hold the abs form
-  int relu;             // ACC_MIN abs-form cells hold 2 sum max(x_j - x_k, 0) (FP64): A needs D_k - D_j
+  int relu;             // ACC_MIN abs-form cells hold 2 sum max(x_j - x_k, 0) (FP64, fixed rows): A needs D_k - D_j
   int gen_abs;          // generalized: M2 holds N = num (FP64) instead of Q (FP32)
   unsigned long long *clamps;  // or null: counts cells whose min-form numerator rounded below 0
   // FP64 calls: the second words of M / M2 and of Dg / Dsp sit this many

@@ -371,51 +371,92 @@ Plan::Dev &plan_dev(Plan *P, int device) {
 
 namespace {
 
+// One sample's tips, for uf_table::Sums.
+struct SampleSum {
+  double dist = 0.0, val_dist = 0.0, length = 0.0, depth = 0.0, low = INFINITY, top = 0.0;
+  void add(double val, const uf_tree::Tip &t) {
+    dist += t.dist;
+    val_dist += val * t.dist;
+    length += t.length;
+    depth += t.depth;
+    low = std::min(low, t.dist);
+    top = std::max(top, t.dist);
+  }
+  void add(const SampleSum &o) {
+    dist += o.dist;
+    val_dist += o.val_dist;
+    length += o.length;
+    depth += o.depth;
+    low = std::min(low, o.low);
+    top = std::max(top, o.top);
+  }
+  void close(double total, const uf_tree *tree, uf_table::Sums *m) const {
+    // D is a mean of the tips' distances: between the nearest's and the
+    // farthest's, which stand for it where its products leave FP64's range
+    const bool ok = total > 1e-200 && total < 1e200 && top < 1e100;
+    const double d = ok ? std::min(val_dist / total, top) : low, w = std::max(top, length);
+    const double b = std::sqrt(std::min(depth, (double)(tree->n_nodes - 1)));
+    m->presence = std::max(m->presence, dist);
+    m->weighted = std::max(m->weighted, ok ? d : top);
+    // (a sample whose branches are all of length 0 holds exact zeros)
+    if (top > 0.0) m->need_weighted = std::max(m->need_weighted, d > 0.0 ? b / d : INFINITY);
+    if (w > 0.0) m->need_presence = std::max(m->need_presence, b / w);
+  }
+};
+void most_of(const uf_table::Sums &a, uf_table::Sums *m) {
+  m->presence = std::max(m->presence, a.presence);
+  m->weighted = std::max(m->weighted, a.weighted);
+  m->need_weighted = std::max(m->need_weighted, a.need_weighted);
+  m->need_presence = std::max(m->need_presence, a.need_presence);
+}
+
+// The sums for a tree: made with the table, or here for another tree.
+uf_table::Sums table_sums(const uf_tree *tree, uf_table *table) {
+  std::lock_guard<std::mutex> g(table->mu);
+  auto it = table->sums.find(tree->id);
+  if (it == table->sums.end()) {
+    // per-sample sums over feature ranges of about equal entries, one per thread
+    const int T = (int)std::max<int64_t>(1, std::min<int64_t>(host_threads(), table->nnz / 200000));
+    std::vector<int64_t> f_lo(T + 1, table->n_features);
+    f_lo[0] = 0;
+    for (int c = 1, f = 0; c < T; c++) {
+      const int64_t want = table->nnz * c / T;
+      while (f < table->n_features && table->col_ptr[f] < want) f++;
+      f_lo[c] = f;
+    }
+    std::vector<std::vector<SampleSum>> part(T, std::vector<SampleSum>(table->n));
+    parallel_for(T, [&](int c) {
+      SampleSum *per = part[c].data();
+      for (int64_t f = f_lo[c]; f < f_lo[c + 1]; f++)
+        for (int64_t q = table->col_ptr[f]; q < table->col_ptr[f + 1]; q++)
+          per[table->col_row[q]].add(table->col_val[q], tree->tips[f]);
+    });
+    uf_table::Sums m;
+    for (int64_t k = 0; k < table->n; k++) {
+      for (int c = 1; c < T; c++) part[0][k].add(part[c][k]);
+      part[0][k].close(table->total[k], tree, &m);
+    }
+    it = table->sums.emplace(tree->id, m).first;
+  }
+  return it->second;
+}
+
 // Upper bound on every value an accumulator of this kind can reach:
-//   l * p embeddings:         D_k = sum_f p_f dist(f) <= max tip distance
+//   l * p embeddings:         D_k = sum_f p_f dist(f): FP64, the largest, its own
+//                             rounding added; FP32, the largest tip distance
 //   l * presence embeddings:  W_k <= min(total length, sum_{f in k} dist(f))
 //   generalized (den, Q):     den <= sum l s^alpha <= 2 (W_k + W_j)
 //   variance-adjusted (den, N): den <= w_max (D_k + D_j), with the weight
 //                             1 / sqrt(m_v (m - m_v)) <= w_max = max(1, 1 / c_min)
 //                             (both factors are sums of counts >= c_min, or 0)
-double accum_bound_of(uf_tree *tree, uf_table *table, int kind) {
-  if (kind == EMB_SCALED) return tree->max_tip_dist;
+// (FP64 sums go by what the table holds: one tip far off that no sample has
+// would coarsen the grid of them all)
+double accum_bound_of(uf_tree *tree, uf_table *table, int kind, bool fp32) {
+  if (kind == EMB_SCALED)
+    return fp32 ? tree->max_tip_dist
+                : std::min(tree->max_tip_dist, table_sums(tree, table).weighted * (1.0 + 1.0 / (1 << 20)));
   if (kind == EMB_VAW) return 2.0 * tree->max_tip_dist * std::max(1.0, 1.0 / table->min_count);
-  double pres;
-  {
-    std::lock_guard<std::mutex> g(table->mu);
-    auto it = table->presence_bound.find(tree->id);
-    if (it == table->presence_bound.end()) {
-      std::vector<int32_t> tip_node(tree->n_tips);
-      for (int64_t v = 0; v < tree->n_nodes; v++)
-        if (tree->tip_of_node[v] >= 0) tip_node[tree->tip_of_node[v]] = (int32_t)v;
-      // per-sample sums over feature ranges of about equal entries, one per thread
-      const int T = (int)std::max<int64_t>(1, std::min<int64_t>(host_threads(), table->nnz / 200000));
-      std::vector<int64_t> f_lo(T + 1, table->n_features);
-      f_lo[0] = 0;
-      for (int c = 1, f = 0; c < T; c++) {
-        const int64_t want = table->nnz * c / T;
-        while (f < table->n_features && table->col_ptr[f] < want) f++;
-        f_lo[c] = f;
-      }
-      std::vector<std::vector<double>> part(T, std::vector<double>(table->n, 0.0));
-      parallel_for(T, [&](int c) {
-        double *per = part[c].data();
-        for (int64_t f = f_lo[c]; f < f_lo[c + 1]; f++) {
-          const double d = tree->dist[tip_node[f]];
-          for (int64_t q = table->col_ptr[f]; q < table->col_ptr[f + 1]; q++) per[table->col_row[q]] += d;
-        }
-      });
-      double mx = 0.0;
-      for (int64_t k = 0; k < table->n; k++) {
-        double x = 0.0;
-        for (int c = 0; c < T; c++) x += part[c][k];
-        mx = std::max(mx, x);
-      }
-      it = table->presence_bound.emplace(tree->id, mx).first;
-    }
-    pres = std::min(tree->total_length, it->second);
-  }
+  const double pres = std::min(tree->total_length, table_sums(tree, table).presence);
   return kind == EMB_PRESENCE ? pres : 4.0 * pres;
 }
 
@@ -441,13 +482,22 @@ uf_status check_args(const uf_tree *tree, const uf_table *table, uf_method metho
 }  // namespace
 
 namespace ufg {
-double accum_bound(const uf_tree *tree, const uf_table *table, int kind) {
-  return accum_bound_of(const_cast<uf_tree *>(tree), const_cast<uf_table *>(table), kind);
+double accum_bound(const uf_tree *tree, const uf_table *table, int kind, bool fp32) {
+  return accum_bound_of(const_cast<uf_tree *>(tree), const_cast<uf_table *>(table), kind, fp32);
+}
+
+double grid_need(const uf_tree *tree, const uf_table *table, int kind) {
+  const uf_table::Sums s = table_sums(tree, const_cast<uf_table *>(table));
+  return kind == EMB_SCALED ? s.need_weighted : s.need_presence;
+}
+
+bool grid_fits(const uf_tree *tree, double need, int g) {
+  return need <= std::ldexp(1.0, g - 52) && std::isfinite(std::ldexp(tree->max_length, g));
 }
 
 // Fixed-point scale 2^F of the accumulators: 2 * bound * 2^F <= 2^61.
-double accum_scale(const uf_tree *tree, const uf_table *table, int kind) {
-  const double B = accum_bound(tree, table, kind);
+double accum_scale(const uf_tree *tree, const uf_table *table, int kind, bool fp32) {
+  const double B = accum_bound(tree, table, kind, fp32);
   int F = 100;
   if (B > 0.0 && std::isfinite(B)) F = std::min(100, std::max(0, 60 - (int)std::ceil(std::log2(B))));
   return std::ldexp(1.0, F);
@@ -643,15 +693,18 @@ uf_status uf_tree_create(int64_t n_nodes, const int64_t *parent, const double *l
     // one pass in reverse order (parents first): root distances, the tips'
     // distances, and the tip ranges that are not contiguous (both set to -1)
     t->dist.assign(n_nodes, 0.0);
-    t->tip_dist.resize(std::max<int32_t>(tips, 1));
+    std::vector<int32_t> depth(n_nodes, 0);
+    t->tips.resize(std::max<int32_t>(tips, 1));
     for (int64_t v = n_nodes - 1; v >= 0; v--) {
       if (v + 1 < n_nodes) {
         t->dist[v] = t->length[v] + t->dist[parent[v]];
+        depth[v] = depth[parent[v]] + 1;
         t->total_length += t->length[v];
+        t->max_length = std::max(t->max_length, t->length[v]);
       }
       if (t->tip_of_node[v] >= 0) {
         t->max_tip_dist = std::max(t->max_tip_dist, t->dist[v]);
-        t->tip_dist[t->tip_of_node[v]] = t->dist[v];
+        t->tips[t->tip_of_node[v]] = {t->dist[v], v + 1 < n_nodes ? t->length[v] : 0.0, (double)depth[v]};
       }
       if ((int64_t)t->tip_hi[v] - t->tip_lo[v] != under[v]) t->tip_lo[v] = t->tip_hi[v] = -1;
     }
@@ -708,15 +761,15 @@ uf_status uf_table_create(int64_t n_samples, int64_t n_features, const int64_t *
     std::vector<int64_t> bad_k(T, -1);
     std::vector<std::string> bad_msg(T);
     std::vector<std::vector<int64_t>> cnt(T);
-    // and the presence bound for this tree: max over samples of the summed
-    // root distances of their tips (accum_bound)
-    std::vector<double> pres(T, 0.0);
+    // and what this tree's branches sum to below the samples (accum_bound, grid_need)
+    std::vector<uf_table::Sums> sums(T);
     std::vector<double> cmin(T, INFINITY);  // the smallest count (variance-adjusted bound)
-    const double *tip_dist = tree->tip_dist.data();
+    const uf_tree::Tip *tips = tree->tips.data();
     parallel_for(T, [&](int c) {
       char buf[160];
       for (int64_t k = k_lo[c]; k < k_lo[c + 1]; k++) {
-        double s = 0.0, w = 0.0;
+        double s = 0.0;
+        SampleSum w;
         for (int64_t q = indptr[k]; q < indptr[k + 1]; q++) {
           if (indices[q] < 0 || indices[q] >= n_features)
             snprintf(buf, sizeof buf, "sample %lld: feature index %d out of range", (long long)k, indices[q]);
@@ -726,7 +779,7 @@ uf_status uf_table_create(int64_t n_samples, int64_t n_features, const int64_t *
             snprintf(buf, sizeof buf, "sample %lld: count %g must be finite and > 0", (long long)k, data[q]);
           else {
             s += data[q];
-            w += tip_dist[indices[q]];
+            w.add(data[q], tips[indices[q]]);
             cmin[c] = std::min(cmin[c], data[q]);
             continue;
           }
@@ -736,13 +789,14 @@ uf_status uf_table_create(int64_t n_samples, int64_t n_features, const int64_t *
         }
         t->total[k] = s;
         t->inv_total_f[k] = (float)(1.0 / s);
-        pres[c] = std::max(pres[c], w);
+        w.close(s, tree, &sums[c]);
       }
     });
     for (int c = 0; c < T; c++)
       if (bad_k[c] >= 0) return fail(UF_ETABLE, "%s", bad_msg[c].c_str());
     t->id = next_id++;
-    t->presence_bound[tree->id] = *std::max_element(pres.begin(), pres.end());
+    for (int c = 1; c < T; c++) most_of(sums[c], &sums[0]);
+    t->sums[tree->id] = sums[0];
     t->min_count = *std::min_element(cmin.begin(), cmin.end());
     // each thread's column counts (a counting sort) and, below, its scatter
     // run over feature blocks: a sample's entries are sorted by feature, so

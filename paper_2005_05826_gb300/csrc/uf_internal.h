@@ -66,16 +66,16 @@ struct TabDesc {
 // A stripe s whose bit (s mod 8) is set in the call's abs mask holds
 // A = sum |x_k - x_j| (abs form) instead of M = sum min(x_k, x_j) (min form).
 // FP32: stripes 1, 3, 5, 7 of every 8, so that the ALU and FMA pipes share
-// the load (see uf_stripe.cu).  FP64: every stripe; its rows are 64-bit fixed
-// point and a cell holds 2 R, R = sum max(x_j - x_k, 0), so that
-// A = 2 R + D_k - D_j in exact integers (k_stripe_u64; FinalArgs::relu).
+// the load (see uf_stripe.cu).  FP64: every stripe; where its rows are 64-bit
+// fixed point (StripeArgs::fixed) a cell holds 2 R, R = sum max(x_j - x_k, 0),
+// so that A = 2 R + D_k - D_j in exact integers (k_stripe_u64; FinalArgs::relu).
 constexpr unsigned FP32_ABS_ROW_MASK = 0xAAu;
 constexpr unsigned FP64_ABS_ROW_MASK = 0xFFu;
 __host__ __device__ constexpr unsigned abs_row_mask(bool fp32) { return fp32 ? FP32_ABS_ROW_MASK : FP64_ABS_ROW_MASK; }
 __host__ __device__ constexpr bool abs_row(unsigned mask, int64_t s) { return (mask >> (s & 7)) & 1u; }
 
 struct StripeArgs {
-  const void *X;        // [rows][pitch] float, double or (FP64 ACC_MIN) 64-bit fixed point,
+  const void *X;        // [rows][pitch] float, double or (`fixed`) 64-bit fixed point,
                         // one segment per table
   const double *len;    // per-row branch length (generalized only), [rows]
   int rows;             // branches in this launch
@@ -96,9 +96,10 @@ struct StripeArgs {
   // this many elements after its first word (M and M2 cells; Dg); the FP32
   // kernels keep one word
   int64_t m_lo_off, d_lo_off;
-  // FP64 ACC_MIN: the rows of X are x * 2^(F + x_shift), 0 <= x_shift <= 32,
-  // with every column's sum over a work unit's rows below 2^63
-  int x_shift;
+  // FP64 ACC_MIN: 1: the rows of X are 64-bit integers x * 2^(F + x_shift),
+  // 0 <= x_shift <= 32, with every column's sum over a work unit's rows below
+  // 2^63; 0: FP64 values
+  int fixed, x_shift;
   // FP32 min kernel: 0xFF runs every stripe in the abs form (methods whose
   // numerator must not come from a difference of sums); anything else the
   // default FP32_ABS_ROW_MASK
@@ -112,6 +113,7 @@ void stripe_tile_shape(int acc, bool fp32, int *tile_s, int *tile_k, int shape =
 int stripe_shapes(int acc, bool fp32, unsigned abs_mask);
 // the shape of small tiles
 int stripe_small_shape(int acc, bool fp32);
+// (fixed: the FP64 ACC_MIN rows are 64-bit fixed point, StripeArgs::fixed)
 // Tile shape and rows per unit for problems that do not fill it: the small
 // tiles where the shape's own pad their tables' stripes and samples out to
 // more work, and units of fewer than `chunk` rows (split) until there are four
@@ -122,16 +124,15 @@ struct SmallPlan {
   int shape, chunk;
   bool split;
 };
-SmallPlan stripe_small_plan(int acc, bool fp32, const int *n, size_t n_tabs, int rows, int chunk,
+SmallPlan stripe_small_plan(int acc, bool fp32, bool fixed, const int *n, size_t n_tabs, int rows, int chunk,
                             int shape, bool shape_free, int sms);
 // default rows per work unit
 int stripe_chunk_rows();
 cudaError_t launch_stripe_acc(int acc, bool fp32, const StripeArgs &a, cudaStream_t st);
-// D[k] += sum of the launch's rows at column k (ACC_MIN only): FP32 with the
-// stripe kernel's operation order, in scratch of diag_scratch_bytes(); FP64
-// rows are integers,
-// summed in any order
-size_t diag_scratch_bytes(bool fp32, int rows, int n_cols);
+// D[k] += sum of the launch's rows at column k (ACC_MIN only): with the
+// stripe kernel's operation order, in scratch of diag_scratch_bytes(); fixed
+// rows are integers, summed in any order
+size_t diag_scratch_bytes(bool fp32, bool fixed, int rows, int n_cols);
 cudaError_t launch_diag(bool fp32, const StripeArgs &a, void *scratch, cudaStream_t st);
 
 }  // namespace ufg
@@ -160,8 +161,19 @@ bool table_host_view(const ::uf_table *t, TableView *v);
 namespace ufg {
 // Upper bound of every accumulated value of an embedding kind, and the
 // fixed-point scale 2^F it gives (uf_host.cpp).
-double accum_bound(const ::uf_tree *tree, const ::uf_table *table, int kind);
-double accum_scale(const ::uf_tree *tree, const ::uf_table *table, int kind);
+double accum_bound(const ::uf_tree *tree, const ::uf_table *table, int kind, bool fp32);
+double accum_scale(const ::uf_tree *tree, const ::uf_table *table, int kind, bool fp32);
+// Whether FP64 values of an embedding kind (EMB_SCALED or EMB_PRESENCE) may be
+// rounded to the grid 2^-g for a table: with need = grid_need() of the table(s).
+// A distance rests on the branches below either sample, b_i + b_j of them at
+// most, each value off by at most half a grid step, so by about
+// sqrt(b_i + b_j) <= sqrt(b_i) + sqrt(b_j) steps in all; and it is measured
+// against D_i + D_j (W_i, W_j: presence).  With need = max_k sqrt(b_k) / D_k that
+// is need * step of it, and the line at 2^-52 keeps the worst of millions of pairs
+// (5 of their 0.3 need * step deviations) below 4e-16, inside the 1e-15 that the
+// FP64 distances are held to.  No length may overflow on the grid.
+bool grid_fits(const ::uf_tree *tree, double need, int g);
+double grid_need(const ::uf_tree *tree, const ::uf_table *table, int kind);
 // Largest StripeArgs::x_shift for FP64 ACC_MIN rows: the sum of any column
 // over the rows of one work unit is at most the accumulator's bound and at
 // most the unit's summed branch lengths (n lengths len[], units of `chunk`

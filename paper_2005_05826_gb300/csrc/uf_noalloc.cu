@@ -121,14 +121,20 @@ uf_status compute_noalloc(const uf_tree *tree, const uf_table *table, uf_method 
   const bool usable = e == cudaSuccess && device >= 0 && device < UF_NOALLOC_MAX_DEVICES &&
                       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) == cudaSuccess;
   const unsigned amask = acc == ACC_MIN ? abs_row_mask(fp32) : 0u;
-  const SmallPlan plan = stripe_small_plan(acc, fp32, &n, 1, (int)std::max<int64_t>(tv.n_nodes - 1, 1),
+  const double scale = accum_scale(tree, table, kind, fp32);
+  // FP64 min kernel: 64-bit fixed-point rows where every distance keeps its
+  // accuracy on their grid (StripeArgs::fixed, x_shift; as in run_batch)
+  const double most = accum_bound(tree, table, kind, fp32);
+  const bool fixed_rows =
+      !fp32 && acc == ACC_MIN &&
+      grid_fits(tree, grid_need(tree, table, kind), std::ilogb(scale) + fixed_row_shift(scale, most, &most, 1, 1));
+  const SmallPlan plan = stripe_small_plan(acc, fp32, fixed_rows, &n, 1, (int)std::max<int64_t>(tv.n_nodes - 1, 1),
                                            stripe_chunk_rows(), 0, true, sms);
   int tile_s = 0, tile_k = 0;
   stripe_tile_shape(acc, fp32, &tile_s, &tile_k, plan.shape);
   const int m_hi = (int)((S - 1) / tile_s);
   const int64_t pitch = round_up(round_up(n, tile_k) + (int64_t)(m_hi + 1) * tile_s, 32);
   const int64_t N = tv.n_nodes, nb = N - 1;
-  const double scale = accum_scale(tree, table, kind);
 
   // one branch block holding every branch; slot and row of node v = v
   std::vector<int32_t> level(N, 0), lists, level_at;
@@ -175,7 +181,7 @@ uf_status compute_noalloc(const uf_tree *tree, const uf_table *table, uf_method 
     p[13] = c.take<unsigned long long>((size_t)S * n * words);  // stripe accumulator
     p[14] = acc == ACC_GEN ? (void *)c.take<unsigned long long>((size_t)S * n * words) : nullptr;  // Q or N
     p[15] = acc == ACC_MIN ? (void *)c.take<unsigned long long>((size_t)n * words) : nullptr;      // diagonal
-    p[16] = acc == ACC_MIN ? (void *)c.take<unsigned char>(diag_scratch_bytes(fp32, std::max(rows, 1), n))
+    p[16] = acc == ACC_MIN ? (void *)c.take<unsigned char>(diag_scratch_bytes(fp32, fixed_rows, std::max(rows, 1), n))
                            : nullptr;                                        // diagonal partials
     p[17] = c.take<int>(1);                                                  // work-unit counter
     p[18] = c.take<TabDesc>(1);                                              // the table's description
@@ -246,10 +252,7 @@ uf_status compute_noalloc(const uf_tree *tree, const uf_table *table, uf_method 
   if (p[14]) UF_TRY(cudaMemsetAsync(p[14], 0, (size_t)S * n * 8 * words, st));
   if (p[15]) UF_TRY(cudaMemsetAsync(p[15], 0, (size_t)n * 8 * words, st));
 
-  // FP64 min kernel: 64-bit fixed-point rows (StripeArgs::x_shift)
-  const bool fixed_rows = !fp32 && acc == ACC_MIN;
-  const int x_shift =
-      fixed_rows ? fixed_row_shift(scale, accum_bound(tree, table, kind), tv.length, nb, plan.chunk) : 0;
+  const int x_shift = fixed_rows ? fixed_row_shift(scale, most, tv.length, nb, plan.chunk) : 0;
 
   const int32_t *d_lists = (const int32_t *)p[5];
   if (rows > 0) {
@@ -300,6 +303,7 @@ uf_status compute_noalloc(const uf_tree *tree, const uf_table *table, uf_method 
     sa.counter = (int *)p[17];
     sa.m_lo_off = fp32 ? 0 : (int64_t)S * n;
     sa.d_lo_off = fp32 ? 0 : n;
+    sa.fixed = fixed_rows;
     sa.x_shift = x_shift;
     UF_TRY(launch_stripe_acc(acc, fp32, sa, st));
     if (acc == ACC_MIN) UF_TRY(launch_diag(fp32, sa, p[16], st));

@@ -869,6 +869,17 @@ int64_t stripe_cells(const BatchJob &J) {
   return c;
 }
 
+// Grid 2^-g of the digits of branch lengths up to `most`: the longest that a
+// sample has below 2^62 on it, no finer than the second words' 2^-(F+32).
+int digit_grid(const uf_tree *tree, const BatchJob &J, double most, double scale) {
+  double bound = 0.0;
+  // (a branch longer than the accumulators' bound is in no sample)
+  for (const TableJob &t : J.tabs) bound = std::max(bound, accum_bound(tree, t.table, EMB_PRESENCE, false));
+  most = std::min(most, bound);
+  const int f = std::ilogb(scale) + 32;
+  return most > 0.0 ? std::min(f, 61 - std::ilogb(most)) : f;  // most < 2^(ilogb + 1)
+}
+
 // Unweighted on the tensor cores (mixed: three BF16 terms per length; FP64:
 // seven exact digits and two-word sums): per branch block, counts
 // -> presence / split-length planes of every table -> tcgen05 gram into the
@@ -900,7 +911,7 @@ uf_status run_gram(uf_tree *tree, const BatchJob &J, int device, double scale) {
   }();
   const std::shared_ptr<const RowSplit> split_p = [&] {
     NvtxRange r("uf: branch split");
-    return get_split(tree, J, in.P, SPLIT_GRAM, J.fp32);
+    return get_split(tree, J, in.P, SPLIT_GRAM, J.fp32, false);
   }();
   const RowSplit &split = *split_p;
   const int64_t K_pad = gram_kpad((int)std::max<int64_t>(split.max_dense, 1));
@@ -942,19 +953,13 @@ uf_status run_gram(uf_tree *tree, const BatchJob &J, int device, double scale) {
     Msp = DevBuf((size_t)cells * 8 * acc_words, st, "alloc sparse stripes");
     ck(cudaMemsetAsync(Msp.p, 0, (size_t)cells * 8 * acc_words, st), "memset");
   }
-  // digits: the lengths' grid 2^-g, the longest dense one below 2^62 on it,
-  // no finer than the second words' 2^-(F+32)
   int digit_shift = 0;
   double digit_scale = 0.0;
   if (digits) {
-    double most = 0.0, bound = 0.0;
+    double most = 0.0;
     for (double l : split.dense_len) most = std::max(most, l);
-    // (a branch longer than the accumulators' bound is in no sample)
-    for (const TableJob &t : J.tabs) bound = std::max(bound, accum_bound(tree, t.table, EMB_PRESENCE));
-    most = std::min(most, bound);
-    const int f = std::ilogb(scale) + 32;
-    const int g = most > 0.0 ? std::min(f, 61 - std::ilogb(most)) : f;  // most < 2^(ilogb + 1)
-    digit_shift = f - g;
+    const int g = digit_grid(tree, J, most, scale);
+    digit_shift = std::ilogb(scale) + 32 - g;
     digit_scale = std::ldexp(1.0, g);
   }
   meta.upload(st);
@@ -1125,9 +1130,10 @@ uf_status run_gram(uf_tree *tree, const BatchJob &J, int device, double scale) {
   return UF_OK;
 }
 
-// Every other method / precision on the CUDA-core stripe kernels.  Throws
-// CudaFail on CUDA errors.
-uf_status run_stripes(uf_tree *tree, const BatchJob &J, int device, uf_method method, double scale) {
+// Every other method / precision on the CUDA-core stripe kernels; fixed_rows:
+// the FP64 min kernels' rows are 64-bit fixed point.  Throws CudaFail on CUDA
+// errors.
+uf_status run_stripes(uf_tree *tree, const BatchJob &J, int device, uf_method method, double scale, bool fixed_rows) {
   const auto t_start = std::chrono::steady_clock::now();
   const size_t nt = J.tabs.size();
   const int acc = acc_of(method), kind = kind_of(method);
@@ -1203,7 +1209,7 @@ uf_status run_stripes(uf_tree *tree, const BatchJob &J, int device, uf_method me
   cudaStream_t st = J.st;
   const std::shared_ptr<const RowSplit> split_p = [&] {
     NvtxRange r("uf: branch split");
-    return get_split(tree, J, in.P, acc, fp32);
+    return get_split(tree, J, in.P, acc, fp32, fixed_rows);
   }();
   const RowSplit &split = *split_p;
   const int64_t xrows = std::max<int64_t>(split.max_dense, 1);
@@ -1252,7 +1258,7 @@ uf_status run_stripes(uf_tree *tree, const BatchJob &J, int device, uf_method me
   std::vector<SpLayout> lay(nt);
   for (size_t t = 0; t < nt; t++) lay[t] = SpLayout{tabs[t].n, tabs[t].off, tabs[t].s_lo, tabs[t].s_hi, tabs[t].m_off};
   SparseScatter sc;
-  sc.prepare(tree, J, in, split, lay, acc, !fp32, !fp32, cells, n_cols, tile_scatter(J, acc, fp32), kind == EMB_PRESENCE,
+  sc.prepare(tree, J, in, split, lay, acc, !fp32, !fp32, cells, n_cols, tile_scatter(J, acc, fixed_rows), kind == EMB_PRESENCE,
              meta, st);
   meta.upload(st);
   const TabDesc *d_tabs = meta.at<TabDesc>(o_tabs);
@@ -1272,7 +1278,7 @@ uf_status run_stripes(uf_tree *tree, const BatchJob &J, int device, uf_method me
     ck(cudaMemsetAsync(M2.p, 0, m_bytes, st), "memset");
   } else {
     Dg = DevBuf(d_bytes, st, "alloc diagonal");
-    diag_tmp = DevBuf(diag_scratch_bytes(fp32, (int)xrows, n_cols), st, "alloc diagonal scratch");
+    diag_tmp = DevBuf(diag_scratch_bytes(fp32, fixed_rows, (int)xrows, n_cols), st, "alloc diagonal scratch");
     ck(cudaMemsetAsync(Dg.p, 0, d_bytes, st), "memset");
   }
   ck(cudaMemsetAsync(M.p, 0, m_bytes, st), "memset");
@@ -1290,15 +1296,14 @@ uf_status run_stripes(uf_tree *tree, const BatchJob &J, int device, uf_method me
   const auto key = tune_key(acc, (fp32 ? (amask == 0xFFu ? 2 : 1) : 0) + 4 * (forced + 1), n_tiles, xrows);
   int chunk = stripe_chunk_rows(), shape = forced > 0 ? forced : 0;
   bool tune = false;
-  // (the FP64 min kernel's sums are exact for any chunk: not tuned)
-  const bool fixed_rows = !fp32 && acc == ACC_MIN;
+  // (fixed rows' sums are exact for any chunk: not tuned)
   // problems too small to fill the GPU: the rule's shape and shorter units, nothing tuned
   int sms = 0;
   ck(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device), "cudaDeviceGetAttribute");
   std::vector<int> ns(nt);
   for (size_t t = 0; t < nt; t++) ns[t] = tabs[t].n;
   auto small_plan = [&](bool shape_free) {
-    return stripe_small_plan(acc, fp32, ns.data(), nt, (int)xrows, chunk, shape, shape_free, sms);
+    return stripe_small_plan(acc, fp32, fixed_rows, ns.data(), nt, (int)xrows, chunk, shape, shape_free, sms);
   };
   const SmallPlan small = small_plan(forced < 0);
   if (g_autotune.load() && !split.dense.empty() && !fixed_rows && !small.split && small.shape != small_shape) {
@@ -1324,9 +1329,9 @@ uf_status run_stripes(uf_tree *tree, const BatchJob &J, int device, uf_method me
   // so that every SM has units (tuned chunks are found with enough of them)
   int unit_rows = small.split && !tune ? small_plan(false).chunk : chunk;
   double acc_most = 0.0;  // bound of the accumulators
-  int x_shift = 0;  // grid of the FP64 min kernel's rows (StripeArgs::x_shift)
+  int x_shift = 0;  // grid of the fixed rows (StripeArgs::x_shift)
   if (fixed_rows) {
-    for (const TableJob &t : J.tabs) acc_most = std::max(acc_most, accum_bound(tree, t.table, kind));
+    for (const TableJob &t : J.tabs) acc_most = std::max(acc_most, accum_bound(tree, t.table, kind, false));
     x_shift = 32;
     for (size_t b = 0; b + 1 < split.dense_ptr.size(); b++)
       x_shift = std::min(x_shift, fixed_row_shift(scale, acc_most, split.dense_len.data() + split.dense_ptr[b],
@@ -1433,6 +1438,7 @@ uf_status run_stripes(uf_tree *tree, const BatchJob &J, int device, uf_method me
     sa.m_lo_off = fp32 ? 0 : cells;
     sa.d_lo_off = fp32 ? 0 : n_cols;
     sa.abs_mask = amask;
+    sa.fixed = fixed_rows;
     sa.x_shift = x_shift;
     if (tune && !tuned) {
       std::vector<const TabDesc *> tp;
@@ -1464,7 +1470,7 @@ uf_status run_stripes(uf_tree *tree, const BatchJob &J, int device, uf_method me
       timer.begin(2);
       ck(launch_diag(fp32, sa, diag_tmp.p, ls), "diagonal accumulate");
       timer.end();
-      kernels += fp32 ? 2 : 1;
+      kernels += fixed_rows ? 1 : 2;
     }
   }
   if (split.n_sparse > 0 && !side.ev_fork) {  // not launched beside a dense block
@@ -1570,9 +1576,17 @@ uf_status run_batch(uf_tree *tree, const BatchJob &J) {
   const int kind = kind_of(method);
   double scale = 0.0;  // one fixed-point scale valid for every table of the call
   for (const TableJob &t : J.tabs) {
-    const double s = accum_scale(tree, t.table, kind);
+    const double s = accum_scale(tree, t.table, kind, J.fp32);
     scale = scale == 0.0 ? s : std::min(scale, s);
   }
+  // FP64 min methods run on integers of one grid (digits of the lengths, 64-bit
+  // rows) where every distance keeps its accuracy on it; samples whose branches
+  // are far shorter than others' take FP64 rows (3.6e12 against 2.6e11 updates/s).
+  // Decided from the coarsest grid the call can get, before its branch split.
+  const bool min64 = !J.fp32 && acc_of(method) == ACC_MIN;
+  double need_grid = 0.0;
+  if (min64)
+    for (const TableJob &t : J.tabs) need_grid = std::max(need_grid, grid_need(tree, t.table, kind));
   // (the unweighted numerator alone stays on the CUDA-core kernels: the gram
   // gives it as W_i + W_j - 2G, rounded relative to W rather than to itself)
   if (method == UF_UNWEIGHTED && g_tensor_path.load()) {
@@ -1582,9 +1596,17 @@ uf_status run_batch(uf_tree *tree, const BatchJob &J) {
     const GramPlan G = gram_plan(J);
     const double need =
         ((double)G.n_tiles * GRAM_TILE_CELLS + (double)stripe_cells(J)) * 8.0 * (J.fp32 ? 1 : 2);
-    if (need <= 0.5 * available_bytes()) return run_gram(tree, J, device, scale);
+    if (need <= 0.5 * available_bytes() &&
+        (J.fp32 || grid_fits(tree, need_grid, digit_grid(tree, J, tree->max_length, scale))))
+      return run_gram(tree, J, device, scale);
   }
-  return run_stripes(tree, J, device, method, scale);
+  bool fixed = false;
+  if (min64) {
+    double most = 0.0;
+    for (const TableJob &t : J.tabs) most = std::max(most, accum_bound(tree, t.table, kind, false));
+    fixed = grid_fits(tree, need_grid, std::ilogb(scale) + fixed_row_shift(scale, most, &most, 1, 1));
+  }
+  return run_stripes(tree, J, device, method, scale, fixed);
 }
 
 void forget_tuned_chunks() {

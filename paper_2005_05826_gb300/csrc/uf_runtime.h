@@ -156,7 +156,7 @@ struct Plan {
 };
 
 struct RowSplit;
-// (table ids, accumulator, FP32, sparse mode, block rows, region budget)
+// (table ids, accumulator, row type, sparse mode, block rows, region budget)
 using SplitKey = std::tuple<std::vector<uint64_t>, int, int, int, int64_t, int64_t>;
 
 }  // namespace rt
@@ -184,8 +184,12 @@ struct uf_tree {
   std::map<ufg::rt::SplitKey, std::shared_ptr<const ufg::rt::RowSplit>> splits;  // dense / sparse branch splits
   // root distance of every node (root: 0), max over tips, total branch length
   std::vector<double> dist;
-  std::vector<double> tip_dist;  // dist of tip number f
-  double max_tip_dist = 0.0, total_length = 0.0;
+  struct Tip {
+    double dist, length;  // from the root, and of its own branch
+    double depth;         // branches from the root
+  };
+  std::vector<Tip> tips;  // by tip number
+  double max_tip_dist = 0.0, total_length = 0.0, max_length = 0.0;
   ~uf_tree() {
     int cur = 0;
     cudaGetDevice(&cur);
@@ -211,7 +215,15 @@ struct uf_table {
   std::vector<int32_t, ufg::rt::NoInit<int32_t>> col_row;
   std::vector<double, ufg::rt::NoInit<double>> col_val;
   std::mutex mu;
-  std::map<uint64_t, double> presence_bound;  // by tree id: max_k sum_{f in k} dist(tip f)
+  // What a tree's branches sum to below the samples, by tree id (uf_host.cpp)
+  struct Sums {
+    double presence = 0.0;       // max_k sum_{f in k} dist(tip f)
+    double weighted = 0.0;       // max_k D_k, D_k = sum_f p_kf dist(tip f)
+    // max_k sqrt(branches below sample k) / D_k and the same over W_k, its
+    // branches' summed lengths, from below (grid_need)
+    double need_weighted = 0.0, need_presence = 0.0;
+  };
+  std::map<uint64_t, Sums> sums;
   double min_count = 1.0;                     // the smallest count of the table
   struct Dev {
     char *base = nullptr;  // one allocation holding the arrays below
@@ -333,15 +345,17 @@ constexpr int64_t LIST_MIN_SAMPLES = 512;
 constexpr int SPLIT_GRAM = 2;
 double sparse_regions(size_t n_tables, int acc, double acc_bytes);
 // Whether a call's scatter runs in shared-memory tiles (uf_sparse.cu): FP64
-// weighted methods (rows on the dense kernel's 64-bit grid) on one table of
+// weighted methods with `fixed` rows (the dense kernel's 64-bit grid) on one table of
 // TILE_MIN_SAMPLES (fewer make too few tiles) to TILE_MAX_SAMPLES (more leave
 // few of a row's samples in a tile) samples
 constexpr int64_t TILE_MIN_SAMPLES = 512, TILE_MAX_SAMPLES = 4096;
-bool tile_scatter(const BatchJob &J, int acc, bool fp32);
+bool tile_scatter(const BatchJob &J, int acc, bool fixed);
 
 
-// The split of a call, cached on the tree (uf_split.cpp).
-std::shared_ptr<const RowSplit> get_split(uf_tree *tree, const BatchJob &J, const Plan *P, int acc, bool fp32);
+// The split of a call, cached on the tree (uf_split.cpp); fixed: its FP64 rows
+// are 64-bit fixed point (StripeArgs::fixed).
+std::shared_ptr<const RowSplit> get_split(uf_tree *tree, const BatchJob &J, const Plan *P, int acc, bool fp32,
+                                          bool fixed);
 
 // Runs one compute call on the current device (uf_run.cpp); throws CudaFail.
 uf_status run_batch(uf_tree *tree, const BatchJob &J);

@@ -13,8 +13,8 @@ double sparse_regions(size_t n_tables, int acc, double acc_bytes) {
   return std::ceil(acc_bytes / budget);
 }
 
-bool tile_scatter(const BatchJob &J, int acc, bool fp32) {
-  if (J.tabs.size() != 1 || fp32 || acc != ACC_MIN || kind_of(J.method) != EMB_SCALED) return false;
+bool tile_scatter(const BatchJob &J, int acc, bool fixed) {
+  if (J.tabs.size() != 1 || !fixed || acc != ACC_MIN || kind_of(J.method) != EMB_SCALED) return false;
   const int64_t n = J.tabs[0].table->n;
   return n >= TILE_MIN_SAMPLES && n <= TILE_MAX_SAMPLES;
 }
@@ -30,7 +30,7 @@ namespace {
 // scatters every branch that fits; mode 0 none.  The choice depends on the
 // tree and the tables only, not on the stripe range, so that a range run
 // gives bitwise the stripes of the full run.
-RowSplit split_rows(const uf_tree *tree, const BatchJob &J, const Plan *P, int acc, bool fp32) {
+RowSplit split_rows(const uf_tree *tree, const BatchJob &J, const Plan *P, int acc, bool fp32, bool fixed) {
   RowSplit R;
   // the variance-adjusted method has no pair-scatter form: every branch dense
   const int mode = acc == ACC_VAW ? 0 : (int)g_sparse.load();
@@ -53,7 +53,7 @@ RowSplit split_rows(const uf_tree *tree, const BatchJob &J, const Plan *P, int a
     }
     // accumulators beyond L2: one table scatters region by region in L2
     // (sparse_regions), several tables scatter straight into HBM-resident cells
-    const bool tiles = tile_scatter(J, acc, fp32);
+    const bool tiles = tile_scatter(J, acc, fixed);
     const bool regions = !tiles && sparse_regions(nt, acc, cells * 8.0 * n_acc) > 1;
     // FP32 terms of one table go through lists even when its accumulators fit
     // in L2: a fused list's pair is one atomic (generalized: two) for three
@@ -71,7 +71,7 @@ RowSplit split_rows(const uf_tree *tree, const BatchJob &J, const Plan *P, int a
     const double n_regions = regions ? sparse_regions(nt, acc, cells * 8.0 * n_acc) : 1.0;
     double dense_rate;  // cell updates per second of the dense kernel
     if (acc == SPLIT_GRAM) dense_rate = fp32 ? 2.5e14 : 2.5e14 * GRAM_SPLITS / GRAM_DIGITS;
-    else dense_rate = fp32 ? (acc == ACC_GEN ? 4e12 : 1.3e13) : (acc == ACC_GEN ? 5e10 : 3.5e12);
+    else dense_rate = fp32 ? (acc == ACC_GEN ? 4e12 : 1.3e13) : (acc == ACC_GEN ? 5e10 : fixed ? 3.5e12 : 2e11);
     const double visit_rate = fp32 ? 2e12 : (acc == ACC_GEN ? 3e10 : 1e12);
     const double job_cost = 5e-10;
     // region lists are fused (a listed branch carries its sparse children,
@@ -217,7 +217,7 @@ RowSplit split_rows(const uf_tree *tree, const BatchJob &J, const Plan *P, int a
   };
   // the lists of the scattered branches (a table's tiles make their own), of
   // the count rows and of the dense rows side by side: none needs another
-  const bool lists = R.lists && R.n_sparse > 0 && !tile_scatter(J, acc, fp32);
+  const bool lists = R.lists && R.n_sparse > 0 && !tile_scatter(J, acc, fixed);
   auto part = [&](int c) {
     if (c == 0 && lists) region_lists(tree, J.tabs[0].table, R);
     if (c == 1) count_rows();
@@ -345,11 +345,12 @@ const RegionLists &region_lists(const uf_tree *tree, const uf_table *table, cons
 
 // The split of a call, cached on the tree by its tables and kind (tables are
 // immutable and their ids are never reused).
-std::shared_ptr<const RowSplit> get_split(uf_tree *tree, const BatchJob &J, const Plan *P, int acc, bool fp32) {
+std::shared_ptr<const RowSplit> get_split(uf_tree *tree, const BatchJob &J, const Plan *P, int acc, bool fp32,
+                                          bool fixed) {
   SplitKey key;
   for (const TableJob &t : J.tabs) std::get<0>(key).push_back(t.table->id);
-  std::get<1>(key) = acc + (tile_scatter(J, acc, fp32) ? 16 : 0);
-  std::get<2>(key) = fp32 ? 1 : 0;
+  std::get<1>(key) = acc + (tile_scatter(J, acc, fixed) ? 16 : 0);
+  std::get<2>(key) = fp32 ? 1 : fixed ? 2 : 0;
   std::get<3>(key) = (int)(g_sparse.load() * 16 + g_sparse_fuse.load());
   std::get<4>(key) = P->block_rows;
   std::get<5>(key) = g_region_bytes.load();
@@ -357,7 +358,7 @@ std::shared_ptr<const RowSplit> get_split(uf_tree *tree, const BatchJob &J, cons
   auto it = tree->splits.find(key);
   if (it != tree->splits.end()) return it->second;
   if (tree->splits.size() >= 16) tree->splits.clear();
-  auto sp = std::make_shared<const RowSplit>(split_rows(tree, J, P, acc, fp32));
+  auto sp = std::make_shared<const RowSplit>(split_rows(tree, J, P, acc, fp32, fixed));
   tree->splits.emplace(key, sp);
   return sp;
 }

@@ -18,7 +18,9 @@
 // point, and its kernel (k_stripe_u64) adds R = sum max(x_j - x_k, 0) in
 // integers, A = 2 R + D_k - D_j: GB300 has 2 FP64 lanes per clock per SM but
 // 64 integer ones, and integer sums are exact, so the only rounding is that
-// of a row's value to the grid, and no difference of two sums cancels.  Generalized UniFrac keeps two
+// of a row's value to the grid, and no difference of two sums cancels.  Where
+// that grid is too coarse for some sample's branches (grid_need) the rows are
+// FP64 values, all in the abs form.  Generalized UniFrac keeps two
 // accumulators, den = sum l s^a and, FP32, Q = sum l min(u, v) s^(a-1) with
 // num = den - 2Q or, FP64, N = sum l |u - v| s^(a-1) = num.
 //
@@ -220,12 +222,11 @@ __device__ __forceinline__ void commit_cells(unsigned long long *M, const Mid *m
   }
 }
 
-// ---- weighted / unweighted, FP32 ----
+// ---- weighted / unweighted on FP32 and FP64 rows ----
 // rows i of the micro-tile with bit i of ABSM clear: M += min(x_k, x_j);
-// with it set: A += |x_k - x_j|
-template <int RD, int RK, int TX, unsigned ABSM, int MINB>
+// with it set: A += |x_k - x_j| (FP64: every row)
+template <typename T, int RD, int RK, int TX, unsigned ABSM, int MINB>
 __global__ void __launch_bounds__(TX *TX, MINB) k_stripe_min(const StripeArgs a) {
-  using T = float;
   using G = Geo<T, RD, RK, 1, TX>;
   constexpr int NT = G::NT;
   using Mid = typename G::Mid;
@@ -279,24 +280,34 @@ __global__ void __launch_bounds__(TX *TX, MINB) k_stripe_min(const StripeArgs a)
         for (int q = 0; q < G::NV; q++)
           *reinterpret_cast<uint4 *>(&v[q * G::VEC]) =
               *reinterpret_cast<const uint4 *>(vrow + swz<T>(w0 + q * G::VEC));
+        if constexpr (sizeof(T) == 8) {
+          // two FP64 instructions per update on 2 lanes per clock per SM bound
+          // it: 2.6e11 updates/s
+          static_assert(ABSM == FP64_ABS_ROW_MASK);
 #pragma unroll
-        for (int i = 0; i < RD; i++)
+          for (int i = 0; i < RD; i++)
 #pragma unroll
-          for (int j = 0; j < RK; j += 2) {
-            if (!((ABSM >> i) & 1u)) {  // two mins, one paired add
-              float2 a2 = make_float2(acc[i][j], acc[i][j + 1]);
-              const float2 m2 = make_float2(fminf(u[j], v[i + j + 1]), fminf(u[j + 1], v[i + j + 2]));
-              a2 = __fadd2_rn(a2, m2);
-              acc[i][j] = a2.x;
-              acc[i][j + 1] = a2.y;
-            } else {  // one paired difference, one paired add of absolute values
-              const float2 d2 = fsub2(make_float2(u[j], u[j + 1]), make_float2(v[i + j + 1], v[i + j + 2]));
-              float2 a2 = make_float2(acc[i][j], acc[i][j + 1]);
-              a2 = __fadd2_rn(a2, make_float2(fabsf(d2.x), fabsf(d2.y)));
-              acc[i][j] = a2.x;
-              acc[i][j + 1] = a2.y;
+            for (int j = 0; j < RK; j++) acc[i][j] += fabs(u[j] - v[i + j + 1]);
+        } else {
+#pragma unroll
+          for (int i = 0; i < RD; i++)
+#pragma unroll
+            for (int j = 0; j < RK; j += 2) {
+              if (!((ABSM >> i) & 1u)) {  // two mins, one paired add
+                float2 a2 = make_float2(acc[i][j], acc[i][j + 1]);
+                const float2 m2 = make_float2(fminf(u[j], v[i + j + 1]), fminf(u[j + 1], v[i + j + 2]));
+                a2 = __fadd2_rn(a2, m2);
+                acc[i][j] = a2.x;
+                acc[i][j + 1] = a2.y;
+              } else {  // one paired difference, one paired add of absolute values
+                const float2 d2 = fsub2(make_float2(u[j], u[j + 1]), make_float2(v[i + j + 1], v[i + j + 2]));
+                float2 a2 = make_float2(acc[i][j], acc[i][j + 1]);
+                a2 = __fadd2_rn(a2, make_float2(fabsf(d2.x), fabsf(d2.y)));
+                acc[i][j] = a2.x;
+                acc[i][j + 1] = a2.y;
+              }
             }
-          }
+        }
       }
       in_sub += G::RB;
       if (in_sub == B1 || it == nst - 1) {
@@ -315,7 +326,7 @@ __global__ void __launch_bounds__(TX *TX, MINB) k_stripe_min(const StripeArgs a)
   }
 }
 
-// ---- weighted / unweighted, FP64: 64-bit fixed-point rows ----
+// ---- weighted / unweighted, FP64 on 64-bit fixed-point rows ----
 // c += max(v - u, 0) for u, v < 2^63: a 64-bit difference, a test of its sign
 // and a predicated 64-bit add, 5 integer instructions.
 __device__ __forceinline__ void add_relu(unsigned long long &c, unsigned long long u, unsigned long long v) {
@@ -721,37 +732,41 @@ __device__ __forceinline__ int table_of_col(const TabDesc *tabs, int n_tabs, int
   return lo;
 }
 
-__global__ void k_diag_partial(const StripeArgs a, float *__restrict__ part) {
+template <typename T>
+__global__ void k_diag_partial(const StripeArgs a, T *__restrict__ part) {
   const int kg = blockIdx.x * blockDim.x + threadIdx.x;
   if (kg >= a.n_cols) return;
   const TabDesc &tb = a.tabs[a.n_tabs == 1 ? 0 : table_of_col(a.tabs, a.n_tabs, kg)];
   const int64_t k = tb.x_col + (kg - tb.off);  // the sample's column in its segment
   const int sb = blockIdx.y;
-  const float *X = (const float *)a.X;
+  const T *X = (const T *)a.X;
   const int per_chunk = (a.chunk + B1 - 1) / B1;
   const int c = sb / per_chunk;
   const int e0 = c * a.chunk + (sb - c * per_chunk) * B1;
   const int e1 = min(min(a.rows, (c + 1) * a.chunk), e0 + B1);
-  float acc = 0.f;
+  T acc = T(0);
   for (int e = e0; e < e1; e++) {
-    const float x = X[(int64_t)e * a.pitch + k];
-    acc += fminf(x, x);
+    const T x = X[(int64_t)e * a.pitch + k];
+    acc += tmin<T>(x, x);
   }
   part[(int64_t)sb * a.n_cols + kg] = acc;
 }
 
-// Phase 2: a chunk's sub-block partials summed in order in FP32, then rounded
-// to fixed point (the stripe kernels' second level); blockIdx.y is the chunk,
-// whose integers add in any order.
-__global__ void k_diag_reduce(const StripeArgs a, const float *__restrict__ part, int n_sb) {
+// Phase 2: a chunk's sub-block partials summed in order in the rows' precision,
+// then rounded to fixed point (the stripe kernels' second level); blockIdx.y is
+// the chunk, whose integers add in any order.
+template <typename T>
+__global__ void k_diag_reduce(const StripeArgs a, const T *__restrict__ part, int n_sb) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= a.n_cols) return;
   const int per_chunk = (a.chunk + B1 - 1) / B1;
   const int sb0 = blockIdx.y * per_chunk, sb1 = min(n_sb, sb0 + per_chunk);
-  float mid = 0.f;
+  T mid = T(0);
 #pragma unroll 8
   for (int sb = sb0; sb < sb1; sb++) mid += part[(int64_t)sb * a.n_cols + k];
-  atomicAdd(a.Dg + k, (unsigned long long)to_fixed(mid, a.scale));
+  const Fx2 d = to_fixed2(mid, a.scale);
+  atomicAdd(a.Dg + k, (unsigned long long)d.hi);
+  if constexpr (sizeof(T) == 8) atomicAdd(a.Dg + k + a.d_lo_off, (unsigned long long)d.lo);
 }
 
 // FP64: the fixed-point rows' sums, each value split into its two words
@@ -795,9 +810,9 @@ cudaError_t run_units(K kernel, int threads, size_t smem, const StripeArgs &a, c
   return launch_k(kernel, dim3(grid), dim3(threads), smem, st, a);
 }
 
-template <int RD, int RK, int TX, unsigned ABSM, int MINB>
+template <typename T, int RD, int RK, int TX, unsigned ABSM, int MINB>
 cudaError_t run_min(const StripeArgs &a, cudaStream_t st) {
-  return run_units(k_stripe_min<RD, RK, TX, ABSM, MINB>, TX * TX, Geo<float, RD, RK, 1, TX>::SMEM, a, st);
+  return run_units(k_stripe_min<T, RD, RK, TX, ABSM, MINB>, TX * TX, Geo<T, RD, RK, 1, TX>::SMEM, a, st);
 }
 template <int RD, int RK, int TX, int MINB>
 cudaError_t run_u64(const StripeArgs &a, cudaStream_t st) {
@@ -834,8 +849,9 @@ int stripe_shapes(int acc, bool fp32, unsigned abs_mask) {
 
 int stripe_chunk_rows() { return 2048; }
 
-SmallPlan stripe_small_plan(int acc, bool fp32, const int *n, size_t n_tabs, int rows, int chunk,
+SmallPlan stripe_small_plan(int acc, bool fp32, bool fixed, const int *n, size_t n_tabs, int rows, int chunk,
                             int shape, bool shape_free, int sms) {
+  const bool fp64 = !fp32 && !fixed;  // bound by the FP64 pipe
   auto tiles_of = [&](int sh, int64_t *cells) {
     int ts = 0, tk = 0;
     stripe_tile_shape(acc, fp32, &ts, &tk, sh);
@@ -849,9 +865,9 @@ SmallPlan stripe_small_plan(int acc, bool fp32, const int *n, size_t n_tabs, int
   int64_t tiles = tiles_of(shape, &cells);
   const int small = stripe_small_shape(acc, fp32);
   if (shape_free && shape != small) {
-    // the small tiles stage twice the bytes per update; FP64 generalized and
-    // variance-adjusted updates are bound by the FP64 pipe either way
-    const double rate = !fp32 && acc != ACC_MIN ? 1.0 : 0.85;
+    // the small tiles stage twice the bytes per update; updates on FP64 rows
+    // are bound by the FP64 pipe either way
+    const double rate = fp64 ? 1.0 : 0.85;
     int64_t cells_s = 0;
     const int64_t tiles_s = tiles_of(small, &cells_s);
     if ((double)cells_s < rate * (double)cells) {
@@ -859,16 +875,17 @@ SmallPlan stripe_small_plan(int acc, bool fp32, const int *n, size_t n_tabs, int
       tiles = tiles_s;
     }
   }
-  // units in flight: CTAs of 256 threads run two per SM (FP64 generalized and
-  // variance-adjusted: one), the small ones eight
-  const int64_t slots = (int64_t)sms * (p.shape == small ? 8 : (!fp32 && acc != ACC_MIN ? 1 : 2)), want = 4 * slots;
+  // units in flight: CTAs of 256 threads run two per SM (FP64 rows: one), the
+  // small ones eight
+  const int64_t slots = (int64_t)sms * (p.shape == small ? 8 : fp64 ? 1 : 2), want = 4 * slots;
   // kernels whose chunk is tuned are cut only where the smallest candidate
   // leaves under two waves (1,003 samples generalized, three waves of tuned
   // units: cut to four they took 2 % longer)
-  const bool tuned = fp32 || acc != ACC_MIN;
+  const bool tuned = !fixed;
   const int64_t least = tuned ? std::min(chunk, 1024) : chunk;
   if (tiles > 0 && tiles * ((rows + least - 1) / least) < (tuned ? 2 * slots : want)) {
-    const int step = acc == ACC_MIN && fp32 ? B1 : 16;
+    // (launch_diag's sub-blocks of B1 rows restart at every chunk)
+    const int step = acc == ACC_MIN && !fixed ? B1 : 16;
     const int64_t c = ((int64_t)rows * tiles / want + step) / step * step;
     p.chunk = (int)std::min<int64_t>(chunk, std::max<int64_t>(c, step));
     p.split = true;
@@ -879,12 +896,15 @@ SmallPlan stripe_small_plan(int acc, bool fp32, const int *n, size_t n_tabs, int
 cudaError_t launch_stripe_acc(int acc, bool fp32, const StripeArgs &a, cudaStream_t st) {
   if (a.rows <= 0 || a.n_tiles <= 0) return cudaSuccess;
   if (acc == ACC_MIN) {
-    if (!fp32) return a.shape == 1 ? run_u64<4, 8, 8, 8>(a, st) : run_u64<4, 8, 16, 2>(a, st);
+    if (!fp32 && a.fixed) return a.shape == 1 ? run_u64<4, 8, 8, 8>(a, st) : run_u64<4, 8, 16, 2>(a, st);
+    if (!fp32)
+      return a.shape == 1 ? run_min<double, 4, 8, 8, FP64_ABS_ROW_MASK, 4>(a, st)
+                          : run_min<double, 4, 8, 16, FP64_ABS_ROW_MASK, 1>(a, st);
     if (a.abs_mask == 0xFFu)
-      return a.shape == 2 ? run_min<4, 8, 8, 0xFFu, 8>(a, st) : run_min<8, 8, 16, 0xFFu, 2>(a, st);
-    if (a.shape == 2) return run_min<4, 8, 8, FP32_ABS_ROW_MASK, 8>(a, st);
-    return a.shape == 1 ? run_min<4, 8, 16, FP32_ABS_ROW_MASK, 3>(a, st)
-                        : run_min<8, 8, 16, FP32_ABS_ROW_MASK, 2>(a, st);
+      return a.shape == 2 ? run_min<float, 4, 8, 8, 0xFFu, 8>(a, st) : run_min<float, 8, 8, 16, 0xFFu, 2>(a, st);
+    if (a.shape == 2) return run_min<float, 4, 8, 8, FP32_ABS_ROW_MASK, 8>(a, st);
+    return a.shape == 1 ? run_min<float, 4, 8, 16, FP32_ABS_ROW_MASK, 3>(a, st)
+                        : run_min<float, 8, 8, 16, FP32_ABS_ROW_MASK, 2>(a, st);
   }
   const bool small = a.shape == 1;
   if (acc == ACC_VAW) {
@@ -900,24 +920,27 @@ cudaError_t launch_stripe_acc(int acc, bool fp32, const StripeArgs &a, cudaStrea
   return half ? run_gen<double, 4, 8, 16, 0, 1>(a, st) : run_gen<double, 4, 8, 16, 1, 1>(a, st);
 }
 
-size_t diag_scratch_bytes(bool fp32, int rows, int n_cols) {
-  if (!fp32) return 0;
+size_t diag_scratch_bytes(bool fp32, bool fixed, int rows, int n_cols) {
+  if (fixed) return 0;
   // one sub-block of B1 rows after another (chunks are multiples of B1)
   const int64_t n_sb = (rows + B1 - 1) / B1;
-  return (size_t)std::max<int64_t>(n_sb, 1) * n_cols * 4;
+  return (size_t)std::max<int64_t>(n_sb, 1) * n_cols * (fp32 ? 4 : 8);
 }
 
 cudaError_t launch_diag(bool fp32, const StripeArgs &a, void *scratch, cudaStream_t st) {
   if (a.rows <= 0) return cudaSuccess;
   const int gx = (a.n_cols + 127) / 128;
-  if (!fp32)
+  if (a.fixed)
     return launch_k(k_diag_u64, dim3(gx, (a.rows + DIAG_ROWS - 1) / DIAG_ROWS), dim3(128), 0, st, a);
   const int per_chunk = (a.chunk + B1 - 1) / B1;
   const int n_chunks = (a.rows + a.chunk - 1) / a.chunk;
   const int n_sb = (n_chunks - 1) * per_chunk + ((a.rows - (n_chunks - 1) * a.chunk) + B1 - 1) / B1;
-  const cudaError_t e = launch_k(k_diag_partial, dim3(gx, n_sb), dim3(128), 0, st, a, (float *)scratch);
-  if (e != cudaSuccess) return e;
-  return launch_k(k_diag_reduce, dim3(gx, n_chunks), dim3(128), 0, st, a, (const float *)scratch, n_sb);
+  auto both = [&](auto partial, auto reduce, auto *part) {
+    const cudaError_t e = launch_k(partial, dim3(gx, n_sb), dim3(128), 0, st, a, part);
+    return e != cudaSuccess ? e : launch_k(reduce, dim3(gx, n_chunks), dim3(128), 0, st, a, part, n_sb);
+  };
+  return fp32 ? both(k_diag_partial<float>, k_diag_reduce<float>, (float *)scratch)
+              : both(k_diag_partial<double>, k_diag_reduce<double>, (double *)scratch);
 }
 
 }  // namespace ufg
