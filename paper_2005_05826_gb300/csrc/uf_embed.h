@@ -62,6 +62,9 @@ cudaError_t launch_embed(int kind, bool fp32, const EmbedArgs &a, const int *lev
 // row of fewer repeats its head so often that a launch over rows
 // (launch_emb_rows) is faster than a thread per column.
 constexpr int EMBED_MIN_SAMPLES = 32;
+// It forms FP64 quotients from a total's reciprocal, which has to be a normal
+// number; a table with another total takes launch_emb_rows, which divides.
+inline bool plain_total(double t) { return t > 1e-290 && t < 1e290; }
 // Embedding rows of branches nodes[0 .. rows) (b0 .. b0 + rows - 1 when
 // nodes is null) for every table segment; EMB_VAW rows hold three planes of
 // `pitch` elements each, l p, c and T - c (a node list is required).  With

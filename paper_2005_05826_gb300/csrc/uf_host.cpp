@@ -798,6 +798,7 @@ uf_status uf_table_create(int64_t n_samples, int64_t n_features, const int64_t *
     for (int c = 1; c < T; c++) most_of(sums[c], &sums[0]);
     t->sums[tree->id] = sums[0];
     t->min_count = *std::min_element(cmin.begin(), cmin.end());
+    t->plain_totals = std::all_of(t->total.begin(), t->total.end(), plain_total);
     // each thread's column counts (a counting sort) and, below, its scatter
     // run over feature blocks: a sample's entries are sorted by feature, so
     // each block's entries of a sample are the run after the previous

@@ -272,7 +272,8 @@ uf_status compute_noalloc(const uf_tree *tree, const uf_table *table, uf_method 
     ea.length = (const double *)p[0];
     ea.total = (const double *)p[9];
     ea.inv_total_f = (const float *)p[10];
-    ea.X = n >= EMBED_MIN_SAMPLES ? p[12] : nullptr;
+    const bool in_slab = n >= EMBED_MIN_SAMPLES && (fp32 || std::all_of(xv.total, xv.total + n, plain_total));
+    ea.X = in_slab ? p[12] : nullptr;
     ea.pitch = pitch;
     ea.tabs = (const TabDesc *)p[18];
     ea.n_tabs = 1;

@@ -1370,7 +1370,9 @@ uf_status run_stripes(uf_tree *tree, const BatchJob &J, int device, uf_method me
     launch_sparse(ss);
     timer.end();
   }
-  const bool rows_in_slab = *std::min_element(ns.begin(), ns.end()) >= EMBED_MIN_SAMPLES;
+  const bool rows_in_slab =
+      *std::min_element(ns.begin(), ns.end()) >= EMBED_MIN_SAMPLES &&
+      (fp32 || std::all_of(J.tabs.begin(), J.tabs.end(), [](const TableJob &t) { return t.table->plain_totals; }));
   bool tuned = false;
   for (size_t b = 0; b < in.P->b0.size(); b++) {
     const int64_t b0 = in.P->b0[b];

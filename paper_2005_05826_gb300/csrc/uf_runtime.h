@@ -225,6 +225,7 @@ struct uf_table {
   };
   std::map<uint64_t, Sums> sums;
   double min_count = 1.0;                     // the smallest count of the table
+  bool plain_totals = true;                   // every total in plain_total()'s range (uf_embed.h)
   struct Dev {
     char *base = nullptr;  // one allocation holding the arrays below
     double *total = nullptr, *col_val = nullptr;
