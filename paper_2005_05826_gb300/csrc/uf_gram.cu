@@ -403,7 +403,9 @@ __global__ void __launch_bounds__(256) k_gram_prep(const int32_t *__restrict__ n
   constexpr int NT = DIGITS ? GRAM_DIGITS : GRAM_SPLITS;
   __shared__ uint32_t mask[GK];
   __shared__ __align__(16) __nv_bfloat16 term[1 + NT][GK];
-  const int e_base = blockIdx.x * GK, k_base = blockIdx.y * 32;  // a table's rows start at multiples of 256
+  // (one grid dimension: more than 65,535 blocks of plane rows or of branches may be asked for)
+  const int n_eb = (rows + GK - 1) / GK, kb = blockIdx.x / n_eb;
+  const int e_base = (blockIdx.x - kb * n_eb) * GK, k_base = kb * 32;  // a table's rows start at multiples of 256
   if (threadIdx.x < GK) {
     const int e = e_base + threadIdx.x;
     const GramTab &tb = tabs[n_tabs == 1 ? 0 : gram_table_of_row(tabs, n_tabs, k_base)];
@@ -638,10 +640,10 @@ void gram_tiles(int n, int64_t s0, int64_t s1, std::vector<int32_t> *bi, std::ve
 cudaError_t launch_gram_prep(const int32_t *nodes, int rows, const int32_t *slot_of_node, const uint32_t *bits,
                              int64_t words, const double *length, const GramTab *tabs, int n_tabs, int npad_tot,
                              int64_t K_pad, void *Pl, double digit_scale, cudaStream_t st) {
-  // K_pad is a multiple of GK, npad_tot of 256
+  // K_pad is a multiple of GK, npad_tot of 256 (the planes' bytes keep the blocks below 2^31)
   return launch_k(digit_scale != 0.0 ? k_gram_prep<true> : k_gram_prep<false>,
-                  dim3((rows + GK - 1) / GK, npad_tot / 32), dim3(256), 0, st, nodes, rows, slot_of_node, bits, words,
-                  length, tabs, n_tabs, npad_tot, K_pad, (__nv_bfloat16 *)Pl, digit_scale);
+                  dim3((unsigned)((int64_t)((rows + GK - 1) / GK) * (npad_tot / 32))), dim3(256), 0, st, nodes, rows,
+                  slot_of_node, bits, words, length, tabs, n_tabs, npad_tot, K_pad, (__nv_bfloat16 *)Pl, digit_scale);
 }
 
 cudaError_t launch_gram(const GramArgs &a0, void *Pl, int64_t K_pad, cudaStream_t st) {

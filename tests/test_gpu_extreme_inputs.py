@@ -1,5 +1,6 @@
 """FP64 calls at the ends of what the handles accept: sample totals so small
-that their reciprocal overflows, and branches of nearly the largest FP64 value."""
+that their reciprocal overflows, branches of nearly the largest FP64 value, and
+more jobs in a call than 65,535 blocks of 32 plane rows hold."""
 import numpy as np
 import pytest
 
@@ -62,3 +63,22 @@ def test_a_branch_of_any_length_that_no_sample_has(n, tensor):
     uf.uf_set_option("tensor_path", tensor)
     check(tree_s, STable.from_dense(counts), ["weighted_normalized", "weighted_unnormalized", "unweighted"],
           f"n={n} absent branch of 1.5e308")
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_many_jobs_on_the_tensor_cores(precision):
+    tree_s = yule_tree(40, seed=2320)
+    tree = uf.Tree(tree_s.parent, tree_s.length)
+    tables, exp = [], []
+    for s in range(3):
+        t = table_iid(2 + s, 40, 0.3, seed=2321 + s)
+        tables.append(uf.Table(t.indptr, t.indices, t.data, tree))
+        exp.append(oracle.condensed(tree_s, t, "unweighted"))
+    jobs = [(tables[q % 3], 0, tables[q % 3].n_samples // 2) for q in range(8200)]
+    outs, reps = uf.uf_compute_ranges(tree, jobs, "unweighted", 1.0, precision)
+    assert reps[0].path == 1
+    for q in (0, 1, 2, 4095, 8191, 8192, 8197, 8198, 8199):
+        assert_close(outs[q], exp[q % 3], "unweighted", precision, f"job {q}")
+    for s in range(3):
+        got = np.stack([np.asarray(o) for o in outs[s::3]])
+        assert (got == got[0]).all()
