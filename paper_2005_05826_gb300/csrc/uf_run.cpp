@@ -674,7 +674,7 @@ struct SparseScatter {
     n_cols = call_cols;
     const size_t nt = J.tabs.size();
     if (sp.n_sparse == 0) return;
-    const int64_t n_regions = (int64_t)sparse_regions(nt, acc, (double)cells * 8.0 * n_acc * (two_word ? 2 : 1));
+    const int64_t n_regions = (int64_t)sparse_regions(J, (double)cells * 8.0 * n_acc * (two_word ? 2 : 1));
     std::vector<int32_t> all;
     tiles = want_tiles && prepare_tiles(tree, J, sp, &all, meta, st);
     region_mode = !tiles && (n_regions > 1 || sp.lists);
@@ -699,7 +699,7 @@ struct SparseScatter {
       le = DevBuf(total_e * sparse_entry_bytes(!fp64_entries, fuse_m, acc, pres), st, "alloc sparse lists");
       lk = DevBuf(total_e * 4, st, "alloc sparse lists");
       // (cursors from one region to the next)
-      if (region_stripes(g_region_bytes.load()) <= (int64_t)lay[0].s_hi - lay[0].s_lo)
+      if (region_stripes(J.region_bytes) <= (int64_t)lay[0].s_hi - lay[0].s_lo)
         cur = DevBuf(total_e * 2 * sizeof(uint16_t), st, "alloc sparse list cursors");
       lz = DevBuf(std::max<size_t>(rows.size(), 1) * 4, st, "alloc sparse lists");
       // rows without entries in the table return before writing their count
@@ -993,7 +993,7 @@ uf_status run_gram(uf_tree *tree, const BatchJob &J, int device, double scale) {
     sp.M = Msp.as<unsigned long long>();
     sp.alpha = 1.0;
     sp.scale = scale;
-    sc.launch(meta, in, sp, ACC_MIN, true, g_region_bytes.load(), sms, ss, &kernels);
+    sc.launch(meta, in, sp, ACC_MIN, true, J.region_bytes, sms, ss, &kernels);
     timer.end();
   }
   for (size_t b = 0; b < in.P->b0.size(); b++) {
@@ -1355,7 +1355,7 @@ uf_status run_stripes(uf_tree *tree, const BatchJob &J, int device, uf_method me
       sp.x_shift = fixed_row_shift(scale, acc_most, &acc_most, 1, 1);
       sp.row_scale = std::ldexp(scale, sp.x_shift);
     }
-    sc.launch(meta, in, sp, acc, !fp32, g_region_bytes.load(), sms, on, &kernels);
+    sc.launch(meta, in, sp, acc, !fp32, J.region_bytes, sms, on, &kernels);
   };
   // with option "sparse_overlap" (default) the sparse-row scatter runs on a
   // side branch beside the count pass, the embeddings and the dense stripe

@@ -38,7 +38,7 @@ namespace rt {
 extern thread_local std::string g_err;   // uf_last_error() text of this thread
 extern thread_local double g_h2d;        // bytes the current call uploaded
 extern std::atomic<int64_t> g_branch_block, g_kernel_timing, g_tensor_path, g_graph, g_autotune, g_sparse, g_overlap,
-    g_tensor_wait_test, g_tile_shape, g_sparse_fuse;
+    g_tensor_wait_test, g_tile_shape, g_sparse_fuse, g_region_bytes;
 
 // Sets the thread's error text and returns st.
 uf_status fail(uf_status st, const char *fmt, ...);
@@ -293,6 +293,10 @@ struct BatchJob {
   int out_is_device, out_fp32;
   cudaStream_t st;
   std::vector<TableJob> tabs;
+  // options that several steps of the call go by, as they are when it starts
+  // (another thread may set them meanwhile): "sparse", "sparse_fuse",
+  // "sparse_region_bytes"
+  int64_t sparse = g_sparse.load(), fuse = g_sparse_fuse.load(), region_bytes = g_region_bytes.load();
 };
 
 // Branches of a call split between the dense stripe kernels and the
@@ -339,12 +343,11 @@ const RegionLists &region_lists(const uf_tree *tree, const uf_table *table, cons
 // exceed the L2 budget scatters region by region (launch_sparse_region) so
 // that every region's cells stay in L2; otherwise one region.
 constexpr double SPARSE_REGION_BYTES_DEFAULT = 48e6;
-extern std::atomic<int64_t> g_region_bytes;
 // Fewest samples of a table whose FP32 scatter goes through (fused) lists when its accumulators fit in L2.
 constexpr int64_t LIST_MIN_SAMPLES = 512;
 // split and region path: ACC_MIN or ACC_GEN (CUDA-core stripe kernels) or SPLIT_GRAM (tensor cores)
 constexpr int SPLIT_GRAM = 2;
-double sparse_regions(size_t n_tables, int acc, double acc_bytes);
+double sparse_regions(const BatchJob &J, double acc_bytes);
 // Whether a call's scatter runs in shared-memory tiles (uf_sparse.cu): FP64
 // weighted methods with `fixed` rows (the dense kernel's 64-bit grid) on one table of
 // TILE_MIN_SAMPLES (fewer make too few tiles) to TILE_MAX_SAMPLES (more leave

@@ -7,9 +7,9 @@
 namespace ufg {
 namespace rt {
 
-double sparse_regions(size_t n_tables, int acc, double acc_bytes) {
-  const double budget = (double)g_region_bytes.load();
-  if (n_tables != 1 || acc_bytes <= budget) return 1.0;
+double sparse_regions(const BatchJob &J, double acc_bytes) {
+  const double budget = (double)J.region_bytes;
+  if (J.tabs.size() != 1 || acc_bytes <= budget) return 1.0;
   return std::ceil(acc_bytes / budget);
 }
 
@@ -33,7 +33,7 @@ namespace {
 RowSplit split_rows(const uf_tree *tree, const BatchJob &J, const Plan *P, int acc, bool fp32, bool fixed) {
   RowSplit R;
   // the variance-adjusted method has no pair-scatter form: every branch dense
-  const int mode = acc == ACC_VAW ? 0 : (int)g_sparse.load();
+  const int mode = acc == ACC_VAW ? 0 : (int)J.sparse;
   const int64_t nb = tree->n_nodes - 1;
   const size_t nt = J.tabs.size();
   constexpr int NC = 6;
@@ -54,7 +54,7 @@ RowSplit split_rows(const uf_tree *tree, const BatchJob &J, const Plan *P, int a
     // accumulators beyond L2: one table scatters region by region in L2
     // (sparse_regions), several tables scatter straight into HBM-resident cells
     const bool tiles = tile_scatter(J, acc, fixed);
-    const bool regions = !tiles && sparse_regions(nt, acc, cells * 8.0 * n_acc) > 1;
+    const bool regions = !tiles && sparse_regions(J, cells * 8.0 * n_acc) > 1;
     // FP32 terms of one table go through lists even when its accumulators fit
     // in L2: a fused list's pair is one atomic (generalized: two) for three
     // branches, and the atomics bound the scatter (2,048 samples weighted 4.73 ->
@@ -62,13 +62,13 @@ RowSplit split_rows(const uf_tree *tree, const BatchJob &J, const Plan *P, int a
     const bool listed =
         nt == 1 && (acc == ACC_MIN || acc == ACC_GEN) && fp32 && J.tabs[0].table->n >= LIST_MIN_SAMPLES;
     R.lists = regions || tiles || listed;
-    R.fuse = (int)(acc == ACC_GEN ? std::min<int64_t>(g_sparse_fuse.load(), 2) : g_sparse_fuse.load());
+    R.fuse = (int)(acc == ACC_GEN ? std::min<int64_t>(J.fuse, 2) : J.fuse);
     // list mode keeps only sort keys in shared memory: longer runs fit
     const int64_t max_entries = R.lists ? SPARSE_LIST_MAX_ENTRIES : SPARSE_MAX_ENTRIES;
     // the scatter runs table by table (its grid's y is the table), so each
     // table's atomics hit L2 when that table's accumulators fit there
     std::vector<double> pair_cost(nt), entry_cost(nt);
-    const double n_regions = regions ? sparse_regions(nt, acc, cells * 8.0 * n_acc) : 1.0;
+    const double n_regions = regions ? sparse_regions(J, cells * 8.0 * n_acc) : 1.0;
     double dense_rate;  // cell updates per second of the dense kernel
     if (acc == SPLIT_GRAM) dense_rate = fp32 ? 2.5e14 : 2.5e14 * GRAM_SPLITS / GRAM_DIGITS;
     else dense_rate = fp32 ? (acc == ACC_GEN ? 4e12 : 1.3e13) : (acc == ACC_GEN ? 5e10 : fixed ? 3.5e12 : 2e11);
@@ -351,9 +351,9 @@ std::shared_ptr<const RowSplit> get_split(uf_tree *tree, const BatchJob &J, cons
   for (const TableJob &t : J.tabs) std::get<0>(key).push_back(t.table->id);
   std::get<1>(key) = acc + (tile_scatter(J, acc, fixed) ? 16 : 0);
   std::get<2>(key) = fp32 ? 1 : fixed ? 2 : 0;
-  std::get<3>(key) = (int)(g_sparse.load() * 16 + g_sparse_fuse.load());
+  std::get<3>(key) = (int)(J.sparse * 16 + J.fuse);
   std::get<4>(key) = P->block_rows;
-  std::get<5>(key) = g_region_bytes.load();
+  std::get<5>(key) = J.region_bytes;
   std::lock_guard<std::mutex> g(tree->mu);
   auto it = tree->splits.find(key);
   if (it != tree->splits.end()) return it->second;
