@@ -653,9 +653,9 @@ struct SparseScatter {
     all->insert(all->end(), listed.begin(), listed.end());
     le = DevBuf((size_t)std::max<int64_t>(entries, 1) * sizeof(TileEnt), st, "alloc sparse lists");
     toff = DevBuf((size_t)(stride * blocks) * 2, st, "alloc list offsets");
-    // per row its place and length, then the running total of entries
-    lz = DevBuf((size_t)(2 * stride + 1) * 4, st, "alloc sparse lists");
-    ck(cudaMemsetAsync(lz.p, 0, (size_t)(2 * stride + 1) * 4, st), "memset");
+    // the running total of entries, then per row its place
+    lz = DevBuf((size_t)(stride + 1) * 4, st, "alloc sparse lists");
+    ck(cudaMemsetAsync(lz.p, 0, 4, st), "memset");
     n_win = (int)win.size();
     o_win = meta.add(win);
     return true;
@@ -771,9 +771,8 @@ struct SparseScatter {
       const int64_t stride = round_up(n_tile_rows, 32);
       SparseArgs sp = base;
       sp.le = le.p;
-      sp.pos = lz.as<uint32_t>();
-      sp.lz = (int *)(sp.pos + stride);
-      sp.total = sp.pos + 2 * stride;
+      sp.total = lz.as<uint32_t>();
+      sp.pos = sp.total + 1;
       sp.off = toff.as<uint16_t>();
       sp.off_stride = stride;
       sp.n_blocks = (lay[0].n + TILE_I - 1) / TILE_I;
@@ -789,7 +788,6 @@ struct SparseScatter {
       TileArgs ta{};
       ta.ent = le.as<TileEnt>();
       ta.pos = sp.pos;
-      ta.z = sp.lz;
       ta.off = toff.as<uint16_t>();
       ta.n_rows = (int)n_tile_rows;
       ta.stride = stride;

@@ -668,8 +668,14 @@ __global__ void __launch_bounds__(256) k_tile_lists(const SparseArgs a) {
   const SpTab tb = a.tabs[0];
   const int64_t q0 = tb.col_ptr[a.tip_lo[v]];
   const int L = (int)(tb.col_ptr[a.tip_hi[v]] - q0);
-  if (L <= 0 || L > a.cap) return;  // the host sizes cap to every run and z starts at 0
   const int tid = threadIdx.x, NT = blockDim.x;
+  // the host lists no empty row and sizes cap to every run; such a row would have
+  // no pairs, and the scatter reads its offsets
+  if (L <= 0 || L > a.cap) {
+    for (int b = tid; b <= a.n_blocks; b += NT) a.off[b * a.off_stride + row] = 0;
+    if (tid == 0) a.pos[row] = 0;
+    return;
+  }
   int P2 = 1;
   while (P2 < L) P2 <<= 1;
   for (int i = tid; i < P2; i += NT)
@@ -701,7 +707,6 @@ __global__ void __launch_bounds__(256) k_tile_lists(const SparseArgs a) {
   if (tid == 0) {
     s_pos = atomicAdd(a.total, (uint32_t)z);
     a.pos[row] = s_pos;
-    a.lz[row] = z;
   }
   __syncthreads();
   TileEnt *le = reinterpret_cast<TileEnt *>(a.le) + s_pos;

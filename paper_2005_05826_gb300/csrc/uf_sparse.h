@@ -93,9 +93,8 @@ struct TileWin {
   int tile0, a_lo, a_n, b_lo, b_n, pad;
 };
 struct TileArgs {
-  const TileEnt *ent;       // the rows' entries in ascending sample, row r's from pos[r] on, z[r] of them
+  const TileEnt *ent;       // the rows' entries in ascending sample, row r's from pos[r] on
   const uint32_t *pos;
-  const int *z;
   const uint16_t *off;      // off[b * stride + r]: entries of row r with a sample below b TILE_I
   int n_rows;
   int64_t stride;           // n_rows rounded up to 32
@@ -111,7 +110,7 @@ struct TileArgs {
 int64_t tile_windows(int n, int s_lo, int s_hi, std::vector<TileWin> *win);
 cudaError_t launch_tile_scatter(const TileArgs &a, cudaStream_t st);
 // List mode of the tile scatter: rows nodes[0 .. n_nodes) write their entries
-// where *total places them (pos and z at row_base + row), and their terms to Dsp
+// where *total places them (pos at row_base + row), and their terms to Dsp
 cudaError_t launch_tile_lists(const SparseArgs &a, cudaStream_t st);
 // largest subtree entry count a sparse row may have: scattered directly from
 // shared memory, or written as a list (one table, keys alone in shared memory)
