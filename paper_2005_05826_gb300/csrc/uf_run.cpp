@@ -606,22 +606,13 @@ struct SparseScatter {
   size_t o_win = 0;
   DevBuf toff;
 
-  // Places the rows of at least `least` entries in the tile scatter's lists
-  // (after the others, class by class) and allocates its buffers; false when
-  // they do not fit the memory at hand.
-  bool prepare_tiles(uf_tree *tree, const BatchJob &J, const RowSplit &sp, std::vector<int32_t> *all, Meta &meta,
+  // Places the rows of at least tile_least() entries in the tile scatter's lists
+  // (after the others, class by class) and allocates its buffers.
+  void prepare_tiles(uf_tree *tree, const BatchJob &J, const RowSplit &sp, std::vector<int32_t> *all, Meta &meta,
                      cudaStream_t st) {
     std::vector<TileWin> win;
     n_tiles = tile_windows(lay[0].n, lay[0].s_lo, lay[0].s_hi, &win);
-    if (n_tiles > INT32_MAX / 2) return false;
-    // a listed row costs a look at its offsets per tile, a direct one an atomic
-    // per pair: both over the full stripe range, so that a range call splits
-    // the rows as the full run does (FP64 lists have a grid of their own)
-    const double n = lay[0].n, full = 0.5 * n * n;
-    const double rate = full * 16.0 <= 64e6 ? 1.15e11 : 1.25e10;
-    const double row_cost = full / (TILE_I * TILE_J) * 4e-13;
-    const int64_t least = std::max<int64_t>(SPARSE_SMALL_ENTRIES + 1,
-                                            std::min<int64_t>(1024, (int64_t)std::sqrt(2.0 * rate * row_cost)));
+    const int64_t least = tile_least(lay[0].n);
     const auto &cp = J.tabs[0].table->col_ptr;
     std::vector<int32_t> listed;
     int64_t entries = 0;
@@ -642,13 +633,6 @@ struct SparseScatter {
     }
     n_tile_rows = (int64_t)listed.size();
     const int64_t stride = round_up(std::max<int64_t>(n_tile_rows, 1), 32), blocks = (lay[0].n + TILE_I - 1) / TILE_I + 1;
-    const double need = (double)entries * sizeof(TileEnt) + (double)stride * blocks * 2.0;
-    if (entries >= (int64_t)UINT32_MAX || (need > 64e6 && need > 0.25 * available_bytes())) {
-      sp_off.clear();
-      cls_n.clear();
-      all->clear();
-      return false;
-    }
     for (int64_t &o : tile_off) o += (int64_t)all->size();
     all->insert(all->end(), listed.begin(), listed.end());
     le = DevBuf((size_t)std::max<int64_t>(entries, 1) * sizeof(TileEnt), st, "alloc sparse lists");
@@ -658,14 +642,13 @@ struct SparseScatter {
     ck(cudaMemsetAsync(lz.p, 0, 4, st), "memset");
     n_win = (int)win.size();
     o_win = meta.add(win);
-    return true;
   }
 
-  // acc: ACC_MIN / ACC_GEN; fp64_entries: terms computed in FP64; want_tiles:
-  // the tile scatter where it fits; presence: the rows hold presence terms
+  // acc: ACC_MIN / ACC_GEN; fp64_entries: terms computed in FP64; in_tiles:
+  // the tile scatter; presence: the rows hold presence terms
   void prepare(uf_tree *tree, const BatchJob &J, const Inputs &in, const RowSplit &sp,
                const std::vector<SpLayout> &layout, int acc, bool fp64_entries, bool two_words,
-               int64_t call_cells, int64_t call_cols, bool want_tiles, bool presence, Meta &meta, cudaStream_t st) {
+               int64_t call_cells, int64_t call_cols, bool in_tiles, bool presence, Meta &meta, cudaStream_t st) {
     split = &sp;
     lay = layout;
     two_word = two_words;
@@ -676,7 +659,8 @@ struct SparseScatter {
     if (sp.n_sparse == 0) return;
     const int64_t n_regions = (int64_t)sparse_regions(J, (double)cells * 8.0 * n_acc * (two_word ? 2 : 1));
     std::vector<int32_t> all;
-    tiles = want_tiles && prepare_tiles(tree, J, sp, &all, meta, st);
+    tiles = in_tiles;
+    if (tiles) prepare_tiles(tree, J, sp, &all, meta, st);
     region_mode = !tiles && (n_regions > 1 || sp.lists);
     pres = presence;
     fuse_m = region_mode ? sp.fuse : 0;
@@ -909,7 +893,7 @@ uf_status run_gram(uf_tree *tree, const BatchJob &J, int device, double scale) {
   }();
   const std::shared_ptr<const RowSplit> split_p = [&] {
     NvtxRange r("uf: branch split");
-    return get_split(tree, J, in.P, SPLIT_GRAM, J.fp32, false);
+    return get_split(tree, J, in.P, SPLIT_GRAM, J.fp32, false, true);
   }();
   const RowSplit &split = *split_p;
   const int64_t K_pad = gram_kpad((int)std::max<int64_t>(split.max_dense, 1));
@@ -1205,9 +1189,13 @@ uf_status run_stripes(uf_tree *tree, const BatchJob &J, int device, uf_method me
     return bind_inputs(tree, J, device, rows);
   }();
   cudaStream_t st = J.st;
+  // (lists past a quarter of the memory at hand: scattered without them)
+  bool may_list = true;
   const std::shared_ptr<const RowSplit> split_p = [&] {
     NvtxRange r("uf: branch split");
-    return get_split(tree, J, in.P, acc, fp32, fixed_rows);
+    std::shared_ptr<const RowSplit> sp = get_split(tree, J, in.P, acc, fp32, fixed_rows, true);
+    may_list = !(sp->list_bytes > 64e6 && sp->list_bytes > 0.25 * available_bytes());
+    return may_list ? sp : get_split(tree, J, in.P, acc, fp32, fixed_rows, false);
   }();
   const RowSplit &split = *split_p;
   const int64_t xrows = std::max<int64_t>(split.max_dense, 1);
@@ -1256,8 +1244,8 @@ uf_status run_stripes(uf_tree *tree, const BatchJob &J, int device, uf_method me
   std::vector<SpLayout> lay(nt);
   for (size_t t = 0; t < nt; t++) lay[t] = SpLayout{tabs[t].n, tabs[t].off, tabs[t].s_lo, tabs[t].s_hi, tabs[t].m_off};
   SparseScatter sc;
-  sc.prepare(tree, J, in, split, lay, acc, !fp32, !fp32, cells, n_cols, tile_scatter(J, acc, fixed_rows), kind == EMB_PRESENCE,
-             meta, st);
+  sc.prepare(tree, J, in, split, lay, acc, !fp32, !fp32, cells, n_cols, may_list && tile_scatter(J, acc, fixed_rows),
+             kind == EMB_PRESENCE, meta, st);
   meta.upload(st);
   const TabDesc *d_tabs = meta.at<TabDesc>(o_tabs);
   const int32_t *d_cnt = meta.at<int32_t>(o_cnt);

@@ -318,6 +318,9 @@ struct RowSplit {
   std::vector<std::vector<int32_t>> sparse;  // sparse branch nodes by capacity class
   std::vector<int> cap;             // shared-memory entries of each class
   bool lists = false;               // sample lists: stripe regions, tiles, or FP32 rows of one table
+  // device bytes of lists that the call can do without (tiles, FP32 rows whose
+  // accumulators fit L2): get_split's may_list
+  double list_bytes = 0.0;
   int64_t n_sparse = 0;
   double pairs = 0.0;               // both-nonzero pairs scattered, at most (sum over tables)
   int64_t max_dense = 0;            // most dense rows in one block
@@ -354,12 +357,15 @@ double sparse_regions(const BatchJob &J, double acc_bytes);
 // few of a row's samples in a tile) samples
 constexpr int64_t TILE_MIN_SAMPLES = 512, TILE_MAX_SAMPLES = 4096;
 bool tile_scatter(const BatchJob &J, int acc, bool fixed);
+// Fewest entries of a row that the tiles of an n-sample table take.
+int64_t tile_least(int64_t n);
 
 
 // The split of a call, cached on the tree (uf_split.cpp); fixed: its FP64 rows
-// are 64-bit fixed point (StripeArgs::fixed).
+// are 64-bit fixed point (StripeArgs::fixed); may_list: lists where they are
+// faster, else only where the accumulators are scattered region by region.
 std::shared_ptr<const RowSplit> get_split(uf_tree *tree, const BatchJob &J, const Plan *P, int acc, bool fp32,
-                                          bool fixed);
+                                          bool fixed, bool may_list);
 
 // Runs one compute call on the current device (uf_run.cpp); throws CudaFail.
 uf_status run_batch(uf_tree *tree, const BatchJob &J);

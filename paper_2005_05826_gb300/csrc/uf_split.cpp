@@ -19,6 +19,17 @@ bool tile_scatter(const BatchJob &J, int acc, bool fixed) {
   return n >= TILE_MIN_SAMPLES && n <= TILE_MAX_SAMPLES;
 }
 
+int64_t tile_least(int64_t n) {
+  // a listed row costs a look at its offsets per tile, a direct one an atomic
+  // per pair: both over the full stripe range, so that a range call splits
+  // the rows as the full run does (FP64 lists have a grid of their own)
+  const double full = 0.5 * (double)n * (double)n;
+  const double rate = full * 16.0 <= 64e6 ? 1.15e11 : 1.25e10;
+  const double row_cost = full / (TILE_I * TILE_J) * 4e-13;
+  return std::max<int64_t>(SPARSE_SMALL_ENTRIES + 1,
+                           std::min<int64_t>(1024, (int64_t)std::sqrt(2.0 * rate * row_cost)));
+}
+
 namespace {
 
 // Per branch v the count entries of table t under v are the CSC run of v's
@@ -30,10 +41,13 @@ namespace {
 // scatters every branch that fits; mode 0 none.  The choice depends on the
 // tree and the tables only, not on the stripe range, so that a range run
 // gives bitwise the stripes of the full run.
-RowSplit split_rows(const uf_tree *tree, const BatchJob &J, const Plan *P, int acc, bool fp32, bool fixed) {
+RowSplit split_rows(const uf_tree *tree, const BatchJob &J, const Plan *P, int acc, bool fp32, bool fixed,
+                    bool may_list) {
   RowSplit R;
+  const bool tiles = may_list && tile_scatter(J, acc, fixed);
   // the variance-adjusted method has no pair-scatter form: every branch dense
   const int mode = acc == ACC_VAW ? 0 : (int)J.sparse;
+  bool can_do_without = false;  // the lists other than tiles
   const int64_t nb = tree->n_nodes - 1;
   const size_t nt = J.tabs.size();
   constexpr int NC = 6;
@@ -53,14 +67,13 @@ RowSplit split_rows(const uf_tree *tree, const BatchJob &J, const Plan *P, int a
     }
     // accumulators beyond L2: one table scatters region by region in L2
     // (sparse_regions), several tables scatter straight into HBM-resident cells
-    const bool tiles = tile_scatter(J, acc, fixed);
     const bool regions = !tiles && sparse_regions(J, cells * 8.0 * n_acc) > 1;
     // FP32 terms of one table go through lists even when its accumulators fit
     // in L2: a fused list's pair is one atomic (generalized: two) for three
     // branches, and the atomics bound the scatter (2,048 samples weighted 4.73 ->
     // 4.29 ms a call, 1,003 generalized 3.13 -> 2.94)
     const bool listed =
-        nt == 1 && (acc == ACC_MIN || acc == ACC_GEN) && fp32 && J.tabs[0].table->n >= LIST_MIN_SAMPLES;
+        may_list && nt == 1 && (acc == ACC_MIN || acc == ACC_GEN) && fp32 && J.tabs[0].table->n >= LIST_MIN_SAMPLES;
     R.lists = regions || tiles || listed;
     R.fuse = (int)(acc == ACC_GEN ? std::min<int64_t>(J.fuse, 2) : J.fuse);
     // list mode keeps only sort keys in shared memory: longer runs fit
@@ -92,6 +105,7 @@ RowSplit split_rows(const uf_tree *tree, const BatchJob &J, const Plan *P, int a
         entry_cost[t] = 3e-11;
       }
     }
+    const int64_t least = tiles ? tile_least(J.tabs[0].table->n) : 0;
     // a row's offsets read by every tile
     const double tile_cost = tiles ? cells / (TILE_I * TILE_J) * 4e-13 : 0.0;
     // a dense row also costs its count row and embedding (or planes) in HBM
@@ -101,7 +115,7 @@ RowSplit split_rows(const uf_tree *tree, const BatchJob &J, const Plan *P, int a
     // their double sums are exact in any order)
     struct Part {
       std::vector<int32_t> cls[NC];
-      int64_t n_sparse = 0;
+      int64_t n_sparse = 0, tile_rows = 0, tile_entries = 0;
       double pairs = 0.0;
     };
     const int T = (int)std::max<int64_t>(1, std::min<int64_t>(host_threads(), nb / 16384));
@@ -143,15 +157,28 @@ RowSplit split_rows(const uf_tree *tree, const BatchJob &J, const Plan *P, int a
           pt.cls[k].push_back((int32_t)v);
           pt.n_sparse++;
           pt.pairs += pairs;
+          if (tiles && mx >= least) {
+            pt.tile_rows++;
+            pt.tile_entries += mx;
+          }
         }
       }
     });
     for (int k = 0; k < NC; k++)
       for (const Part &pt : part) R.sparse[k].insert(R.sparse[k].end(), pt.cls[k].begin(), pt.cls[k].end());
+    int64_t tile_rows = 0, tile_entries = 0;
     for (const Part &pt : part) {
       R.n_sparse += pt.n_sparse;
       R.pairs += pt.pairs;
+      tile_rows += pt.tile_rows;
+      tile_entries += pt.tile_entries;
     }
+    if (tiles)  // (their places are 32-bit)
+      R.list_bytes = tile_entries >= (int64_t)UINT32_MAX
+                         ? INFINITY
+                         : (double)tile_entries * sizeof(TileEnt) +
+                               (double)(tile_rows + 31) * (J.tabs[0].table->n / TILE_I + 2) * sizeof(uint16_t);
+    can_do_without = listed && !regions;
   }
   auto count_rows = [&] {
     const int64_t root = tree->n_nodes - 1;
@@ -217,7 +244,7 @@ RowSplit split_rows(const uf_tree *tree, const BatchJob &J, const Plan *P, int a
   };
   // the lists of the scattered branches (a table's tiles make their own), of
   // the count rows and of the dense rows side by side: none needs another
-  const bool lists = R.lists && R.n_sparse > 0 && !tile_scatter(J, acc, fixed);
+  const bool lists = R.lists && R.n_sparse > 0 && !tiles;
   auto part = [&](int c) {
     if (c == 0 && lists) region_lists(tree, J.tabs[0].table, R);
     if (c == 1) count_rows();
@@ -226,6 +253,9 @@ RowSplit split_rows(const uf_tree *tree, const BatchJob &J, const Plan *P, int a
   if (nb >= 16384) parallel_for(3, part);
   else
     for (int c = 0; c < 3; c++) part(c);
+  if (lists && can_do_without)
+    R.list_bytes = (double)R.region->entry_off.back() *
+                   (double)(sparse_entry_bytes(fp32, R.fuse, acc, kind_of(J.method) == EMB_PRESENCE) + sizeof(int));
   R.cnt_xrow.resize(R.cnt_lists.size());
   for (size_t q = 0; q < R.cnt_lists.size(); q++) {
     const int32_t v = R.cnt_lists[q];
@@ -346,10 +376,10 @@ const RegionLists &region_lists(const uf_tree *tree, const uf_table *table, cons
 // The split of a call, cached on the tree by its tables and kind (tables are
 // immutable and their ids are never reused).
 std::shared_ptr<const RowSplit> get_split(uf_tree *tree, const BatchJob &J, const Plan *P, int acc, bool fp32,
-                                          bool fixed) {
+                                          bool fixed, bool may_list) {
   SplitKey key;
   for (const TableJob &t : J.tabs) std::get<0>(key).push_back(t.table->id);
-  std::get<1>(key) = acc + (tile_scatter(J, acc, fixed) ? 16 : 0);
+  std::get<1>(key) = acc + (tile_scatter(J, acc, fixed) ? 16 : 0) + (may_list ? 0 : 32);
   std::get<2>(key) = fp32 ? 1 : fixed ? 2 : 0;
   std::get<3>(key) = (int)(J.sparse * 16 + J.fuse);
   std::get<4>(key) = P->block_rows;
@@ -358,7 +388,7 @@ std::shared_ptr<const RowSplit> get_split(uf_tree *tree, const BatchJob &J, cons
   auto it = tree->splits.find(key);
   if (it != tree->splits.end()) return it->second;
   if (tree->splits.size() >= 16) tree->splits.clear();
-  auto sp = std::make_shared<const RowSplit>(split_rows(tree, J, P, acc, fp32, fixed));
+  auto sp = std::make_shared<const RowSplit>(split_rows(tree, J, P, acc, fp32, fixed, may_list));
   tree->splits.emplace(key, sp);
   return sp;
 }
