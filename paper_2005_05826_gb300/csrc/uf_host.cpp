@@ -373,34 +373,28 @@ namespace {
 
 // One sample's tips, for uf_table::Sums.
 struct SampleSum {
-  double dist = 0.0, val_dist = 0.0, length = 0.0, depth = 0.0, low = INFINITY, top = 0.0;
+  double dist = 0.0, val_dist = 0.0, length = 0.0;
   void add(double val, const uf_tree::Tip &t) {
     dist += t.dist;
     val_dist += val * t.dist;
     length += t.length;
-    depth += t.depth;
-    low = std::min(low, t.dist);
-    top = std::max(top, t.dist);
   }
   void add(const SampleSum &o) {
     dist += o.dist;
     val_dist += o.val_dist;
     length += o.length;
-    depth += o.depth;
-    low = std::min(low, o.low);
-    top = std::max(top, o.top);
   }
-  void close(double total, const uf_tree *tree, uf_table::Sums *m) const {
-    // D is a mean of the tips' distances: between the nearest's and the
-    // farthest's, which stand for it where its products leave FP64's range
-    const bool ok = total > 1e-200 && total < 1e200 && top < 1e100;
-    const double d = ok ? std::min(val_dist / total, top) : low, w = std::max(top, length);
-    const double b = std::sqrt(std::min(depth, (double)(tree->n_nodes - 1)));
+  void close(int64_t n_tips, double total, const uf_tree *tree, uf_table::Sums *m) const {
     m->presence = std::max(m->presence, dist);
-    m->weighted = std::max(m->weighted, ok ? d : top);
-    // (a sample whose branches are all of length 0 holds exact zeros)
-    if (top > 0.0) m->need_weighted = std::max(m->need_weighted, d > 0.0 ? b / d : INFINITY);
-    if (w > 0.0) m->need_presence = std::max(m->need_presence, b / w);
+    if (!(dist > 0.0)) return;  // branches of length 0 alone: exact zeros
+    // (counts or lengths whose products may leave FP64's range: not summed)
+    const bool ok = total > 1e-200 && total < 1e200 && dist < 1e100;
+    const double d = ok ? std::min(val_dist / total, tree->max_tip_dist) : 0.0;
+    m->weighted = std::max(m->weighted, ok ? d : tree->max_tip_dist);
+    const double b = std::sqrt(std::min((double)n_tips * tree->max_depth, (double)(tree->n_nodes - 1)));
+    m->need_weighted = std::max(m->need_weighted, d > 0.0 ? b / d : INFINITY);
+    // its farthest tip's path is among its branches, and so are all its tips' own
+    m->need_presence = std::max(m->need_presence, b / std::max(dist / (double)n_tips, length));
   }
 };
 void most_of(const uf_table::Sums &a, uf_table::Sums *m) {
@@ -425,16 +419,22 @@ uf_table::Sums table_sums(const uf_tree *tree, uf_table *table) {
       f_lo[c] = f;
     }
     std::vector<std::vector<SampleSum>> part(T, std::vector<SampleSum>(table->n));
+    std::vector<std::vector<int64_t>> tips(T, std::vector<int64_t>(table->n, 0));
     parallel_for(T, [&](int c) {
       SampleSum *per = part[c].data();
       for (int64_t f = f_lo[c]; f < f_lo[c + 1]; f++)
-        for (int64_t q = table->col_ptr[f]; q < table->col_ptr[f + 1]; q++)
+        for (int64_t q = table->col_ptr[f]; q < table->col_ptr[f + 1]; q++) {
           per[table->col_row[q]].add(table->col_val[q], tree->tips[f]);
+          tips[c][table->col_row[q]]++;
+        }
     });
     uf_table::Sums m;
     for (int64_t k = 0; k < table->n; k++) {
-      for (int c = 1; c < T; c++) part[0][k].add(part[c][k]);
-      part[0][k].close(table->total[k], tree, &m);
+      for (int c = 1; c < T; c++) {
+        part[0][k].add(part[c][k]);
+        tips[0][k] += tips[c][k];
+      }
+      part[0][k].close(tips[0][k], table->total[k], tree, &m);
     }
     it = table->sums.emplace(tree->id, m).first;
   }
@@ -690,24 +690,38 @@ uf_status uf_tree_create(int64_t n_nodes, const int64_t *parent, const double *l
       const int64_t p = parent[i];
       t->child_idx[t->child_ptr[p + 1] - nchild[p]--] = (int32_t)i;  // ascending child order
     }
-    // one pass in reverse order (parents first): root distances, the tips'
-    // distances, and the tip ranges that are not contiguous (both set to -1)
-    t->dist.assign(n_nodes, 0.0);
-    std::vector<int32_t> depth(n_nodes, 0);
+    // one pass in reverse order (parents first): root distances and depths, the
+    // tips' distances, and the tip ranges that are not contiguous (both set to -1)
+    struct FromRoot {
+      double dist;
+      int32_t depth;
+    };
+    std::vector<FromRoot, NoInit<FromRoot>> at(n_nodes);
     t->tips.resize(std::max<int32_t>(tips, 1));
+    double total = 0.0, longest = 0.0, farthest = 0.0;
+    int32_t deepest = 0;
     for (int64_t v = n_nodes - 1; v >= 0; v--) {
+      double l = 0.0;
+      FromRoot r{0.0, 0};
       if (v + 1 < n_nodes) {
-        t->dist[v] = t->length[v] + t->dist[parent[v]];
-        depth[v] = depth[parent[v]] + 1;
-        t->total_length += t->length[v];
-        t->max_length = std::max(t->max_length, t->length[v]);
+        l = t->length[v];
+        const FromRoot &up = at[parent[v]];
+        r = {l + up.dist, up.depth + 1};
+        total += l;
+        longest = std::max(longest, l);
       }
+      at[v] = r;
       if (t->tip_of_node[v] >= 0) {
-        t->max_tip_dist = std::max(t->max_tip_dist, t->dist[v]);
-        t->tips[t->tip_of_node[v]] = {t->dist[v], v + 1 < n_nodes ? t->length[v] : 0.0, (double)depth[v]};
+        farthest = std::max(farthest, r.dist);
+        deepest = std::max(deepest, r.depth);
+        t->tips[t->tip_of_node[v]] = {r.dist, l};
       }
       if ((int64_t)t->tip_hi[v] - t->tip_lo[v] != under[v]) t->tip_lo[v] = t->tip_hi[v] = -1;
     }
+    t->total_length = total;
+    t->max_length = longest;
+    t->max_tip_dist = farthest;
+    t->max_depth = deepest;
     *out = t.release();
     return UF_OK;
   } catch (const std::bad_alloc &) {
@@ -789,7 +803,7 @@ uf_status uf_table_create(int64_t n_samples, int64_t n_features, const int64_t *
         }
         t->total[k] = s;
         t->inv_total_f[k] = (float)(1.0 / s);
-        w.close(s, tree, &sums[c]);
+        w.close(indptr[k + 1] - indptr[k], s, tree, &sums[c]);
       }
     });
     for (int c = 0; c < T; c++)

@@ -182,13 +182,12 @@ struct uf_tree {
   std::map<int, Dev> dev;
   std::map<int64_t, std::unique_ptr<ufg::rt::Plan>> plans;  // by block rows
   std::map<ufg::rt::SplitKey, std::shared_ptr<const ufg::rt::RowSplit>> splits;  // dense / sparse branch splits
-  // root distance of every node (root: 0), max over tips, total branch length
-  std::vector<double> dist;
   struct Tip {
     double dist, length;  // from the root, and of its own branch
-    double depth;         // branches from the root
   };
   std::vector<Tip> tips;  // by tip number
+  int32_t max_depth = 0;  // most branches between a tip and the root
+  // the farthest tip's distance; every branch together; the longest
   double max_tip_dist = 0.0, total_length = 0.0, max_length = 0.0;
   ~uf_tree() {
     int cur = 0;
@@ -220,7 +219,7 @@ struct uf_table {
     double presence = 0.0;       // max_k sum_{f in k} dist(tip f)
     double weighted = 0.0;       // max_k D_k, D_k = sum_f p_kf dist(tip f)
     // max_k sqrt(branches below sample k) / D_k and the same over W_k, its
-    // branches' summed lengths, from below (grid_need)
+    // branches' summed lengths, both from above (grid_need)
     double need_weighted = 0.0, need_presence = 0.0;
   };
   std::map<uint64_t, Sums> sums;

@@ -105,7 +105,6 @@ RowSplit split_rows(const uf_tree *tree, const BatchJob &J, const Plan *P, int a
         entry_cost[t] = 3e-11;
       }
     }
-    const int64_t least = tiles ? tile_least(J.tabs[0].table->n) : 0;
     // a row's offsets read by every tile
     const double tile_cost = tiles ? cells / (TILE_I * TILE_J) * 4e-13 : 0.0;
     // a dense row also costs its count row and embedding (or planes) in HBM
@@ -115,7 +114,7 @@ RowSplit split_rows(const uf_tree *tree, const BatchJob &J, const Plan *P, int a
     // their double sums are exact in any order)
     struct Part {
       std::vector<int32_t> cls[NC];
-      int64_t n_sparse = 0, tile_rows = 0, tile_entries = 0;
+      int64_t n_sparse = 0;
       double pairs = 0.0;
     };
     const int T = (int)std::max<int64_t>(1, std::min<int64_t>(host_threads(), nb / 16384));
@@ -157,27 +156,29 @@ RowSplit split_rows(const uf_tree *tree, const BatchJob &J, const Plan *P, int a
           pt.cls[k].push_back((int32_t)v);
           pt.n_sparse++;
           pt.pairs += pairs;
-          if (tiles && mx >= least) {
-            pt.tile_rows++;
-            pt.tile_entries += mx;
-          }
         }
       }
     });
     for (int k = 0; k < NC; k++)
       for (const Part &pt : part) R.sparse[k].insert(R.sparse[k].end(), pt.cls[k].begin(), pt.cls[k].end());
-    int64_t tile_rows = 0, tile_entries = 0;
     for (const Part &pt : part) {
       R.n_sparse += pt.n_sparse;
       R.pairs += pt.pairs;
-      tile_rows += pt.tile_rows;
-      tile_entries += pt.tile_entries;
     }
-    if (tiles)  // (their places are 32-bit)
-      R.list_bytes = tile_entries >= (int64_t)UINT32_MAX
+    if (tiles) {
+      const auto &cp = J.tabs[0].table->col_ptr;
+      const int64_t n = J.tabs[0].table->n, least = tile_least(n);
+      int64_t rows = 0, entries = 0;
+      for (const auto &c : R.sparse)
+        for (int32_t v : c) {
+          const int64_t ub = cp[tree->tip_hi[v]] - cp[tree->tip_lo[v]];
+          rows += ub >= least;
+          entries += ub >= least ? ub : 0;
+        }
+      R.list_bytes = entries >= (int64_t)UINT32_MAX  // (their places are 32-bit)
                          ? INFINITY
-                         : (double)tile_entries * sizeof(TileEnt) +
-                               (double)(tile_rows + 31) * (J.tabs[0].table->n / TILE_I + 2) * sizeof(uint16_t);
+                         : (double)entries * sizeof(TileEnt) + (double)(rows + 31) * (n / TILE_I + 2) * sizeof(uint16_t);
+    }
     can_do_without = listed && !regions;
   }
   auto count_rows = [&] {
