@@ -135,8 +135,9 @@ typedef struct {
     double t_diag_ms;      /* diagonal accumulate launches */
     double t_finalize_ms;  /* finalize */
     int64_t acc_launches;  /* accumulate launches timed in t_accumulate_ms */
-    int64_t chunk_rows;    /* branches per accumulate work unit (autotuned; calls too
-                              small to fill the GPU cut a unit into shorter ones) */
+    int64_t chunk_rows;    /* branches per accumulate work unit, the longest of a call
+                              (CUDA cores: autotuned, and calls too small to fill the
+                              GPU cut a unit into shorter ones) */
     int32_t graph;         /* 1: the launch sequence ran as one CUDA graph */
     int32_t reserved2;
     int64_t dense_rows;    /* branches run through the dense stripe kernels */

@@ -30,6 +30,7 @@ constexpr int GRAM_PAIRS = (GRAM_DIGITS + 1) / 2;
 // A digit's sum over a unit is an integer of at most 256 x GRAM_DIGIT_KC:
 // below 2^23, so that FP32 accumulation is exact.
 constexpr int GRAM_DIGIT_KC = 16384;
+constexpr int GRAM_KC = 4096;  // branches per unit, mixed
 struct GramArgs {
   int digits;           // 1: FP64 (digit planes, exact sums), 0: mixed
   int k_len;            // branches of this block, rounded up to 64

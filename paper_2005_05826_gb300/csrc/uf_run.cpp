@@ -958,6 +958,7 @@ uf_status run_gram(uf_tree *tree, const BatchJob &J, int device, double scale) {
   }
   Outputs o = bind_outputs(J, st);
   double exec_flops = 0.0;
+  int64_t unit_rows = GRAM_KC;  // reported: the longest of any block
   Capture cap(g_graph.load() != 0 && !timer.on, st, device);
   const cudaStream_t ls = cap.stream();
   // the sparse-row scatters need no count rows or planes: first, on a side
@@ -1014,12 +1015,13 @@ uf_status run_gram(uf_tree *tree, const BatchJob &J, int device, double scale) {
     GramArgs ga{};
     ga.digits = digits;
     ga.k_len = (int)round_up(nd, 64);
-    ga.kc = 4096;
+    ga.kc = GRAM_KC;
     if (digits) {
       // the longest units (a drain per unit is not hidden) that still give
       // four waves of them
       const int64_t units = (int64_t)n_tiles * GRAM_PAIRS, want = 4 * (int64_t)sms;
       ga.kc = (int)std::min<int64_t>(GRAM_DIGIT_KC, std::max<int64_t>(512, round_up(ga.k_len * units / want, 64)));
+      unit_rows = std::max<int64_t>(acc_launches > 0 ? unit_rows : 0, ga.kc);
     }
     ga.gt_lo = digits ? gt_cells : 0;
     ga.digit_shift = digit_shift;
@@ -1100,7 +1102,7 @@ uf_status run_gram(uf_tree *tree, const BatchJob &J, int device, double scale) {
                GRAM_TM, std::chrono::duration<double>(std::chrono::steady_clock::now() - t_start).count());
   for (const TableJob &t : J.tabs)
     if (t.rep) {
-      t.rep->chunk_rows = 4096;
+      t.rep->chunk_rows = unit_rows;
       t.rep->graph = cap.on ? 1 : 0;
       t.rep->dense_rows = (int64_t)split.dense.size();
       t.rep->sparse_rows = split.n_sparse;

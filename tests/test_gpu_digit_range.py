@@ -82,7 +82,7 @@ def test_longest_units(lengths):
     table_s = STable(n, tips, np.asarray(indptr, dtype=np.int64), idx, np.ones(idx.size))
     h = handles(tree_s, table_s)
     got, rep = compute(h, 0, 1)
-    assert rep.dense_rows > 16_384
+    assert rep.chunk_rows == 16_384 and rep.dense_rows > 16_384
     i, j = np.triu_indices(n, k=1)
     q = rng.choice(i.size, 3000, replace=False)
     exp = oracle.pairs(tree_s, table_s, "unweighted", 1.0, i[q], j[q])[0]
