@@ -164,7 +164,8 @@ typedef struct {
  *                    diagonal tiles included)
  *                    and the sparse rows' stripe cells fit in half the device
  *                    memory that is free or held unused by the stream-ordered
- *                    pool, else on the CUDA-core stripe kernels
+ *                    pool (UF_FP64: and its grid of lengths holds every
+ *                    distance, see UF_FP64), else on the CUDA-core stripe kernels
  *                    (report path 0); 0: always on the CUDA-core kernels
  *   "graph"          1 (default): a call's branch-block launch sequence is
  *                    captured into a CUDA graph and launched as one graph

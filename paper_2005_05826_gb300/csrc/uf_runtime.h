@@ -345,15 +345,23 @@ const RegionLists &region_lists(const uf_tree *tree, const uf_table *table, cons
 // exceed the L2 budget scatters region by region (launch_sparse_region) so
 // that every region's cells stay in L2; otherwise one region.
 constexpr double SPARSE_REGION_BYTES_DEFAULT = 48e6;
-// Fewest samples of a table whose FP32 scatter goes through (fused) lists when its accumulators fit in L2.
+// Fewest samples of a table whose FP32 scatter goes through (fused) lists when its
+// accumulators fit in L2: fewer pairs a branch do not repay writing the lists.
+// Time of the direct scatter's call over the lists' (20,000 and 50,000 tips,
+// prevalence Beta(0.5, 20) and 1 %): weighted 0.85 - 0.90 at 96 samples, 0.91 -
+// 1.14 at 256, 0.98 - 1.16 at 512, 1.03 - 1.19 at 768; generalized 0.83 - 1.06,
+// 0.78 - 1.11, 0.94 - 1.06, 0.99 - 1.06.
 constexpr int64_t LIST_MIN_SAMPLES = 512;
 // split and region path: ACC_MIN or ACC_GEN (CUDA-core stripe kernels) or SPLIT_GRAM (tensor cores)
 constexpr int SPLIT_GRAM = 2;
 double sparse_regions(const BatchJob &J, double acc_bytes);
 // Whether a call's scatter runs in shared-memory tiles (uf_sparse.cu): FP64
 // weighted methods with `fixed` rows (the dense kernel's 64-bit grid) on one table of
-// TILE_MIN_SAMPLES (fewer make too few tiles) to TILE_MAX_SAMPLES (more leave
-// few of a row's samples in a tile) samples
+// TILE_MIN_SAMPLES (fewer make too few tiles) to TILE_MAX_SAMPLES samples.  Time of
+// the direct scatter's call over the tiles' on the same tables: 0.73 - 0.97 at 256
+// samples, 0.93 - 1.01 at 512, 1.08 - 1.35 at 768.  The upper line is no turning
+// point: over region lists the tiles gain 1.39 - 1.51 at 3,000 samples, 1.45 - 1.54
+// at 4,096 and 1.56 - 1.64 at 12,000.
 constexpr int64_t TILE_MIN_SAMPLES = 512, TILE_MAX_SAMPLES = 4096;
 bool tile_scatter(const BatchJob &J, int acc, bool fixed);
 // Fewest entries of a row that the tiles of an n-sample table take.

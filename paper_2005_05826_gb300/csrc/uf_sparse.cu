@@ -745,8 +745,8 @@ __global__ void __launch_bounds__(256) k_tile_lists(const SparseArgs a) {
 // accumulators once per tile.  Without tiles every pair was two 64-bit atomics
 // into L2, 1.5e11 pairs/s on 1,531 samples; here 4.2e11.  One-word FP32 terms are
 // one L2 atomic a pair, 2.3e11/s, and no faster in tiles (3.2e11/s less the
-// lists), and with 25,000 samples (8 pairs per row and tile) tiles are slower
-// than regions: tile_scatter() says which calls come here.
+// lists), and with 25,000 samples (8 pairs per row and tile) slower than in
+// regions: tile_scatter() says which calls come here.
 constexpr int TS_THREADS = 512, TS_WARPS = TS_THREADS / 32, TS_QUEUE = 64;
 constexpr size_t TS_SMEM = (size_t)TILE_I * TILE_J * 8 + (size_t)TS_WARPS * TS_QUEUE * sizeof(uint4);
 
