@@ -17,7 +17,7 @@
 // (the common 2^F cancels); weighted_unnormalized returns num * 2^-F.  FP64
 // accumulators have two words (uf_device.cuh); they are combined here into
 // one 128-bit integer in units of 2^-(F+32).
-// A ratio with den == 0 is 0.  An abs-form numerator is a sum of
+// A ratio with den == 0 is 0 (generalized in FP32: den at most gen_den_floor).  An abs-form numerator is a sum of
 // nonnegative integers and never negative; a min-form numerator (FP32 only)
 // can round a hair below 0 for two nearly identical samples and is then
 // raised to 0 (and counted when the caller asks).
@@ -25,6 +25,7 @@
 // diagonal is D + R, an abs-form cell gains R_k + R_j, and the generalized
 // den and N gain R_k + R_j.
 #include <algorithm>
+#include <cmath>
 
 #include "uf_internal.h"
 #include "uf_finalize.h"
@@ -109,7 +110,7 @@ __global__ void k_finalize(const FinalArgs a) {
         clamped++;
         num = 0;
       }
-      val = den > 0 ? to_double(num) / to_double(den) : 0.0;
+      val = den > (I)a.den_floor ? to_double(num) / to_double(den) : 0.0;
     } break;
     }
     if (a.unnormalized) val = to_double(num) * inv_scale;
@@ -124,6 +125,13 @@ __global__ void k_finalize(const FinalArgs a) {
     else ((double *)a.out)[idx] = val;
   }
   if (clamped && a.clamps) atomicAdd(a.clamps, clamped);
+}
+
+int64_t gen_den_floor(bool fp32, double alpha, double length, double scale, int64_t units) {
+  if (!fp32 || alpha != 0.5) return 0;  // (other alpha: an absent pair's terms are zeroed)
+  // (the kernel's FP32 sums and reciprocal square roots are within 1e-4)
+  const double most = length * std::sqrt(2e-30) * (1.0 + 1e-4) * scale + 0.5 * (double)units;
+  return most < 4e18 ? (int64_t)most + 1 : 0;
 }
 
 cudaError_t launch_finalize(const FinalArgs &a, cudaStream_t st) {

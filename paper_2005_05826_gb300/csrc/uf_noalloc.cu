@@ -318,6 +318,11 @@ uf_status compute_noalloc(const uf_tree *tree, const uf_table *table, uf_method 
   fa.abs_mask = amask;
   fa.relu = fixed_rows;
   fa.gen_abs = acc == ACC_GEN && !fp32;
+  if (acc == ACC_GEN) {
+    double length = 0.0;
+    for (int64_t v = 0; v < nb; v++) length += tv.length[v];
+    fa.den_floor = gen_den_floor(fp32, alpha, length, scale, (rows + plan.chunk - 1) / plan.chunk);
+  }
   fa.M = (const unsigned long long *)p[13];
   fa.M2 = (const unsigned long long *)p[14];
   fa.Dg = (const unsigned long long *)p[15];

@@ -1470,8 +1470,18 @@ uf_status run_stripes(uf_tree *tree, const BatchJob &J, int device, uf_method me
   }
   side.join();
   timer.begin(3);
+  int64_t den_floor = 0;
+  if (acc == ACC_GEN) {
+    double length = 0.0;
+    int64_t units = 0;
+    for (double l : split.dense_len) length += l;
+    for (size_t b = 0; b + 1 < split.dense_ptr.size(); b++)
+      units += (split.dense_ptr[b + 1] - split.dense_ptr[b] + unit_rows - 1) / unit_rows;
+    den_floor = gen_den_floor(fp32, J.alpha, length, scale, units);
+  }
   for (size_t t = 0; t < nt; t++) {
     FinalArgs fa{};
+    fa.den_floor = den_floor;
     fa.method = acc == ACC_MIN ? (kind == EMB_PRESENCE ? 0 : 2) : 3;
     fa.unnormalized = unnormalized(method);
     fa.n = tabs[t].n;
